@@ -497,19 +497,19 @@ def run_ours(args):
         return
     R = results[modes[0]]
     # Roofline of the secondary trace kernel (k_trace_bvh2): the algorithmic node + triangle
-    # bytes per secondary ray (32 ray + 4 queue + 8 hit + 64 per node visit + 48 per triangle
+    # bytes per secondary ray (32 ray + 4 queue + 8 hit + 32 per node visit + 48 per triangle
     # test, visits and tests from the counting pass) times the rays of one launch, over the
     # launch's CUDA-event time, against the measured HBM copy bandwidth (the headline) and
     # the measured L2 read roof.  Above the HBM roof means caches serve node fetches again
     # (coherence); the DRAM traffic the kernel really causes is the "traffic" key (ncu).
-    # ncu shows the kernel bound by instruction issue (7-8 active lanes per warp
-    # instruction), so the issue and FP32-ALU roofs are reported beside it.
+    # ncu shows the kernel bound by instruction issue and load latency, so the issue and
+    # FP32-ALU roofs are reported beside it.
     # With "+bvh8q" ("+bvh4") first, the figures describe k_trace_bvh8 (k_trace_bvh4) instead:
     # 80 B and 8 box tests (112 B and 4) per node visit, and no ncu-derived keys (the committed
     # summary is the BVH2 kernel's).
     layout0 = parse(modes[0])[3]
     plain = layout0 == cr.CR_BVH2
-    node_b = {cr.CR_BVH2: 64, cr.CR_BVH8Q: 80, cr.CR_BVH4: 112}
+    node_b = {cr.CR_BVH2: 32, cr.CR_BVH8Q: 80, cr.CR_BVH4: 112}
     boxes = {cr.CR_BVH2: 2, cr.CR_BVH8Q: 8, cr.CR_BVH4: 4}
     launches = BOUNCES
     n_sm = torch.cuda.get_device_properties(local).multi_processor_count  # cudaDevAttrMultiProcessorCount
@@ -524,6 +524,9 @@ def run_ours(args):
     clk = (clocks or {}).get("sm_mhz") or 2070.0
     peak_ops = n_sm * 128 * clk * 1e6 / 1e12
     bytes_per_ray = node_bytes_per_ray(R, layout0)
+    # secondary rays per second of closest-hit trace time (the committed instruction count covers
+    # the step's primary trace too)
+    closest_mrays = R["secondary_rays_per_step"] / ((R["ms_trace_primary"] + R["ms_trace_secondary"]) * 1e3)
     achieved = bytes_per_ray * rays_per_launch / (ms_per_launch / 1e3) / 1e9
     peak, peak_kind = load_peaks()
     traffic = profile_traffic() if plain else None
@@ -567,7 +570,7 @@ def run_ours(args):
                          "unit": "TOP/s (FP32 ALU operations)", "frac": round(achieved_ops / peak_ops, 4),
                          "ops_per_ray": round(ops_per_ray, 1),
                          "peak_source": f"{n_sm} SMs (device attribute) x 128 FP32 lanes x {clk:.0f} MHz (sampled)"},
-        "roofline_issue": issue_roof(R, clk, n_sm) if plain else None,
+        "roofline_issue": issue_roof({"trace_mrays": closest_mrays}, clk, n_sm) if plain else None,
         "roofline_l2": {"achieved": round(achieved, 1), "peak": round(l2_gbs, 1), "unit": "GB/s",
                         "frac": round(achieved / l2_gbs, 4),
                         "peak_source": "cr_measure_l2_read: read-only kernel over an L2-resident 48 MB buffer, CUDA events",
@@ -614,15 +617,16 @@ def run_ours(args):
 
 def trace_bytes_per_ray(nodes_per_ray: float, tris_per_ray: float, node_bytes: int = 64) -> float:
     """Algorithmic bytes one secondary ray moves through the trace kernel: its ray record
-    (32 B), the queue entry (4 B) and the hit (8 B), every node visited (64 B for a BVH2
-    node, 80 for BVH8-Q, 112 for BVH4) and every triangle tested (48 B)."""
+    (32 B), the queue entry (4 B) and the hit (8 B), every node visited (node_bytes: 32 for a
+    BVH2 record, 80 for BVH8-Q, 112 for BVH4) and every triangle tested (48 B)."""
     return 32 + 4 + 8 + node_bytes * nodes_per_ray + 48 * tris_per_ray
 
 
 def issue_roof(R, clk, n_sm):
     """The trace kernel's binding roof (ncu: issue-bound): warp instructions per second
     against one instruction per scheduler per clock (n_sm SMs x 4 schedulers).  Instructions
-    per ray come from the committed ncu capture; the ray rate is this run's."""
+    per secondary ray come from the committed ncu capture and cover all closest-hit launches of
+    a step; the ray rate (secondary rays per second of that trace time) is this run's."""
     ipr = profile_traffic("warp_instructions_per_ray")
     peak = n_sm * 4 * clk * 1e6 / 1e12
     if ipr is None:
@@ -630,7 +634,7 @@ def issue_roof(R, clk, n_sm):
     ach = ipr * R["trace_mrays"] * 1e6 / 1e12
     return {"achieved": round(ach, 3), "peak": round(peak, 3), "unit": "T warp instructions/s",
             "frac": round(ach / peak, 4), "instructions_per_ray": ipr,
-            "source": "warp instructions per ray from profiles/k_trace_bvh2.landscape.txt x this run's trace-only rate"}
+            "source": "warp instructions per ray from profiles/k_trace_bvh2.landscape.txt x this run's secondary rays per second of closest-hit trace time"}
 
 
 def l2_read_bandwidth(cr, mb=48, reps=100):

@@ -17,6 +17,7 @@
 #include <cstring>
 #include <functional>
 #include <mutex>
+#include <system_error>
 #include <thread>
 
 #include "cr_internal.h"
@@ -329,6 +330,84 @@ HostBVH2 build_bvh2(const float* v, uint32_t n_tri, int n_threads) {
 } // namespace cr
 
 // ------------------------------------------------------------------------------------
+// The BVH2 in the kernels' 32-byte records (DevBVH2).
+namespace cr {
+namespace {
+
+float bits_float(uint32_t b) {
+    float f;
+    std::memcpy(&f, &b, 4);
+    return f;
+}
+
+float plane_value(uint32_t q) { return bits_float(0x3f000000u | q << 8); }
+
+// The largest code whose plane lies at or below g, the smallest whose plane lies at or above it
+// (0.5 <= g < 2).
+uint32_t plane_below(double g) {
+    const double q = g < 1.0 ? (g - 0.5) * 65536.0 : 32768.0 + (g - 1.0) * 32768.0;
+    uint32_t c = (uint32_t)std::min(65535.0, std::max(0.0, std::floor(q)));
+    while (c > 0 && (double)plane_value(c) > g) --c;
+    return c;
+}
+uint32_t plane_above(double g) {
+    uint32_t c = plane_below(g);
+    while (c < 65535 && (double)plane_value(c) < g) ++c;
+    return c;
+}
+
+} // namespace
+
+DevBVH2 pack_bvh2(const HostBVH2& b, int n_threads) {
+    DevBVH2 out;
+    double big = 0.0, far = 0.0;
+    for (int k = 0; k < 3; ++k) {
+        big = std::max(big, (double)b.hi[k] - (double)b.lo[k]);
+        far = std::max(far, std::max(std::fabs((double)b.lo[k]), std::fabs((double)b.hi[k])));
+    }
+    for (int k = 0; k < 3; ++k) {
+        // a flat axis takes 2^-12 of the largest extent, a point a few units of its coordinates;
+        // a margin of at least 2^-11 on both sides keeps the enlarged boxes inside the grid
+        const double ext = std::max({(double)b.hi[k] - (double)b.lo[k], big * 0x1.0p-12, far * 0x1.0p-22, 1e-30});
+        const double want = (double)b.lo[k] - ext * 0x1.0p-11;
+        out.lo[k] = (float)want;
+        if ((double)out.lo[k] > want) out.lo[k] = std::nextafterf(out.lo[k], -INFINITY);
+        out.scale[k] = (float)std::min(1.498 / ((double)b.lo[k] + ext - (double)out.lo[k]), 1e30);
+    }
+    out.words.resize((size_t)kDevNode2Words * b.n_nodes);
+    auto run = [&](uint32_t first, uint32_t last) {
+        for (uint32_t i = first; i < last; ++i) {
+            const float* o = &b.nodes[16 * (size_t)i];
+            uint32_t* w = &out.words[(size_t)kDevNode2Words * i];
+            static const int at[3][2] = {{0, 4}, {2, 6}, {8, 10}}; // lower plane of (axis, child)
+            for (int c = 0; c < 2; ++c)
+                for (int a = 0; a < 3; ++a) {
+                    const double lo = 0.5 + ((double)o[at[a][c]] - (double)out.lo[a]) * (double)out.scale[a];
+                    const double hi = 0.5 + ((double)o[at[a][c] + 1] - (double)out.lo[a]) * (double)out.scale[a];
+                    w[3 * c + a] = plane_below(lo - kGridSlack) | plane_above(hi + kGridSlack) << 16;
+                }
+            std::memcpy(&w[6], &o[12], 4);
+            std::memcpy(&w[7], &o[13], 4);
+        }
+    };
+    const uint32_t nt = (uint32_t)std::max(1, std::min(n_threads, (int)(b.n_nodes / 16384u)));
+    std::vector<std::thread> th;
+    for (uint32_t t = 0; t < nt; ++t) {
+        const uint32_t first = (uint32_t)((uint64_t)b.n_nodes * t / nt), last = (uint32_t)((uint64_t)b.n_nodes * (t + 1) / nt);
+        try {
+            if (t + 1 == nt) run(first, last);
+            else th.emplace_back(run, first, last);
+        } catch (const std::system_error&) { // no thread to be had
+            run(first, last);
+        }
+    }
+    for (auto& t : th) t.join();
+    return out;
+}
+
+} // namespace cr
+
+// ------------------------------------------------------------------------------------
 // Host verification of the BVH2 (used by cr_debug_bvh_check).
 namespace cr {
 namespace {
@@ -384,6 +463,21 @@ void check_bvh2(const HostBVH2& b, const float* v, uint32_t n_tri, uint32_t& cov
             }
         }
     }
+    // the kernels' records: the same links, and boxes (as the kernels decode them) that contain
+    // each child box and kGridSlack around it
+    const DevBVH2 d = pack_bvh2(b, 2);
+    for (uint32_t i = 0; i < b.n_nodes; ++i)
+        for (int w = 0; w < 2; ++w) {
+            const Child2 c = child2_of(b, i, w);
+            const uint32_t* rec = &d.words[(size_t)kDevNode2Words * i];
+            if (rec[6 + w] != (uint32_t)c.link) ++violations;
+            for (int k = 0; k < 3; ++k) {
+                const double lo = 0.5 + ((double)c.lo[k] - (double)d.lo[k]) * (double)d.scale[k] - kGridSlack;
+                const double hi = 0.5 + ((double)c.hi[k] - (double)d.lo[k]) * (double)d.scale[k] + kGridSlack;
+                const uint32_t q = rec[3 * w + k];
+                if ((double)plane_value(q & 0xffffu) > lo || (double)plane_value(q >> 16) < hi) ++violations;
+            }
+        }
     covered = 0;
     for (uint32_t t = 0; t < n_tri; ++t) covered += seen[t] >= 1 ? 1u : 0u;
     // the root-leaf case emits the same triangles twice on purpose; count distinct coverage

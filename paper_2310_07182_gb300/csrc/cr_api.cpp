@@ -213,6 +213,12 @@ extern "C" cr_status cr_scene_create(const float* tri_xyz, uint32_t n_tri, const
     if (b2.depth >= kBvh2StackCapacity)
         return fail(CR_ERR_STACK_OVERFLOW, "cr_scene_create: BVH2 depth %u needs a deeper traversal stack (%u)", b2.depth,
                     kBvh2StackCapacity);
+    DevBVH2 d2;
+    try {
+        d2 = pack_bvh2(b2, hc ? (int)hc : 4);
+    } catch (const std::bad_alloc&) {
+        return fail(CR_ERR_OOM, "cr_scene_create: host allocation during BVH build");
+    }
     // triangles in leaf order: v0 | original index, v1 | material, v2 | 0
     std::vector<float> tris(12 * (size_t)n_tri);
     for (uint32_t i = 0; i < n_tri; ++i) {
@@ -301,10 +307,10 @@ extern "C" cr_status cr_scene_create(const float* tri_xyz, uint32_t n_tri, const
     }
     const auto t1 = std::chrono::steady_clock::now();
     DevMem dn, dt, dm;
-    CR_CUDA(dn.alloc(b2.nodes.size() * sizeof(float)));
+    CR_CUDA(dn.alloc(d2.words.size() * sizeof(uint32_t)));
     CR_CUDA(dt.alloc(tris.size() * sizeof(float)));
     CR_CUDA(dm.alloc(mt.size() * sizeof(float)));
-    CR_CUDA(cudaMemcpy(dn.p, b2.nodes.data(), dn.bytes, cudaMemcpyHostToDevice));
+    CR_CUDA(cudaMemcpy(dn.p, d2.words.data(), dn.bytes, cudaMemcpyHostToDevice));
     CR_CUDA(cudaMemcpy(dt.p, tris.data(), dt.bytes, cudaMemcpyHostToDevice));
     CR_CUDA(cudaMemcpy(dm.p, mt.data(), dm.bytes, cudaMemcpyHostToDevice));
     DevMem dn8, dt8;
@@ -345,7 +351,11 @@ extern "C" cr_status cr_scene_create(const float* tri_xyz, uint32_t n_tri, const
     s->dev.n_nodes4 = b4.n_nodes;
     s->dev.nodes8 = static_cast<const uint4*>(s->d_nodes8);
     s->dev.tris8 = static_cast<const float4*>(s->d_tris8);
-    s->dev.nodes2 = static_cast<const float4*>(s->d_nodes2);
+    s->dev.nodes2 = static_cast<const uint32_t*>(s->d_nodes2);
+    for (int k = 0; k < 3; ++k) {
+        s->dev.grid_lo[k] = d2.lo[k];
+        s->dev.grid_scale[k] = d2.scale[k];
+    }
     s->dev.tris = static_cast<const float4*>(s->d_tris);
     s->dev.mats = static_cast<const float4*>(s->d_mats);
     for (int k = 0; k < 3; ++k) {
@@ -377,7 +387,7 @@ extern "C" cr_status cr_scene_create(const float* tri_xyz, uint32_t n_tri, const
     s->info.n_nodes8 = b8.n_nodes;
     s->info.n_nodes4 = b4.n_nodes;
     s->info.depth4 = b4.depth;
-    s->info.device_bytes = b2.nodes.size() * 4 + tris.size() * 4 + mt.size() * 4 + b8.nodes.size() * 4 + tris8.size() * 4 +
+    s->info.device_bytes = d2.words.size() * 4 + tris.size() * 4 + mt.size() * 4 + b8.nodes.size() * 4 + tris8.size() * 4 +
                            b4.nodes.size() * 4 + lrec.size() * 4 + lcdf.size() * 4;
     s->info.n_lights = n_lights;
     s->info.light_area = s->dev.light_total;

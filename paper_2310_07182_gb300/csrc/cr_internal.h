@@ -28,6 +28,24 @@ struct HostBVH2 {
     float lo[3], hi[3];
 };
 
+// The BVH2 as the kernels read it: one 32-byte record per inner node, which a single 256-bit
+// load fetches (word w of the record = words[8 * node + w]):
+//   words 0-2  planes of child 0 along x, y, z: the lower plane's 16-bit code in the low half,
+//              the upper plane's in the high half;   words 3-5  those of child 1
+//   words 6, 7 links of child 0 and 1, as in HostBVH2
+// Coordinates are those of a per-scene grid, g = 0.5 + (x - lo) * scale per axis, which maps the
+// scene into [0.5, 2).  A code q is the float with the bits 0x3f000000 | q << 8 (steps of 2^-16
+// below 1 and 2^-15 above).  Lower planes are rounded down and upper planes up, so that the
+// record's box contains the exact child box and kGridSlack beyond it on every side.
+struct DevBVH2 {
+    std::vector<uint32_t> words; // 8 per inner node
+    float lo[3], scale[3];
+};
+// Boxes are enlarged by this much on every side (grid units); see grid_ray in trace_common.cuh.
+constexpr double kGridSlack = 0x1.0p-18;
+constexpr uint32_t kDevNode2Words = 8;
+DevBVH2 pack_bvh2(const HostBVH2& b, int n_threads);
+
 // SAH build (exact sweep up to 1024 triangles, 32 bins per axis above; SAH-chosen leaves
 // of <= 4 triangles; median splits below depth 40 so the depth stays <= 64).
 HostBVH2 build_bvh2(const float* tri_xyz, uint32_t n_tri, int n_threads);
@@ -78,7 +96,8 @@ void check_bvh8(const HostBVH8& b, const float* v, uint32_t n_tri, uint32_t& cov
 // ------------------------------------------------------------------------------------
 // Device-side scene description (host copy kept in the scene handle).
 struct DevScene {
-    const float4* nodes2 = nullptr; // 4 per node
+    const uint32_t* nodes2 = nullptr; // 8 words per node (DevBVH2)
+    float grid_lo[3] = {0, 0, 0}, grid_scale[3] = {1, 1, 1}; // grid of its boxes
     const uint4* nodes8 = nullptr;  // 5 per node
     const float4* nodes4 = nullptr; // 8 per node (BVH4, if built)
     const float4* tris = nullptr;   // 3 per triangle in leaf order: v0|orig, v1|mat, v2|0
@@ -98,7 +117,8 @@ struct DevScene {
 
 // One entry of the device scene table a pass reads (tris in the order of the BVH traversed).
 struct SceneDev {
-    const float4* nodes2;
+    const uint32_t* nodes2; // BVH2 records (DevBVH2) and the grid of their boxes
+    float grid_lo[3], grid_scale[3];
     const uint4* nodes8;
     const float4* nodes4; // BVH4 (with the BVH2's triangle records), or NULL
     const float4* tris;
@@ -184,9 +204,9 @@ struct LaunchCount {
 
 // Saved traversal of a ray suspended by the two-phase trace (128 bytes).
 struct TraceState {
-    int node, sp, leaf, orig;
+    int node, sp, leaf;
     float t;
-    int pad[3];
+    int pad[4];
     int stack[24];
 };
 // Buffers of the two-phase trace (per slot: state, flag; per queue entry: second queue).

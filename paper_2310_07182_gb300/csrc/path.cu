@@ -1092,41 +1092,44 @@ __global__ void __launch_bounds__(kCompactBlock) k_compact_scatter(const int32_t
 constexpr uint32_t kHcutLevels = 15;
 constexpr float kHcutLambda = 0.125f;
 
-__device__ __forceinline__ float box_dist2(float px, float py, float pz, float lox, float hix, float loy, float hiy,
-                                           float loz, float hiz) {
-    const float dx = fmaxf(fmaxf(lox - px, px - hix), 0.0f);
-    const float dy = fmaxf(fmaxf(loy - py, py - hiy), 0.0f);
-    const float dz = fmaxf(fmaxf(loz - pz, pz - hiz), 0.0f);
-    return dx * dx + dy * dy + dz * dz;
-}
-
 // Path bits of point p through the BVH2 (root = node 0): at each node the child whose box is
 // nearer to p (distance 0 inside), ties (p in both) to the child whose box centre is nearer;
-// levels below a leaf add zero bits.
-__device__ __forceinline__ uint32_t hcut_path(const float4* __restrict__ nodes, float px, float py, float pz) {
+// levels below a leaf add zero bits.  Boxes are the record's, in grid coordinates; each axis is
+// scaled back to the scene's units.
+__device__ __forceinline__ uint32_t hcut_path(const SceneDev& sc, float px, float py, float pz) {
     uint32_t code = 0;
     int node = 0;
+    const float p[3] = {px, py, pz};
+    float pg[3], inv[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        pg[k] = fmaf(p[k] - sc.grid_lo[k], sc.grid_scale[k], 0.5f);
+        inv[k] = 1.0f / sc.grid_scale[k];
+    }
     for (uint32_t l = 0; l < kHcutLevels; ++l) {
         code <<= 1;
         if (node < 0) continue;
-        const float4 n0 = __ldg(&nodes[4 * node + 0]);
-        const float4 n1 = __ldg(&nodes[4 * node + 1]);
-        const float4 n2 = __ldg(&nodes[4 * node + 2]);
-        const float4 n3 = __ldg(&nodes[4 * node + 3]);
-        const float d0 = box_dist2(px, py, pz, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y);
-        const float d1 = box_dist2(px, py, pz, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w);
-        bool right;
-        if (d0 != d1) {
-            right = d1 < d0;
-        } else {
-            const float c0 = box_dist2(px, py, pz, 0.5f * (n0.x + n0.y), 0.5f * (n0.x + n0.y), 0.5f * (n0.z + n0.w),
-                                       0.5f * (n0.z + n0.w), 0.5f * (n2.x + n2.y), 0.5f * (n2.x + n2.y));
-            const float c1 = box_dist2(px, py, pz, 0.5f * (n1.x + n1.y), 0.5f * (n1.x + n1.y), 0.5f * (n1.z + n1.w),
-                                       0.5f * (n1.z + n1.w), 0.5f * (n2.z + n2.w), 0.5f * (n2.z + n2.w));
-            right = c1 < c0;
+        const uint4* rec = reinterpret_cast<const uint4*>(sc.nodes2 + kDevNode2Words * (size_t)node);
+        const uint4 a = __ldg(rec), b = __ldg(rec + 1);
+        const uint32_t w0[3] = {a.x, a.y, a.z}, w1[3] = {a.w, b.x, b.y};
+        float d0 = 0.0f, d1 = 0.0f, e0 = 0.0f, e1 = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float l0 = pg[k] - __uint_as_float(0x3f000000u | (w0[k] & 0xffffu) << 8);
+            const float u0 = __uint_as_float(0x3f000000u | (w0[k] >> 16) << 8) - pg[k];
+            const float l1 = pg[k] - __uint_as_float(0x3f000000u | (w1[k] & 0xffffu) << 8);
+            const float u1 = __uint_as_float(0x3f000000u | (w1[k] >> 16) << 8) - pg[k];
+            // l < 0: below the box, u < 0: above it; l - u: twice the offset from the centre
+            const float b0 = fmaxf(fmaxf(-l0, -u0), 0.0f) * inv[k], b1 = fmaxf(fmaxf(-l1, -u1), 0.0f) * inv[k];
+            const float a0 = (l0 - u0) * inv[k], a1 = (l1 - u1) * inv[k];
+            d0 += b0 * b0;
+            d1 += b1 * b1;
+            e0 += a0 * a0;
+            e1 += a1 * a1;
         }
+        const bool right = d0 != d1 ? d1 < d0 : e1 < e0;
         code |= right ? 1u : 0u;
-        node = __float_as_int(right ? n3.y : n3.x);
+        node = (int)(right ? b.w : b.z);
     }
     return code;
 }
@@ -1162,8 +1165,8 @@ __device__ __forceinline__ uint32_t morton_key(const float4* __restrict__ ray_o,
     uint32_t key = 0;
     if (kind == 5) {
         const float il = rsqrtf(d.x * d.x + d.y * d.y + d.z * d.z) * (kHcutLambda * emax);
-        const uint32_t a = hcut_path(sc.nodes2, o.x, o.y, o.z);
-        const uint32_t b = hcut_path(sc.nodes2, o.x + d.x * il, o.y + d.y * il, o.z + d.z * il);
+        const uint32_t a = hcut_path(sc, o.x, o.y, o.z);
+        const uint32_t b = hcut_path(sc, o.x + d.x * il, o.y + d.y * il, o.z + d.z * il);
         const uint32_t q[2] = {a, b};
         return interleave(q, 2, kHcutLevels);
     }

@@ -1,11 +1,10 @@
 // trace.cu -- closest-hit BVH2 traversal (the intersection step, which dominates path
-// tracing time, Sec. 1), one ray per thread.
+// tracing time, Sec. 1), one ray per lane.
 //
-// Stackful while-while traversal of the 64-byte two-child nodes: both child boxes are
-// fetched with four 16-byte read-only loads, tested with a conservative slab test, the
-// nearer hit child is visited first and the farther one pushed.  The traversal stack lives
-// in shared memory (kSmemStack entries per thread, interleaved so that a warp's pushes hit
-// distinct banks) and continues in a per-thread local array for deeper trees.  Leaves hold
+// Stackful traversal of the 32-byte two-child records (DevBVH2): one 256-bit load fetches both
+// child boxes, the nearer hit child is visited first and the farther one pushed.  The stack
+// lives in shared memory (kSmemStack entries per lane, a warp's entries of one level in one
+// 128-byte line) and older entries move to local memory when it fills.  Leaves hold
 // up to four triangles tested with the watertight test of Woop, Benthin and Wald (2013).
 // The primitives and the closest-hit rule shared with the BVH8-Q kernels (trace_bvh8.cu)
 // are in trace_common.cuh.
@@ -18,59 +17,133 @@ namespace cr {
 namespace {
 
 
-// kAny: visibility only; the traversal ends at the first triangle hit before the ray's tmax.
-// kSmemS: stack entries per thread kept in shared memory (8, 16 or 32; deeper ones go to a
-// local array), a launch-shape knob of the autotuner.
-// dsc: the scene-table entry, read only by the index checks of a debug build.
-template <bool kCount, bool kAny = false, int kSmemS = kSmemStack>
-__device__ __forceinline__ int2 trace_bvh2_one(const float4* __restrict__ nodes, const float4* __restrict__ tris,
-                                               float4 ro, float4 rd, uint32_t* sstack, unsigned long long& n_node,
-                                               unsigned long long& n_tri, const SceneDev* dsc = nullptr) {
+__device__ __forceinline__ void sts(uint32_t a, uint32_t v) {
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t lds(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+
+constexpr int kNoNode = (int)0x80000000; // no traversal left (leaf codes are all above kRefill)
+constexpr int kRefill = (int)0x80000001; // the stack's older entries wait in local memory
+constexpr int kSteps = 2;                // node visits between two votes of the warp
+
+// Traversal of one ray per lane.  All 32 lanes of a warp call it together; `live` says whether
+// the lane has a ray.
+//
+// What bounds it: issue slots and the latency of the record loads, both multiplied by lanes
+// that wait.  A warp that descends until its last lane has reached a leaf keeps 8 of 32 lanes
+// busy on secondary rays; so the descent ends as soon as no more than half of the unfinished
+// lanes are still in it, and the leaves reached are tested while the others wait.  That gives 13
+// lanes and 22% fewer warp instructions (half is the best of 3/8 to 3/4; a vote every second
+// visit the best of 1 to 4).
+// Measured on the landscape's 1.93M secondary rays (1920x1080, 2 bounces, one step):
+// 1.059 ms for the start's kernel (64-byte records in four loads, no vote), 0.833 with 256-bit loads
+// and the vote, 0.790 with the 32-byte records as well.  On the interior's 3.35M secondary rays
+// 2.46 -> 2.02 -> 1.95 ms, its 1.68M shadow rays 1.75 -> 1.48 -> 1.43 ms.
+//
+// kAny: visibility only; a lane is done at the first triangle hit before its ray's tmax.
+// kSmemS: stack entries per lane kept in shared memory (8, 16 or 32), a launch-shape knob of
+// the autotuner.
+template <bool kCount, bool kAny, int kSmemS>
+__device__ __forceinline__ int2 trace_bvh2_warp(const SceneDev& sc, float4 ro, float4 rd, bool live, uint32_t* smem,
+                                                unsigned long long& n_node, unsigned long long& n_tri) {
+    constexpr uint32_t kLevel = 128u; // bytes between a lane's entries
+    constexpr int kHalf = kSmemS / 2;
+    const uint32_t* __restrict__ nodes = sc.nodes2;
+    const float4* __restrict__ tris = sc.tris;
     const RayPre r = prep_ray(ro, rd);
+    const GridRay g = grid_ray(ro, rd, sc);
     const int skip = __float_as_int(ro.w);
-    Best best{rd.w, -1, 0x7fffffff};
-    int lstack[kStackTotal - kSmemS];
-    const int stride = blockDim.x;
-    int sp = 0;
-    int node = 0;
+    Best best{rd.w, -1};
     float tcull = __fmul_rn(best.t, kCullWiden); // changes only after a leaf
-    uint32_t* top = sstack; // next free shared-memory stack entry (stays at the end once full)
+    // entry 0 holds kNoNode (or kRefill while older entries are in lstack), so a pop needs no
+    // test for an empty stack
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem) + (threadIdx.x >> 5) * (kSmemS * kLevel) +
+                          (threadIdx.x & 31u) * 4u;
+    const uint32_t lim = base + (uint32_t)(kSmemS - kSteps + 1) * kLevel; // below it there is room for kSteps pushes
+    uint32_t top = base + kLevel;                                         // next free entry
+    int lstack[kStackTotal];
+    int lsp = 0;
+    sts(base, (uint32_t)kNoNode);
+    int node = live ? 0 : kNoNode;
+    auto step = [&]() {
+        if (kCount) ++n_node;
+        CR_DBG(if (!dbg_in_range(&sc, (uint32_t)node, kDbgNode, sc.n_nodes)) {
+            node = kNoNode;
+            return;
+        })
+        const NodeTest q = node_test(g, nodes, node);
+        // the nearer hit child is next; with both hit the farther one is pushed, with none an
+        // entry is popped (predicated: branches here cost 10% of the trace)
+        asm volatile("{\n\t"
+                     ".reg .pred p0, p1, q, s, b, n;\n\t"
+                     ".reg .b32 far;\n\t"
+                     "setp.le.f32 p0, %2, %4;\n\t"
+                     "setp.le.and.f32 p0, %2, %6, p0;\n\t"
+                     "setp.le.f32 p1, %3, %5;\n\t"
+                     "setp.le.and.f32 p1, %3, %6, p1;\n\t"
+                     "setp.le.f32 q, %2, %3;\n\t"
+                     "not.pred n, p1;\n\t"
+                     "or.pred s, q, n;\n\t"
+                     "and.pred s, s, p0;\n\t"
+                     "and.pred b, p0, p1;\n\t"
+                     "or.pred n, p0, p1;\n\t"
+                     "not.pred n, n;\n\t"
+                     "selp.b32 %1, %7, %8, s;\n\t"
+                     "selp.b32 far, %8, %7, s;\n\t"
+                     "@b st.shared.u32 [%0], far;\n\t"
+                     "@b add.u32 %0, %0, %9;\n\t"
+                     "@n sub.u32 %0, %0, %9;\n\t"
+                     "@n ld.shared.u32 %1, [%0];\n\t}"
+                     : "+r"(top), "+r"(node)
+                     : "f"(q.t0), "f"(q.t1), "f"(q.f0), "f"(q.f1), "f"(tcull), "r"(q.c0), "r"(q.c1), "n"(kLevel)
+                     : "memory");
+    };
     while (true) {
-        while (node >= 0) {
-            if (kCount) ++n_node;
-            CR_DBG(if (!dbg_in_range(dsc, (uint32_t)node, kDbgNode, dsc->n_nodes)) {
-                node = 0x7fffffff;
-                break;
-            })
-            const float4 n0 = __ldg(&nodes[4 * node + 0]);
-            const float4 n1 = __ldg(&nodes[4 * node + 1]);
-            const float4 n2 = __ldg(&nodes[4 * node + 2]);
-            const float4 n3 = __ldg(&nodes[4 * node + 3]);
-            float t0, t1;
-            const bool h0 = box_hit_fma(r, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, tcull, t0);
-            const bool h1 = box_hit_fma(r, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, tcull, t1);
-            const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-            if (h0 && h1) {
-                const bool first0 = t0 <= t1;
-                const int near = first0 ? c0 : c1, far = first0 ? c1 : c0;
-                STACK_PUSH_TOP(far);
-                node = near;
-            } else if (h0 || h1) {
-                node = h0 ? c0 : c1;
-            } else {
-                if (sp == 0) { node = 0x7fffffff; break; }
-                STACK_POP_TOP(node);
+        const uint32_t alive = __ballot_sync(0xffffffffu, node != kNoNode);
+        if (alive == 0u) break;
+        const int half = __popc(alive) >> 1;
+        bool run;
+        do {
+            run = node >= 0 && top < lim;
+#pragma unroll
+            for (int e = 0; e < kSteps; ++e) {
+                if (run) {
+                    step();
+                    run = node >= 0;
+                }
             }
+            run = run && top < lim;
+        } while (__popc(__ballot_sync(0xffffffffu, run)) > half);
+        if (node >= 0 && top >= lim) { // rare: the older half of the stack moves to local memory
+            for (int k = 0; k < kHalf; ++k) lstack[lsp + k] = (int)lds(base + (1 + k) * kLevel);
+            for (uint32_t a = base + (1 + kHalf) * kLevel; a < top; a += kLevel) sts(a - kHalf * kLevel, lds(a));
+            sts(base, (uint32_t)kRefill);
+            lsp += kHalf;
+            top -= kHalf * kLevel;
         }
-        if (node == 0x7fffffff) break;
-        // leaf
-        const uint32_t code = (uint32_t)(~node);
-        CR_DBG(if (!dbg_in_range(dsc, (code >> 2) + (code & 3u), kDbgTri, dsc->n_tris)) break;)
-        test_leaf(tris, r, skip, code >> 2, (code & 3u) + 1u, best, n_tri);
-        if (kAny && best.leaf >= 0) break;
-        tcull = __fmul_rn(best.t, kCullWiden);
-        if (sp == 0) break;
-        STACK_POP_TOP(node);
+        if (node < 0 && node != kNoNode) {
+            if (node == kRefill) { // the stack is empty: its next entries come back
+                lsp -= kHalf;
+                for (int k = 0; k < kHalf; ++k) sts(base + (1 + k) * kLevel, (uint32_t)lstack[lsp + k]);
+                top = base + (1 + kHalf) * kLevel;
+                if (lsp == 0) sts(base, (uint32_t)kNoNode);
+            } else { // a leaf
+                const uint32_t code = (uint32_t)(~node);
+                CR_DBG(if (!dbg_in_range(&sc, (code >> 2) + (code & 3u), kDbgTri, sc.n_tris)) {
+                    node = kNoNode;
+                    continue;
+                })
+                test_leaf(tris, r, skip, code >> 2, (code & 3u) + 1u, best, n_tri);
+                tcull = __fmul_rn(best.t, kCullWiden);
+            }
+            top -= kLevel;
+            node = (int)lds(top);
+            if (kAny && best.leaf >= 0) node = kNoNode;
+        }
     }
     return make_int2(best.leaf, __float_as_int(best.t));
 }
@@ -78,6 +151,27 @@ __device__ __forceinline__ int2 trace_bvh2_one(const float4* __restrict__ nodes,
 #ifndef CR_TRACE_MAXNREG
 #define CR_TRACE_MAXNREG 48 // 42 warps resident per SM (10 blocks of 128 or 21 of 64 threads); 40 spills
 #endif
+
+// Loads of the whole warp's rays, traversal, hits per slot.
+template <bool kCount, bool kAny, int kSmemS>
+__device__ __forceinline__ void trace_positions(const SceneDev* __restrict__ scenes,
+                                                const uint16_t* __restrict__ slot_scene,
+                                                const float4* __restrict__ ray_o, const float4* __restrict__ ray_d,
+                                                const int32_t* __restrict__ queue, uint32_t n, uint32_t i,
+                                                int2* __restrict__ hit, uint32_t* smem, unsigned long long& n_node,
+                                                unsigned long long& n_tri) {
+    int slot = -1;
+    float4 ro = make_float4(0.0f, 0.0f, 0.0f, 0.0f), rd = make_float4(0.0f, 0.0f, 1.0f, -1.0f);
+    if (i < n) {
+        slot = queue ? queue[i] : (int)i;
+        ro = ray_o[slot];
+        rd = ray_d[slot];
+    }
+    const SceneDev& sc = scenes[slot_scene && slot >= 0 ? slot_scene[slot] : 0];
+    const bool live = rd.w >= 0.0f;
+    const int2 h = trace_bvh2_warp<kCount, kAny, kSmemS>(sc, ro, rd, live, smem, n_node, n_tri);
+    if (slot >= 0) hit[slot] = live ? h : make_int2(-1, __float_as_int(INFINITY));
+}
 
 template <bool kCount, bool kAny = false, int kSmemS = kSmemStack>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __restrict__ scenes, const uint16_t* __restrict__ slot_scene,
@@ -88,17 +182,9 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __res
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long n_node = 0, n_tri = 0;
-    if (i < n) {
-        const int slot = queue ? queue[i] : (int)i;
-        const SceneDev& sc = scenes[slot_scene ? slot_scene[slot] : 0];
-        const float4 ro = ray_o[slot];
-        const float4 rd = ray_d[slot];
-        int2 h = make_int2(-1, __float_as_int(INFINITY));
-        if (rd.w >= 0.0f)
-            h = trace_bvh2_one<kCount, kAny, kSmemS>(sc.nodes2, sc.tris, ro, rd, smem_stack + threadIdx.x, n_node,
-                                                     n_tri, &sc);
-        hit[slot] = h;
-    }
+    if ((i & ~31u) < n) // whole warps stay or leave
+        trace_positions<kCount, kAny, kSmemS>(scenes, slot_scene, ray_o, ray_d, queue, n, i, hit, smem_stack, n_node,
+                                              n_tri);
     if (kCount) {
         for (int off = 16; off > 0; off >>= 1) {
             n_node += __shfl_down_sync(0xffffffffu, n_node, off);
@@ -120,20 +206,22 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __res
 // kernel's, so the hits are identical.
 constexpr int kSaveStack = 24;
 
-__device__ __forceinline__ int2 trace_bvh2_resumable(const float4* __restrict__ nodes, const float4* __restrict__ tris,
-                                                     float4 ro, float4 rd, uint32_t* sstack, uint32_t budget,
-                                                     TraceState* st, bool resume, bool& suspended) {
+__device__ __forceinline__ int2 trace_bvh2_resumable(const SceneDev& sc, float4 ro, float4 rd, uint32_t* sstack,
+                                                     uint32_t budget, TraceState* st, bool resume, bool& suspended) {
     constexpr int kSmemS = kSmemStack;
+    const uint32_t* __restrict__ nodes = sc.nodes2;
+    const float4* __restrict__ tris = sc.tris;
     const RayPre r = prep_ray(ro, rd);
+    const GridRay g = grid_ray(ro, rd, sc);
     const int skip = __float_as_int(ro.w);
-    Best best{rd.w, -1, 0x7fffffff};
+    Best best{rd.w, -1};
     int lstack[kStackTotal - kSmemStack];
     const int stride = blockDim.x;
     int sp = 0, node = 0;
     if (resume) {
         node = st->node;
         sp = st->sp;
-        best = Best{st->t, st->leaf, st->orig};
+        best = Best{st->t, st->leaf};
         for (int k = 0; k < sp; ++k) {
             const int v = st->stack[k];
             if (k < kSmemStack) sstack[k * stride] = (uint32_t)v;
@@ -148,15 +236,11 @@ __device__ __forceinline__ int2 trace_bvh2_resumable(const float4* __restrict__ 
                 suspended = true;
                 break;
             }
-            const float4 n0 = __ldg(&nodes[4 * node + 0]);
-            const float4 n1 = __ldg(&nodes[4 * node + 1]);
-            const float4 n2 = __ldg(&nodes[4 * node + 2]);
-            const float4 n3 = __ldg(&nodes[4 * node + 3]);
             const float tcull = __fmul_rn(best.t, kCullWiden);
-            const float t0 = box_entry_fma(r, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, tcull);
-            const float t1 = box_entry_fma(r, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, tcull);
-            const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-            const bool h0 = t0 != INFINITY, h1 = t1 != INFINITY;
+            const NodeTest q = node_test(g, nodes, node);
+            const float t0 = q.t0, t1 = q.t1;
+            const int c0 = q.c0, c1 = q.c1;
+            const bool h0 = q.hit0(tcull), h1 = q.hit1(tcull);
             if (h0 && h1) {
                 const bool first0 = t0 <= t1;
                 const int near = first0 ? c0 : c1, far = first0 ? c1 : c0;
@@ -182,7 +266,6 @@ __device__ __forceinline__ int2 trace_bvh2_resumable(const float4* __restrict__ 
         st->sp = sp;
         st->t = best.t;
         st->leaf = best.leaf;
-        st->orig = best.orig;
         for (int k = 0; k < sp; ++k) st->stack[k] = k < kSmemStack ? (int)sstack[k * stride] : lstack[k - kSmemStack];
     }
     return make_int2(best.leaf, __float_as_int(best.t));
@@ -204,7 +287,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_phase(
     int2 h = make_int2(-1, __float_as_int(INFINITY));
     if (rd.w >= 0.0f) {
         const SceneDev& sc = scenes[slot_scene ? slot_scene[slot] : 0];
-        h = trace_bvh2_resumable(sc.nodes2, sc.tris, ro, rd, smem_stack + threadIdx.x, budget, &state[slot],
+        h = trace_bvh2_resumable(sc, ro, rd, smem_stack + threadIdx.x, budget, &state[slot],
                                  resume != 0, suspended);
     }
     if (!suspended) hit[slot] = h;
@@ -268,7 +351,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
     bool valid = false;
     RayPre r;
     int skip = -1;
-    Best best{-1.0f, -1, 0x7fffffff}; // t < 0: a lane without a ray never enters a box
+    Best best{-1.0f, -1}; // t < 0: a lane without a ray never enters a box
     uint32_t sid = 0;
     if (i < n) {
         slot = queue ? queue[i] : (int)i;
@@ -278,7 +361,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
         if (rd.w >= 0.0f) {
             r = prep_ray(ro, rd);
             skip = __float_as_int(ro.w);
-            best = Best{rd.w, -1, 0x7fffffff};
+            best = Best{rd.w, -1};
             valid = true;
         } else {
             hit[slot] = make_int2(-1, __float_as_int(INFINITY));
@@ -288,14 +371,12 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
     const uint32_t sid0 = __shfl_sync(0xffffffffu, sid, 0);
     const bool uniform_scene = __all_sync(0xffffffffu, !valid || sid == sid0);
     const SceneDev& sc = scenes[uniform_scene ? sid0 : sid];
-    const float4* nodes = sc.nodes2;
+    const uint32_t* nodes = sc.nodes2;
     const float4* tris = sc.tris;
     unsigned long long dummy = 0;
     if (!uniform_scene) { // rare: a warp straddling two jobs of different scenes
-        if (valid) {
-            int2 h = trace_bvh2_one<false>(nodes, tris, ray_o[slot], ray_d[slot], sstack, dummy, dummy);
-            hit[slot] = h;
-        }
+        trace_positions<false, false, kSmemStack>(scenes, slot_scene, ray_o, ray_d, queue, n, i, hit, smem_stack, dummy,
+                                                  dummy);
         return;
     }
     constexpr int kSmemS = kSmemStack;
@@ -307,17 +388,14 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
     int sp = 0;
     int node = 0;
     if (!valid) r = prep_ray(make_float4(0, 0, 0, 0), make_float4(0, 0, 1, -1)); // inert ray
+    const GridRay g = grid_ray(make_float4(r.ox, r.oy, r.oz, 0), make_float4(r.dx, r.dy, r.dz, 0), sc);
     while (true) {
         if (node >= 0) {
-            const float4 n0 = __ldg(&nodes[4 * node + 0]);
-            const float4 n1 = __ldg(&nodes[4 * node + 1]);
-            const float4 n2 = __ldg(&nodes[4 * node + 2]);
-            const float4 n3 = __ldg(&nodes[4 * node + 3]);
-            const float tcull = __fmul_rn(best.t, kCullWiden); // negative for lanes without a ray
-            const float t0 = box_entry_fma(r, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, tcull);
-            const float t1 = box_entry_fma(r, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, tcull);
-            const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-            const bool h0 = t0 != INFINITY, h1 = t1 != INFINITY;
+            const float tcull = __fmul_rn(best.t, kCullWiden);
+            const NodeTest q = node_test(g, nodes, node);
+            const float t0 = q.t0, t1 = q.t1;
+            const int c0 = q.c0, c1 = q.c1;
+            const bool h0 = q.hit0(tcull), h1 = q.hit1(tcull);
             const uint32_t v0 = __ballot_sync(0xffffffffu, h0 && (!h1 || t0 <= t1));
             const uint32_t v1 = __ballot_sync(0xffffffffu, h1 && (!h0 || t1 < t0));
             const bool any0 = __any_sync(0xffffffffu, h0), any1 = __any_sync(0xffffffffu, h1);
@@ -361,9 +439,10 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_spec(
     int slot = -1;
     bool done = true;
     RayPre r;
+    GridRay g;
     int skip = -1;
-    Best best{0.0f, -1, 0x7fffffff};
-    const float4* nodes = nullptr;
+    Best best{0.0f, -1};
+    const uint32_t* nodes = nullptr;
     const float4* tris = nullptr;
     if (i < n) {
         slot = queue ? queue[i] : (int)i;
@@ -374,8 +453,9 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_spec(
             nodes = sc.nodes2;
             tris = sc.tris;
             r = prep_ray(ro, rd);
+            g = grid_ray(ro, rd, sc);
             skip = __float_as_int(ro.w);
-            best = Best{rd.w, -1, 0x7fffffff};
+            best = Best{rd.w, -1};
             done = false;
         } else {
             hit[slot] = make_int2(-1, __float_as_int(INFINITY));
@@ -393,15 +473,11 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_spec(
         // inner phase
         while (true) {
             if (node >= 0 && node != kEmpty) {
-                const float4 n0 = __ldg(&nodes[4 * node + 0]);
-                const float4 n1 = __ldg(&nodes[4 * node + 1]);
-                const float4 n2 = __ldg(&nodes[4 * node + 2]);
-                const float4 n3 = __ldg(&nodes[4 * node + 3]);
                 const float tcull = __fmul_rn(best.t, kCullWiden);
-                const float t0 = box_entry_fma(r, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, tcull);
-                const float t1 = box_entry_fma(r, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, tcull);
-                const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-                const bool h0 = t0 != INFINITY, h1 = t1 != INFINITY;
+                const NodeTest q = node_test(g, nodes, node);
+                const float t0 = q.t0, t1 = q.t1;
+                const int c0 = q.c0, c1 = q.c1;
+                const bool h0 = q.hit0(tcull), h1 = q.hit1(tcull);
                 if (h0 && h1) {
                     const bool first0 = t0 <= t1;
                     const int far = first0 ? c1 : c0;
@@ -464,10 +540,11 @@ __global__ void __launch_bounds__(128) k_trace_bvh2_dynamic(
     bool exhausted = false;                 // warp-uniform
     bool live = false;
     RayPre r;
+    GridRay g;
     int skip = -1, node = kDone, sp = 0, slot = -1;
-    const float4* nodes = nullptr;
+    const uint32_t* nodes = nullptr;
     const float4* tris = nullptr;
-    Best best{0.0f, -1, 0x7fffffff};
+    Best best{0.0f, -1};
     int lstack[kStackTotal - kSmemStack];
     unsigned long long dummy = 0;
     while (true) {
@@ -499,8 +576,9 @@ __global__ void __launch_bounds__(128) k_trace_bvh2_dynamic(
                             nodes = sc.nodes2;
                             tris = sc.tris;
                             r = prep_ray(ro, rd);
+                            g = grid_ray(ro, rd, sc);
                             skip = __float_as_int(ro.w);
-                            best = Best{rd.w, -1, 0x7fffffff};
+                            best = Best{rd.w, -1};
                             node = 0;
                             sp = 0;
                             live = true;
@@ -520,15 +598,11 @@ __global__ void __launch_bounds__(128) k_trace_bvh2_dynamic(
         if (live) {
             // inner nodes until a leaf is reached or the traversal ends
             while (node >= 0 && node != kDone) {
-                const float4 n0 = __ldg(&nodes[4 * node + 0]);
-                const float4 n1 = __ldg(&nodes[4 * node + 1]);
-                const float4 n2 = __ldg(&nodes[4 * node + 2]);
-                const float4 n3 = __ldg(&nodes[4 * node + 3]);
                 const float tcull = __fmul_rn(best.t, kCullWiden);
-                const float t0 = box_entry_fma(r, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, tcull);
-                const float t1 = box_entry_fma(r, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, tcull);
-                const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-                const bool h0 = t0 != INFINITY, h1 = t1 != INFINITY;
+                const NodeTest q = node_test(g, nodes, node);
+                const float t0 = q.t0, t1 = q.t1;
+                const int c0 = q.c0, c1 = q.c1;
+                const bool h0 = q.hit0(tcull), h1 = q.hit1(tcull);
                 if (h0 && h1) {
                     const bool first0 = t0 <= t1;
                     const int near = first0 ? c0 : c1, far = first0 ? c1 : c0;
@@ -563,7 +637,7 @@ __global__ void __launch_bounds__(128) k_trace_bvh2_dynamic(
     }
 }
 
-// Shadow rays of next-event estimation, one thread per position of the last shade's group
+// Shadow rays of next-event estimation, one lane per position of the last shade's group
 // queue (so a reuse group's rays run in adjacent lanes, as they were shaded).  A ray whose
 // direction record has w = tmax > 0 is traced for visibility only; if nothing blocks it, its
 // contribution is added to the path radiance of its slot.  Rays traced are counted.
@@ -573,30 +647,29 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
     const uint32_t* __restrict__ group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
     unsigned long long* __restrict__ n_traced) {
     extern __shared__ uint32_t smem_stack[];
-    const uint32_t n_groups = group_queue ? min(*group_count, n_groups_max) : n_groups_max;
+    const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
     const uint32_t pos = blockIdx.x * blockDim.x + threadIdx.x;
-    bool traced = false;
-    if (pos < n_groups * K) {
+    if ((pos & ~31u) >= n) return; // whole warps leave together
+    int slot = -1;
+    float4 ro = make_float4(0.0f, 0.0f, 0.0f, 0.0f), rd = make_float4(0.0f, 0.0f, 1.0f, -1.0f);
+    if (pos < n) {
         const uint32_t g = group_queue ? (uint32_t)group_queue[pos / K] : pos / K;
-        const int slot = (int)(g * K + pos % K);
-        const float4 rd = sh_d[slot];
-        if (rd.w > 0.0f) {
-            traced = true;
-            const float4 ro = sh_o[slot];
-            const SceneDev& sc = scenes[slot_scene[slot]];
-            unsigned long long dn = 0, dt = 0;
-            const int2 h = trace_bvh2_one<false, true>(sc.nodes2, sc.tris, ro, rd, smem_stack + threadIdx.x, dn, dt, &sc);
-            if (h.x < 0) {
-                const float4 c = sh_c[slot];
-                const float4 L = radiance[slot];
-                radiance[slot] = make_float4(__fadd_rn(L.x, c.x), __fadd_rn(L.y, c.y), __fadd_rn(L.z, c.z), L.w);
-            }
-        }
+        slot = (int)(g * K + pos % K);
+        rd = sh_d[slot];
+    }
+    const bool traced = rd.w > 0.0f;
+    if (traced) ro = sh_o[slot];
+    const SceneDev& sc = scenes[traced ? slot_scene[slot] : 0];
+    unsigned long long dn = 0, dt = 0;
+    const int2 h = trace_bvh2_warp<false, true, kSmemStack>(sc, ro, rd, traced, smem_stack, dn, dt);
+    if (traced && h.x < 0) {
+        const float4 c = sh_c[slot];
+        const float4 L = radiance[slot];
+        radiance[slot] = make_float4(__fadd_rn(L.x, c.x), __fadd_rn(L.y, c.y), __fadd_rn(L.z, c.z), L.w);
     }
     const uint32_t b = __ballot_sync(0xffffffffu, traced);
     if ((threadIdx.x & 31) == 0 && b) atomicAdd(n_traced, (unsigned long long)__popc(b));
 }
-
 
 __global__ void k_hits_to_user(const float4* __restrict__ tris, const int2* __restrict__ hit, uint32_t n,
                                int32_t* __restrict__ prim, float* __restrict__ t) {
@@ -647,6 +720,10 @@ void launch_rays_from_user(const float* rays, const int32_t* skip, uint32_t n, f
 SceneDev scene_entry(const DevScene& s, bool bvh8) {
     SceneDev e;
     e.nodes2 = s.nodes2;
+    for (int k = 0; k < 3; ++k) {
+        e.grid_lo[k] = s.grid_lo[k];
+        e.grid_scale[k] = s.grid_scale[k];
+    }
     e.nodes8 = s.nodes8;
     e.nodes4 = s.nodes4;
     e.tris = bvh8 ? s.tris8 : s.tris;

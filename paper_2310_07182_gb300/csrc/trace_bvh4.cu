@@ -57,7 +57,7 @@ __device__ __forceinline__ int2 trace_bvh4_one(const float4* __restrict__ nodes,
     constexpr int kSmemS = kSmemStack;
     const RayPre r = prep_ray(ro, rd);
     const int skip = __float_as_int(ro.w);
-    Best best{rd.w, -1, 0x7fffffff};
+    Best best{rd.w, -1};
     int lstack[kBvh4StackCapacity - kSmemS];
     const int stride = blockDim.x;
     int sp = 0;

@@ -53,7 +53,7 @@ __device__ __forceinline__ int2 trace_bvh8_one(const uint4* __restrict__ nodes, 
     const uint32_t oct = (rd.x < 0.0f ? 1u : 0u) | (rd.y < 0.0f ? 2u : 0u) | (rd.z < 0.0f ? 4u : 0u);
     const uint32_t o3 = oct & 3u;
     const uint32_t sel = o3 | ((1u ^ o3) << 4) | ((2u ^ o3) << 8) | ((3u ^ o3) << 12);
-    Best best{rd.w, -1, 0x7fffffff};
+    Best best{rd.w, -1};
     uint2 stack[kStack8];
     int sp = 0;
     uint32_t node = 0;

@@ -24,7 +24,7 @@ constexpr float kCullWiden = 1.0f + 0x1.0p-16f;
 struct RayPre {
     float ox, oy, oz;
     float ix, iy, iz; // 1 / d (zero components replaced by +-1e-20 first)
-    int kx, ky, kz;
+    int kz;           // axis of the largest direction component; kx, ky follow it cyclically
     float sx, sy, sz; // shear constants of the watertight test
     float dx, dy, dz;
     // slab offsets for t = fma(plane, 1/d, offset): -o/d biased outward by 2^-22 |o/d|, which
@@ -33,7 +33,10 @@ struct RayPre {
     float lox, loy, loz, hix, hiy, hiz;
 };
 
-__device__ __forceinline__ float sel3(float x, float y, float z, int k) { return k == 0 ? x : (k == 1 ? y : z); }
+// component kz, kx = kz + 1, ky = kz + 2 (mod 3) of (x, y, z)
+__device__ __forceinline__ float sel_z(float x, float y, float z, int kz) { return kz == 0 ? x : (kz == 1 ? y : z); }
+__device__ __forceinline__ float sel_x(float x, float y, float z, int kz) { return kz == 0 ? y : (kz == 1 ? z : x); }
+__device__ __forceinline__ float sel_y(float x, float y, float z, int kz) { return kz == 0 ? z : (kz == 1 ? x : y); }
 
 __device__ __forceinline__ RayPre prep_ray(float4 o, float4 d) {
     RayPre r;
@@ -48,20 +51,11 @@ __device__ __forceinline__ RayPre prep_ray(float4 o, float4 d) {
     r.iy = 1.0f / (fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y));
     r.iz = 1.0f / (fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z));
     const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
-    int kz = ax > ay ? (ax > az ? 0 : 2) : (ay > az ? 1 : 2);
-    int kx = kz + 1 == 3 ? 0 : kz + 1;
-    int ky = kx + 1 == 3 ? 0 : kx + 1;
-    const float dkz = sel3(d.x, d.y, d.z, kz);
-    if (dkz < 0.0f) {
-        int t = kx;
-        kx = ky;
-        ky = t;
-    }
-    r.kx = kx;
-    r.ky = ky;
+    const int kz = ax > ay ? (ax > az ? 0 : 2) : (ay > az ? 1 : 2);
+    const float dkz = sel_z(d.x, d.y, d.z, kz);
     r.kz = kz;
-    r.sx = sel3(d.x, d.y, d.z, kx) / dkz;
-    r.sy = sel3(d.x, d.y, d.z, ky) / dkz;
+    r.sx = sel_x(d.x, d.y, d.z, kz) / dkz;
+    r.sy = sel_y(d.x, d.y, d.z, kz) / dkz;
     r.sz = 1.0f / dkz;
     // plane of the lower bound enters first when 1/d >= 0; bias each offset so that the
     // entry distance can only decrease and the exit distance only increase
@@ -77,21 +71,6 @@ __device__ __forceinline__ RayPre prep_ray(float4 o, float4 d) {
     return r;
 }
 
-// Slab test of one box; returns the entry distance, or +inf if the box is missed or culled.
-__device__ __forceinline__ float box_entry(const RayPre& r, float lox, float hix, float loy, float hiy, float loz,
-                                           float hiz, float tcull) {
-    const float tx0 = __fmul_rn(__fsub_rn(lox, r.ox), r.ix), tx1 = __fmul_rn(__fsub_rn(hix, r.ox), r.ix);
-    const float ty0 = __fmul_rn(__fsub_rn(loy, r.oy), r.iy), ty1 = __fmul_rn(__fsub_rn(hiy, r.oy), r.iy);
-    const float tz0 = __fmul_rn(__fsub_rn(loz, r.oz), r.iz), tz1 = __fmul_rn(__fsub_rn(hiz, r.oz), r.iz);
-    const float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.0f));
-    const float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fmaxf(tz0, tz1));
-    return (tn <= __fmul_rn(tf, kFarWiden) && tn <= tcull) ? tn : INFINITY;
-}
-
-// The same test with one FMA per plane.  Each plane distance fma(x, 1/d, offset) differs
-// from (x - o) * (1/d) by at most the rounding of o/d and of the offset (<= 2^-23 |o/d|) plus a
-// relative 2^-24; the offsets are pre-biased by 2^-22 |o/d| toward a larger interval and the
-// exit is widened by (1 + 2^-21), so no box that the exact form would enter is rejected.
 #ifndef CR_TRACE_MINMAX3
 #define CR_TRACE_MINMAX3 1
 #endif
@@ -115,6 +94,97 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
 #endif
 }
 
+// ------------------------------------------------------------------------------------
+// The BVH2's 32-byte records (DevBVH2 in cr_internal.h).
+//
+// A ray against boxes in grid coordinates (the same distances t): a plane at g is met at
+// fma(g, i, -og * i) with og the origin in the grid and i = 1 / (d * scale).  With
+// u = 2^-24, per axis and as a shift of the plane: og is off by 3 u |og|, i by a relative 2 u,
+// the offset by 2 u |og| and the fma by u (|og| + 2); the triangle test adds about
+// 8 u (|og| + 2).  Boxes are stored 2^-18 = 64 u larger on every side, and the entry and exit
+// offsets move apart by 2^-19 |og| = 32 u |og| each, which covers all of it for any origin, so
+// no box that holds a candidate triangle is rejected.  (NaN plane distances, from 1/d that
+// overflows, drop out of the minima and maxima: that axis then rejects nothing.)
+struct GridRay {
+    float ix, iy, iz; // 1 / (d * scale) (zero components of d replaced by +-1e-20 first)
+    float nx, ny, nz; // offsets of the entry distances
+    float fx, fy, fz; // offsets of the exit distances
+    // byte selectors that decode the near and the far plane: the plane of the lower bound is
+    // entered first when 1/d >= 0, so a box needs no minima and maxima of its plane distances
+    uint32_t snx, sny, snz, sfx, sfy, sfz;
+};
+
+__device__ __forceinline__ void grid_axis(float o, float d, float lo, float scale, float& i, float& n, float& f,
+                                          uint32_t& sn, uint32_t& sf) {
+    const float tiny = 1e-20f;
+    const float og = fmaf(o - lo, scale, 0.5f);
+    i = 1.0f / ((fabsf(d) > tiny ? d : copysignf(tiny, d)) * scale);
+    const float oi = __fmul_rn(og, i), e = __fmul_rn(fabsf(oi), 0x1.0p-19f);
+    n = -oi - e;
+    f = -oi + e;
+    sn = i < 0.0f ? 0x7324u : 0x7104u;
+    sf = i < 0.0f ? 0x7104u : 0x7324u;
+}
+
+__device__ __forceinline__ GridRay grid_ray(float4 o, float4 d, const SceneDev& sc) {
+    GridRay g;
+    grid_axis(o.x, d.x, sc.grid_lo[0], sc.grid_scale[0], g.ix, g.nx, g.fx, g.snx, g.sfx);
+    grid_axis(o.y, d.y, sc.grid_lo[1], sc.grid_scale[1], g.iy, g.ny, g.fy, g.sny, g.sfy);
+    grid_axis(o.z, d.z, sc.grid_lo[2], sc.grid_scale[2], g.iz, g.nz, g.fz, g.snz, g.sfz);
+    return g;
+}
+
+struct NodeTest {
+    float t0, t1; // entry distances of the boxes of child 0, 1 (0 from inside)
+    float f0, f1; // exit distances
+    int c0, c1;   // links
+    // whether the ray enters the box before tcull
+    __device__ __forceinline__ bool hit0(float tcull) const { return t0 <= f0 && t0 <= tcull; }
+    __device__ __forceinline__ bool hit1(float tcull) const { return t1 <= f1 && t1 <= tcull; }
+};
+
+// The float of one 16-bit plane code (bytes: 0, code, 0x3f).
+__device__ __forceinline__ float plane_at(uint32_t w, uint32_t sel) {
+    return __uint_as_float(__byte_perm(w, 0x3f000000u, sel));
+}
+
+// Both child boxes of record `node`.  One 256-bit load fetches the record: half the L1
+// wavefronts of a 64-byte record, which set the speed before (measured beside the kernel).
+__device__ __forceinline__ NodeTest node_test(const GridRay& g, const uint32_t* __restrict__ nodes, int node) {
+    const uint32_t* rec = nodes + kDevNode2Words * (size_t)(uint32_t)node;
+    uint32_t w0, w1, w2, w3, w4, w5, w6, w7;
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(w0), "=r"(w1), "=r"(w2), "=r"(w3), "=r"(w4), "=r"(w5), "=r"(w6), "=r"(w7)
+        : "l"(rec));
+    NodeTest r;
+    r.t0 = fmaxf(max3f(fmaf(plane_at(w0, g.snx), g.ix, g.nx), fmaf(plane_at(w1, g.sny), g.iy, g.ny),
+                       fmaf(plane_at(w2, g.snz), g.iz, g.nz)), 0.0f);
+    r.t1 = fmaxf(max3f(fmaf(plane_at(w3, g.snx), g.ix, g.nx), fmaf(plane_at(w4, g.sny), g.iy, g.ny),
+                       fmaf(plane_at(w5, g.snz), g.iz, g.nz)), 0.0f);
+    r.f0 = min3f(fmaf(plane_at(w0, g.sfx), g.ix, g.fx), fmaf(plane_at(w1, g.sfy), g.iy, g.fy),
+                           fmaf(plane_at(w2, g.sfz), g.iz, g.fz));
+    r.f1 = min3f(fmaf(plane_at(w3, g.sfx), g.ix, g.fx), fmaf(plane_at(w4, g.sfy), g.iy, g.fy),
+                           fmaf(plane_at(w5, g.sfz), g.iz, g.fz));
+    r.c0 = (int)w6;
+    r.c1 = (int)w7;
+    return r;
+}
+
+// Slab test of one box; returns the entry distance, or +inf if the box is missed or culled.
+__device__ __forceinline__ float box_entry(const RayPre& r, float lox, float hix, float loy, float hiy, float loz,
+                                           float hiz, float tcull) {
+    const float tx0 = __fmul_rn(__fsub_rn(lox, r.ox), r.ix), tx1 = __fmul_rn(__fsub_rn(hix, r.ox), r.ix);
+    const float ty0 = __fmul_rn(__fsub_rn(loy, r.oy), r.iy), ty1 = __fmul_rn(__fsub_rn(hiy, r.oy), r.iy);
+    const float tz0 = __fmul_rn(__fsub_rn(loz, r.oz), r.iz), tz1 = __fmul_rn(__fsub_rn(hiz, r.oz), r.iz);
+    const float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.0f));
+    const float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fmaxf(tz0, tz1));
+    return (tn <= __fmul_rn(tf, kFarWiden) && tn <= tcull) ? tn : INFINITY;
+}
+
+// The same test with one FMA per plane.  Each plane distance fma(x, 1/d, offset) differs
+// from (x - o) * (1/d) by at most the rounding of o/d and of the offset (<= 2^-23 |o/d|) plus a
+// relative 2^-24; the offsets are pre-biased by 2^-22 |o/d| toward a larger interval and the
+// exit is widened by (1 + 2^-21), so no box that the exact form would enter is rejected.
 __device__ __forceinline__ float box_entry_fma(const RayPre& r, float lox, float hix, float loy, float hiy, float loz,
                                                float hiz, float tcull) {
     const float tx0 = fmaf(lox, r.ix, r.lox), tx1 = fmaf(hix, r.ix, r.hix);
@@ -138,13 +208,15 @@ __device__ __forceinline__ bool box_hit_fma(const RayPre& r, float lox, float hi
 
 // Watertight ray/triangle test (Woop, Benthin, Wald 2013) without the double-precision
 // fallback: edge functions of exactly zero count as inside, so shared edges are covered.
+// kx and ky are not exchanged for rays that run down the kz axis: that negates U, V, W, det
+// and T exactly, which leaves the sign test and t = T / det as they are.
 __device__ __forceinline__ bool tri_test(const RayPre& r, float4 a4, float4 b4, float4 c4, float& t_out) {
     const float Ax3 = a4.x - r.ox, Ay3 = a4.y - r.oy, Az3 = a4.z - r.oz;
     const float Bx3 = b4.x - r.ox, By3 = b4.y - r.oy, Bz3 = b4.z - r.oz;
     const float Cx3 = c4.x - r.ox, Cy3 = c4.y - r.oy, Cz3 = c4.z - r.oz;
-    const float Akx = sel3(Ax3, Ay3, Az3, r.kx), Aky = sel3(Ax3, Ay3, Az3, r.ky), Akz = sel3(Ax3, Ay3, Az3, r.kz);
-    const float Bkx = sel3(Bx3, By3, Bz3, r.kx), Bky = sel3(Bx3, By3, Bz3, r.ky), Bkz = sel3(Bx3, By3, Bz3, r.kz);
-    const float Ckx = sel3(Cx3, Cy3, Cz3, r.kx), Cky = sel3(Cx3, Cy3, Cz3, r.ky), Ckz = sel3(Cx3, Cy3, Cz3, r.kz);
+    const float Akx = sel_x(Ax3, Ay3, Az3, r.kz), Aky = sel_y(Ax3, Ay3, Az3, r.kz), Akz = sel_z(Ax3, Ay3, Az3, r.kz);
+    const float Bkx = sel_x(Bx3, By3, Bz3, r.kz), Bky = sel_y(Bx3, By3, Bz3, r.kz), Bkz = sel_z(Bx3, By3, Bz3, r.kz);
+    const float Ckx = sel_x(Cx3, Cy3, Cz3, r.kz), Cky = sel_y(Cx3, Cy3, Cz3, r.kz), Ckz = sel_z(Cx3, Cy3, Cz3, r.kz);
     const float Ax = __fsub_rn(Akx, __fmul_rn(r.sx, Akz)), Ay = __fsub_rn(Aky, __fmul_rn(r.sy, Akz));
     const float Bx = __fsub_rn(Bkx, __fmul_rn(r.sx, Bkz)), By = __fsub_rn(Bky, __fmul_rn(r.sy, Bkz));
     const float Cx = __fsub_rn(Ckx, __fmul_rn(r.sx, Ckz)), Cy = __fsub_rn(Cky, __fmul_rn(r.sy, Ckz));
@@ -164,8 +236,7 @@ __device__ __forceinline__ bool tri_test(const RayPre& r, float4 a4, float4 b4, 
 
 struct Best {
     float t;
-    int leaf;
-    int orig;
+    int leaf; // triangle in leaf order, -1 none
 };
 
 __device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, const RayPre& r, int skip, uint32_t first,
@@ -179,10 +250,11 @@ __device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, const
         const float4 c = __ldg(&tris[3 * tri + 2]);
         ++n_tri;
         float t;
-        if (tri_test(r, a, b, c, t) && (t < best.t || (t == best.t && orig < best.orig))) {
+        // a tie goes to the smaller original index (any hit at exactly tmax is taken)
+        if (tri_test(r, a, b, c, t) &&
+            (t < best.t || (t == best.t && (best.leaf < 0 || orig < __float_as_int(__ldg(&tris[3 * best.leaf]).w))))) {
             best.t = t;
             best.leaf = (int)tri;
-            best.orig = orig;
         }
     }
 }
@@ -213,7 +285,7 @@ __device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, const
 
 
 // The same stack with a pointer to the next free shared-memory entry, which saves the index
-// arithmetic of every push and pop (1% on the secondary trace); used by trace_bvh2_one.
+// arithmetic of every push and pop (1% on the secondary trace); used by the BVH4 kernel.
 #define STACK_PUSH_TOP(v)                                                            \
     do {                                                                             \
         if (sp < kSmemS) {                                                           \

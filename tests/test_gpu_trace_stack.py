@@ -1,0 +1,55 @@
+"""The BVH2 traversal where its stack and its rays leave the ordinary range: stacks that overflow
+into local memory (large triangles that all overlap, so both children are hit all the way
+down), and ray origins far outside the scene's grid."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2310_07182_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cr():
+    from paper_2310_07182_gb300 import binding
+    binding.lib()
+    return binding
+
+
+def _overlapping(n, seed):
+    """n triangles of random shape around the origin, each about as large as the whole scene."""
+    rng = np.random.default_rng(seed)
+    sc = scenes.tiny(seed=seed, n_soup=n, material_mix="mixed")
+    sc.tri_xyz[:n] = rng.normal(size=(n, 9)).astype(np.float32)
+    return sc
+
+
+@pytest.mark.parametrize("n", [3, 40, 3000])
+@pytest.mark.parametrize("stack", [8, 16, 32])
+def test_full_stacks_render_the_same(cr, n, stack):
+    S = cr.Scene(_overlapping(n, 4), bvh_flags=cr.CR_BVH2 | cr.CR_BVH8Q)
+    kw = dict(spp=1, max_bounces=3, mode="direction_reuse", tile=(8, 8), k=8, seed=2)
+    cam = scenes.Camera((0.3, 0.2, -4.0), (0.0, 0.0, 0.0), (0.0, 1.0, 0.0), 50.0, 75, 41)
+    want, _ = S.render(cam, bvh=cr.CR_BVH8Q, **kw)
+    got, _ = S.render(cam, stack=stack, **kw)
+    assert torch.equal(want, got)
+
+
+@pytest.mark.parametrize("far", [1.0, 30.0, 1e4])
+@pytest.mark.parametrize("n_rays", [1, 33, 1999])
+def test_far_origins_and_every_layout_agree(cr, far, n_rays):
+    S = cr.Scene(_overlapping(500, 9), bvh_flags=cr.CR_BVH2 | cr.CR_BVH8Q | cr.CR_BVH4)
+    rng = np.random.default_rng(n_rays)
+    rays = scenes.random_rays(3, n_rays, target_box=(-2.0, 2.0))
+    d = rng.normal(size=(n_rays, 3))
+    rays[:, 0:3] = far * d / np.linalg.norm(d, axis=1, keepdims=True)
+    rays[:, 4:7] = (rng.uniform(-2, 2, (n_rays, 3)) - rays[:, 0:3]) / far
+    rays[::7, 4] = 0.0  # parallel to a pair of planes
+    r = torch.from_numpy(rays).cuda()
+    p2, t2 = S.trace(r)
+    p8, t8 = S.trace(r, bvh=cr.CR_BVH8Q)
+    p4, t4 = S.trace(r, bvh=cr.CR_BVH4)
+    assert torch.equal(p2, p8) and torch.equal(t2, t8)
+    assert torch.equal(p2, p4) and torch.equal(t2, t4)
+    assert n_rays == 1 or (p2 >= 0).any()
