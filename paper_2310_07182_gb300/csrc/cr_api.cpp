@@ -821,9 +821,8 @@ cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, cons
     ta.hit = b.hit;
     ta.block = eo.block;
     ta.stack = eo.stack;
-    ta.persistent = eo.persistent;
+    ta.one_scene = p.scenes.size() == 1;
     ta.speculative = eo.speculative;
-    ta.work_counter = b.counts + 2;
     ta.bvh8 = p.bvh8;
     ta.bvh4 = p.bvh4;
     ta.scenes = dev.d_scenes;
@@ -841,6 +840,7 @@ cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, cons
         P.n_tiles = ps.n_tiles;
         P.npx = eo.debug_npx;
         P.nee = p.nee;
+        P.one_scene = p.scenes.size() == 1;
         P.accum_mode = fused_out ? 3u : 0u;
         const uint32_t n_slots = ps.n_tiles * p.m;
         b.n_groups = n_slots / p.k;
@@ -851,7 +851,9 @@ cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, cons
         ta.queue_count = nullptr;
         ta.n_max = n_slots;
         ta.counters = nullptr;
-        if (ta.persistent) check(cudaMemsetAsync(ta.work_counter, 0, 4, stream), "memset");
+        // primary rays of a warp end together: lanes that take new rays on their own mix pixel blocks
+        // and cost 20% of this trace
+        ta.work = eo.persistent ? b.counts + kWorkWord : nullptr;
         ta.packet = eo.packet_primary;
         ta.block = eo.block;
         ev.begin(stream, times ? &times->trace_primary : &dummy, "cr trace primary", true);
@@ -883,7 +885,7 @@ cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, cons
                 ev.end();
             }
             ta.counters = eo.count ? b.counters : nullptr;
-            if (ta.persistent) check(cudaMemsetAsync(ta.work_counter, 0, 4, stream), "memset");
+            ta.work = b.counts + kWorkWord + bnc;
             ta.two_phase = eo.phase_budget > 0 && ws.phase.state;
             ta.phase = ws.phase;
             ta.phase.budget = eo.phase_budget;
@@ -1147,7 +1149,6 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
     ta.hit = hit.as<int2>();
     ta.n_max = n;
     ta.block = block;
-    ta.persistent = (o.flags & CR_OPT_PERSISTENT) != 0;
     ta.speculative = (o.flags & CR_OPT_SPECULATIVE) != 0;
     ta.packet = (o.flags & (CR_OPT_PACKET_PRIMARY | CR_OPT_PACKET_SECONDARY)) != 0;
     ta.any_hit = (o.flags & CR_OPT_ANY_HIT) != 0;
@@ -1155,7 +1156,8 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
     ta.bvh4 = use4;
     ta.scenes = dev_scene_entry(s, use8);
     ta.slot_scene = nullptr;
-    ta.work_counter = wc.as<uint32_t>();
+    ta.one_scene = true;
+    ta.work = (o.flags & CR_OPT_PERSISTENT) ? wc.as<uint32_t>() : nullptr;
     ta.counters = (o.flags & CR_OPT_COUNT) ? reinterpret_cast<unsigned long long*>(wc.as<uint32_t>() + 4) : nullptr;
     cudaEvent_t e0, e1;
     if (o.stats) {

@@ -182,6 +182,7 @@ struct PassArgs {
     uint32_t bounce = 0;   // shade: 1..B (B + 1 = final)
     uint32_t npx = 0;      // pixels of the debug capture (single-job renders)
     bool nee = false;      // some job of the plan uses next-event estimation
+    bool one_scene = false; // the scene table has one entry
     // bit 0: a job's first sample writes its pixel sums without reading them (the buffer is
     // not cleared first); bit 1: its last sample writes the output instead of the sums
     uint32_t accum_mode = 0;
@@ -232,10 +233,11 @@ struct TraceArgs {
     const SceneDev* scenes = nullptr;  // scene table
     const uint16_t* slot_scene = nullptr; // per-slot scene index (NULL: scene 0)
     unsigned long long* counters = nullptr; // [0] node visits, [1] triangle tests (counting pass)
-    uint32_t* work_counter = nullptr;       // persistent mode: atomic ray counter (zeroed)
+    // device counter, zero before the launch: warps of a resident grid take further rays as
+    // theirs end (BVH2); NULL: one ray per lane
+    uint32_t* work = nullptr;
+    bool one_scene = false; // every ray is in scenes[0]
     int block = 128;
-    uint32_t refill = 0; // persistent mode: refill a warp's idle lanes when at least this many (0 = 8)
-    bool persistent = false;
     bool speculative = false; // parked-leaf speculative traversal (BVH2)
     bool packet = false;      // warp-packet traversal (BVH2)
     bool any_hit = false;     // stop at the first hit before tmax (visibility)
@@ -267,11 +269,14 @@ struct PathBuffers {
     uint8_t* alive = nullptr;   // 1 while the path continues
     int32_t* ray_queue = nullptr;   // alive slots in slot order
     int32_t* group_queue = nullptr; // groups with an alive member (2 x n_groups, double-buffered)
-    // counts (kCountsWords words): [2] persistent work counter; [kQueueErrWord] queue
+    // counts (kCountsWords words): [kQueueErrWord] queue
     // overflow flag; [8 + 2b], [8 + 2b + 1] ray and group queue lengths after the compaction
     // of bounce b (kQueueCountWords words, zeroed by raygen each pass); from word kStatWord, 64-bit
     // running totals of rays traced per bounce (index b); from kCounterWord, 64-bit node
-    // visits and triangle tests of the counting pass.
+    // visits and triangle tests of the counting pass; from kWorkWord, the work counters of the
+    // closest-hit traces (index b) and, 32 words on, of the shadow traces (kWorkWords words,
+    // zeroed by raygen each pass).  Rolling wavefront: four words per parity from word 8 (rays,
+    // groups, closest-hit and shadow work counter), zeroed by the iteration that appends to them.
     uint32_t* counts = nullptr;
     uint32_t* block_counts = nullptr; // compaction scratch (2 per block) + offsets
     // next-event estimation (allocated on first use): shadow ray origin|skip, direction|tmax
@@ -291,6 +296,7 @@ struct PathBuffers {
 };
 
 constexpr uint32_t kCountsWords = 256, kStatWord = 64, kCounterWord = 128, kShadowWord = 200;
+constexpr uint32_t kWorkWord = 136, kWorkWords = 64;
 constexpr uint32_t kQueueErrWord = 5, kQueueCountWords = kStatWord - 8;
 // Shadow rays of the last shade (positions of its group queue): any-hit traversal, and the
 // contribution of each unblocked one added to the path radiance.
@@ -303,7 +309,7 @@ void launch_shadow_rays_bvh8(const SceneDev* scenes, const uint16_t* slot_scene,
 void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
                         const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count,
                         uint32_t n_groups_max, uint32_t K, float4* radiance, unsigned long long* n_traced, bool bvh8,
-                        cudaStream_t st, LaunchCount& lc);
+                        bool one_scene, uint32_t* work, cudaStream_t st, LaunchCount& lc);
 
 void launch_raygen(const PassArgs& p, PathBuffers& b, cudaStream_t st, LaunchCount& lc);
 // raygen leaves the primary trace's visiting order (row-major pixels per tile) in the ray queue

@@ -123,8 +123,10 @@ __global__ void k_raygen(PassArgs p, int32_t* __restrict__ pixel, uint16_t* __re
     extern __shared__ uint16_t inv[];
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_base[2];
-    // the shade kernels append to the per-bounce queue counters: zero them for this pass
+    // the shade kernels append to the per-bounce queue counters, the traces take their rays by the
+    // work counters: zero them for this pass
     if (!p.rolling && blockIdx.x == 0 && threadIdx.x < kQueueCountWords) queue_counts[threadIdx.x] = 0;
+    if (!p.rolling && blockIdx.x == 0 && threadIdx.x < kWorkWords) queue_counts[kWorkWord - 8 + threadIdx.x] = 0;
     const uint32_t m = p.m;
     const uint32_t tiles_per_block = blockDim.x / m;
     const uint32_t tl = threadIdx.x / m, j = threadIdx.x % m;
@@ -1706,7 +1708,7 @@ void launch_shadow(const PassArgs& p, PathBuffers& b, bool first, bool bvh8, cud
     const ShadeArgs a = shade_args(p, b, first, false, nullptr);
     launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
                        a.n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
-                       bvh8, st, lc);
+                       bvh8, p.one_scene, b.counts + kWorkWord + 32 + p.bounce, st, lc);
 }
 
 void launch_shade(const PassArgs& p, PathBuffers& b, bool first, bool compact, const cr_debug* dbg,
@@ -1721,8 +1723,9 @@ void launch_shade(const PassArgs& p, PathBuffers& b, bool first, bool compact, c
     lc.n++;
 }
 
-// Rolling wavefront.  Queue words: pair q = counts + 8 + 2 q holds (rays, groups) appended
-// for the iteration that reads group queue q; the caller zeroes the pair an iteration appends
+// Rolling wavefront.  Queue words: counts + 8 + 4 q holds (rays, groups) appended
+// for the iteration that reads group queue q, then the work counters of the closest-hit and the shadow
+// trace of the iteration that appends; the caller zeroes the four words an iteration appends
 // to before its first launch.
 void launch_raygen_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_tiles, cudaStream_t st, LaunchCount& lc) {
     if (!n_tiles) return;
@@ -1740,10 +1743,10 @@ void launch_raygen_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_tiles, 
 static ShadeArgs shade_args_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max) {
     ShadeArgs a = shade_args(p, b, false, true, nullptr);
     a.group_queue = b.group_queue + (size_t)parity * b.n_groups;
-    a.group_count = b.counts + 8 + 2 * parity + 1;
+    a.group_count = b.counts + 8 + 4 * parity + 1;
     a.n_groups_max = n_groups_max;
     a.group_queue_out = b.group_queue + (size_t)(parity ^ 1u) * b.n_groups;
-    a.queue_counts = b.counts + 8 + 2 * (parity ^ 1u);
+    a.queue_counts = b.counts + 8 + 4 * (parity ^ 1u);
     a.rays_queued = reinterpret_cast<unsigned long long*>(b.counts + kStatWord) + 1;
     a.ray_cap = b.n_groups * p.k;
     a.group_cap = b.n_groups;
@@ -1769,7 +1772,7 @@ void launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, u
     const ShadeArgs a = shade_args_rolling(p, b, parity, n_groups_max);
     launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
                        n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
-                       bvh8, st, lc);
+                       bvh8, p.one_scene, b.counts + 8 + 4 * (parity ^ 1u) + 3, st, lc);
 }
 
 void launch_finish_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_slots, cudaStream_t st, LaunchCount& lc) {

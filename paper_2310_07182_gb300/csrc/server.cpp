@@ -467,8 +467,9 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
     P.nee = nee;
     P.rolling = true;
     P.accum_mode = 3u;
-    uint32_t* qn = b.counts + 8 + 2 * (par ^ 1u); // (rays, groups) appended for the next iteration
-    cudaMemsetAsync(qn, 0, 8, L.stream);
+    // (rays, groups) appended for the next iteration, then this iteration's work counters
+    uint32_t* qn = b.counts + 8 + 4 * (par ^ 1u);
+    cudaMemsetAsync(qn, 0, 16, L.stream);
     launch_shade_rolling(P, b, par, n_groups, L.stream, lc);
     launch_shadow_rolling(P, b, par, n_groups, po.bvh8, L.stream, lc);
     if (n_fin) {
@@ -505,8 +506,9 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
         ta.slot_scene = b.slot_scene;
         ta.queue = b.ray_queue;
         ta.queue_count = qn;
+        ta.work = qn + 2;
         ta.n_max = trace_max;
-        if (sort) ta.queue = launch_morton_sort(P, b, par ^ 1u, eo.sort_key, L.stream, lc);
+        if (sort) ta.queue = launch_morton_sort(P, b, 2u * (par ^ 1u), eo.sort_key, L.stream, lc);
         launch_trace(ta, L.stream, lc);
     }
     // the ray total and the error word, read back every kDepth-th iteration (the copies

@@ -53,3 +53,19 @@ def test_far_origins_and_every_layout_agree(cr, far, n_rays):
     assert torch.equal(p2, p8) and torch.equal(t2, t8)
     assert torch.equal(p2, p4) and torch.equal(t2, t4)
     assert n_rays == 1 or (p2 >= 0).any()
+
+
+@pytest.mark.parametrize("n_rays", [1, 31, 33, 4097, 400003])
+@pytest.mark.parametrize("dead", ["none", "some", "runs", "all"])
+def test_lanes_that_take_new_rays(cr, n_rays, dead):
+    """Rays handed out lane by lane (more of them than lanes resident at once, chunks without any
+    ray, single dead rays) give the hits of one ray per lane."""
+    S = cr.Scene(scenes.tiny(seed=5, n_soup=700, material_mix="mixed"))
+    rays = torch.from_numpy(scenes.random_rays(7, n_rays)).cuda()
+    i = torch.arange(n_rays, device="cuda")
+    off = {"none": i < 0, "some": i % 5 == 2, "runs": (i // 96) % 3 != 0, "all": i >= 0}[dead]
+    rays[off, 7] = -1.0
+    want_p, want_t = S.trace(rays)
+    got_p, got_t = S.trace(rays, flags=cr.CR_OPT_PERSISTENT)
+    assert torch.equal(want_p, got_p) and torch.equal(want_t, got_t)
+    assert (got_p[off] == -1).all() and (n_rays < 100 or dead in ("all",) or (got_p >= 0).any())
