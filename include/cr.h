@@ -490,8 +490,9 @@ cr_status cr_debug_bvh_check(const float* tri_xyz, uint32_t n_tri, uint32_t flag
  * forbids raw cudaMalloc, a latency-critical loop that cannot afford the device-wide
  * synchronisation of cudaMalloc/cudaFree, or a process that has reserved nearly all device
  * memory, so an allocation could fail mid-frame.  cr_trace_rays_static computes exactly
- * what cr_trace_rays computes (same kernels, BVH2, block 128) but keeps its scratch (ray and
- * hit records, 40 bytes per ray) in one file-scope device array sized for
+ * what cr_trace_rays computes (same kernels, BVH2, block 128), straight from the rays to the
+ * hit arrays.  Only hit arrays that overlap the rays or skip ids need scratch (ray and
+ * hit records, 40 bytes per ray), kept in one file-scope device array sized for
  * CR_TRACE_STATIC_MAX_RAYS rays (2.5 MiB), which every GPU that loads the library holds
  * until the process exits.  It calls no cudaMalloc, cudaFree or allocating library routine.
  *   rays, skip_prim (or NULL), prim, t: DEVICE pointers of the current device with the
@@ -500,10 +501,10 @@ cr_status cr_debug_bvh_check(const float* tri_xyz, uint32_t n_tri, uint32_t flag
  *   n: 0..CR_TRACE_STATIC_MAX_RAYS; larger n returns CR_ERR_INVALID_ARG (trace in chunks).
  *   stream: cudaStream_t to run on (NULL = legacy default stream).  The call synchronises
  *   this stream before it returns.
- * The first call on a device looks up the array's device address (cudaGetSymbolAddress,
- * with that device current); make that first call before any stream capture.  All calls
- * share the one array and it keeps the last call's contents: calls that overlap on the GPU
- * (other host threads, or other streams) race on it, so serialise them.
+ * The first call on a device that needs the array looks up its device address
+ * (cudaGetSymbolAddress, with that device current); make that first call before any stream
+ * capture.  Such calls share the one array and it keeps the last call's contents: those that
+ * overlap on the GPU (other host threads, or other streams) race on it, so serialise them.
  * Errors: CR_ERR_INVALID_ARG, CR_ERR_CUDA. */
 #define CR_TRACE_STATIC_MAX_RAYS 65536u
 cr_status cr_trace_rays_static(cr_scene* scene, const float* rays, const int32_t* skip_prim, uint32_t n,

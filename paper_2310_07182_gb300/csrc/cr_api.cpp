@@ -125,6 +125,7 @@ struct cr_scene {
     void* d_mats = nullptr;
     void* d_lights = nullptr; // emitter records and their running areas (one allocation)
     cr::SceneDev* d_entries = nullptr; // [0] BVH2 layout, [1] BVH8-Q layout (scene-table entries)
+    uint32_t* d_work = nullptr;        // 8 words of cr_trace_rays: work counter, counting pass
     int device = -1;                   // the CUDA device the scene's memory lives on
     // render workspace and job tables, grown on demand
     cr::Workspace ws;
@@ -369,14 +370,16 @@ extern "C" cr_status cr_scene_create(const float* tri_xyz, uint32_t n_tri, const
     s->dev.n_nodes8 = (bvh_flags & CR_BVH8Q) ? b8.n_nodes : 0u;
     {
         // the two scene-table entries, then the scene's error word (index checks of a debug build)
+        // and, 16 bytes on, the work words of cr_trace_rays
         DevMem de;
-        CR_CUDA(de.alloc(2 * sizeof(SceneDev) + 16));
+        CR_CUDA(de.alloc(2 * sizeof(SceneDev) + 64));
         s->dev.err = reinterpret_cast<uint32_t*>(static_cast<char*>(de.p) + 2 * sizeof(SceneDev));
         CR_CUDA(cudaMemset(s->dev.err, 0, 4));
         SceneDev ent[2] = {scene_entry(s->dev, false), scene_entry(s->dev, s->dev.nodes8 != nullptr)};
         ent[0].n_nodes4 = ent[1].n_nodes4 = s->dev.n_nodes4;
         CR_CUDA(cudaMemcpy(de.p, ent, sizeof(ent), cudaMemcpyHostToDevice));
         s->d_entries = static_cast<SceneDev*>(de.p);
+        s->d_work = reinterpret_cast<uint32_t*>(static_cast<char*>(de.p) + 2 * sizeof(SceneDev) + 16);
         de.p = nullptr;
     }
     std::memset(&s->info, 0, sizeof(s->info));
@@ -1134,19 +1137,12 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
     CR_CUDA(stage_in(s_in, skip_prim, sizeof(int32_t) * (size_t)n, stream));
     CR_CUDA(stage_out(p_out, prim, sizeof(int32_t) * (size_t)n));
     CR_CUDA(stage_out(t_out, t, sizeof(float) * (size_t)n));
-    DevMem ro, rd, hit, wc;
-    CR_CUDA(ro.alloc(16 * (size_t)n));
-    CR_CUDA(rd.alloc(16 * (size_t)n));
-    CR_CUDA(hit.alloc(8 * (size_t)n));
-    CR_CUDA(wc.alloc(16 * 4));
-    CR_CUDA(cudaMemsetAsync(wc.p, 0, 64, stream));
+    const float* d_rays = static_cast<const float*>(r_in.dev);
+    const int32_t* d_skip = static_cast<const int32_t*>(s_in.dev);
+    int32_t* d_prim = static_cast<int32_t*>(p_out.dev);
+    float* d_t = static_cast<float*>(t_out.dev);
     LaunchCount lc;
-    launch_rays_from_user(r_in.dev ? static_cast<const float*>(r_in.dev) : nullptr,
-                          static_cast<const int32_t*>(s_in.dev), n, ro.as<float4>(), rd.as<float4>(), stream, lc);
     TraceArgs ta;
-    ta.ray_o = ro.as<float4>();
-    ta.ray_d = rd.as<float4>();
-    ta.hit = hit.as<int2>();
     ta.n_max = n;
     ta.block = block;
     ta.speculative = (o.flags & CR_OPT_SPECULATIVE) != 0;
@@ -1157,8 +1153,34 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
     ta.scenes = dev_scene_entry(s, use8);
     ta.slot_scene = nullptr;
     ta.one_scene = true;
-    ta.work = (o.flags & CR_OPT_PERSISTENT) ? wc.as<uint32_t>() : nullptr;
-    ta.counters = (o.flags & CR_OPT_COUNT) ? reinterpret_cast<unsigned long long*>(wc.as<uint32_t>() + 4) : nullptr;
+    // four work words of the scene: the rays taken (more rays than resident lanes only), then the
+    // counts of a counting pass
+    const bool count = (o.flags & CR_OPT_COUNT) != 0;
+    if (count || n > kTraceWorkMin) {
+        CR_CUDA(cudaMemsetAsync(s->d_work, 0, 32, stream));
+        ta.work = s->d_work;
+        if (count) ta.counters = reinterpret_cast<unsigned long long*>(s->d_work + 4);
+    }
+    // the traversal variants, and hit arrays that overlap the rays, go through ray and hit records
+    const bool records = ((ta.speculative || ta.packet) && !use8 && !use4 && !ta.any_hit && !count) ||
+                         !user_rays_apart(d_rays, d_skip, n, d_prim, d_t);
+    DevMem ro, rd, hit;
+    if (records) {
+        CR_CUDA(ro.alloc(16 * (size_t)n));
+        CR_CUDA(rd.alloc(16 * (size_t)n));
+        CR_CUDA(hit.alloc(8 * (size_t)n));
+        launch_rays_from_user(d_rays, d_skip, n, ro.as<float4>(), rd.as<float4>(), stream, lc);
+        ta.ray_o = ro.as<float4>();
+        ta.ray_d = rd.as<float4>();
+        ta.hit = hit.as<int2>();
+        if (!(o.flags & CR_OPT_PERSISTENT)) ta.work = nullptr;
+    } else {
+        ta.user.rays = d_rays;
+        ta.user.skip = d_skip;
+        ta.user.prim = d_prim;
+        ta.user.t = d_t;
+        ta.user.aligned = ((uintptr_t)d_rays & 15u) == 0;
+    }
     cudaEvent_t e0, e1;
     if (o.stats) {
         CR_CUDA(cudaEventCreate(&e0));
@@ -1167,7 +1189,7 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
     }
     launch_trace(ta, stream, lc);
     if (o.stats) CR_CUDA(cudaEventRecord(e1, stream));
-    launch_hits_to_user(tris, hit.as<int2>(), n, static_cast<int32_t*>(p_out.dev), static_cast<float*>(t_out.dev), stream, lc);
+    if (records) launch_hits_to_user(tris, hit.as<int2>(), n, d_prim, d_t, stream, lc);
     CR_CUDA(cudaGetLastError());
     CR_CUDA(finish_out(p_out, stream));
     CR_CUDA(finish_out(t_out, stream));

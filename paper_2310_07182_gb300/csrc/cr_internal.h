@@ -222,8 +222,18 @@ struct PhaseBuffers {
 // Exclusive scan of per-block counts (column 0 of 2) into offsets; total -> *total.
 void launch_scan_counts(uint32_t* block_counts, uint32_t n_blocks, uint32_t* total, cudaStream_t st);
 
-// Arguments of one trace launch over a queue of slots.
+// A caller's rays (cr_trace_rays): 8 floats each, optional skip ids, and its hit arrays.
+struct UserRays {
+    const float* rays = nullptr;
+    const int32_t* skip = nullptr;
+    int32_t* prim = nullptr;
+    float* t = nullptr;
+    bool aligned = false; // rays lie on a 16-byte boundary
+};
+
+// Arguments of one trace launch over a queue of slots, or over a caller's rays.
 struct TraceArgs {
+    UserRays user; // rays != NULL: [0, n_max) of these instead of slots (scene 0 of the table)
     const float4* ray_o = nullptr; // slot-indexed (o.xyz, skip original index as int bits)
     const float4* ray_d = nullptr; // slot-indexed (d.xyz, tmax); tmax < 0: no ray
     const int32_t* queue = nullptr;     // slots to trace; NULL = slots [0, n_max)
@@ -247,8 +257,14 @@ struct TraceArgs {
     bool bvh8 = false;
     bool bvh4 = false; // closest hits through the BVH4 (any-hit queries stay on the BVH2)
 };
+// Rays of a cr_trace_rays call above which a work counter is prepared (a GB300 has 175,104 trace lanes
+// resident; launches with fewer rays do not use the counter).
+constexpr uint32_t kTraceWorkMin = 65536;
 void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc);
 void launch_trace_bvh4(const TraceArgs& a, cudaStream_t st, LaunchCount& lc);
+// Whether trace launches may read `rays` and `skip` (NULL: none) of n rays while they write `prim`
+// and `t`: none of the arrays overlap.
+bool user_rays_apart(const float* rays, const int32_t* skip, uint32_t n, const int32_t* prim, const float* t);
 // Map leaf-order triangle indices of hits to original indices and split (prim, t).
 void launch_hits_to_user(const float4* tris, const int2* hit, uint32_t n, int32_t* prim, float* t,
                          cudaStream_t st, LaunchCount& lc);

@@ -32,47 +32,6 @@ __device__ __forceinline__ uint32_t lds(uint32_t a) {
 constexpr int kNoNode = (int)0x80000000; // no traversal left (leaf codes are all above kRefill)
 constexpr int kRefill = (int)0x80000001; // the stack's older entries wait in local memory
 constexpr int kSteps = 2;                // node visits between two votes of the warp
-constexpr uint32_t kTraceChunk = 32;     // positions a warp takes at a time
-constexpr int kTraceIdle = 8;            // idle lanes of a warp at which they get new rays
-
-// Where a warp's rays come from: positions of a list of n, kTraceChunk at a time.  A source adds
-// load() (the ray at a position; false: none there) and store() (its hit).
-// kMore: lanes whose ray has ended get further positions of the warp's range, and the warp takes
-// another range from `work` (a device counter, zero before the launch) when its own runs out.
-// Otherwise the first range is all the warp traces.
-template <bool kMore_>
-struct WarpRange {
-    static constexpr bool kMore = kMore_;
-    uint32_t n, next, end;
-    uint32_t* work;
-    uint32_t first_free; // the first position that `work` hands out
-    __device__ __forceinline__ WarpRange(uint32_t n_, uint32_t* work_) : n(n_), work(work_) {
-        const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-        next = min(w * kTraceChunk, n);
-        end = min(next + kTraceChunk, n);
-        first_free = (gridDim.x * blockDim.x >> 5) * kTraceChunk;
-    }
-    __device__ __forceinline__ bool more() const { return next < n; }
-    // The idle lanes (a mask) get the next positions in lane order, n where the range ends.
-    __device__ __forceinline__ uint32_t take(uint32_t idle) {
-        const uint32_t lane = threadIdx.x & 31u;
-        const uint32_t i = next + __popc(idle & ((1u << lane) - 1u)), e = end;
-        if (kMore) {
-            next += __popc(idle);
-            if (next >= e) {
-                next = n;
-                if (first_free < n) { // else the first ranges were all there is (a short queue)
-                    uint32_t got = 0;
-                    if (lane == 0) got = atomicAdd(work, kTraceChunk);
-                    got = __shfl_sync(0xffffffffu, got, 0);
-                    next = min(got + first_free, n);
-                    end = min(next + kTraceChunk, n);
-                }
-            }
-        }
-        return i < e ? i : n;
-    }
-};
 
 // Traversal of a warp's rays, one ray per lane; all 32 lanes call it together.
 //
@@ -181,7 +140,11 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
         if (Src::kMore && 32 - __popc(alive) >= refill) {
             fill(alive);
             alive = __ballot_sync(0xffffffffu, node != kNoNode);
-            refill = !src.more() ? 33 : alive == 0u ? 32 : kTraceIdle;
+            if (Src::kProbe) {
+                const uint32_t oct = (g.ix < 0.0f ? 1u : 0u) | (g.iy < 0.0f ? 2u : 0u) | (g.iz < 0.0f ? 4u : 0u);
+                src.probe(node != kNoNode, oct);
+            }
+            refill = !src.more() ? 33 : alive == 0u ? 32 : src.idle;
             if (alive == 0u && refill == 32) continue; // the positions taken held no rays
         }
         if (alive == 0u) {
@@ -234,34 +197,6 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
     }
 }
 
-// Rays of a queue of slots (or of the slots in order), hits per slot.
-template <bool kMore>
-struct QueueSrc : WarpRange<kMore> {
-    const uint16_t* __restrict__ slot_scene;
-    const float4* __restrict__ ray_o;
-    const float4* __restrict__ ray_d;
-    const int32_t* __restrict__ queue;
-    int2* __restrict__ hit;
-    __device__ __forceinline__ QueueSrc(uint32_t n, uint32_t* work, const uint16_t* ss, const float4* o, const float4* d,
-                                        const int32_t* q, int2* h)
-        : WarpRange<kMore>(n, work), slot_scene(ss), ray_o(o), ray_d(d), queue(q), hit(h) {}
-    __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) const {
-        const int slot = queue ? queue[i] : (int)i;
-        ro = ray_o[slot];
-        rd = ray_d[slot];
-        if (!(rd.w >= 0.0f)) {
-            hit[slot] = make_int2(-1, __float_as_int(INFINITY));
-            return false;
-        }
-        key = slot;
-        return true;
-    }
-    __device__ __forceinline__ uint32_t scene(int key) const { return slot_scene ? slot_scene[key] : 0u; }
-    __device__ __forceinline__ void store(int key, int leaf, float t, const float4*) const {
-        hit[key] = make_int2(leaf, __float_as_int(t));
-    }
-};
-
 #ifndef CR_TRACE_MAXNREG
 #define CR_TRACE_MAXNREG 56 // 36 warps resident per SM, no spills; 48 and 64 are within 1%, 40 costs 4%
 #endif
@@ -280,16 +215,21 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __res
     unsigned long long n_node = 0, n_tri = 0;
     QueueSrc<kMore> src(n, work, slot_scene, ray_o, ray_d, queue, hit);
     if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemS, kOne>(scenes, src, smem_stack, n_node, n_tri);
-    if (kCount) {
-        for (int off = 16; off > 0; off >>= 1) {
-            n_node += __shfl_down_sync(0xffffffffu, n_node, off);
-            n_tri += __shfl_down_sync(0xffffffffu, n_tri, off);
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicAdd(&counters[0], n_node);
-            atomicAdd(&counters[1], n_tri);
-        }
-    }
+    if (kCount) add_counts(counters, n_node, n_tri);
+}
+
+// A caller's rays and hit arrays, no scratch between: cr_trace_rays used to copy the rays into the
+// render path's records, trace, and copy the hits out, in buffers allocated per call (1M surface
+// rays 952 us against 503, 300k camera rays 456 against 146, 1,000 rays 69 against 51).
+template <bool kCount, bool kAny, bool kMore>
+__global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_user(const SceneDev* __restrict__ scene, UserRays rays,
+                                                                uint32_t n, unsigned long long* counters,
+                                                                uint32_t* work) {
+    extern __shared__ uint32_t smem_stack[];
+    unsigned long long n_node = 0, n_tri = 0;
+    UserSrc<kMore> src(n, work, rays);
+    if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemStack, true>(scene, src, smem_stack, n_node, n_tri);
+    if (kCount) add_counts(counters, n_node, n_tri);
 }
 
 // Two-phase variant: phase 1 traverses every ray for at most `budget` node and leaf visits;
@@ -624,6 +564,9 @@ struct ShadowSrc : WarpRange<kMore> {
     const int32_t* __restrict__ group_queue;
     float4* __restrict__ radiance;
     uint32_t K, traced;
+    static constexpr int idle = kTraceIdle;
+    static constexpr bool kProbe = false;
+    __device__ __forceinline__ void probe(bool, uint32_t) {}
     __device__ __forceinline__ ShadowSrc(uint32_t n, uint32_t* work) : WarpRange<kMore>(n, work) {}
     __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) {
         const uint32_t g = group_queue ? (uint32_t)group_queue[i / K] : i / K;
@@ -742,6 +685,16 @@ void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, cons
     lc.n++;
 }
 
+bool user_rays_apart(const float* rays, const int32_t* skip, uint32_t n, const int32_t* prim, const float* t) {
+    const auto apart = [](const void* a, size_t na, const void* b, size_t nb) {
+        const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+        return x + na <= y || y + nb <= x;
+    };
+    const size_t w = 4 * (size_t)n;
+    return apart(rays, 8 * w, prim, w) && apart(rays, 8 * w, t, w) && apart(prim, w, t, w) &&
+           (!skip || (apart(skip, w, prim, w) && apart(skip, w, t, w)));
+}
+
 void launch_rays_from_user(const float* rays, const int32_t* skip, uint32_t n, float4* ray_o, float4* ray_d,
                            cudaStream_t st, LaunchCount& lc) {
     if (n == 0) return;
@@ -807,8 +760,26 @@ static void launch_bvh2(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     else launch_bvh2_scenes<false, kCount, kAny, kSmemS>(a, st, lc);
 }
 
+template <bool kCount, bool kAny>
+static void launch_bvh2_user(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
+    const size_t smem = (size_t)kSmemStack * a.block * sizeof(uint32_t);
+    const uint32_t need = blocks_for(a.n_max, a.block);
+    const uint32_t most = a.work ? resident_blocks<k_trace_bvh2_user<kCount, kAny, true>>(a.block, smem) : 0u;
+    if (most && need > most)
+        k_trace_bvh2_user<kCount, kAny, true><<<most, a.block, smem, st>>>(a.scenes, a.user, a.n_max, a.counters, a.work);
+    else
+        k_trace_bvh2_user<kCount, kAny, false><<<need, a.block, smem, st>>>(a.scenes, a.user, a.n_max, a.counters, nullptr);
+    lc.n++;
+}
+
 void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     if (a.n_max == 0) return;
+    if (a.user.rays && !a.bvh8 && !(a.bvh4 && !a.any_hit)) { // a caller's rays through the BVH2
+        if (a.any_hit) launch_bvh2_user<false, true>(a, st, lc);
+        else if (a.counters) launch_bvh2_user<true, false>(a, st, lc);
+        else launch_bvh2_user<false, false>(a, st, lc);
+        return;
+    }
     const int block = a.block;
     const size_t smem = (size_t)kSmemStack * block * sizeof(uint32_t);
     if (a.bvh8) { // BVH8-Q kernels (trace_bvh8.cu)

@@ -130,6 +130,22 @@ __device__ __forceinline__ int2 trace_bvh4_one(const float4* __restrict__ nodes,
     return make_int2(best.leaf, __float_as_int(best.t));
 }
 
+// One ray per lane of a queue or of a caller's rays.
+template <bool kCount, class Src>
+__device__ __forceinline__ void trace_bvh4_rays(const SceneDev* __restrict__ scenes, Src src, uint32_t* smem,
+                                                unsigned long long* counters) {
+    unsigned long long n_node = 0, n_tri = 0;
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    int key = -1;
+    float4 ro, rd;
+    if (i < src.n && src.load(i, key, ro, rd)) {
+        const SceneDev& sc = scenes[src.scene(key)];
+        const int2 h = trace_bvh4_one<kCount>(sc.nodes4, sc.tris, ro, rd, smem + threadIdx.x, n_node, n_tri, &sc);
+        src.store(key, h.x, __int_as_float(h.y), sc.tris);
+    }
+    if (kCount) add_counts(counters, n_node, n_tri);
+}
+
 template <bool kCount>
 __global__ void __maxnreg__(CR_TRACE4_MAXNREG) k_trace_bvh4(const SceneDev* __restrict__ scenes,
                                                              const uint16_t* __restrict__ slot_scene,
@@ -140,28 +156,14 @@ __global__ void __maxnreg__(CR_TRACE4_MAXNREG) k_trace_bvh4(const SceneDev* __re
                                                              int2* __restrict__ hit, unsigned long long* counters) {
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long n_node = 0, n_tri = 0;
-    if (i < n) {
-        const int slot = queue ? queue[i] : (int)i;
-        const SceneDev& sc = scenes[slot_scene ? slot_scene[slot] : 0];
-        const float4 ro = ray_o[slot];
-        const float4 rd = ray_d[slot];
-        int2 h = make_int2(-1, __float_as_int(INFINITY));
-        if (rd.w >= 0.0f)
-            h = trace_bvh4_one<kCount>(sc.nodes4, sc.tris, ro, rd, smem_stack + threadIdx.x, n_node, n_tri, &sc);
-        hit[slot] = h;
-    }
-    if (kCount) {
-        for (int off = 16; off > 0; off >>= 1) {
-            n_node += __shfl_down_sync(0xffffffffu, n_node, off);
-            n_tri += __shfl_down_sync(0xffffffffu, n_tri, off);
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicAdd(&counters[0], n_node);
-            atomicAdd(&counters[1], n_tri);
-        }
-    }
+    trace_bvh4_rays<kCount>(scenes, QueueSrc<false>(n, nullptr, slot_scene, ray_o, ray_d, queue, hit), smem_stack, counters);
+}
+
+template <bool kCount>
+__global__ void __maxnreg__(CR_TRACE4_MAXNREG) k_trace_bvh4_user(const SceneDev* __restrict__ scene, UserRays rays,
+                                                                 uint32_t n, unsigned long long* counters) {
+    extern __shared__ uint32_t smem_stack[];
+    trace_bvh4_rays<kCount>(scene, UserSrc<false>(n, nullptr, rays), smem_stack, counters);
 }
 
 } // namespace
@@ -172,7 +174,11 @@ void launch_trace_bvh4(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     const int block = a.block;
     const uint32_t grid = (a.n_max + block - 1) / block;
     const size_t smem = (size_t)block * kSmemStack * sizeof(uint32_t);
-    if (a.counters)
+    if (a.user.rays && a.counters)
+        k_trace_bvh4_user<true><<<grid, block, smem, st>>>(a.scenes, a.user, a.n_max, a.counters);
+    else if (a.user.rays)
+        k_trace_bvh4_user<false><<<grid, block, smem, st>>>(a.scenes, a.user, a.n_max, nullptr);
+    else if (a.counters)
         k_trace_bvh4<true><<<grid, block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue, a.queue_count,
                                                        a.n_max, a.hit, a.counters);
     else

@@ -173,6 +173,22 @@ __device__ __forceinline__ int2 trace_bvh8_one(const uint4* __restrict__ nodes, 
 #define CR_BVH8_MIN_BLOCKS 8 // resident 128-thread blocks per SM the register budget is sized for
 #endif
 
+// One ray per lane of a queue or of a caller's rays.
+template <bool kCount, bool kAny, class Src>
+__device__ __forceinline__ void trace_bvh8_rays(const SceneDev* __restrict__ scenes, Src src,
+                                                unsigned long long* counters) {
+    unsigned long long n_node = 0, n_tri = 0;
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    int key = -1;
+    float4 ro, rd;
+    if (i < src.n && src.load(i, key, ro, rd)) {
+        const SceneDev& sc = scenes[src.scene(key)];
+        const int2 h = trace_bvh8_one<kCount, kAny>(sc.nodes8, sc.tris, ro, rd, n_node, n_tri, &sc);
+        src.store(key, h.x, __int_as_float(h.y), sc.tris);
+    }
+    if (kCount) add_counts(counters, n_node, n_tri);
+}
+
 template <bool kCount, bool kAny = false>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8(const SceneDev* __restrict__ scenes,
                              const uint16_t* __restrict__ slot_scene,
@@ -180,27 +196,14 @@ __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8(const Sc
                              const int32_t* __restrict__ queue, const uint32_t* __restrict__ queue_count,
                              uint32_t n_max, int2* __restrict__ hit, unsigned long long* counters) {
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long n_node = 0, n_tri = 0;
-    if (i < n) {
-        const int slot = queue ? queue[i] : (int)i;
-        const SceneDev& sc = scenes[slot_scene ? slot_scene[slot] : 0];
-        const float4 ro = ray_o[slot];
-        const float4 rd = ray_d[slot];
-        int2 h = make_int2(-1, __float_as_int(INFINITY));
-        if (rd.w >= 0.0f) h = trace_bvh8_one<kCount, kAny>(sc.nodes8, sc.tris, ro, rd, n_node, n_tri, &sc);
-        hit[slot] = h;
-    }
-    if (kCount) {
-        for (int off = 16; off > 0; off >>= 1) {
-            n_node += __shfl_down_sync(0xffffffffu, n_node, off);
-            n_tri += __shfl_down_sync(0xffffffffu, n_tri, off);
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicAdd(&counters[0], n_node);
-            atomicAdd(&counters[1], n_tri);
-        }
-    }
+    trace_bvh8_rays<kCount, kAny>(scenes, QueueSrc<false>(n, nullptr, slot_scene, ray_o, ray_d, queue, hit), counters);
+}
+
+template <bool kCount, bool kAny = false>
+__global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8_user(const SceneDev* __restrict__ scene,
+                                                                             UserRays rays, uint32_t n,
+                                                                             unsigned long long* counters) {
+    trace_bvh8_rays<kCount, kAny>(scene, UserSrc<false>(n, nullptr, rays), counters);
 }
 
 // Shadow rays of next-event estimation over the BVH8-Q, one thread per position of the last shade's group
@@ -243,7 +246,13 @@ void launch_trace_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     const int block = a.block;
     const size_t smem = 0;
     const uint32_t grid = (a.n_max + block - 1) / block;
-    if (a.any_hit)
+    if (a.user.rays && a.any_hit)
+        k_trace_bvh8_user<false, true><<<grid, block, smem, st>>>(a.scenes, a.user, a.n_max, nullptr);
+    else if (a.user.rays && a.counters)
+        k_trace_bvh8_user<true><<<grid, block, smem, st>>>(a.scenes, a.user, a.n_max, a.counters);
+    else if (a.user.rays)
+        k_trace_bvh8_user<false><<<grid, block, smem, st>>>(a.scenes, a.user, a.n_max, nullptr);
+    else if (a.any_hit)
         k_trace_bvh8<false, true><<<grid, block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
                                                              a.queue_count, a.n_max, a.hit, nullptr);
     else if (a.counters)

@@ -307,5 +307,130 @@ __device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, const
         }                                                                            \
     } while (0)
 
+// ------------------------------------------------------------------------------------
+// Ray sources of the trace kernels.
+constexpr uint32_t kTraceChunk = 32; // positions a warp takes at a time
+constexpr int kTraceIdle = 8;        // idle lanes of a warp at which they get new rays
+
+// Where a warp's rays come from: positions of a list of n, kTraceChunk at a time.  A source adds
+// load() (the ray at a position; false: none there) and store() (its hit).
+// kMore: lanes whose ray has ended get further positions of the warp's range, and the warp takes
+// another range from `work` (a device counter, zero before the launch) when its own runs out.
+// Otherwise the first range is all the warp traces.
+template <bool kMore_>
+struct WarpRange {
+    static constexpr bool kMore = kMore_;
+    uint32_t n, next, end;
+    uint32_t* work;
+    uint32_t first_free; // the first position that `work` hands out
+    __device__ __forceinline__ WarpRange(uint32_t n_, uint32_t* work_) : n(n_), work(work_) {
+        const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+        next = min(w * kTraceChunk, n);
+        end = min(next + kTraceChunk, n);
+        first_free = (gridDim.x * blockDim.x >> 5) * kTraceChunk;
+    }
+    __device__ __forceinline__ bool more() const { return next < n; }
+    // The idle lanes (a mask) get the next positions in lane order, n where the range ends.
+    __device__ __forceinline__ uint32_t take(uint32_t idle) {
+        const uint32_t lane = threadIdx.x & 31u;
+        const uint32_t i = next + __popc(idle & ((1u << lane) - 1u)), e = end;
+        if (kMore) {
+            next += __popc(idle);
+            if (next >= e) {
+                next = n;
+                if (first_free < n) { // else the first ranges were all there is (a short queue)
+                    uint32_t got = 0;
+                    if (lane == 0) got = atomicAdd(work, kTraceChunk);
+                    got = __shfl_sync(0xffffffffu, got, 0);
+                    next = min(got + first_free, n);
+                    end = min(next + kTraceChunk, n);
+                }
+            }
+        }
+        return i < e ? i : n;
+    }
+};
+
+// Rays of a queue of slots (or of the slots in order), hits per slot.
+template <bool kMore>
+struct QueueSrc : WarpRange<kMore> {
+    const uint16_t* __restrict__ slot_scene;
+    const float4* __restrict__ ray_o;
+    const float4* __restrict__ ray_d;
+    const int32_t* __restrict__ queue;
+    int2* __restrict__ hit;
+    static constexpr int idle = kTraceIdle;
+    static constexpr bool kProbe = false;
+    __device__ __forceinline__ void probe(bool, uint32_t) {}
+    __device__ __forceinline__ QueueSrc(uint32_t n, uint32_t* work, const uint16_t* ss, const float4* o, const float4* d,
+                                        const int32_t* q, int2* h)
+        : WarpRange<kMore>(n, work), slot_scene(ss), ray_o(o), ray_d(d), queue(q), hit(h) {}
+    __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) const {
+        const int slot = queue ? queue[i] : (int)i;
+        ro = ray_o[slot];
+        rd = ray_d[slot];
+        if (!(rd.w >= 0.0f)) {
+            hit[slot] = make_int2(-1, __float_as_int(INFINITY));
+            return false;
+        }
+        key = slot;
+        return true;
+    }
+    __device__ __forceinline__ uint32_t scene(int key) const { return slot_scene ? slot_scene[key] : 0u; }
+    __device__ __forceinline__ void store(int key, int leaf, float t, const float4*) const {
+        hit[key] = make_int2(leaf, __float_as_int(t));
+    }
+};
+
+// A caller's rays (8 floats each), optional skip ids and hit arrays.
+template <bool kMore>
+struct UserSrc : WarpRange<kMore>, UserRays {
+    int idle = kTraceIdle;
+    // A warp whose rays all run into one octant is taken for a coherent one (camera rays), whose
+    // rays end together: it gets new rays only when all of its own have ended (the rule of
+    // the render path's camera rays, which the caller's list does not say).
+    static constexpr bool kProbe = true;
+    __device__ __forceinline__ void probe(bool live, uint32_t oct) {
+        idle = __popc(__reduce_or_sync(0xffffffffu, live ? 1u << oct : 0u)) <= 1 ? 32 : kTraceIdle;
+    }
+    __device__ __forceinline__ UserSrc(uint32_t n, uint32_t* work, const UserRays& u) : WarpRange<kMore>(n, work), UserRays(u) {}
+    __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) const {
+        const float* r = rays + 8 * (size_t)i;
+        if (aligned) {
+            ro = *reinterpret_cast<const float4*>(r);
+            rd = *reinterpret_cast<const float4*>(r + 4);
+        } else {
+            ro = make_float4(r[0], r[1], r[2], 0.0f);
+            rd = make_float4(r[4], r[5], r[6], r[7]);
+        }
+        ro.w = __int_as_float(skip ? skip[i] : -1);
+        if (!(rd.w >= 0.0f)) {
+            prim[i] = -1;
+            t[i] = INFINITY;
+            return false;
+        }
+        key = (int)i;
+        return true;
+    }
+    __device__ __forceinline__ uint32_t scene(int) const { return 0u; }
+    __device__ __forceinline__ void store(int key, int leaf, float tt, const float4* __restrict__ tris) const {
+        prim[key] = leaf >= 0 ? __float_as_int(__ldg(&tris[3 * leaf]).w) : -1;
+        t[key] = leaf >= 0 ? tt : INFINITY; // a miss of a bounded ray reports inf, not tmax
+    }
+};
+
+// Node visits and triangle tests of a counting pass, summed over the warp.
+__device__ __forceinline__ void add_counts(unsigned long long* counters, unsigned long long n_node,
+                                           unsigned long long n_tri) {
+    for (int off = 16; off > 0; off >>= 1) {
+        n_node += __shfl_down_sync(0xffffffffu, n_node, off);
+        n_tri += __shfl_down_sync(0xffffffffu, n_tri, off);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&counters[0], n_node);
+        atomicAdd(&counters[1], n_tri);
+    }
+}
+
 } // namespace
 } // namespace cr

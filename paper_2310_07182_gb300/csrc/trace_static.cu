@@ -1,12 +1,13 @@
 // trace_static.cu -- closest-hit tracing that allocates nothing.
 //
-// cr_trace_rays stages its rays and hits through device buffers it allocates per call.
-// Some callers cannot allow that: a host framework that owns all device memory through its
+// cr_trace_rays may allocate device buffers (for host arrays, traversal variants, and hits that
+// overwrite the rays).  Some callers cannot allow that: a host framework that owns all device memory through its
 // own pool allocator and forbids raw cudaMalloc, a latency-critical loop that cannot afford
 // the implicit device synchronisation of cudaMalloc/cudaFree, or a process that has already
 // reserved nearly all device memory so an allocation could fail mid-frame.  For them this
-// file keeps the trace kernel's scratch (ray origin/direction records and hit records for up
-// to CR_TRACE_STATIC_MAX_RAYS rays, 40 bytes each) in one file-scope __device__ array.  Every
+// call traces straight from the caller's rays into its hit arrays; only where these overlap do ray
+// origin/direction and hit records (up
+// to CR_TRACE_STATIC_MAX_RAYS rays, 40 bytes each) lie between, in one file-scope __device__ array.  Every
 // GPU that loads the library holds that array until the process exits.
 #include <cuda_runtime.h>
 
@@ -96,32 +97,42 @@ extern "C" cr_status cr_trace_rays_static(cr_scene* scene, const float* rays, co
         set_last_error("cr_trace_rays_static: rays, skip_prim, prim and t must be device pointers of the current device");
         return CR_ERR_INVALID_ARG;
     }
-    void* base = nullptr;
-    cudaError_t e = scratch_on_current_device(&base);
-    if (e != cudaSuccess) {
-        snprintf(msg, sizeof(msg), "cr_trace_rays_static: cudaGetSymbolAddress: %s", cudaGetErrorString(e));
-        set_last_error(msg);
-        return CR_ERR_CUDA;
-    }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    unsigned char* b = static_cast<unsigned char*>(base);
-    float4* ro = reinterpret_cast<float4*>(b + kOffRayO);
-    float4* rd = reinterpret_cast<float4*>(b + kOffRayD);
-    int2* hit = reinterpret_cast<int2*>(b + kOffHit);
-    const DevScene& ds = *dev_scene_of(scene);
+    cudaError_t e = cudaSuccess;
     LaunchCount lc;
     // the scene's device table entry was made by cr_scene_create, so nothing is allocated here
-    // every scratch record read below is written first by this call, so nothing needs clearing
-    launch_rays_from_user(rays, skip_prim, n, ro, rd, st, lc);
     TraceArgs ta;
-    ta.ray_o = ro;
-    ta.ray_d = rd;
-    ta.hit = hit;
     ta.n_max = n;
     ta.block = 128;
     ta.scenes = dev_scene_entry(scene, false);
-    launch_trace(ta, st, lc);
-    launch_hits_to_user(ds.tris, hit, n, prim, t, st, lc);
+    ta.one_scene = true;
+    if (user_rays_apart(rays, skip_prim, n, prim, t)) {
+        ta.user.rays = rays;
+        ta.user.skip = skip_prim;
+        ta.user.prim = prim;
+        ta.user.t = t;
+        ta.user.aligned = ((uintptr_t)rays & 15u) == 0;
+        launch_trace(ta, st, lc);
+    } else { // hits that overwrite the rays: through the scratch
+        void* base = nullptr;
+        e = scratch_on_current_device(&base);
+        if (e != cudaSuccess) {
+            snprintf(msg, sizeof(msg), "cr_trace_rays_static: cudaGetSymbolAddress: %s", cudaGetErrorString(e));
+            set_last_error(msg);
+            return CR_ERR_CUDA;
+        }
+        unsigned char* b = static_cast<unsigned char*>(base);
+        float4* ro = reinterpret_cast<float4*>(b + kOffRayO);
+        float4* rd = reinterpret_cast<float4*>(b + kOffRayD);
+        int2* hit = reinterpret_cast<int2*>(b + kOffHit);
+        // every scratch record read below is written first by this call, so nothing needs clearing
+        launch_rays_from_user(rays, skip_prim, n, ro, rd, st, lc);
+        ta.ray_o = ro;
+        ta.ray_d = rd;
+        ta.hit = hit;
+        launch_trace(ta, st, lc);
+        launch_hits_to_user(dev_scene_of(scene)->tris, hit, n, prim, t, st, lc);
+    }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {

@@ -59,13 +59,23 @@ def test_far_origins_and_every_layout_agree(cr, far, n_rays):
 @pytest.mark.parametrize("dead", ["none", "some", "runs", "all"])
 def test_lanes_that_take_new_rays(cr, n_rays, dead):
     """Rays handed out lane by lane (more of them than lanes resident at once, chunks without any
-    ray, single dead rays) give the hits of one ray per lane."""
-    S = cr.Scene(scenes.tiny(seed=5, n_soup=700, material_mix="mixed"))
+    ray, single dead rays), read from aligned and unaligned lists, give the hits of one ray per
+    lane through the BVH8-Q; so do hits that are written over the rays."""
+    S = cr.Scene(scenes.tiny(seed=5, n_soup=700, material_mix="mixed"), bvh_flags=cr.CR_BVH2 | cr.CR_BVH8Q)
     rays = torch.from_numpy(scenes.random_rays(7, n_rays)).cuda()
     i = torch.arange(n_rays, device="cuda")
     off = {"none": i < 0, "some": i % 5 == 2, "runs": (i // 96) % 3 != 0, "all": i >= 0}[dead]
     rays[off, 7] = -1.0
-    want_p, want_t = S.trace(rays)
-    got_p, got_t = S.trace(rays, flags=cr.CR_OPT_PERSISTENT)
-    assert torch.equal(want_p, got_p) and torch.equal(want_t, got_t)
-    assert (got_p[off] == -1).all() and (n_rays < 100 or dead in ("all",) or (got_p >= 0).any())
+    want_p, want_t = S.trace(rays, bvh=cr.CR_BVH8Q)
+    moved = torch.empty(8 * n_rays + 1, device="cuda")[1:].view(n_rays, 8)
+    moved.copy_(rays)
+    for r in (rays, moved):
+        for flags in (0, cr.CR_OPT_PERSISTENT):
+            got_p, got_t = S.trace(r, flags=flags)
+            assert torch.equal(want_p, got_p) and torch.equal(want_t, got_t)
+    assert (want_p[off] == -1).all() and (n_rays < 100 or dead == "all" or (want_p >= 0).any())
+    over = rays.clone().view(-1)
+    cr.cr_trace_rays(S.handle, over.view(n_rays, 8), None, over[:n_rays].view(torch.int32), over[n_rays:2 * n_rays],
+                     cr.make_opts())
+    assert torch.equal(want_p, over[:n_rays].view(torch.int32)) and torch.equal(want_t, over[n_rays:2 * n_rays])
+    assert bool(((want_p >= 0) == (S.trace(rays, any_hit=True)[0] >= 0)).all())
