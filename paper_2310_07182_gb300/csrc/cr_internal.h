@@ -321,7 +321,7 @@ void launch_trace_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc);
 void launch_shadow_rays_bvh8(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o,
                              const float4* sh_d, const float4* sh_c, const int32_t* group_queue,
                              const uint32_t* group_count, uint32_t n_groups_max, uint32_t K, float4* radiance,
-                             unsigned long long* n_traced, cudaStream_t st, LaunchCount& lc);
+                             unsigned long long* n_traced, uint32_t* work, cudaStream_t st, LaunchCount& lc);
 void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
                         const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count,
                         uint32_t n_groups_max, uint32_t K, float4* radiance, unsigned long long* n_traced, bool bvh8,

@@ -10,7 +10,6 @@
 // are in trace_common.cuh.
 #include <cuda_runtime.h>
 
-#include <atomic>
 #include <type_traits>
 
 #include "cr_internal.h"
@@ -551,42 +550,6 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_spec(
     }
 }
 
-// Shadow rays of next-event estimation, by position of the last shade's group queue (so a
-// reuse group's rays run in adjacent lanes, as they were shaded).  A ray whose
-// direction record has w = tmax > 0 is traced for visibility only; if nothing blocks it, its
-// contribution is added to the path radiance of its slot.  Rays traced are counted.
-template <bool kMore>
-struct ShadowSrc : WarpRange<kMore> {
-    const uint16_t* __restrict__ slot_scene;
-    const float4* __restrict__ sh_o;
-    const float4* __restrict__ sh_d;
-    const float4* __restrict__ sh_c;
-    const int32_t* __restrict__ group_queue;
-    float4* __restrict__ radiance;
-    uint32_t K, traced;
-    static constexpr int idle = kTraceIdle;
-    static constexpr bool kProbe = false;
-    __device__ __forceinline__ void probe(bool, uint32_t) {}
-    __device__ __forceinline__ ShadowSrc(uint32_t n, uint32_t* work) : WarpRange<kMore>(n, work) {}
-    __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) {
-        const uint32_t g = group_queue ? (uint32_t)group_queue[i / K] : i / K;
-        const int slot = (int)(g * K + i % K);
-        rd = sh_d[slot];
-        if (!(rd.w > 0.0f)) return false;
-        ro = sh_o[slot];
-        key = slot;
-        ++traced;
-        return true;
-    }
-    __device__ __forceinline__ uint32_t scene(int key) const { return slot_scene[key]; }
-    __device__ __forceinline__ void store(int key, int leaf, float, const float4*) const {
-        if (leaf >= 0) return;
-        const float4 c = sh_c[key];
-        const float4 L = radiance[key];
-        radiance[key] = make_float4(__fadd_rn(L.x, c.x), __fadd_rn(L.y, c.y), __fadd_rn(L.z, c.z), L.w);
-    }
-};
-
 template <bool kOne, bool kMore>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
     const SceneDev* __restrict__ scenes, const uint16_t* __restrict__ slot_scene, const float4* __restrict__ sh_o,
@@ -595,20 +558,11 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
     unsigned long long* __restrict__ n_traced, uint32_t* work) {
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
-    ShadowSrc<kMore> src(n, work);
+    ShadowSrc<kMore> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
     if (!src.more()) return;
-    src.slot_scene = slot_scene;
-    src.sh_o = sh_o;
-    src.sh_d = sh_d;
-    src.sh_c = sh_c;
-    src.group_queue = group_queue;
-    src.radiance = radiance;
-    src.K = K;
-    src.traced = 0u;
     unsigned long long dn = 0, dt = 0;
     trace_bvh2_warp<false, true, kSmemStack, kOne>(scenes, src, smem_stack, dn, dt);
-    const uint32_t b = __reduce_add_sync(0xffffffffu, src.traced);
-    if ((threadIdx.x & 31) == 0 && b) atomicAdd(n_traced, (unsigned long long)b);
+    src.add_traced(n_traced);
 }
 
 __global__ void k_hits_to_user(const float4* __restrict__ tris, const int2* __restrict__ hit, uint32_t n,
@@ -631,29 +585,6 @@ __global__ void k_rays_from_user(const float* __restrict__ rays, const int32_t* 
 
 } // namespace
 
-// Blocks of a trace kernel that are resident on the current device at once (0: unknown).
-template <auto kKernel>
-static uint32_t resident_blocks(int block, size_t smem) {
-    // per device and block size (block sizes are multiples of 32 up to 512)
-    static std::atomic<uint32_t> known[64][17];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    std::atomic<uint32_t>& r = known[dev][block / 32];
-    uint32_t v = r.load(std::memory_order_relaxed);
-    if (!v) {
-        int sms = 0, nb = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kKernel, block, smem) != cudaSuccess || sms <= 0 || nb <= 0)
-            return 0;
-        v = (uint32_t)sms * (uint32_t)nb;
-        r.store(v, std::memory_order_relaxed);
-    }
-    return v;
-}
-
-// Blocks for n positions, one per lane.
-static uint32_t blocks_for(uint32_t n, int block) { return n / (uint32_t)block + (n % (uint32_t)block ? 1u : 0u); }
-
 void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
                         const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count,
                         uint32_t n_groups_max, uint32_t K, float4* radiance, unsigned long long* n_traced, bool bvh8,
@@ -662,7 +593,7 @@ void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, cons
     if (n_pos == 0) return;
     if (bvh8) {
         launch_shadow_rays_bvh8(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count, n_groups_max, K,
-                                radiance, n_traced, st, lc);
+                                radiance, n_traced, work, st, lc);
         return;
     }
     const int block = kSecondaryBlock;

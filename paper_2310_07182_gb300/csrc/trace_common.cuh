@@ -10,6 +10,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "cr_internal.h"
 #include "debug_checks.cuh"
 
@@ -419,6 +421,48 @@ struct UserSrc : WarpRange<kMore>, UserRays {
     }
 };
 
+// Shadow rays of next-event estimation, by position of the last shade's group queue (so a
+// reuse group's rays run in adjacent lanes, as they were shaded).  A ray whose
+// direction record has w = tmax > 0 is traced for visibility only; if nothing blocks it, its
+// contribution is added to the path radiance of its slot.  Rays traced are counted.
+template <bool kMore>
+struct ShadowSrc : WarpRange<kMore> {
+    const uint16_t* __restrict__ slot_scene;
+    const float4* __restrict__ sh_o;
+    const float4* __restrict__ sh_d;
+    const float4* __restrict__ sh_c;
+    const int32_t* __restrict__ group_queue;
+    float4* __restrict__ radiance;
+    uint32_t K, traced = 0;
+    static constexpr int idle = kTraceIdle;
+    static constexpr bool kProbe = false;
+    __device__ __forceinline__ void probe(bool, uint32_t) {}
+    __device__ __forceinline__ ShadowSrc(uint32_t n, uint32_t* work, const uint16_t* ss, const float4* o, const float4* d,
+                                         const float4* c, const int32_t* gq, float4* rad, uint32_t k)
+        : WarpRange<kMore>(n, work), slot_scene(ss), sh_o(o), sh_d(d), sh_c(c), group_queue(gq), radiance(rad), K(k) {}
+    __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) {
+        const uint32_t g = group_queue ? (uint32_t)group_queue[i / K] : i / K;
+        const int slot = (int)(g * K + i % K);
+        rd = sh_d[slot];
+        if (!(rd.w > 0.0f)) return false;
+        ro = sh_o[slot];
+        key = slot;
+        ++traced;
+        return true;
+    }
+    __device__ __forceinline__ uint32_t scene(int key) const { return slot_scene[key]; }
+    __device__ __forceinline__ void store(int key, int leaf, float, const float4*) const {
+        if (leaf >= 0) return;
+        const float4 c = sh_c[key];
+        const float4 L = radiance[key];
+        radiance[key] = make_float4(__fadd_rn(L.x, c.x), __fadd_rn(L.y, c.y), __fadd_rn(L.z, c.z), L.w);
+    }
+    __device__ __forceinline__ void add_traced(unsigned long long* n_traced) const {
+        const uint32_t b = __reduce_add_sync(0xffffffffu, traced);
+        if ((threadIdx.x & 31) == 0 && b) atomicAdd(n_traced, (unsigned long long)b);
+    }
+};
+
 // Node visits and triangle tests of a counting pass, summed over the warp.
 __device__ __forceinline__ void add_counts(unsigned long long* counters, unsigned long long n_node,
                                            unsigned long long n_tri) {
@@ -431,6 +475,29 @@ __device__ __forceinline__ void add_counts(unsigned long long* counters, unsigne
         atomicAdd(&counters[1], n_tri);
     }
 }
+
+// Blocks of a trace kernel that are resident on the current device at once (0: unknown).
+template <auto kKernel>
+static uint32_t resident_blocks(int block, size_t smem) {
+    // per device and block size (block sizes are multiples of 32 up to 512)
+    static std::atomic<uint32_t> known[64][17];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    std::atomic<uint32_t>& r = known[dev][block / 32];
+    uint32_t v = r.load(std::memory_order_relaxed);
+    if (!v) {
+        int sms = 0, nb = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kKernel, block, smem) != cudaSuccess || sms <= 0 || nb <= 0)
+            return 0;
+        v = (uint32_t)sms * (uint32_t)nb;
+        r.store(v, std::memory_order_relaxed);
+    }
+    return v;
+}
+
+// Blocks for n positions, one per lane.
+static uint32_t blocks_for(uint32_t n, int block) { return n / (uint32_t)block + (n % (uint32_t)block ? 1u : 0u); }
 
 } // namespace
 } // namespace cr
