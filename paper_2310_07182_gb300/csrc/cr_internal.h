@@ -247,6 +247,7 @@ struct TraceArgs {
     // theirs end (BVH2); NULL: one ray per lane
     uint32_t* work = nullptr;
     bool one_scene = false; // every ray is in scenes[0]
+    bool alone = true;      // no other launches of the library run beside this one
     int block = 128;
     bool speculative = false; // parked-leaf speculative traversal (BVH2)
     bool packet = false;      // warp-packet traversal (BVH2)
@@ -325,7 +326,8 @@ void launch_shadow_rays_bvh8(const SceneDev* scenes, const uint16_t* slot_scene,
 void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
                         const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count,
                         uint32_t n_groups_max, uint32_t K, float4* radiance, unsigned long long* n_traced, bool bvh8,
-                        bool one_scene, uint32_t* work, cudaStream_t st, LaunchCount& lc);
+                        bool one_scene, bool alone, uint32_t* work, cudaStream_t st,
+                        LaunchCount& lc);
 
 void launch_raygen(const PassArgs& p, PathBuffers& b, cudaStream_t st, LaunchCount& lc);
 // raygen leaves the primary trace's visiting order (row-major pixels per tile) in the ray queue

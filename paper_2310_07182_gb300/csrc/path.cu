@@ -1708,7 +1708,7 @@ void launch_shadow(const PassArgs& p, PathBuffers& b, bool first, bool bvh8, cud
     const ShadeArgs a = shade_args(p, b, first, false, nullptr);
     launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
                        a.n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
-                       bvh8, p.one_scene, b.counts + kWorkWord + 32 + p.bounce, st, lc);
+                       bvh8, p.one_scene, true, b.counts + kWorkWord + 32 + p.bounce, st, lc);
 }
 
 void launch_shade(const PassArgs& p, PathBuffers& b, bool first, bool compact, const cr_debug* dbg,
@@ -1772,7 +1772,7 @@ void launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, u
     const ShadeArgs a = shade_args_rolling(p, b, parity, n_groups_max);
     launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
                        n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
-                       bvh8, p.one_scene, b.counts + 8 + 4 * (parity ^ 1u) + 3, st, lc);
+                       bvh8, p.one_scene, false, b.counts + 8 + 4 * (parity ^ 1u) + 3, st, lc);
 }
 
 void launch_finish_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_slots, cudaStream_t st, LaunchCount& lc) {

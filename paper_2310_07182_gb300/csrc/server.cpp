@@ -507,6 +507,7 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
         ta.queue = b.ray_queue;
         ta.queue_count = qn;
         ta.work = qn + 2;
+        ta.alone = false;
         ta.n_max = trace_max;
         if (sort) ta.queue = launch_morton_sort(P, b, 2u * (par ^ 1u), eo.sort_key, L.stream, lc);
         launch_trace(ta, L.stream, lc);

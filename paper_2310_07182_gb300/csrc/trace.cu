@@ -31,11 +31,14 @@ __device__ __forceinline__ uint32_t lds(uint32_t a) {
 constexpr int kNoNode = (int)0x80000000; // no traversal left (leaf codes are all above kRefill)
 constexpr int kRefill = (int)0x80000001; // the stack's older entries wait in local memory
 constexpr int kSteps = 2;                // node visits between two votes of the warp
+constexpr int kStealIdle = 16;           // idle lanes of a warp at which they take over parts of other lanes' rays
+// Shared-memory bytes of one warp: the lanes' stacks, three more words each.
+__host__ __device__ constexpr uint32_t warp_smem(int entries) { return (uint32_t)(entries + 3) * 128u; }
 
 // Traversal of a warp's rays, one ray per lane; all 32 lanes call it together.
 //
 // What bounds it: issue slots and the latency of the record loads, both multiplied by lanes
-// that wait (at the start 8 of 32 lanes were busy on secondary rays).  Two rules keep lanes busy:
+// that wait (at the start 8 of 32 lanes were busy on secondary rays).  Three rules keep lanes busy:
 //  - The descent ends as soon as no more than half of the warp's unfinished lanes are still in it,
 //    and the leaves reached are tested while the others wait (half is the best of 3/8 to 3/4, a
 //    vote every second visit the best of 1 to 4).
@@ -44,16 +47,25 @@ constexpr int kSteps = 2;                // node visits between two votes of the
 //    the queue stay together, and the records are small enough for the wider spread of
 //    addresses.  Camera rays are traced without: a warp's rays are one pixel block, which
 //    ends together, and taking rays one by one mixes blocks (0.35 to 0.40 ms against 0.28).
+//  - kSteal: once the queue is empty and 16 lanes of the warp have nothing to do (8 to 24 are alike),
+//    each of them takes the oldest stack entry of a lane that has one, with a copy of its ray, and
+//    hands its hit back at the end; a word per ray carries the smallest distance found so far, by
+//    which all of its lanes cull.  The closest hit does not depend on the order of visits, so it
+//    stays the same.  Short launches spread their rays over the whole device first (two to a
+//    warp or more): their time is that of their longest ray, one dependent load after another.
 // Landscape frame (1920x1080, 1.93M secondary rays): secondary trace 1.059 ms at the start (64-byte
-// records in four loads, neither rule), 0.74 with 32-byte records and the first rule, 0.63 with both;
-// primary trace 0.357 -> 0.280 ms.  Interior (3.35M secondary, 1.68M shadow rays): 2.46 -> 1.84 ->
-// 1.52 ms and 1.75 -> 1.39 -> 0.92 ms.
+// records in four loads, none of the rules), 0.74 with 32-byte records and the first rule, 0.63 with the
+// second; primary trace 0.357 -> 0.280 ms.  Interior (3.35M secondary, 1.68M shadow rays): 2.46 ->
+// 1.84 -> 1.52 ms and 1.75 -> 1.39 -> 0.92, 0.89 ms with the third.  A 500x333 frame of 4 samples and 8
+// bounces (17,600 rays per launch): secondary trace 2.03 ms without the third rule, 1.26 with it;
+// the two traces of 4,096 and 1,987 rays of a 64x64 frame 26 and 33 us (with 6 us of events
+// each), 21 and 24 with it.
 //
 // kAny: visibility only; a lane is done at the first triangle hit before its ray's tmax.
 // kSmemS: stack entries per lane kept in shared memory (8, 16 or 32), a launch-shape knob of
 // the autotuner.
 // kOne: every ray is in scenes[0], whose pointers then take no registers per lane.
-template <bool kCount, bool kAny, int kSmemS, bool kOne, class Src>
+template <bool kCount, bool kAny, int kSmemS, bool kOne, bool kSteal, class Src>
 __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ scenes, Src& src, uint32_t* smem,
                                                 unsigned long long& n_node, unsigned long long& n_tri) {
     constexpr uint32_t kLevel = 128u; // bytes between a lane's entries
@@ -68,12 +80,18 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
     int skip = -1, key = -1;
     // entry 0 holds kNoNode (or kRefill while older entries are in lstack), so a pop needs no
     // test for an empty stack
-    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem) + (threadIdx.x >> 5) * (kSmemS * kLevel) +
-                          (threadIdx.x & 31u) * 4u;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem) + (threadIdx.x >> 5) * warp_smem(kSmemS) + lane * 4u;
+    // kSteal: three more words per lane
+    const uint32_t lent = base + kSmemS * kLevel;      // lanes that trace part of this lane's ray
+    const uint32_t bound = lent + kLevel;              // the smallest distance found for this lane's ray
+    const uint32_t list = bound + kLevel - lane * 4u;  // scratch list of the warp
     const uint32_t lim = base + (uint32_t)(kSmemS - kSteps + 1) * kLevel; // below it there is room for kSteps pushes
     uint32_t top = base + kLevel;                                         // next free entry
     int lstack[kStackTotal];
     int lsp = 0;
+    uint32_t bot = base; // the entry that holds kNoNode or kRefill
+    uint32_t owner = lane; // kSteal: the lane whose ray this lane traces (part of)
     int node = kNoNode;
     auto step = [&]() {
         if (kCount) ++n_node;
@@ -126,15 +144,43 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
                 skip = __float_as_int(ro.w);
                 best = Best{rd.w, -1};
                 tcull = __fmul_rn(best.t, kCullWiden);
-                sts(base, (uint32_t)kNoNode);
+                bot = base;
+                sts(bot, (uint32_t)kNoNode);
                 top = base + kLevel;
+                if (kSteal) {
+                    sts(lent, 0u);
+                    sts(bound, __float_as_uint(rd.w));
+                }
                 node = 0;
             }
         }
     };
     if (!Src::kMore) fill(0u);
-    int refill = 32; // idle lanes at which rays are taken; 33: none are left
+    int refill = Src::kMore ? 32 : 33; // idle lanes at which rays are taken; 33: none are left
     while (true) {
+        if (kSteal && refill == 33) {
+            // a lane that has finished its part of another lane's ray hands its hit over
+            uint32_t done = __ballot_sync(0xffffffffu, node == kNoNode && owner != lane);
+            while (done) {
+                const int h = __ffs(done) - 1;
+                done &= done - 1u;
+                const uint32_t o = __shfl_sync(0xffffffffu, owner, h);
+                const float t = __shfl_sync(0xffffffffu, best.t, h);
+                const int leaf = __shfl_sync(0xffffffffu, best.leaf, h);
+                if (lane == o) {
+                    sts(lent, lds(lent) - 1u);
+                    if (leaf >= 0 && (best.leaf < 0 || t < best.t ||
+                                      (t == best.t && __float_as_int(__ldg(&tris[3 * leaf]).w) <
+                                                          __float_as_int(__ldg(&tris[3 * best.leaf]).w))))
+                        best = Best{t, leaf};
+                }
+                if (lane == (uint32_t)h) owner = lane;
+            }
+            if (node == kNoNode && key >= 0 && lds(lent) == 0u) {
+                src.store(key, best.leaf, best.t, tris);
+                key = -1;
+            }
+        }
         uint32_t alive = __ballot_sync(0xffffffffu, node != kNoNode);
         if (Src::kMore && 32 - __popc(alive) >= refill) {
             fill(alive);
@@ -150,6 +196,82 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
             if (key >= 0) src.store(key, best.leaf, best.t, tris);
             return;
         }
+        if (kSteal && refill == 33 && 32 - __popc(alive) >= kStealIdle) {
+            // lanes without a ray take the oldest stack entry of a lane that has one
+            const bool free = node == kNoNode && key < 0;
+            const bool gives = node != kNoNode && node != kRefill && lsp == 0 && top > bot + kLevel;
+            const uint32_t takers = __ballot_sync(0xffffffffu, free), givers = __ballot_sync(0xffffffffu, gives);
+            const int n_moves = min(__popc(takers), __popc(givers));
+            if (n_moves) {
+                const uint32_t below = (1u << lane) - 1u;
+                const int rank = __popc((gives ? givers : takers) & below);
+                if (gives && rank < n_moves) {
+                    sts(list + 4u * rank, lane);
+                    asm volatile("red.shared.min.s32 [%0], %1;" ::"r"(bound + (owner - lane) * 4u), "r"(__float_as_int(best.t)) : "memory");
+                }
+                __syncwarp();
+                const bool takes = free && rank < n_moves;
+                const uint32_t from = takes ? lds(list + 4u * rank) : lane;
+                const uint32_t their_bot = __shfl_sync(0xffffffffu, bot, from);
+                const uint32_t their_owner = __shfl_sync(0xffffffffu, owner, from);
+                r.ox = __shfl_sync(0xffffffffu, r.ox, from);
+                r.oy = __shfl_sync(0xffffffffu, r.oy, from);
+                r.oz = __shfl_sync(0xffffffffu, r.oz, from);
+                r.sx = __shfl_sync(0xffffffffu, r.sx, from);
+                r.sy = __shfl_sync(0xffffffffu, r.sy, from);
+                r.sz = __shfl_sync(0xffffffffu, r.sz, from);
+                r.kz = __shfl_sync(0xffffffffu, r.kz, from);
+                g.ix = __shfl_sync(0xffffffffu, g.ix, from);
+                g.iy = __shfl_sync(0xffffffffu, g.iy, from);
+                g.iz = __shfl_sync(0xffffffffu, g.iz, from);
+                g.nx = __shfl_sync(0xffffffffu, g.nx, from);
+                g.ny = __shfl_sync(0xffffffffu, g.ny, from);
+                g.nz = __shfl_sync(0xffffffffu, g.nz, from);
+                g.fx = __shfl_sync(0xffffffffu, g.fx, from);
+                g.fy = __shfl_sync(0xffffffffu, g.fy, from);
+                g.fz = __shfl_sync(0xffffffffu, g.fz, from);
+                g.snx = __shfl_sync(0xffffffffu, g.snx, from);
+                g.sny = __shfl_sync(0xffffffffu, g.sny, from);
+                g.snz = __shfl_sync(0xffffffffu, g.snz, from);
+                g.sfx = __shfl_sync(0xffffffffu, g.sfx, from);
+                g.sfy = __shfl_sync(0xffffffffu, g.sfy, from);
+                g.sfz = __shfl_sync(0xffffffffu, g.sfz, from);
+                skip = __shfl_sync(0xffffffffu, skip, from);
+                const float their_t = __shfl_sync(0xffffffffu, best.t, from);
+                if (!kOne) {
+                    const unsigned long long their_sc = __shfl_sync(0xffffffffu, (unsigned long long)sc, from);
+                    if (takes) {
+                        sc = (const SceneDev*)their_sc;
+                        nodes = sc->nodes2;
+                        tris = sc->tris;
+                    }
+                }
+                if (takes) {
+                    node = (int)lds(their_bot + kLevel);
+                    owner = their_owner;
+                    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(lent + (owner - lane) * 4u) : "memory");
+                    best = Best{their_t, -1};
+                    bot = base;
+                    sts(bot, (uint32_t)kNoNode);
+                    top = base + kLevel;
+                    lsp = 0;
+                }
+                __syncwarp();
+                if (gives && rank < n_moves) {
+                    bot += kLevel;
+                    sts(bot, (uint32_t)kNoNode);
+                }
+                alive = __ballot_sync(0xffffffffu, node != kNoNode);
+            }
+        }
+        if (kSteal && refill == 33) { // what the other lanes of this ray have found
+            const float b = __uint_as_float(lds(bound + (owner - lane) * 4u));
+            tcull = __fmul_rn(fminf(best.t, b), kCullWiden);
+            if (kAny && b < 0.0f) { // one of them was blocked
+                node = kNoNode;
+                lsp = 0;
+            }
+        }
         const int half = __popc(alive) >> 1;
         bool run;
         do {
@@ -163,7 +285,12 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
             }
             run = run && top < lim;
         } while (__popc(__ballot_sync(0xffffffffu, run)) > half);
-        if (node >= 0 && top >= lim) { // rare: the older half of the stack moves to local memory
+        if (kSteal && node >= 0 && top >= lim && bot != base) { // the room of entries given away
+            const uint32_t by = bot - base;
+            for (uint32_t a = bot; a < top; a += kLevel) sts(a - by, lds(a));
+            bot = base;
+            top -= by;
+        } else if (node >= 0 && top >= lim) { // rare: the older half of the stack moves to local memory
             for (int k = 0; k < kHalf; ++k) lstack[lsp + k] = (int)lds(base + (1 + k) * kLevel);
             for (uint32_t a = base + (1 + kHalf) * kLevel; a < top; a += kLevel) sts(a - kHalf * kLevel, lds(a));
             sts(base, (uint32_t)kRefill);
@@ -185,6 +312,10 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
                 })
                 test_leaf(tris, r, skip, code >> 2, (code & 3u) + 1u, best, n_tri);
                 tcull = __fmul_rn(best.t, kCullWiden);
+                if (kSteal && refill == 33 && best.leaf >= 0)
+                    asm volatile("red.shared.min.s32 [%0], %1;" ::"r"(bound + (owner - lane) * 4u),
+                                 "r"(__float_as_int(kAny ? -1.0f : best.t))
+                                 : "memory");
             }
             top -= kLevel;
             node = (int)lds(top);
@@ -200,7 +331,7 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
 #define CR_TRACE_MAXNREG 56 // 36 warps resident per SM, no spills; 48 and 64 are within 1%, 40 costs 4%
 #endif
 
-template <bool kCount, bool kAny, int kSmemS, bool kOne, bool kMore>
+template <bool kCount, bool kAny, int kSmemS, bool kOne, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __restrict__ scenes,
                                                            const uint16_t* __restrict__ slot_scene,
                                                            const float4* __restrict__ ray_o,
@@ -212,22 +343,22 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __res
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     unsigned long long n_node = 0, n_tri = 0;
-    QueueSrc<kMore> src(n, work, slot_scene, ray_o, ray_d, queue, hit);
-    if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemS, kOne>(scenes, src, smem_stack, n_node, n_tri);
+    QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit);
+    if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemS, kOne, !kCount && !kAny && kKind != kPlain>(scenes, src, smem_stack, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
 }
 
 // A caller's rays and hit arrays, no scratch between: cr_trace_rays used to copy the rays into the
 // render path's records, trace, and copy the hits out, in buffers allocated per call (1M surface
 // rays 952 us against 503, 300k camera rays 456 against 146, 1,000 rays 69 against 51).
-template <bool kCount, bool kAny, bool kMore>
+template <bool kCount, bool kAny, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_user(const SceneDev* __restrict__ scene, UserRays rays,
                                                                 uint32_t n, unsigned long long* counters,
                                                                 uint32_t* work) {
     extern __shared__ uint32_t smem_stack[];
     unsigned long long n_node = 0, n_tri = 0;
-    UserSrc<kMore> src(n, work, rays);
-    if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemStack, true>(scene, src, smem_stack, n_node, n_tri);
+    UserSrc<kKind> src(n, work, rays);
+    if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemStack, true, !kCount && !kAny && kKind != kPlain>(scene, src, smem_stack, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
 }
 
@@ -409,8 +540,8 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
     const float4* tris = sc.tris;
     unsigned long long dummy = 0;
     if (!uniform_scene) { // rare: a warp straddling two jobs of different scenes
-        QueueSrc<false> src(n, nullptr, slot_scene, ray_o, ray_d, queue, hit);
-        trace_bvh2_warp<false, false, kSmemStack, false>(scenes, src, smem_stack, dummy, dummy);
+        QueueSrc<kPlain> src(n, nullptr, slot_scene, ray_o, ray_d, queue, hit);
+        trace_bvh2_warp<false, false, kSmemStack, false, false>(scenes, src, smem_stack, dummy, dummy);
         return;
     }
     constexpr int kSmemS = kSmemStack;
@@ -550,7 +681,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_spec(
     }
 }
 
-template <bool kOne, bool kMore>
+template <bool kOne, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
     const SceneDev* __restrict__ scenes, const uint16_t* __restrict__ slot_scene, const float4* __restrict__ sh_o,
     const float4* __restrict__ sh_d, const float4* __restrict__ sh_c, const int32_t* __restrict__ group_queue,
@@ -558,10 +689,10 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
     unsigned long long* __restrict__ n_traced, uint32_t* work) {
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
-    ShadowSrc<kMore> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
+    ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
     if (!src.more()) return;
     unsigned long long dn = 0, dt = 0;
-    trace_bvh2_warp<false, true, kSmemStack, kOne>(scenes, src, smem_stack, dn, dt);
+    trace_bvh2_warp<false, true, kSmemStack, kOne, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
     src.add_traced(n_traced);
 }
 
@@ -588,7 +719,8 @@ __global__ void k_rays_from_user(const float* __restrict__ rays, const int32_t* 
 void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
                         const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count,
                         uint32_t n_groups_max, uint32_t K, float4* radiance, unsigned long long* n_traced, bool bvh8,
-                        bool one_scene, uint32_t* work, cudaStream_t st, LaunchCount& lc) {
+                        bool one_scene, bool alone, uint32_t* work, cudaStream_t st,
+                        LaunchCount& lc) {
     const uint32_t n_pos = n_groups_max * K;
     if (n_pos == 0) return;
     if (bvh8) {
@@ -597,19 +729,18 @@ void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, cons
         return;
     }
     const int block = kSecondaryBlock;
-    const size_t smem = (size_t)kSmemStack * block * sizeof(uint32_t);
-    // rays handed out lane by lane only where there are more of them than resident lanes (as below)
-    const uint32_t need = blocks_for(n_pos, block);
+    const size_t smem = (size_t)warp_smem(kSmemStack) * (block / 32);
+    const uint32_t need = blocks_for(n_pos, block); // the kinds of range as below
     auto go = [&](auto one) {
         constexpr bool kOne = decltype(one)::value;
-        const uint32_t most = work ? resident_blocks<k_trace_shadow<kOne, true>>(block, smem) : 0u;
-        if (most && need > most)
-            k_trace_shadow<kOne, true><<<most, block, smem, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue,
-                                                                 group_count, n_groups_max, K, radiance, n_traced, work);
-        else
-            k_trace_shadow<kOne, false><<<need, block, smem, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue,
-                                                                  group_count, n_groups_max, K, radiance, n_traced,
-                                                                  nullptr);
+        const uint32_t most = resident_blocks<k_trace_shadow<kOne, kMore>>(block, smem);
+        auto run = [&](auto kernel, uint32_t grid) {
+            kernel<<<grid, block, smem, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count,
+                                              n_groups_max, K, radiance, n_traced, work);
+        };
+        if (need <= most && alone) run(k_trace_shadow<kOne, kFew>, spread_blocks(n_pos, block, most));
+        else if (work && most && need > most) run(k_trace_shadow<kOne, kMore>, most);
+        else run(k_trace_shadow<kOne, kPlain>, need);
     };
     if (one_scene) go(std::true_type());
     else go(std::false_type());
@@ -663,7 +794,7 @@ SceneDev scene_entry(const DevScene& s, bool bvh8) {
 
 template <auto kKernel, int kSmemS>
 static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t st, LaunchCount& lc) {
-    const size_t smem = (size_t)kSmemS * a.block * sizeof(uint32_t);
+    const size_t smem = (size_t)warp_smem(kSmemS) * (a.block / 32);
     if (smem > 48 * 1024) // 512-thread blocks with 32 entries need the opt-in beyond 48 KB
         cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     kKernel<<<grid, a.block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue, a.queue_count, a.n_max, a.hit,
@@ -671,17 +802,20 @@ static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t s
     lc.n++;
 }
 
-// Rays are handed out lane by lane (kMore) where a.work allows it and the launch may hold more
-// rays than lanes are resident at once; with fewer, every lane has its ray from the start and
-// the plain variant is 3.5% faster (a 500x333 frame of 8 bounces: 2.76 against 2.86 ms).
+// The kind of range.  A launch that may hold more rays than lanes are resident at once hands them
+// out lane by lane where a.work allows it (kMore), else one per lane of as many blocks as it takes
+// (kPlain).  With fewer rays they are spread over all resident warps (kFew), unless other launches
+// share the device (a server's lanes): 24 requests took 6.65 ms against 6.54.
 template <bool kOne, bool kCount, bool kAny, int kSmemS>
 static void launch_bvh2_scenes(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
+    constexpr auto kM = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kMore>;
+    constexpr auto kF = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kFew>;
+    constexpr auto kP = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kPlain>;
     const uint32_t need = blocks_for(a.n_max, a.block);
-    constexpr auto kDynamic = k_trace_bvh2<kCount, kAny, kSmemS, kOne, true>;
-    constexpr auto kPlain = k_trace_bvh2<kCount, kAny, kSmemS, kOne, false>;
-    const uint32_t most = a.work ? resident_blocks<kDynamic>(a.block, (size_t)kSmemS * a.block * sizeof(uint32_t)) : 0u;
-    if (most && need > most) launch_bvh2_kernel<kDynamic, kSmemS>(a, most, st, lc);
-    else launch_bvh2_kernel<kPlain, kSmemS>(a, need, st, lc);
+    const uint32_t most = resident_blocks<kM>(a.block, (size_t)warp_smem(kSmemS) * (a.block / 32));
+    if (need <= most && a.alone) launch_bvh2_kernel<kF, kSmemS>(a, spread_blocks(a.n_max, a.block, most), st, lc);
+    else if (a.work && most && need > most) launch_bvh2_kernel<kM, kSmemS>(a, most, st, lc);
+    else launch_bvh2_kernel<kP, kSmemS>(a, need, st, lc);
 }
 
 // kOneScene: whether launches over a single scene have a variant of their own.
@@ -693,13 +827,15 @@ static void launch_bvh2(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
 
 template <bool kCount, bool kAny>
 static void launch_bvh2_user(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    const size_t smem = (size_t)kSmemStack * a.block * sizeof(uint32_t);
+    const size_t smem = (size_t)warp_smem(kSmemStack) * (a.block / 32);
     const uint32_t need = blocks_for(a.n_max, a.block);
-    const uint32_t most = a.work ? resident_blocks<k_trace_bvh2_user<kCount, kAny, true>>(a.block, smem) : 0u;
-    if (most && need > most)
-        k_trace_bvh2_user<kCount, kAny, true><<<most, a.block, smem, st>>>(a.scenes, a.user, a.n_max, a.counters, a.work);
-    else
-        k_trace_bvh2_user<kCount, kAny, false><<<need, a.block, smem, st>>>(a.scenes, a.user, a.n_max, a.counters, nullptr);
+    const uint32_t most = resident_blocks<k_trace_bvh2_user<kCount, kAny, kMore>>(a.block, smem);
+    auto run = [&](auto kernel, uint32_t grid) {
+        kernel<<<grid, a.block, smem, st>>>(a.scenes, a.user, a.n_max, a.counters, a.work);
+    };
+    if (need <= most) run(k_trace_bvh2_user<kCount, kAny, kFew>, spread_blocks(a.n_max, a.block, most));
+    else if (a.work && most) run(k_trace_bvh2_user<kCount, kAny, kMore>, most);
+    else run(k_trace_bvh2_user<kCount, kAny, kPlain>, need);
     lc.n++;
 }
 
@@ -712,7 +848,7 @@ void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
         return;
     }
     const int block = a.block;
-    const size_t smem = (size_t)kSmemStack * block * sizeof(uint32_t);
+    const size_t smem = (size_t)warp_smem(kSmemStack) * (block / 32);
     if (a.bvh8) { // BVH8-Q kernels (trace_bvh8.cu)
         launch_trace_bvh8(a, st, lc);
         return;

@@ -156,14 +156,14 @@ __global__ void __maxnreg__(CR_TRACE4_MAXNREG) k_trace_bvh4(const SceneDev* __re
                                                              int2* __restrict__ hit, unsigned long long* counters) {
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
-    trace_bvh4_rays<kCount>(scenes, QueueSrc<false>(n, nullptr, slot_scene, ray_o, ray_d, queue, hit), smem_stack, counters);
+    trace_bvh4_rays<kCount>(scenes, QueueSrc<kPlain>(n, nullptr, slot_scene, ray_o, ray_d, queue, hit), smem_stack, counters);
 }
 
 template <bool kCount>
 __global__ void __maxnreg__(CR_TRACE4_MAXNREG) k_trace_bvh4_user(const SceneDev* __restrict__ scene, UserRays rays,
                                                                  uint32_t n, unsigned long long* counters) {
     extern __shared__ uint32_t smem_stack[];
-    trace_bvh4_rays<kCount>(scene, UserSrc<false>(n, nullptr, rays), smem_stack, counters);
+    trace_bvh4_rays<kCount>(scene, UserSrc<kPlain>(n, nullptr, rays), smem_stack, counters);
 }
 
 } // namespace

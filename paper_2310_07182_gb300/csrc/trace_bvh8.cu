@@ -218,7 +218,7 @@ __device__ __forceinline__ void trace_bvh8_warp(const SceneDev* __restrict__ sce
 #define CR_BVH8_MIN_BLOCKS 8 // resident 128-thread blocks per SM the register budget is sized for
 #endif
 
-template <bool kCount, bool kAny, bool kMore>
+template <bool kCount, bool kAny, RangeKind kKind>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8(const SceneDev* __restrict__ scenes,
                              const uint16_t* __restrict__ slot_scene,
                              const float4* __restrict__ ray_o, const float4* __restrict__ ray_d,
@@ -226,30 +226,30 @@ __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8(const Sc
                              uint32_t n_max, int2* __restrict__ hit, unsigned long long* counters, uint32_t* work) {
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     unsigned long long n_node = 0, n_tri = 0;
-    QueueSrc<kMore> src(n, work, slot_scene, ray_o, ray_d, queue, hit);
+    QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit);
     if (src.more()) trace_bvh8_warp<kCount, kAny>(scenes, src, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
 }
 
-template <bool kCount, bool kAny, bool kMore>
+template <bool kCount, bool kAny, RangeKind kKind>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8_user(const SceneDev* __restrict__ scene,
                                                                              UserRays rays, uint32_t n,
                                                                              unsigned long long* counters, uint32_t* work) {
     unsigned long long n_node = 0, n_tri = 0;
-    UserSrc<kMore> src(n, work, rays);
+    UserSrc<kKind> src(n, work, rays);
     if (src.more()) trace_bvh8_warp<kCount, kAny>(scene, src, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
 }
 
 // Shadow rays of next-event estimation over the BVH8-Q (see k_trace_shadow).
-template <bool kMore>
+template <RangeKind kKind>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_shadow8(
     const SceneDev* __restrict__ scenes, const uint16_t* __restrict__ slot_scene, const float4* __restrict__ sh_o,
     const float4* __restrict__ sh_d, const float4* __restrict__ sh_c, const int32_t* __restrict__ group_queue,
     const uint32_t* __restrict__ group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
     unsigned long long* __restrict__ n_traced, uint32_t* work) {
     const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
-    ShadowSrc<kMore> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
+    ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
     if (!src.more()) return;
     unsigned long long dn = 0, dt = 0;
     trace_bvh8_warp<false, true>(scenes, src, dn, dt);
@@ -264,18 +264,18 @@ template <bool kCount, bool kAny>
 static void launch_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     const uint32_t need = blocks_for(a.n_max, a.block);
     if (a.user.rays) {
-        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8_user<kCount, kAny, true>>(a.block, 0) : 0u;
+        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8_user<kCount, kAny, kMore>>(a.block, 0) : 0u;
         if (most && need > most)
-            k_trace_bvh8_user<kCount, kAny, true><<<most, a.block, 0, st>>>(a.scenes, a.user, a.n_max, a.counters, a.work);
+            k_trace_bvh8_user<kCount, kAny, kMore><<<most, a.block, 0, st>>>(a.scenes, a.user, a.n_max, a.counters, a.work);
         else
-            k_trace_bvh8_user<kCount, kAny, false><<<need, a.block, 0, st>>>(a.scenes, a.user, a.n_max, a.counters, nullptr);
+            k_trace_bvh8_user<kCount, kAny, kPlain><<<need, a.block, 0, st>>>(a.scenes, a.user, a.n_max, a.counters, nullptr);
     } else {
-        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8<kCount, kAny, true>>(a.block, 0) : 0u;
+        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8<kCount, kAny, kMore>>(a.block, 0) : 0u;
         if (most && need > most)
-            k_trace_bvh8<kCount, kAny, true><<<most, a.block, 0, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
+            k_trace_bvh8<kCount, kAny, kMore><<<most, a.block, 0, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
                                                                       a.queue_count, a.n_max, a.hit, a.counters, a.work);
         else
-            k_trace_bvh8<kCount, kAny, false><<<need, a.block, 0, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
+            k_trace_bvh8<kCount, kAny, kPlain><<<need, a.block, 0, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
                                                                        a.queue_count, a.n_max, a.hit, a.counters,
                                                                        nullptr);
     }
@@ -294,12 +294,12 @@ void launch_shadow_rays_bvh8(const SceneDev* scenes, const uint16_t* slot_scene,
                              unsigned long long* n_traced, uint32_t* work, cudaStream_t st, LaunchCount& lc) {
     const int block = 128;
     const uint32_t need = blocks_for(n_groups_max * K, block);
-    const uint32_t most = work ? resident_blocks<k_trace_shadow8<true>>(block, 0) : 0u;
+    const uint32_t most = work ? resident_blocks<k_trace_shadow8<kMore>>(block, 0) : 0u;
     if (most && need > most)
-        k_trace_shadow8<true><<<most, block, 0, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count,
+        k_trace_shadow8<kMore><<<most, block, 0, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count,
                                                       n_groups_max, K, radiance, n_traced, work);
     else
-        k_trace_shadow8<false><<<need, block, 0, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count,
+        k_trace_shadow8<kPlain><<<need, block, 0, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count,
                                                        n_groups_max, K, radiance, n_traced, nullptr);
     lc.n++;
 }

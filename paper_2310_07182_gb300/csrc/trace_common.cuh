@@ -312,24 +312,31 @@ __device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, const
 // ------------------------------------------------------------------------------------
 // Ray sources of the trace kernels.
 constexpr uint32_t kTraceChunk = 32; // positions a warp takes at a time
+constexpr uint32_t kTraceShare = 2;  // positions of a warp at least (below, warps are spread over the device)
 constexpr int kTraceIdle = 8;        // idle lanes of a warp at which they get new rays
 
-// Where a warp's rays come from: positions of a list of n, kTraceChunk at a time.  A source adds
+// Where a warp's rays come from: positions of a list of n.  A source adds
 // load() (the ray at a position; false: none there) and store() (its hit).
-// kMore: lanes whose ray has ended get further positions of the warp's range, and the warp takes
-// another range from `work` (a device counter, zero before the launch) when its own runs out.
-// Otherwise the first range is all the warp traces.
-template <bool kMore_>
+//   kPlain  kTraceChunk positions, one per lane, are all a warp traces (grids of any size).
+//   kMore   lanes whose ray has ended get further positions of the warp's range, and the warp takes
+//           another kTraceChunk from `work` (a device counter, zero before the launch) when its own
+//           run out (resident grids, more positions than lanes).
+//   kFew    the n positions are spread evenly over the warps of a resident grid, which has more lanes.
+enum RangeKind { kPlain, kMore, kFew };
+
+template <RangeKind kKind>
 struct WarpRange {
-    static constexpr bool kMore = kMore_;
+    static constexpr bool kMore = kKind == RangeKind::kMore;
     uint32_t n, next, end;
     uint32_t* work;
     uint32_t first_free; // the first position that `work` hands out
     __device__ __forceinline__ WarpRange(uint32_t n_, uint32_t* work_) : n(n_), work(work_) {
-        const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-        next = min(w * kTraceChunk, n);
-        end = min(next + kTraceChunk, n);
-        first_free = (gridDim.x * blockDim.x >> 5) * kTraceChunk;
+        const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, warps = gridDim.x * blockDim.x >> 5;
+        // fewer positions than lanes: the same share for every warp
+        const uint32_t each = kKind == RangeKind::kPlain ? kTraceChunk : min(max((n + warps - 1u) / warps, kTraceShare), kTraceChunk);
+        next = min(w * each, n);
+        end = min(next + each, n);
+        first_free = warps * each;
     }
     __device__ __forceinline__ bool more() const { return next < n; }
     // The idle lanes (a mask) get the next positions in lane order, n where the range ends.
@@ -354,8 +361,8 @@ struct WarpRange {
 };
 
 // Rays of a queue of slots (or of the slots in order), hits per slot.
-template <bool kMore>
-struct QueueSrc : WarpRange<kMore> {
+template <RangeKind kKind>
+struct QueueSrc : WarpRange<kKind> {
     const uint16_t* __restrict__ slot_scene;
     const float4* __restrict__ ray_o;
     const float4* __restrict__ ray_d;
@@ -366,7 +373,7 @@ struct QueueSrc : WarpRange<kMore> {
     __device__ __forceinline__ void probe(bool, uint32_t) {}
     __device__ __forceinline__ QueueSrc(uint32_t n, uint32_t* work, const uint16_t* ss, const float4* o, const float4* d,
                                         const int32_t* q, int2* h)
-        : WarpRange<kMore>(n, work), slot_scene(ss), ray_o(o), ray_d(d), queue(q), hit(h) {}
+        : WarpRange<kKind>(n, work), slot_scene(ss), ray_o(o), ray_d(d), queue(q), hit(h) {}
     __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) const {
         const int slot = queue ? queue[i] : (int)i;
         ro = ray_o[slot];
@@ -385,8 +392,8 @@ struct QueueSrc : WarpRange<kMore> {
 };
 
 // A caller's rays (8 floats each), optional skip ids and hit arrays.
-template <bool kMore>
-struct UserSrc : WarpRange<kMore>, UserRays {
+template <RangeKind kKind>
+struct UserSrc : WarpRange<kKind>, UserRays {
     int idle = kTraceIdle;
     // A warp whose rays all run into one octant is taken for a coherent one (camera rays), whose
     // rays end together: it gets new rays only when all of its own have ended (the rule of
@@ -395,7 +402,7 @@ struct UserSrc : WarpRange<kMore>, UserRays {
     __device__ __forceinline__ void probe(bool live, uint32_t oct) {
         idle = __popc(__reduce_or_sync(0xffffffffu, live ? 1u << oct : 0u)) <= 1 ? 32 : kTraceIdle;
     }
-    __device__ __forceinline__ UserSrc(uint32_t n, uint32_t* work, const UserRays& u) : WarpRange<kMore>(n, work), UserRays(u) {}
+    __device__ __forceinline__ UserSrc(uint32_t n, uint32_t* work, const UserRays& u) : WarpRange<kKind>(n, work), UserRays(u) {}
     __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) const {
         const float* r = rays + 8 * (size_t)i;
         if (aligned) {
@@ -425,8 +432,8 @@ struct UserSrc : WarpRange<kMore>, UserRays {
 // reuse group's rays run in adjacent lanes, as they were shaded).  A ray whose
 // direction record has w = tmax > 0 is traced for visibility only; if nothing blocks it, its
 // contribution is added to the path radiance of its slot.  Rays traced are counted.
-template <bool kMore>
-struct ShadowSrc : WarpRange<kMore> {
+template <RangeKind kKind>
+struct ShadowSrc : WarpRange<kKind> {
     const uint16_t* __restrict__ slot_scene;
     const float4* __restrict__ sh_o;
     const float4* __restrict__ sh_d;
@@ -439,7 +446,7 @@ struct ShadowSrc : WarpRange<kMore> {
     __device__ __forceinline__ void probe(bool, uint32_t) {}
     __device__ __forceinline__ ShadowSrc(uint32_t n, uint32_t* work, const uint16_t* ss, const float4* o, const float4* d,
                                          const float4* c, const int32_t* gq, float4* rad, uint32_t k)
-        : WarpRange<kMore>(n, work), slot_scene(ss), sh_o(o), sh_d(d), sh_c(c), group_queue(gq), radiance(rad), K(k) {}
+        : WarpRange<kKind>(n, work), slot_scene(ss), sh_o(o), sh_d(d), sh_c(c), group_queue(gq), radiance(rad), K(k) {}
     __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) {
         const uint32_t g = group_queue ? (uint32_t)group_queue[i / K] : i / K;
         const int slot = (int)(g * K + i % K);
@@ -497,7 +504,12 @@ static uint32_t resident_blocks(int block, size_t smem) {
 }
 
 // Blocks for n positions, one per lane.
-static uint32_t blocks_for(uint32_t n, int block) { return n / (uint32_t)block + (n % (uint32_t)block ? 1u : 0u); }
+static inline uint32_t blocks_for(uint32_t n, int block) { return n / (uint32_t)block + (n % (uint32_t)block ? 1u : 0u); }
+// Blocks for n positions spread kTraceShare to a warp, at most `most`.
+static inline uint32_t spread_blocks(uint32_t n, int block, uint32_t most) {
+    const uint32_t want = blocks_for(n, block / 32 * (int)kTraceShare);
+    return want < most ? want : most;
+}
 
 } // namespace
 } // namespace cr

@@ -79,3 +79,18 @@ def test_lanes_that_take_new_rays(cr, n_rays, dead):
                      cr.make_opts())
     assert torch.equal(want_p, over[:n_rays].view(torch.int32)) and torch.equal(want_t, over[n_rays:2 * n_rays])
     assert bool(((want_p >= 0) == (S.trace(rays, any_hit=True)[0] >= 0)).all())
+
+
+@pytest.mark.parametrize("copies,n_rays", [(2, 500), (9, 70), (9, 200000)])
+def test_ties_between_lanes_that_share_a_ray(cr, copies, n_rays):
+    """Every triangle several times over: lanes that trace parts of one ray find the same distance
+    on different copies, and the smallest index wins."""
+    base = _overlapping(300, 12)
+    order = np.random.default_rng(copies).permutation(copies * base.n_tri)
+    sc = scenes.Scene("copies", np.tile(base.tri_xyz, (copies, 1))[order], np.tile(base.tri_mat, copies)[order],
+                      base.mat_type, base.mat_params, base.env, base.camera)
+    S = cr.Scene(sc, bvh_flags=cr.CR_BVH2 | cr.CR_BVH8Q)
+    rays = torch.from_numpy(scenes.random_rays(2, n_rays)).cuda()
+    p, t = S.trace(rays)
+    p8, t8 = S.trace(rays, bvh=cr.CR_BVH8Q)
+    assert torch.equal(p, p8) and torch.equal(t, t8) and (p >= 0).any()
