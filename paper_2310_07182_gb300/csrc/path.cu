@@ -168,8 +168,10 @@ __global__ void k_raygen(PassArgs p, int32_t* __restrict__ pixel, uint16_t* __re
             pixel[slot] = (int32_t)pix;
             ray_o[slot] = make_float4(J.cam.pos[0], J.cam.pos[1], J.cam.pos[2], __int_as_float(-1));
             ray_d[slot] = make_float4(d.x, d.y, d.z, INFINITY);
-            beta[slot] = make_float4(1.0f, 1.0f, 1.0f, 0.0f); // w: direction density, 0 for camera rays
-            radiance[slot] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (p.rolling) { // otherwise the pass's first shade starts both
+                beta[slot] = make_float4(1.0f, 1.0f, 1.0f, 0.0f); // w: direction density, 0 for camera rays
+                radiance[slot] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
             alive[slot] = 1;
             live = true;
         } else {
@@ -243,6 +245,12 @@ struct ShadeArgs {
     uint32_t ray_cap, group_cap;
 };
 
+// Whether the launch shades camera rays (the first shade of a pass): throughput 1 and radiance 0 are
+// known, so ray generation does not write them and this shade does not read them (32 B each way
+// per slot); later shades write the radiance of the paths that end.  Shade time of the landscape frame
+// 0.168 -> 0.160 ms, of an interior sample 0.348 -> 0.339 ms.  A rolling wavefront mixes bounces in a launch and keeps them in memory.
+__device__ __forceinline__ bool camera_paths(const PassArgs& p) { return !p.rolling && p.bounce == 1; }
+
 struct Member {
     int pix;
     bool alive;
@@ -252,6 +260,7 @@ struct Member {
     bool nee;        // the job uses next-event estimation
     bool nee_shared; // ... with one light point per group
     bool hdonor;     // hybrid groups: diffuse members reuse the first diffuse member's sample
+    bool ended;      // the environment or an emitter has just been added to the path's radiance
     bool cosgl;      // a GGX point in the diffuse class while reusing: cosine samples, pi f weights
     uint32_t scene;  // scene table index
     uint32_t type;   // material type of the shading point
@@ -332,6 +341,7 @@ __device__ __forceinline__ void setup_member(const ShadeArgs& a, const PassArgs&
     if (a.dbg.ray) capture_trace(a.dbg, (p.bounce - 1) * a.npx + (uint32_t)mb.pix, a.ray_o[slot], d4, h, bt);
     if (h.x < 0) { // miss: environment
         add_environment(sc, bt, L);
+        mb.ended = true;
         mb.alive = false;
         return;
     }
@@ -353,6 +363,7 @@ __device__ __forceinline__ void setup_member(const ShadeArgs& a, const PassArgs&
     mb.orig = __float_as_int(v0.w);
     if (type == kMatEmitter) {
         add_emission(sc, v0, v1, v2, m1, bt, h, d4, mb.nee, L);
+        mb.ended = true;
         mb.alive = false;
         return;
     }
@@ -557,7 +568,8 @@ __device__ __forceinline__ bool finish_member(const ShadeArgs& a, const PassArgs
         a.dbg.world[3 * di + 2] = ww.z;
     }
     if (!was_alive) return false;
-    a.radiance[slot] = make_float4(L.x, L.y, L.z, 0.0f);
+    // the radiance changes only where the path has just ended (the first shade writes all)
+    if (camera_paths(p) || mb.ended) a.radiance[slot] = make_float4(L.x, L.y, L.z, 0.0f);
     if (mb.alive && mb.valid) {
         const V3 o = spawn_point(a, slot, mb.wl.z < 0.0f ? v3(-mb.n.x, -mb.n.y, -mb.n.z) : mb.n);
         const V3 dw = local_to_world(mb.t, mb.b, mb.n, mb.wl);
@@ -650,6 +662,7 @@ __global__ void k_shade_warp(ShadeArgs a, PassArgs p) {
     const uint32_t pos = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t gq = pos / K, lane_g = pos % K;
     const bool active = gq < n_groups;
+    const bool fresh = camera_paths(p); // ray generation has left throughput and radiance to this shade
     int slot = -1;
     Member mb;
     mb.pix = -1;
@@ -667,6 +680,7 @@ __global__ void k_shade_warp(ShadeArgs a, PassArgs p) {
     mb.nee = false;
     mb.nee_shared = false;
     mb.hdonor = false;
+    mb.ended = false;
     mb.cosgl = false;
     mb.type = kMatLambert;
     mb.hemi = 1.0f;
@@ -681,8 +695,8 @@ __global__ void k_shade_warp(ShadeArgs a, PassArgs p) {
         const bool alive_in = a.alive[slot] != 0;
         const int2 h = a.hit[slot];
         const float4 d4 = a.ray_d[slot];
-        const float4 b4 = a.beta[slot];
-        const float4 r4 = a.radiance[slot];
+        const float4 b4 = fresh ? make_float4(1.0f, 1.0f, 1.0f, 0.0f) : a.beta[slot];
+        const float4 r4 = fresh ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : a.radiance[slot];
         const JobDev* Jp = nullptr;
         if (mb.pix >= 0) { // every valid slot knows whether its job is past its last bounce
             Jp = &a.jobs[jid];
@@ -798,6 +812,7 @@ __global__ void __launch_bounds__(256, CR_SHADE_BLOCK_MIN_BLOCKS) k_shade_block(
     const uint32_t pos = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t gq = pos / K, lane_g = pos % K;
     const bool active = gq < n_groups;
+    const bool fresh = camera_paths(p); // ray generation has left throughput and radiance to this shade
     int slot = -1;
     Member mb;
     mb.pix = -1;
@@ -815,6 +830,7 @@ __global__ void __launch_bounds__(256, CR_SHADE_BLOCK_MIN_BLOCKS) k_shade_block(
     mb.nee = false;
     mb.nee_shared = false;
     mb.hdonor = false;
+    mb.ended = false;
     mb.cosgl = false;
     mb.type = kMatLambert;
     mb.hemi = 1.0f;
@@ -829,8 +845,8 @@ __global__ void __launch_bounds__(256, CR_SHADE_BLOCK_MIN_BLOCKS) k_shade_block(
         const bool alive_in = a.alive[slot] != 0;
         const int2 h = a.hit[slot];
         const float4 d4 = a.ray_d[slot];
-        const float4 b4 = a.beta[slot];
-        const float4 r4 = a.radiance[slot];
+        const float4 b4 = fresh ? make_float4(1.0f, 1.0f, 1.0f, 0.0f) : a.beta[slot];
+        const float4 r4 = fresh ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : a.radiance[slot];
         const JobDev* Jp = nullptr;
         if (mb.pix >= 0) { // every valid slot knows whether its job is past its last bounce
             Jp = &a.jobs[jid];
