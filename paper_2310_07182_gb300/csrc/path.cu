@@ -1616,6 +1616,27 @@ __global__ void k_output_one(const float4* __restrict__ accum, uint32_t npx, flo
     out[3 * i + 2] = a.z * inv_spp;
 }
 
+// Sums of sample regions, in sample order: the same additions as one sample after another.
+__global__ void k_sum_samples(const float4* __restrict__ regions, uint32_t n, uint32_t npx, uint32_t first,
+                              float4* __restrict__ sum, float inv_spp, float* __restrict__ out) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= npx) return;
+    float4 a = first ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : sum[i];
+    for (uint32_t k = 0; k < n; ++k) {
+        const float4 r = regions[(size_t)k * npx + i];
+        a.x += r.x;
+        a.y += r.y;
+        a.z += r.z;
+    }
+    if (out) {
+        out[3 * (size_t)i + 0] = a.x * inv_spp;
+        out[3 * (size_t)i + 1] = a.y * inv_spp;
+        out[3 * (size_t)i + 2] = a.z * inv_spp;
+    } else {
+        sum[i] = a;
+    }
+}
+
 __global__ void k_philox(uint64_t seed, const uint32_t* __restrict__ ctr, uint32_t n, uint32_t* __restrict__ out) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -1821,6 +1842,12 @@ void launch_finish_accumulate(const PassArgs& p, PathBuffers& b, const cr_debug*
     k_finish_accumulate<<<(n_slots + 255) / 256, 256, 0, st>>>(p, b.pixel, b.slot_job, b.alive, b.hit, b.ray_o,
                                                                b.ray_d, b.beta, b.radiance, n_slots, b.accum,
                                                                dbg ? *dbg : cr_debug{}, p.npx);
+    lc.n++;
+}
+
+void launch_sum_samples(const float4* regions, uint32_t n, uint32_t npx, bool first, float4* sum, float inv_spp,
+                        float* out, cudaStream_t st, LaunchCount& lc) {
+    k_sum_samples<<<(npx + 255) / 256, 256, 0, st>>>(regions, n, npx, first ? 1u : 0u, sum, inv_spp, out);
     lc.n++;
 }
 

@@ -94,3 +94,21 @@ def test_ties_between_lanes_that_share_a_ray(cr, copies, n_rays):
     p, t = S.trace(rays)
     p8, t8 = S.trace(rays, bvh=cr.CR_BVH8Q)
     assert torch.equal(p, p8) and torch.equal(t, t8) and (p >= 0).any()
+
+
+@pytest.mark.parametrize("mode", ["direction_reuse", "morton_sort"])
+@pytest.mark.parametrize("size,spp", [((1, 1), 2), ((33, 17), 3), ((1500, 1100), 4)])
+def test_samples_that_share_a_pass_sum_in_order(cr, mode, size, spp):
+    """Samples rendered side by side in a pass (all of them, or fewer than the image has: the largest
+    size) give the float sums of one sample after another, and the same ray counts."""
+    S = cr.Scene(scenes.tiny(seed=6, n_soup=300, material_mix="transmissive"))
+    cam = scenes.Camera((0.0, 0.0, -3.0), (0.0, 0.0, 0.0), (0.0, 1.0, 0.0), 60.0, *size)
+    kw = dict(max_bounces=2, mode=mode, tile=(8, 8), k=8, seed=9)
+    img, st = S.render(cam, spp=spp, stats=True, **kw)
+    total, rays = torch.zeros_like(img), 0
+    for s in range(spp):
+        one, st1 = S.render(cam, spp=1, frame_base=s, stats=True, **kw)
+        total += one
+        rays += st1["secondary_rays"]
+    assert torch.equal(img, total * torch.tensor(1.0 / spp, dtype=torch.float32, device="cuda"))
+    assert st["secondary_rays"] == rays
