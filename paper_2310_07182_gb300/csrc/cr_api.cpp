@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
@@ -680,8 +681,17 @@ JobDev job_dev(const cr_job& j, const PlanOpts& po, uint32_t scene_idx, uint32_t
     d.inv_spp = 1.0f / (float)j.spp;
     d.sample_flags = (sample == 0 ? 1u : 0u) | (sample + 1 == j.spp ? 2u : 0u);
     d.diffuse_rough = j.diffuse_roughness;
+    d.spp = j.spp;
     return d;
 }
+
+// Slots up to which samples of a plan's jobs share a pass (1.6 GB of path state with light samples).  A
+// trace launch costs about 90 us beyond its rays at full rate (the device fills, then drains to the
+// longest rays).  1280x720, 16 samples, 4 bounces, light samples: 48.2 ms with a pass per sample,
+// 42.1 / 38.9 / 37.3 with 2^21 / 2^22 / 2^23 slots; 853x479 with 4 samples through the BVH8-Q: 7.42 ms,
+// 5.58 with 2^21 or more; 500x333 with 4 samples and 8 bounces: 1.92 ms, 0.82 from 2^20 on;
+// a batch of 16 jobs of 1.6M slots and 4 samples: 6.75 ms, 5.41 with all four in a pass.
+constexpr uint64_t kPassSlots = 1ull << 23;
 
 cr_status build_plan(const cr_job* jobs, uint32_t n_jobs, const PlanOpts& po, RenderPlan& plan) {
     if (n_jobs == 0 || n_jobs > 65535) return fail(CR_ERR_INVALID_ARG, "n_jobs %u not in [1, 65535]", n_jobs);
@@ -739,29 +749,46 @@ cr_status build_plan(const cr_job* jobs, uint32_t n_jobs, const PlanOpts& po, Re
             return fail(CR_ERR_INVALID_ARG, "tile range [%u, %u) is not within the image's %llu tiles", po.tile_begin,
                         po.tile_end, (unsigned long long)all);
     }
-    if (po.samples > 1 && n_jobs == 1 && po.tile_end == 0 && jobs[0].spp > 1) {
-        const cr_job& j = jobs[0];
-        plan.regions = std::min(po.samples, j.spp);
+    if (po.tile_end == 0 && max_spp > 1) { // samples of a job side by side
+        uint64_t slots = 0;
+        for (uint32_t i = 0; i < n_jobs; ++i)
+            slots += (uint64_t)((jobs[i].camera.width + po.tile_w - 1) / po.tile_w) *
+                     ((jobs[i].camera.height + po.tile_h - 1) / po.tile_h) * m;
+        uint64_t r = po.samples ? po.samples : std::max<uint64_t>(1, kPassSlots / slots);
+        r = std::min<uint64_t>({r, max_spp, 65535u / n_jobs, (1ull << 27) / slots, ((1ull << 28) / px) - 1});
+        plan.regions = (uint32_t)std::max<uint64_t>(1, r);
+    }
+    if (plan.regions > 1) {
         plan.npx = px;
         plan.npx_total = px * (plan.regions + 1);
-        plan.out = j.out_rgb;
-        plan.inv_spp = 1.0f / (float)j.spp;
-        const uint32_t tiles = ((j.camera.width + po.tile_w - 1) / po.tile_w) * ((j.camera.height + po.tile_h - 1) / po.tile_h);
-        plan.nee = (j.flags & CR_JOB_NEE) != 0;
-        for (uint32_t s0 = 0; s0 < j.spp; s0 += plan.regions) {
-            Pass ps;
-            ps.job_offset = (uint32_t)plan.jobs.size();
-            ps.n_jobs = std::min(plan.regions, j.spp - s0);
-            ps.n_tiles = tiles * ps.n_jobs;
-            for (uint32_t k = 0; k < ps.n_jobs; ++k) {
-                JobDev d = job_dev(j, po, 0, s0 + k);
-                d.tile_base = d.slot_tile = k * tiles;
-                d.px_base = k * px;
+        plan.n_jobs = n_jobs;
+    }
+    for (uint32_t p = 0; p < max_spp && plan.regions > 1; p += plan.regions) {
+        Pass ps;
+        ps.job_offset = (uint32_t)plan.jobs.size();
+        uint32_t tiles = 0;
+        for (uint32_t k = 0; k < plan.regions; ++k)
+            for (uint32_t i = 0; i < n_jobs; ++i) {
+                const cr_job& j = jobs[i];
+                if (j.spp <= p + k) continue;
+                JobDev d = job_dev(j, po, scene_idx[i], p + k);
+                d.tile_base = d.slot_tile = tiles;
+                d.px_base = k * px + pxb[i];
                 d.sample_flags = 1u; // each sample starts the sum of its own region
+                if (d.nee) plan.nee = true;
+                tiles += d.tiles_x * ((j.camera.height + po.tile_h - 1) / po.tile_h);
                 plan.jobs.push_back(d);
             }
-            plan.max_slots = std::max(plan.max_slots, ps.n_tiles * m);
-            plan.passes.push_back(ps);
+        ps.n_jobs = (uint32_t)plan.jobs.size() - ps.job_offset;
+        ps.n_tiles = tiles;
+        plan.max_slots = std::max(plan.max_slots, tiles * m);
+        plan.passes.push_back(ps);
+    }
+    if (plan.regions > 1) {
+        plan.sum_offset = (uint32_t)plan.jobs.size();
+        for (uint32_t i = 0; i < n_jobs; ++i) {
+            plan.jobs.push_back(job_dev(jobs[i], po, scene_idx[i], 0));
+            plan.jobs.back().px_base = pxb[i];
         }
         return CR_OK;
     }
@@ -925,11 +952,9 @@ cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, cons
         P.bounce = p.max_bounces + 1;
         ev.begin(stream, times ? &times->accum : &dummy, "cr accumulate");
         launch_finish_accumulate(P, b, eo.debug, stream, lc);
-        if (p.regions > 1) {
-            const bool last_pass = &ps == &p.passes.back();
-            launch_sum_samples(b.accum, ps.n_jobs, p.npx, &ps == &p.passes.front(), b.accum + (size_t)p.regions * p.npx,
-                               p.inv_spp, last_pass ? p.out : nullptr, stream, lc);
-        }
+        if (p.regions > 1)
+            launch_sum_samples(dev.d_jobs + p.sum_offset, p.n_jobs, b.accum, p.regions, p.npx,
+                               (uint32_t)(&ps - p.passes.data()) * p.regions, stream, lc);
         ev.end();
     }
     // pass 0 holds every job (spp >= 1), with the px_base and output of each
@@ -945,13 +970,6 @@ cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, cons
 }
 
 } // namespace cr
-
-// Slots up to which samples of one image share a pass (0.8 GB of path state with light samples).  A
-// trace launch costs about 90 us beyond its rays at full rate (the device fills, then drains to the
-// longest rays).  1280x720, 16 samples, 4 bounces, light samples: 48.2 ms with a pass per sample,
-// 42.1 / 38.9 / 37.3 with 2^21 / 2^22 / 2^23 slots; 853x479 with 4 samples through the BVH8-Q: 7.42 ms,
-// 5.58 with 2^21 or more; 500x333 with 4 samples and 8 bounces: 1.92 ms, 0.82 from 2^20 on.
-constexpr uint64_t kPassSlots = 1ull << 22;
 
 extern "C" cr_status cr_render_ex(cr_scene* s, const cr_camera* cam, uint32_t spp, uint32_t max_bounces,
                                   cr_reuse_mode mode, uint32_t group_w, uint32_t group_h, float* out_rgb,
@@ -1013,21 +1031,14 @@ extern "C" cr_status cr_render_ex(cr_scene* s, const cr_camera* cam, uint32_t sp
         po.tile_end = o.tile_end;
         if (po.tile_end == 0) return fail(CR_ERR_INVALID_ARG, "cr_render: tile_end is 0 with tile_begin %u", o.tile_begin);
     }
-    // Samples of small images share passes, up to kPassSlots slots: a pass costs what its longest rays
-    // cost at every bounce, and a few ten thousand rays leave the device half empty.
-    if (spp > 1 && group_w && group_h && !o.debug) {
-        const uint64_t slots = (uint64_t)((cam->width + group_w - 1) / group_w) * ((cam->height + group_h - 1) / group_h) *
-                               group_w * group_h;
-        po.samples = (uint32_t)std::min<uint64_t>(spp, std::max<uint64_t>(1, kPassSlots / slots));
-    }
     RenderPlan plan;
-    for (bool again = false;; again = true) {
+    while (true) {
         st = build_plan(&job, 1, po, plan);
         if (st != CR_OK) return st;
         st = s->ws.ensure(plan.max_slots, plan.npx_total);
         if (st == CR_OK && plan.nee) st = s->ws.ensure_nee(plan.max_slots);
         if (st == CR_OK) break;
-        if (st != CR_ERR_OOM || po.samples == 1 || again) return st;
+        if (st != CR_ERR_OOM || plan.regions == 1) return st;
         s->ws.release(); // one sample per pass needs less memory
         po.samples = 1;
     }
@@ -1491,19 +1502,22 @@ extern "C" cr_status cr_batch_create(const cr_job* jobs, uint32_t n_jobs, const 
     if (!b) return fail(CR_ERR_OOM, "cr_batch_create: host allocation");
     b->jobs.assign(jobs, jobs + n_jobs);
     b->opts = *opts;
-    st = build_plan(b->jobs.data(), n_jobs, po, b->plan);
-    if (st != CR_OK) return st;
+    while (true) {
+        st = build_plan(b->jobs.data(), n_jobs, po, b->plan);
+        if (st != CR_OK) return st;
+        st = b->ws.ensure(b->plan.max_slots, b->plan.npx_total);
+        if (st == CR_OK && b->plan.nee) st = b->ws.ensure_nee(b->plan.max_slots);
+        if (st == CR_OK) break;
+        if (st != CR_ERR_OOM || b->plan.regions == 1) return st;
+        b->ws.release(); // one sample per pass needs less memory
+        po.samples = 1;
+    }
+    g_err.clear();
     if (opts->stream) {
         b->stream = static_cast<cudaStream_t>(opts->stream);
     } else {
         CR_CUDA(cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking));
         b->own_stream = true;
-    }
-    st = b->ws.ensure(b->plan.max_slots, b->plan.npx_total);
-    if (st != CR_OK) return st;
-    if (b->plan.nee) {
-        st = b->ws.ensure_nee(b->plan.max_slots);
-        if (st != CR_OK) return st;
     }
     st = b->dev.upload(b->plan, b->stream);
     if (st != CR_OK) return st;

@@ -170,6 +170,7 @@ struct JobDev {
     // slot_tile = first tile of the job's slot range (slot = (slot_tile + t) m + i)
     uint32_t step;
     uint32_t slot_tile;
+    uint32_t spp;         // samples of the job
 };
 
 // Launch-uniform description of a pass.
@@ -360,10 +361,10 @@ void launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, u
 void launch_finish_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_slots, cudaStream_t st, LaunchCount& lc);
 void launch_finish_accumulate(const PassArgs& p, PathBuffers& b, const cr_debug* dbg, cudaStream_t st,
                               LaunchCount& lc);
-// The pixels' sums of n sample regions of npx pixels (RenderPlan::regions), on top of `sum` unless
-// `first`; to `out` (times inv_spp) if not NULL, else to `sum`.
-void launch_sum_samples(const float4* regions, uint32_t n, uint32_t npx, bool first, float4* sum, float inv_spp,
-                        float* out, cudaStream_t st, LaunchCount& lc);
+// After the pass of samples [s0, s0 + regions) (RenderPlan::regions): each job's regions added to its
+// pixels' sums, the output written where its last sample is among them.
+void launch_sum_samples(const JobDev* jobs, uint32_t n_jobs, float4* accum, uint32_t regions, uint32_t npx, uint32_t s0,
+                        cudaStream_t st, LaunchCount& lc);
 // out[job] = accum / spp for every job of the table (all pixels of all jobs, one launch).
 void launch_output(const JobDev* jobs, uint32_t n_jobs, const float4* accum, uint32_t npx_total, cudaStream_t st,
                    LaunchCount& lc);
@@ -402,7 +403,9 @@ struct PlanOpts {
     bool bvh8 = false;
     bool bvh4 = false; // closest-hit traces through the BVH4 (single renders; shadow rays stay on the BVH2)
     uint32_t tile_begin = 0, tile_end = 0; // single-job plans: render only these tiles (0, 0 = all)
-    uint32_t samples = 1; // single-job plans of whole images: samples of one pass (RenderPlan::regions)
+    // samples of each job that share a pass (RenderPlan::regions; whole images only): 0 = as many as
+    // keep a pass within kPassSlots slots
+    uint32_t samples = 0;
 };
 struct Pass {
     uint32_t job_offset = 0, n_jobs = 0, n_tiles = 0;
@@ -413,12 +416,11 @@ struct RenderPlan {
     bool bvh4 = false;
     bool nee = false; // some job uses next-event estimation
     uint32_t max_bounces = 0, max_slots = 0, npx_total = 0;
-    // > 1: a pass renders up to `regions` samples of the one job, each as a table entry of its own with
-    // its own region of npx pixels in the accumulation buffer; after each pass the regions are added
-    // in sample order to a running sum in the region after them (the last pass writes the output)
-    uint32_t regions = 1, npx = 0;
-    float* out = nullptr;
-    float inv_spp = 0.0f;
+    // > 1: a pass renders up to `regions` samples of every job, each as a table entry of its own.  The
+    // accumulation buffer then has `regions` regions of npx pixels (all jobs'), one per sample of
+    // the pass; after each pass they are added in sample order to the running sums in the region
+    // after them, and a job's last pass writes its output.  jobs[sum_offset ...] has one entry per job.
+    uint32_t regions = 1, npx = 0, sum_offset = 0, n_jobs = 0;
     std::vector<JobDev> jobs;     // all passes' tables, pass by pass
     std::vector<SceneDev> scenes; // scene table
     std::vector<Pass> passes;

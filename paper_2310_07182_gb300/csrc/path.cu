@@ -1617,23 +1617,29 @@ __global__ void k_output_one(const float4* __restrict__ accum, uint32_t npx, flo
 }
 
 // Sums of sample regions, in sample order: the same additions as one sample after another.
-__global__ void k_sum_samples(const float4* __restrict__ regions, uint32_t n, uint32_t npx, uint32_t first,
-                              float4* __restrict__ sum, float inv_spp, float* __restrict__ out) {
+// One thread per pixel of all jobs; reads 16 B per region, HBM-bound.
+__global__ void k_sum_samples(const JobDev* __restrict__ jobs, uint32_t n_jobs, float4* __restrict__ accum,
+                              uint32_t regions, uint32_t npx, uint32_t s0) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= npx) return;
-    float4 a = first ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : sum[i];
+    const JobDev& J = jobs[job_of_pixel(jobs, n_jobs, i)];
+    if (J.spp <= s0) return; // done in an earlier pass
+    const uint32_t n = min(regions, J.spp - s0);
+    float4* const sum = accum + (size_t)regions * npx + i;
+    float4 a = s0 == 0 ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : *sum;
     for (uint32_t k = 0; k < n; ++k) {
-        const float4 r = regions[(size_t)k * npx + i];
+        const float4 r = accum[(size_t)k * npx + i];
         a.x += r.x;
         a.y += r.y;
         a.z += r.z;
     }
-    if (out) {
-        out[3 * (size_t)i + 0] = a.x * inv_spp;
-        out[3 * (size_t)i + 1] = a.y * inv_spp;
-        out[3 * (size_t)i + 2] = a.z * inv_spp;
+    if (s0 + n == J.spp) {
+        float* const o = J.out + 3 * (size_t)(i - J.px_base);
+        o[0] = a.x * J.inv_spp;
+        o[1] = a.y * J.inv_spp;
+        o[2] = a.z * J.inv_spp;
     } else {
-        sum[i] = a;
+        *sum = a;
     }
 }
 
@@ -1845,9 +1851,9 @@ void launch_finish_accumulate(const PassArgs& p, PathBuffers& b, const cr_debug*
     lc.n++;
 }
 
-void launch_sum_samples(const float4* regions, uint32_t n, uint32_t npx, bool first, float4* sum, float inv_spp,
-                        float* out, cudaStream_t st, LaunchCount& lc) {
-    k_sum_samples<<<(npx + 255) / 256, 256, 0, st>>>(regions, n, npx, first ? 1u : 0u, sum, inv_spp, out);
+void launch_sum_samples(const JobDev* jobs, uint32_t n_jobs, float4* accum, uint32_t regions, uint32_t npx, uint32_t s0,
+                        cudaStream_t st, LaunchCount& lc) {
+    k_sum_samples<<<(npx + 255) / 256, 256, 0, st>>>(jobs, n_jobs, accum, regions, npx, s0);
     lc.n++;
 }
 
