@@ -145,7 +145,8 @@ typedef struct {
     uint64_t node_visits, tri_tests; /* counting pass only (CR_OPT_COUNT) */
     uint64_t shadow_rays;      /* shadow rays of next-event estimation (CR_OPT_NEE) */
     double ms_trace_shadow;    /* their any-hit trace */
-    uint64_t h2d_bytes;        /* bytes the call copied host to device (job and scene tables) */
+    uint64_t h2d_bytes;        /* bytes the call sent host to device (its job table, as launch
+                                * arguments or copied; a large plan's scene table) */
     uint64_t d2h_bytes;        /* bytes it copied device to host (a host out_rgb) */
 } cr_stats;
 

@@ -823,22 +823,28 @@ cr_status build_plan(const cr_job* jobs, uint32_t n_jobs, const PlanOpts& po, Re
     return CR_OK;
 }
 
+// Room for the tables, grown on demand (they are reused across calls).
+cr_status Plan::reserve(size_t bj, size_t bs) {
+    if (bj <= cap_jobs && bs <= cap_scenes) return CR_OK;
+    cudaDeviceSynchronize();
+    release();
+    cudaError_t e = cudaMalloc(&d_jobs, bj);
+    if (e == cudaSuccess && bs) e = cudaMalloc(&d_scenes, bs);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        release();
+        return fail(CR_ERR_OOM, "job tables: %s", cudaGetErrorString(e));
+    }
+    cap_jobs = bj;
+    cap_scenes = bs;
+    return CR_OK;
+}
+
 cr_status Plan::upload(const RenderPlan& p, cudaStream_t st) {
     size_t bj = sizeof(JobDev) * p.jobs.size(), bs = sizeof(SceneDev) * p.scenes.size();
+    cr_status rs = reserve(bj, bs);
+    if (rs != CR_OK) return rs;
     cudaError_t e = cudaSuccess;
-    if (bj > cap_jobs || bs > cap_scenes) { // grow (the tables are reused across calls)
-        cudaDeviceSynchronize();
-        release();
-        e = cudaMalloc(&d_jobs, bj);
-        if (e == cudaSuccess) e = cudaMalloc(&d_scenes, bs);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            release();
-            return fail(CR_ERR_OOM, "job tables: %s", cudaGetErrorString(e));
-        }
-        cap_jobs = bj;
-        cap_scenes = bs;
-    }
     e = cudaMemcpyAsync(d_jobs, p.jobs.data(), bj, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_scenes, p.scenes.data(), bs, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return fail(CR_ERR_CUDA, "job tables: %s", cudaGetErrorString(e));
@@ -855,8 +861,8 @@ void Plan::release() {
 
 // Enqueue every stage of a plan on one stream (all passes, all bounces, then the output).
 // Nothing here synchronises the host, so the sequence can also be captured into a graph.
-cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, const ExecOpts& eo, cudaStream_t stream,
-                       LaunchCount& lc, StageTimes* times) {
+cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev* d_scenes, Workspace& ws,
+                       const ExecOpts& eo, cudaStream_t stream, LaunchCount& lc, StageTimes* times) {
     PathBuffers& b = ws.pb;
     StageEvents ev;
     ev.on = times != nullptr;
@@ -865,7 +871,7 @@ cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, cons
     auto check = [&](cudaError_t e, const char* what) {
         if (e != cudaSuccess && failst == CR_OK) failst = fail(CR_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
     };
-    check(cudaMemsetAsync(b.counts, 0, 4 * kCountsWords, stream), "memset counts");
+    if (!eo.counts_cleared) check(cudaMemsetAsync(b.counts, 0, 4 * kCountsWords, stream), "memset counts");
     // a fresh render writes its first samples' sums and its outputs from the accumulation
     // kernel; otherwise (the server's resident sums) the buffer is cleared / output as asked
     const bool fused_out = eo.clear_accum && eo.write_output;
@@ -881,14 +887,14 @@ cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, cons
     ta.speculative = eo.speculative;
     ta.bvh8 = p.bvh8;
     ta.bvh4 = p.bvh4;
-    ta.scenes = dev.d_scenes;
+    ta.scenes = d_scenes;
     ta.slot_scene = b.slot_scene;
     double dummy = 0.0;
     for (const Pass& ps : p.passes) {
         PassArgs P;
-        P.jobs = dev.d_jobs + ps.job_offset;
+        P.jobs = d_jobs + ps.job_offset;
         P.n_jobs = ps.n_jobs;
-        P.scenes = dev.d_scenes;
+        P.scenes = d_scenes;
         P.tile_w = p.tile_w;
         P.tile_h = p.tile_h;
         P.m = p.m;
@@ -953,13 +959,13 @@ cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, cons
         ev.begin(stream, times ? &times->accum : &dummy, "cr accumulate");
         launch_finish_accumulate(P, b, eo.debug, stream, lc);
         if (p.regions > 1)
-            launch_sum_samples(dev.d_jobs + p.sum_offset, p.n_jobs, b.accum, p.regions, p.npx,
+            launch_sum_samples(d_jobs + p.sum_offset, p.n_jobs, b.accum, p.regions, p.npx,
                                (uint32_t)(&ps - p.passes.data()) * p.regions, stream, lc);
         ev.end();
     }
     // pass 0 holds every job (spp >= 1), with the px_base and output of each
     if (eo.write_output && !fused_out)
-        launch_output(dev.d_jobs, p.passes[0].n_jobs, b.accum, p.npx_total, stream, lc);
+        launch_output(d_jobs, p.passes[0].n_jobs, b.accum, p.npx_total, stream, lc);
     check(cudaGetLastError(), "launch");
     if (times) {
         // the caller synchronises the stream before reading; resolve needs completed events
@@ -1043,10 +1049,15 @@ extern "C" cr_status cr_render_ex(cr_scene* s, const cr_camera* cam, uint32_t sp
         po.samples = 1;
     }
     g_err.clear();
+    // the job table (the scene's own entry is its scene table): from the arguments of a first launch
+    // where it is small
     Plan& dev = s->plan_dev;
-    st = dev.upload(plan, stream);
+    const bool setup = plan.jobs.size() <= kSetupJobs;
+    st = setup ? dev.reserve(sizeof(JobDev) * plan.jobs.size(), 0) : dev.upload(plan, stream);
     if (st != CR_OK) return st;
+    const SceneDev* d_scenes = setup ? dev_scene_entry(s, use8) : dev.d_scenes;
     ExecOpts eo;
+    eo.counts_cleared = setup;
     eo.block = block;
     eo.block_secondary = o.block ? block : kSecondaryBlock;
     if (o.stack != 0 && o.stack != 8 && o.stack != 16 && o.stack != 32)
@@ -1078,7 +1089,8 @@ extern "C" cr_status cr_render_ex(cr_scene* s, const cr_camera* cam, uint32_t sp
     }
     if (!out_dev && po.tile_end != 0) // pixels outside the range keep the caller's values
         CR_CUDA(cudaMemcpyAsync(s->d_out, out_rgb, sizeof(float) * 3 * (size_t)npx, cudaMemcpyHostToDevice, stream));
-    st = enqueue_plan(plan, dev, s->ws, eo, stream, lc,
+    if (setup) launch_setup(plan.jobs.data(), (uint32_t)plan.jobs.size(), dev.d_jobs, s->ws.pb.counts, stream, lc);
+    st = enqueue_plan(plan, dev.d_jobs, d_scenes, s->ws, eo, stream, lc,
                       (o.stats && (o.flags & (CR_OPT_STATS | CR_OPT_STATS_TRACES))) ? &times : nullptr);
     if (st != CR_OK) return st;
     if (!out_dev) CR_CUDA(cudaMemcpyAsync(out_rgb, s->d_out, sizeof(float) * 3 * (size_t)npx, cudaMemcpyDeviceToHost, stream));
@@ -1107,7 +1119,7 @@ extern "C" cr_status cr_render_ex(cr_scene* s, const cr_camera* cam, uint32_t sp
         stats.tri_tests = ctr[1];
         stats.shadow_rays = host_counts[kShadowWord / 2];
         stats.ms_trace_shadow = times.trace_shadow;
-        stats.h2d_bytes = sizeof(JobDev) * plan.jobs.size() + sizeof(SceneDev) * plan.scenes.size() +
+        stats.h2d_bytes = sizeof(JobDev) * plan.jobs.size() + (setup ? 0 : sizeof(SceneDev) * plan.scenes.size()) +
                           ((!out_dev && po.tile_end != 0) ? sizeof(float) * 3 * (size_t)npx : 0);
         stats.d2h_bytes = out_dev ? 0 : sizeof(float) * 3 * (uint64_t)npx;
         stats.primary_rays = (uint64_t)npx * spp;
@@ -1525,7 +1537,7 @@ extern "C" cr_status cr_batch_create(const cr_job* jobs, uint32_t n_jobs, const 
     if (opts->flags & CR_BATCH_GRAPH) {
         LaunchCount lc;
         CR_CUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-        st = enqueue_plan(b->plan, b->dev, b->ws, eo, b->stream, lc, nullptr);
+        st = enqueue_plan(b->plan, b->dev.d_jobs, b->dev.d_scenes, b->ws, eo, b->stream, lc, nullptr);
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(b->stream, &g);
         if (st != CR_OK) {
@@ -1559,7 +1571,7 @@ extern "C" cr_status cr_batch_run(cr_batch* b, cr_stats* stats) {
         CR_CUDA(cudaGraphLaunch(b->exec, b->stream));
     } else {
         LaunchCount lc;
-        st = enqueue_plan(b->plan, b->dev, b->ws, eo, b->stream, lc, nullptr);
+        st = enqueue_plan(b->plan, b->dev.d_jobs, b->dev.d_scenes, b->ws, eo, b->stream, lc, nullptr);
         if (st != CR_OK) return st;
         launches = lc.n;
     }

@@ -330,6 +330,11 @@ void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, cons
                         bool one_scene, bool alone, uint32_t* work, cudaStream_t st,
                         LaunchCount& lc);
 
+// A small job table (at most kSetupJobs entries) written from the launch's own arguments, and the
+// counts words cleared.
+constexpr uint32_t kSetupJobs = 24;
+void launch_setup(const JobDev* host_jobs, uint32_t n_jobs, JobDev* jobs, uint32_t* counts, cudaStream_t st,
+                  LaunchCount& lc);
 void launch_raygen(const PassArgs& p, PathBuffers& b, cudaStream_t st, LaunchCount& lc);
 // raygen leaves the primary trace's visiting order (row-major pixels per tile) in the ray queue
 bool primary_pixel_order();
@@ -430,6 +435,7 @@ struct Plan {
     JobDev* d_jobs = nullptr;
     SceneDev* d_scenes = nullptr;
     size_t cap_jobs = 0, cap_scenes = 0;
+    cr_status reserve(size_t bytes_jobs, size_t bytes_scenes);
     cr_status upload(const RenderPlan& p, cudaStream_t st);
     void release();
     ~Plan() { release(); }
@@ -449,6 +455,7 @@ struct ExecOpts {
     bool clear_accum = true; // zero the accumulation buffer first
     bool stats_traces_only = false; // stage events only around the trace launches
     bool write_output = true; // write every job's output after the last pass
+    bool counts_cleared = false; // the counts words are zero already (launch_setup)
     bool ordered_queues = false; // three-launch order-preserving compaction instead of appends
     const cr_debug* debug = nullptr;
     uint32_t debug_npx = 0;
@@ -463,8 +470,8 @@ JobDev job_dev(const cr_job& j, const PlanOpts& po, uint32_t scene_idx, uint32_t
 cr_status queue_status(const uint64_t* host_counts);
 cr_status check_job(const cr_job& j, uint32_t tile_w, uint32_t tile_h);
 bool scene_has_bvh8(const cr_scene* s);
-cr_status enqueue_plan(const RenderPlan& p, const Plan& dev, Workspace& ws, const ExecOpts& eo, cudaStream_t stream,
-                       LaunchCount& lc, StageTimes* times);
+cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev* d_scenes, Workspace& ws,
+                       const ExecOpts& eo, cudaStream_t stream, LaunchCount& lc, StageTimes* times);
 
 // Thread-local message returned by cr_last_error(); handle -> device scene.
 void set_last_error(const char* msg);

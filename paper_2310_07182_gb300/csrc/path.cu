@@ -108,6 +108,21 @@ __device__ __forceinline__ uint32_t launch_entry(const uint32_t* prefix, uint32_
     return lo;
 }
 
+// The start of a render: its job table out of the kernel's arguments, the counts words cleared.  One
+// launch instead of two copies from pageable host memory and a memset (render of 64 x 64 pixels,
+// one sample: 103 -> 96 us).
+struct JobTable {
+    JobDev jobs[kSetupJobs];
+};
+__global__ void k_setup(const __grid_constant__ JobTable t, uint32_t n_jobs, JobDev* __restrict__ jobs,
+                        uint32_t* __restrict__ counts) {
+    static_assert(sizeof(JobDev) % 4 == 0, "copied by words");
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(&t);
+    for (uint32_t i = threadIdx.x; i < n_jobs * (uint32_t)(sizeof(JobDev) / 4); i += blockDim.x)
+        reinterpret_cast<uint32_t*>(jobs)[i] = src[i];
+    for (uint32_t i = threadIdx.x; i < kCountsWords; i += blockDim.x) counts[i] = 0u;
+}
+
 // One block covers blockDim / m whole tiles: every thread finds sigma of its pixel, the
 // inverse map is built in shared memory, then thread j writes slot j of its tile so the
 // slot arrays are written contiguously.
@@ -1689,6 +1704,14 @@ __global__ void k_sample(uint32_t kind, uint32_t n, const float* __restrict__ wo
 
 // ------------------------------------------------------------------------------------
 // Launchers.
+void launch_setup(const JobDev* host_jobs, uint32_t n_jobs, JobDev* jobs, uint32_t* counts, cudaStream_t st,
+                  LaunchCount& lc) {
+    JobTable t;
+    for (uint32_t i = 0; i < n_jobs; ++i) t.jobs[i] = host_jobs[i];
+    k_setup<<<1, 256, 0, st>>>(t, n_jobs, jobs, counts);
+    lc.n++;
+}
+
 void launch_raygen(const PassArgs& p, PathBuffers& b, cudaStream_t st, LaunchCount& lc) {
     const uint32_t block = p.m > 256 ? p.m : 256;
     const uint32_t tiles_per_block = block / p.m;

@@ -112,3 +112,20 @@ def test_samples_that_share_a_pass_sum_in_order(cr, mode, size, spp):
         rays += st1["secondary_rays"]
     assert torch.equal(img, total * torch.tensor(1.0 / spp, dtype=torch.float32, device="cuda"))
     assert st["secondary_rays"] == rays
+
+
+@pytest.mark.parametrize("spp", [1, 11, 22, 23, 24, 25, 40])
+def test_small_and_large_job_tables(cr, spp):
+    """A render's job table (an entry per sample side by side, one more for the sums) comes from launch
+    arguments where it is small and is copied where it is not; a batch of the same job copies it."""
+    S = cr.Scene(scenes.tiny(seed=6, n_soup=300, material_mix="mixed"))
+    cam = scenes.Camera((0.0, 0.0, -3.0), (0.0, 0.0, 0.0), (0.0, 1.0, 0.0), 60.0, 40, 24)
+    kw = dict(spp=spp, max_bounces=3, mode="direction_reuse", seed=9)
+    img, _ = S.render(cam, tile=(8, 8), **kw)
+    out = torch.full_like(img, -1.0)
+    b = cr.cr_batch_create([cr.make_job(S.handle, cam, out, **kw)], cr.make_batch_opts(tile=(8, 8)))
+    try:
+        cr.cr_batch_run(b)
+        assert torch.equal(img, out)
+    finally:
+        cr.cr_batch_destroy(b)
