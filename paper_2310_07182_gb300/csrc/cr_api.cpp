@@ -889,9 +889,13 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
     ta.bvh4 = p.bvh4;
     ta.scenes = d_scenes;
     ta.slot_scene = b.slot_scene;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool chained = cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    ta.chained = chained;
     double dummy = 0.0;
     for (const Pass& ps : p.passes) {
         PassArgs P;
+        P.chained = chained;
         P.jobs = d_jobs + ps.job_offset;
         P.n_jobs = ps.n_jobs;
         P.scenes = d_scenes;
@@ -960,7 +964,7 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
         launch_finish_accumulate(P, b, eo.debug, stream, lc);
         if (p.regions > 1)
             launch_sum_samples(d_jobs + p.sum_offset, p.n_jobs, b.accum, p.regions, p.npx,
-                               (uint32_t)(&ps - p.passes.data()) * p.regions, stream, lc);
+                               (uint32_t)(&ps - p.passes.data()) * p.regions, chained, stream, lc);
         ev.end();
     }
     // pass 0 holds every job (spp >= 1), with the px_base and output of each

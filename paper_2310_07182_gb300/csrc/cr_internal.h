@@ -184,6 +184,7 @@ struct PassArgs {
     uint32_t npx = 0;      // pixels of the debug capture (single-job renders)
     bool nee = false;      // some job of the plan uses next-event estimation
     bool one_scene = false; // the scene table has one entry
+    bool chained = false;   // launches may be set up while the one before ends (launch_step)
     // bit 0: a job's first sample writes its pixel sums without reading them (the buffer is
     // not cleared first); bit 1: its last sample writes the output instead of the sums
     uint32_t accum_mode = 0;
@@ -249,6 +250,7 @@ struct TraceArgs {
     uint32_t* work = nullptr;
     bool one_scene = false; // every ray is in scenes[0]
     bool alone = true;      // no other launches of the library run beside this one
+    bool chained = false;   // may be set up while the launch before ends (launch_step)
     int block = 128;
     bool speculative = false; // parked-leaf speculative traversal (BVH2)
     bool packet = false;      // warp-packet traversal (BVH2)
@@ -323,11 +325,11 @@ void launch_trace_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc);
 void launch_shadow_rays_bvh8(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o,
                              const float4* sh_d, const float4* sh_c, const int32_t* group_queue,
                              const uint32_t* group_count, uint32_t n_groups_max, uint32_t K, float4* radiance,
-                             unsigned long long* n_traced, uint32_t* work, cudaStream_t st, LaunchCount& lc);
+                             unsigned long long* n_traced, bool chained, uint32_t* work, cudaStream_t st, LaunchCount& lc);
 void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
                         const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count,
                         uint32_t n_groups_max, uint32_t K, float4* radiance, unsigned long long* n_traced, bool bvh8,
-                        bool one_scene, bool alone, uint32_t* work, cudaStream_t st,
+                        bool one_scene, bool alone, bool chained, uint32_t* work, cudaStream_t st,
                         LaunchCount& lc);
 
 // A small job table (at most kSetupJobs entries) written from the launch's own arguments, and the
@@ -369,7 +371,7 @@ void launch_finish_accumulate(const PassArgs& p, PathBuffers& b, const cr_debug*
 // After the pass of samples [s0, s0 + regions) (RenderPlan::regions): each job's regions added to its
 // pixels' sums, the output written where its last sample is among them.
 void launch_sum_samples(const JobDev* jobs, uint32_t n_jobs, float4* accum, uint32_t regions, uint32_t npx, uint32_t s0,
-                        cudaStream_t st, LaunchCount& lc);
+                        bool chained, cudaStream_t st, LaunchCount& lc);
 // out[job] = accum / spp for every job of the table (all pixels of all jobs, one launch).
 void launch_output(const JobDev* jobs, uint32_t n_jobs, const float4* accum, uint32_t npx_total, cudaStream_t st,
                    LaunchCount& lc);

@@ -12,6 +12,7 @@
 #include "cr_internal.h"
 #include "debug_checks.cuh"
 #include "device_math.cuh"
+#include "launch_next.cuh"
 
 namespace cr {
 namespace {
@@ -135,6 +136,7 @@ __global__ void k_raygen(PassArgs p, int32_t* __restrict__ pixel, uint16_t* __re
                          uint16_t* __restrict__ slot_scene, float4* __restrict__ ray_o, float4* __restrict__ ray_d,
                          float4* __restrict__ beta, float4* __restrict__ radiance, uint8_t* __restrict__ alive,
                          int32_t* __restrict__ primary_queue, uint32_t* __restrict__ queue_counts) {
+    start_of_step();
     extern __shared__ uint16_t inv[];
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_base[2];
@@ -672,6 +674,7 @@ __global__ void __launch_bounds__(CR_SHADE_WARP_BLOCK, CR_SHADE_MIN_BLOCKS * 128
 #else
 __global__ void k_shade_warp(ShadeArgs a, PassArgs p) {
 #endif
+    start_of_step();
     const uint32_t K = p.k;
     const uint32_t n_groups = a.group_queue ? min(*a.group_count, a.n_groups_max) : a.n_groups_max;
     const uint32_t pos = blockIdx.x * blockDim.x + threadIdx.x;
@@ -816,6 +819,7 @@ __global__ void k_shade_warp(ShadeArgs a, PassArgs p) {
 // members' samples go through shared memory and the hybrid sum is a pairwise tree over the
 // group's slots.
 __global__ void __launch_bounds__(256, CR_SHADE_BLOCK_MIN_BLOCKS) k_shade_block(ShadeArgs a, PassArgs p) {
+    start_of_step();
     __shared__ uint32_t s_bd[8], s_bg[8], s_ba[8];
     __shared__ float s_own[3][256];
     __shared__ float s_sum[3][256];
@@ -1539,12 +1543,11 @@ __global__ void __launch_bounds__(kOsThreads, 3) k_sort_coop(uint32_t* __restric
 // and passes run in sample order, so the sum keeps that order.  With p.accum_mode, a job's
 // first sample starts the sum (no cleared buffer is read) and its last sample writes the
 // output, sum / spp, instead of the sum.
-__global__ void k_finish_accumulate(PassArgs p, const int32_t* __restrict__ pixel,
-                                    const uint16_t* __restrict__ slot_job, const uint8_t* __restrict__ alive,
-                                    const int2* __restrict__ hit, const float4* __restrict__ ray_o,
-                                    const float4* __restrict__ ray_d, const float4* __restrict__ beta,
-                                    const float4* __restrict__ radiance, uint32_t n_slots,
-                                    float4* __restrict__ accum, cr_debug dbg, uint32_t dbg_npx) {
+__global__ void k_finish_accumulate(PassArgs p, const int32_t* pixel, const uint16_t* slot_job, const uint8_t* alive,
+                                    const int2* hit, const float4* ray_o, const float4* ray_d, const float4* beta,
+                                    const float4* radiance, uint32_t n_slots, float4* __restrict__ accum,
+                                    cr_debug dbg, uint32_t dbg_npx) {
+    start_of_step();
     const uint32_t u = blockIdx.x * blockDim.x + threadIdx.x;
     if (u >= n_slots) return;
     uint32_t s = u;
@@ -1633,8 +1636,9 @@ __global__ void k_output_one(const float4* __restrict__ accum, uint32_t npx, flo
 
 // Sums of sample regions, in sample order: the same additions as one sample after another.
 // One thread per pixel of all jobs; reads 16 B per region, HBM-bound.
-__global__ void k_sum_samples(const JobDev* __restrict__ jobs, uint32_t n_jobs, float4* __restrict__ accum,
+__global__ void k_sum_samples(const JobDev* jobs, uint32_t n_jobs, float4* __restrict__ accum,
                               uint32_t regions, uint32_t npx, uint32_t s0) {
+    start_of_step();
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= npx) return;
     const JobDev& J = jobs[job_of_pixel(jobs, n_jobs, i)];
@@ -1720,10 +1724,9 @@ void launch_raygen(const PassArgs& p, PathBuffers& b, cudaStream_t st, LaunchCou
 #define CR_PRIMARY_PIXEL_ORDER 1
 #endif
     // the ray queue is free until the first compaction: it carries the primary trace's order
-    k_raygen<<<grid, block, block * sizeof(uint16_t), st>>>(p, b.pixel, b.slot_job, b.slot_scene, b.ray_o, b.ray_d,
-                                                             b.beta, b.radiance, b.alive,
-                                                             CR_PRIMARY_PIXEL_ORDER ? b.ray_queue : nullptr,
-                                                             b.counts + 8);
+    launch_step(p.chained, k_raygen, grid, block, block * sizeof(uint16_t), st, p, b.pixel, b.slot_job, b.slot_scene,
+                b.ray_o, b.ray_d, b.beta, b.radiance, b.alive, CR_PRIMARY_PIXEL_ORDER ? b.ray_queue : nullptr,
+                b.counts + 8);
     lc.n++;
 }
 
@@ -1774,7 +1777,7 @@ void launch_shadow(const PassArgs& p, PathBuffers& b, bool first, bool bvh8, cud
     const ShadeArgs a = shade_args(p, b, first, false, nullptr);
     launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
                        a.n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
-                       bvh8, p.one_scene, true, b.counts + kWorkWord + 32 + p.bounce, st, lc);
+                       bvh8, p.one_scene, true, p.chained, b.counts + kWorkWord + 32 + p.bounce, st, lc);
 }
 
 void launch_shade(const PassArgs& p, PathBuffers& b, bool first, bool compact, const cr_debug* dbg,
@@ -1782,9 +1785,10 @@ void launch_shade(const PassArgs& p, PathBuffers& b, bool first, bool compact, c
     ShadeArgs a = shade_args(p, b, first, compact, dbg);
     const uint32_t n_pos = b.n_groups * p.k;
     if (p.k <= 32) {
-        k_shade_warp<<<(n_pos + CR_SHADE_WARP_BLOCK - 1) / CR_SHADE_WARP_BLOCK, CR_SHADE_WARP_BLOCK, 0, st>>>(a, p);
+        launch_step(p.chained, k_shade_warp, (n_pos + CR_SHADE_WARP_BLOCK - 1) / CR_SHADE_WARP_BLOCK,
+                    CR_SHADE_WARP_BLOCK, 0, st, a, p);
     } else {
-        k_shade_block<<<(n_pos + 255) / 256, 256, 0, st>>>(a, p);
+        launch_step(p.chained, k_shade_block, (n_pos + 255) / 256, 256, 0, st, a, p);
     }
     lc.n++;
 }
@@ -1801,8 +1805,8 @@ void launch_raygen_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_tiles, 
     const uint32_t tiles_per_block = block / p.m;
     const uint32_t grid = (n_tiles + tiles_per_block - 1) / tiles_per_block;
     // shared memory: the inverse shuffle (2 B per thread), then one live flag per group
-    k_raygen<<<grid, block, block * (sizeof(uint16_t) + sizeof(uint32_t)) + 4, st>>>(
-        q, b.pixel, b.slot_job, b.slot_scene, b.ray_o, b.ray_d, b.beta, b.radiance, b.alive, nullptr, nullptr);
+    launch_step(p.chained, k_raygen, grid, block, block * (sizeof(uint16_t) + sizeof(uint32_t)) + 4, st, q, b.pixel,
+                b.slot_job, b.slot_scene, b.ray_o, b.ray_d, b.beta, b.radiance, b.alive, nullptr, nullptr);
     lc.n++;
 }
 
@@ -1825,9 +1829,10 @@ void launch_shade_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, ui
     ShadeArgs a = shade_args_rolling(p, b, parity, n_groups_max);
     const uint32_t n_pos = n_groups_max * p.k;
     if (p.k <= 32) {
-        k_shade_warp<<<(n_pos + CR_SHADE_WARP_BLOCK - 1) / CR_SHADE_WARP_BLOCK, CR_SHADE_WARP_BLOCK, 0, st>>>(a, p);
+        launch_step(p.chained, k_shade_warp, (n_pos + CR_SHADE_WARP_BLOCK - 1) / CR_SHADE_WARP_BLOCK,
+                    CR_SHADE_WARP_BLOCK, 0, st, a, p);
     } else {
-        k_shade_block<<<(n_pos + 255) / 256, 256, 0, st>>>(a, p);
+        launch_step(p.chained, k_shade_block, (n_pos + 255) / 256, 256, 0, st, a, p);
     }
     lc.n++;
 }
@@ -1838,14 +1843,13 @@ void launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, u
     const ShadeArgs a = shade_args_rolling(p, b, parity, n_groups_max);
     launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
                        n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
-                       bvh8, p.one_scene, false, b.counts + 8 + 4 * (parity ^ 1u) + 3, st, lc);
+                       bvh8, p.one_scene, false, p.chained, b.counts + 8 + 4 * (parity ^ 1u) + 3, st, lc);
 }
 
 void launch_finish_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_slots, cudaStream_t st, LaunchCount& lc) {
     if (!n_slots) return;
-    k_finish_accumulate<<<(n_slots + 255) / 256, 256, 0, st>>>(p, b.pixel, b.slot_job, b.alive, b.hit, b.ray_o,
-                                                               b.ray_d, b.beta, b.radiance, n_slots, b.accum,
-                                                               cr_debug{}, 0);
+    launch_step(p.chained, k_finish_accumulate, (n_slots + 255) / 256, 256, 0, st, p, b.pixel, b.slot_job, b.alive,
+                b.hit, b.ray_o, b.ray_d, b.beta, b.radiance, n_slots, b.accum, cr_debug{}, 0u);
     lc.n++;
 }
 
@@ -1868,15 +1872,14 @@ void launch_compact(const PassArgs& p, PathBuffers& b, bool first, cudaStream_t 
 void launch_finish_accumulate(const PassArgs& p, PathBuffers& b, const cr_debug* dbg, cudaStream_t st,
                               LaunchCount& lc) {
     const uint32_t n_slots = p.n_tiles * p.m;
-    k_finish_accumulate<<<(n_slots + 255) / 256, 256, 0, st>>>(p, b.pixel, b.slot_job, b.alive, b.hit, b.ray_o,
-                                                               b.ray_d, b.beta, b.radiance, n_slots, b.accum,
-                                                               dbg ? *dbg : cr_debug{}, p.npx);
+    launch_step(p.chained, k_finish_accumulate, (n_slots + 255) / 256, 256, 0, st, p, b.pixel, b.slot_job, b.alive,
+                b.hit, b.ray_o, b.ray_d, b.beta, b.radiance, n_slots, b.accum, dbg ? *dbg : cr_debug{}, p.npx);
     lc.n++;
 }
 
 void launch_sum_samples(const JobDev* jobs, uint32_t n_jobs, float4* accum, uint32_t regions, uint32_t npx, uint32_t s0,
-                        cudaStream_t st, LaunchCount& lc) {
-    k_sum_samples<<<(npx + 255) / 256, 256, 0, st>>>(jobs, n_jobs, accum, regions, npx, s0);
+                        bool chained, cudaStream_t st, LaunchCount& lc) {
+    launch_step(chained, k_sum_samples, (npx + 255) / 256, 256, 0, st, jobs, n_jobs, accum, regions, npx, s0);
     lc.n++;
 }
 

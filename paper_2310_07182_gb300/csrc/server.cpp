@@ -466,6 +466,7 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
     P.k = K;
     P.nee = nee;
     P.rolling = true;
+    P.chained = true;
     P.accum_mode = 3u;
     // (rays, groups) appended for the next iteration, then this iteration's work counters
     uint32_t* qn = b.counts + 8 + 4 * (par ^ 1u);
@@ -508,6 +509,7 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
         ta.queue_count = qn;
         ta.work = qn + 2;
         ta.alone = false;
+        ta.chained = true;
         ta.n_max = trace_max;
         if (sort) ta.queue = launch_morton_sort(P, b, 2u * (par ^ 1u), eo.sort_key, L.stream, lc);
         launch_trace(ta, L.stream, lc);

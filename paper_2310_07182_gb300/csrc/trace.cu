@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "cr_internal.h"
+#include "launch_next.cuh"
 #include "trace_common.cuh"
 
 namespace cr {
@@ -333,13 +334,14 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
 
 template <bool kCount, bool kAny, int kSmemS, bool kOne, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __restrict__ scenes,
-                                                           const uint16_t* __restrict__ slot_scene,
-                                                           const float4* __restrict__ ray_o,
-                                                           const float4* __restrict__ ray_d,
-                                                           const int32_t* __restrict__ queue,
-                                                           const uint32_t* __restrict__ queue_count, uint32_t n_max,
+                                                           chained_ptr<kOne, uint16_t> slot_scene,
+                                                           chained_ptr<kOne, float4> ray_o,
+                                                           chained_ptr<kOne, float4> ray_d,
+                                                           chained_ptr<kOne, int32_t> queue,
+                                                           chained_ptr<kOne, uint32_t> queue_count, uint32_t n_max,
                                                            int2* __restrict__ hit, unsigned long long* counters,
                                                            uint32_t* work) {
+    if (kOne) start_of_step();
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     unsigned long long n_node = 0, n_tri = 0;
@@ -683,10 +685,11 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_spec(
 
 template <bool kOne, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
-    const SceneDev* __restrict__ scenes, const uint16_t* __restrict__ slot_scene, const float4* __restrict__ sh_o,
-    const float4* __restrict__ sh_d, const float4* __restrict__ sh_c, const int32_t* __restrict__ group_queue,
-    const uint32_t* __restrict__ group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
+    const SceneDev* __restrict__ scenes, chained_ptr<kOne, uint16_t> slot_scene, chained_ptr<kOne, float4> sh_o,
+    chained_ptr<kOne, float4> sh_d, chained_ptr<kOne, float4> sh_c, chained_ptr<kOne, int32_t> group_queue,
+    chained_ptr<kOne, uint32_t> group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
     unsigned long long* __restrict__ n_traced, uint32_t* work) {
+    if (kOne) start_of_step();
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
     ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
@@ -719,13 +722,13 @@ __global__ void k_rays_from_user(const float* __restrict__ rays, const int32_t* 
 void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
                         const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count,
                         uint32_t n_groups_max, uint32_t K, float4* radiance, unsigned long long* n_traced, bool bvh8,
-                        bool one_scene, bool alone, uint32_t* work, cudaStream_t st,
+                        bool one_scene, bool alone, bool chained, uint32_t* work, cudaStream_t st,
                         LaunchCount& lc) {
     const uint32_t n_pos = n_groups_max * K;
     if (n_pos == 0) return;
     if (bvh8) {
         launch_shadow_rays_bvh8(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count, n_groups_max, K,
-                                radiance, n_traced, work, st, lc);
+                                radiance, n_traced, chained, work, st, lc);
         return;
     }
     const int block = kSecondaryBlock;
@@ -735,8 +738,8 @@ void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, cons
         constexpr bool kOne = decltype(one)::value;
         const uint32_t most = resident_blocks<k_trace_shadow<kOne, kMore>>(block, smem);
         auto run = [&](auto kernel, uint32_t grid) {
-            kernel<<<grid, block, smem, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count,
-                                              n_groups_max, K, radiance, n_traced, work);
+            launch_step(kOne && chained, kernel, grid, block, smem, st, scenes, slot_scene, sh_o, sh_d, sh_c,
+                        group_queue, group_count, n_groups_max, K, radiance, n_traced, work);
         };
         if (need <= most && alone) run(k_trace_shadow<kOne, kFew>, spread_blocks(n_pos, block, most));
         else if (work && most && need > most) run(k_trace_shadow<kOne, kMore>, most);
@@ -792,13 +795,13 @@ SceneDev scene_entry(const DevScene& s, bool bvh8) {
     return e;
 }
 
-template <auto kKernel, int kSmemS>
+template <bool kOne, auto kKernel, int kSmemS>
 static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t st, LaunchCount& lc) {
     const size_t smem = (size_t)warp_smem(kSmemS) * (a.block / 32);
     if (smem > 48 * 1024) // 512-thread blocks with 32 entries need the opt-in beyond 48 KB
         cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kKernel<<<grid, a.block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue, a.queue_count, a.n_max, a.hit,
-                                         a.counters, a.work);
+    launch_step(kOne && a.chained, kKernel, grid, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
+                a.queue_count, a.n_max, a.hit, a.counters, a.work);
     lc.n++;
 }
 
@@ -813,12 +816,14 @@ static void launch_bvh2_scenes(const TraceArgs& a, cudaStream_t st, LaunchCount&
     constexpr auto kP = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kPlain>;
     const uint32_t need = blocks_for(a.n_max, a.block);
     const uint32_t most = resident_blocks<kM>(a.block, (size_t)warp_smem(kSmemS) * (a.block / 32));
-    if (need <= most && a.alone) launch_bvh2_kernel<kF, kSmemS>(a, spread_blocks(a.n_max, a.block, most), st, lc);
-    else if (a.work && most && need > most) launch_bvh2_kernel<kM, kSmemS>(a, most, st, lc);
-    else launch_bvh2_kernel<kP, kSmemS>(a, need, st, lc);
+    if (need <= most && a.alone) launch_bvh2_kernel<kOne, kF, kSmemS>(a, spread_blocks(a.n_max, a.block, most), st, lc);
+    else if (a.work && most && need > most) launch_bvh2_kernel<kOne, kM, kSmemS>(a, most, st, lc);
+    else launch_bvh2_kernel<kOne, kP, kSmemS>(a, need, st, lc);
 }
 
-// kOneScene: whether launches over a single scene have a variant of their own.
+// kOneScene: whether launches over a single scene have a variant of their own.  Only these are set up
+// while the launch before ends: the plain pointers that this takes make launches over several scenes
+// 1% slower (16-job batch 5424 -> 5472 us) and those over one scene 1% faster (1024 x 1024 1185 -> 1175).
 template <bool kOneScene, bool kCount, bool kAny, int kSmemS>
 static void launch_bvh2(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     if (kOneScene && a.one_scene) launch_bvh2_scenes<kOneScene, kCount, kAny, kSmemS>(a, st, lc);

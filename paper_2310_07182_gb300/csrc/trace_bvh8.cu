@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "cr_internal.h"
+#include "launch_next.cuh"
 #include "trace_common.cuh"
 
 namespace cr {
@@ -220,10 +221,10 @@ __device__ __forceinline__ void trace_bvh8_warp(const SceneDev* __restrict__ sce
 
 template <bool kCount, bool kAny, RangeKind kKind>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8(const SceneDev* __restrict__ scenes,
-                             const uint16_t* __restrict__ slot_scene,
-                             const float4* __restrict__ ray_o, const float4* __restrict__ ray_d,
-                             const int32_t* __restrict__ queue, const uint32_t* __restrict__ queue_count,
+                             const uint16_t* slot_scene, const float4* ray_o, const float4* ray_d,
+                             const int32_t* queue, const uint32_t* queue_count,
                              uint32_t n_max, int2* __restrict__ hit, unsigned long long* counters, uint32_t* work) {
+    start_of_step();
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     unsigned long long n_node = 0, n_tri = 0;
     QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit);
@@ -244,10 +245,10 @@ __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8_user(con
 // Shadow rays of next-event estimation over the BVH8-Q (see k_trace_shadow).
 template <RangeKind kKind>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_shadow8(
-    const SceneDev* __restrict__ scenes, const uint16_t* __restrict__ slot_scene, const float4* __restrict__ sh_o,
-    const float4* __restrict__ sh_d, const float4* __restrict__ sh_c, const int32_t* __restrict__ group_queue,
-    const uint32_t* __restrict__ group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
+    const SceneDev* __restrict__ scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
+    const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
     unsigned long long* __restrict__ n_traced, uint32_t* work) {
+    start_of_step();
     const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
     ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
     if (!src.more()) return;
@@ -272,12 +273,11 @@ static void launch_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     } else {
         const uint32_t most = a.work ? resident_blocks<k_trace_bvh8<kCount, kAny, kMore>>(a.block, 0) : 0u;
         if (most && need > most)
-            k_trace_bvh8<kCount, kAny, kMore><<<most, a.block, 0, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
-                                                                      a.queue_count, a.n_max, a.hit, a.counters, a.work);
+            launch_step(a.chained, k_trace_bvh8<kCount, kAny, kMore>, most, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
+                        a.ray_d, a.queue, a.queue_count, a.n_max, a.hit, a.counters, a.work);
         else
-            k_trace_bvh8<kCount, kAny, kPlain><<<need, a.block, 0, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
-                                                                       a.queue_count, a.n_max, a.hit, a.counters,
-                                                                       nullptr);
+            launch_step(a.chained, k_trace_bvh8<kCount, kAny, kPlain>, need, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
+                        a.ray_d, a.queue, a.queue_count, a.n_max, a.hit, a.counters, nullptr);
     }
     lc.n++;
 }
@@ -291,16 +291,17 @@ void launch_trace_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
 void launch_shadow_rays_bvh8(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o,
                              const float4* sh_d, const float4* sh_c, const int32_t* group_queue,
                              const uint32_t* group_count, uint32_t n_groups_max, uint32_t K, float4* radiance,
-                             unsigned long long* n_traced, uint32_t* work, cudaStream_t st, LaunchCount& lc) {
+                             unsigned long long* n_traced, bool chained, uint32_t* work, cudaStream_t st,
+                             LaunchCount& lc) {
     const int block = 128;
     const uint32_t need = blocks_for(n_groups_max * K, block);
     const uint32_t most = work ? resident_blocks<k_trace_shadow8<kMore>>(block, 0) : 0u;
     if (most && need > most)
-        k_trace_shadow8<kMore><<<most, block, 0, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count,
-                                                      n_groups_max, K, radiance, n_traced, work);
+        launch_step(chained, k_trace_shadow8<kMore>, most, block, 0, st, scenes, slot_scene, sh_o, sh_d, sh_c, group_queue,
+                    group_count, n_groups_max, K, radiance, n_traced, work);
     else
-        k_trace_shadow8<kPlain><<<need, block, 0, st>>>(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count,
-                                                       n_groups_max, K, radiance, n_traced, nullptr);
+        launch_step(chained, k_trace_shadow8<kPlain>, need, block, 0, st, scenes, slot_scene, sh_o, sh_d, sh_c, group_queue,
+                    group_count, n_groups_max, K, radiance, n_traced, nullptr);
     lc.n++;
 }
 

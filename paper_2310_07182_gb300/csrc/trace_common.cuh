@@ -363,10 +363,10 @@ struct WarpRange {
 // Rays of a queue of slots (or of the slots in order), hits per slot.
 template <RangeKind kKind>
 struct QueueSrc : WarpRange<kKind> {
-    const uint16_t* __restrict__ slot_scene;
-    const float4* __restrict__ ray_o;
-    const float4* __restrict__ ray_d;
-    const int32_t* __restrict__ queue;
+    const uint16_t* slot_scene;
+    const float4* ray_o;
+    const float4* ray_d;
+    const int32_t* queue;
     int2* __restrict__ hit;
     static constexpr int idle = kTraceIdle;
     static constexpr bool kProbe = false;
@@ -434,11 +434,11 @@ struct UserSrc : WarpRange<kKind>, UserRays {
 // contribution is added to the path radiance of its slot.  Rays traced are counted.
 template <RangeKind kKind>
 struct ShadowSrc : WarpRange<kKind> {
-    const uint16_t* __restrict__ slot_scene;
-    const float4* __restrict__ sh_o;
-    const float4* __restrict__ sh_d;
-    const float4* __restrict__ sh_c;
-    const int32_t* __restrict__ group_queue;
+    const uint16_t* slot_scene;
+    const float4* sh_o;
+    const float4* sh_d;
+    const float4* sh_c;
+    const int32_t* group_queue;
     float4* __restrict__ radiance;
     uint32_t K, traced = 0;
     static constexpr int idle = kTraceIdle;

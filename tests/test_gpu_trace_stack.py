@@ -129,3 +129,28 @@ def test_small_and_large_job_tables(cr, spp):
         assert torch.equal(img, out)
     finally:
         cr.cr_batch_destroy(b)
+
+
+@pytest.mark.parametrize("bvh", ["CR_BVH2", "CR_BVH8Q"])
+@pytest.mark.parametrize("k,size,spp", [(8, (8, 8), 1), (8, (200, 120), 3), (64, (200, 120), 2)])
+def test_chained_launches_and_a_graph_agree(cr, bvh, k, size, spp):
+    """Launches set up while the one before ends (render, direct batch; many calls back to back) and the
+    ordinary ones of a captured graph give the same image."""
+    S = cr.Scene(scenes.tiny(seed=6, n_soup=300, material_mix="mixed"), bvh_flags=cr.CR_BVH2 | cr.CR_BVH8Q)
+    cam = scenes.Camera((0.0, 0.0, -3.0), (0.0, 0.0, 0.0), (0.0, 1.0, 0.0), 60.0, *size)
+    kw = dict(spp=spp, max_bounces=4, mode="direction_reuse", seed=9)
+    out = torch.empty((size[1], size[0], 3), device="cuda")
+    jobs = [cr.make_job(S.handle, cam, out, **kw)]
+    images = []
+    for flags in (cr.CR_BATCH_GRAPH, 0):
+        b = cr.cr_batch_create(jobs, cr.make_batch_opts(tile=(8, 8), k=k, bvh=getattr(cr, bvh), flags=flags))
+        try:
+            for _ in range(3):
+                out.fill_(-1.0)
+                cr.cr_batch_run(b)
+                images.append(out.clone())
+        finally:
+            cr.cr_batch_destroy(b)
+    for _ in range(20):
+        images.append(S.render(cam, tile=(8, 8), k=k, bvh=getattr(cr, bvh), **kw)[0])
+    assert all(torch.equal(images[0], i) for i in images[1:])
