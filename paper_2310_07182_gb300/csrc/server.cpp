@@ -680,6 +680,13 @@ extern "C" cr_status cr_server_create(const cr_server_opts* o, cr_server** out) 
             st = CR_ERR_CUDA;
         }
     }
+    // the lanes' streams do not wait for the legacy stream, on which the clears run (behind whatever
+    // the caller has queued there)
+    if (st == CR_OK && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+        cudaGetLastError();
+        set_last_error("cr_server_create: clearing the counters failed");
+        st = CR_ERR_CUDA;
+    }
     if (st != CR_OK) {
         cleanup();
         return st;

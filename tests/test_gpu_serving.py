@@ -212,3 +212,24 @@ def test_express_lane_fallbacks(cr, world):
         assert torch.equal(small, ref)
     finally:
         cr.cr_server_destroy(srv)
+
+
+def test_a_server_made_while_the_default_stream_is_busy(cr, world):
+    """The counters of a new server are cleared before its first iteration, also when the caller has work queued
+    on the default stream (the render streams do not wait for that one)."""
+    sc, S = world
+    cam = _cam(sc["tiny"].camera, 64, 48)
+    kw = dict(spp=2, max_bounces=3, seed=4)
+    ref, _ = S["tiny"].render(cam, tile=(8, 8), k=8, **kw)
+    out = torch.empty((48, 64, 3), device="cuda")
+    junk = torch.empty(1 << 28, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for v in range(100):
+            junk.fill_(v)  # about 20 ms
+        srv = cr.cr_server_create(256 << 20, tile=(8, 8), k=8)
+        try:
+            cr.cr_server_wait(srv, cr.cr_server_submit(srv, cr.make_job(S["tiny"].handle, cam, out, **kw)), 60000)
+            assert torch.equal(out, ref)
+        finally:
+            cr.cr_server_destroy(srv)
