@@ -895,7 +895,8 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
     double dummy = 0.0;
     for (const Pass& ps : p.passes) {
         PassArgs P;
-        P.chained = chained;
+        // behind a kernel: the call's first launch, or a pass before this one
+        P.chained = chained && (&ps != &p.passes[0] || (eo.counts_cleared && (fused_out || !eo.clear_accum)));
         P.jobs = d_jobs + ps.job_offset;
         P.n_jobs = ps.n_jobs;
         P.scenes = d_scenes;
@@ -912,11 +913,13 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
         b.n_groups = n_slots / p.k;
         ev.begin(stream, times ? &times->raygen : &dummy, "cr raygen");
         launch_raygen(P, b, stream, lc);
+        P.chained = chained;
         ev.end();
         ta.queue = primary_pixel_order() ? b.ray_queue : nullptr; // written by raygen: pixel order per tile
         ta.queue_count = nullptr;
         ta.n_max = n_slots;
         ta.counters = nullptr;
+        ta.beside = false;
         // primary rays of a warp end together: lanes that take new rays on their own mix pixel blocks
         // and cost 20% of this trace
         ta.work = eo.persistent ? b.counts + kWorkWord : nullptr;
@@ -932,9 +935,10 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
             ev.begin(stream, times ? &times->shade : &dummy, "cr shade");
             launch_shade(P, b, bnc == 1, !eo.ordered_queues, eo.debug, stream, lc);
             ev.end();
+            bool shadow = false;
             if (P.nee && b.shadow_d) {
                 ev.begin(stream, times ? &times->trace_shadow : &dummy, "cr trace shadow", true);
-                launch_shadow(P, b, bnc == 1, p.bvh8, stream, lc);
+                shadow = launch_shadow(P, b, bnc == 1, p.bvh8, stream, lc);
                 ev.end();
             }
             if (eo.ordered_queues) {
@@ -952,6 +956,7 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
             }
             ta.counters = eo.count ? b.counters : nullptr;
             ta.work = b.counts + kWorkWord + bnc;
+            ta.beside = shadow && !eo.ordered_queues && !p.sort; // nothing was launched in between
             ta.two_phase = eo.phase_budget > 0 && ws.phase.state;
             ta.phase = ws.phase;
             ta.phase.budget = eo.phase_budget;

@@ -251,6 +251,7 @@ struct TraceArgs {
     bool one_scene = false; // every ray is in scenes[0]
     bool alone = true;      // no other launches of the library run beside this one
     bool chained = false;   // may be set up while the launch before ends (launch_step)
+    bool beside = false;    // the launch before is launch_shadow's of the same bounce (next_may_start)
     int block = 128;
     bool speculative = false; // parked-leaf speculative traversal (BVH2)
     bool packet = false;      // warp-packet traversal (BVH2)
@@ -320,7 +321,8 @@ constexpr uint32_t kWorkWord = 136, kWorkWords = 64;
 constexpr uint32_t kQueueErrWord = 5, kQueueCountWords = kStatWord - 8;
 // Shadow rays of the last shade (positions of its group queue): any-hit traversal, and the
 // contribution of each unblocked one added to the path radiance.
-void launch_shadow(const PassArgs& p, PathBuffers& b, bool first, bool bvh8, cudaStream_t st, LaunchCount& lc);
+// launch_shadow*: false where nothing was launched (no light samples)
+bool launch_shadow(const PassArgs& p, PathBuffers& b, bool first, bool bvh8, cudaStream_t st, LaunchCount& lc);
 void launch_trace_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc);
 void launch_shadow_rays_bvh8(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o,
                              const float4* sh_d, const float4* sh_c, const int32_t* group_queue,
@@ -363,7 +365,7 @@ void launch_rays_from_user(const float* rays, const int32_t* skip, uint32_t n, f
 void launch_raygen_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_tiles, cudaStream_t st, LaunchCount& lc);
 void launch_shade_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max,
                           cudaStream_t st, LaunchCount& lc);
-void launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max, bool bvh8,
+bool launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max, bool bvh8,
                            cudaStream_t st, LaunchCount& lc);
 void launch_finish_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_slots, cudaStream_t st, LaunchCount& lc);
 void launch_finish_accumulate(const PassArgs& p, PathBuffers& b, const cr_debug* dbg, cudaStream_t st,

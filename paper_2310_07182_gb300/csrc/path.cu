@@ -1772,12 +1772,13 @@ static ShadeArgs shade_args(const PassArgs& p, PathBuffers& b, bool first, bool 
     return a;
 }
 
-void launch_shadow(const PassArgs& p, PathBuffers& b, bool first, bool bvh8, cudaStream_t st, LaunchCount& lc) {
-    if (!p.nee || !b.shadow_d) return;
+bool launch_shadow(const PassArgs& p, PathBuffers& b, bool first, bool bvh8, cudaStream_t st, LaunchCount& lc) {
+    if (!p.nee || !b.shadow_d || !b.n_groups) return false;
     const ShadeArgs a = shade_args(p, b, first, false, nullptr);
     launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
                        a.n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
                        bvh8, p.one_scene, true, p.chained, b.counts + kWorkWord + 32 + p.bounce, st, lc);
+    return true;
 }
 
 void launch_shade(const PassArgs& p, PathBuffers& b, bool first, bool compact, const cr_debug* dbg,
@@ -1837,13 +1838,14 @@ void launch_shade_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, ui
     lc.n++;
 }
 
-void launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max, bool bvh8,
+bool launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max, bool bvh8,
                            cudaStream_t st, LaunchCount& lc) {
-    if (!p.nee || !b.shadow_d || !n_groups_max) return;
+    if (!p.nee || !b.shadow_d || !n_groups_max) return false;
     const ShadeArgs a = shade_args_rolling(p, b, parity, n_groups_max);
     launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
                        n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
                        bvh8, p.one_scene, false, p.chained, b.counts + 8 + 4 * (parity ^ 1u) + 3, st, lc);
+    return true;
 }
 
 void launch_finish_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_slots, cudaStream_t st, LaunchCount& lc) {

@@ -466,18 +466,19 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
     P.k = K;
     P.nee = nee;
     P.rolling = true;
-    P.chained = true;
+    P.chained = false; // behind the copies' event and the memset; then behind a kernel
     P.accum_mode = 3u;
     // (rays, groups) appended for the next iteration, then this iteration's work counters
     uint32_t* qn = b.counts + 8 + 4 * (par ^ 1u);
     cudaMemsetAsync(qn, 0, 16, L.stream);
     launch_shade_rolling(P, b, par, n_groups, L.stream, lc);
-    launch_shadow_rolling(P, b, par, n_groups, po.bvh8, L.stream, lc);
+    P.chained = n_groups != 0;
     if (n_fin) {
         P.launch_job = L.d_lists[set];
         P.launch_prefix = L.d_lists[set] + kMaxRuns;
         P.n_launch = n_fin;
         launch_finish_rolling(P, b, fin_slots, L.stream, lc);
+        P.chained = host_copies.empty();
     }
     {
         std::lock_guard<std::mutex> lk(mu);
@@ -494,7 +495,10 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
         P.ray_queue = b.ray_queue;
         P.group_queue_out = b.group_queue + (size_t)(par ^ 1u) * b.n_groups;
         launch_raygen_rolling(P, b, start_tiles, L.stream, lc);
+        P.chained = true;
     }
+    // after the sums and the new samples' rays, which it does not touch, so that the trace runs beside it
+    const bool shadow = launch_shadow_rolling(P, b, par, n_groups, po.bvh8, L.stream, lc);
     if (trace_max) {
         TraceArgs ta;
         ta.ray_o = b.ray_o;
@@ -509,7 +513,8 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
         ta.queue_count = qn;
         ta.work = qn + 2;
         ta.alone = false;
-        ta.chained = true;
+        ta.chained = P.chained;
+        ta.beside = shadow && !sort;
         ta.n_max = trace_max;
         if (sort) ta.queue = launch_morton_sort(P, b, 2u * (par ^ 1u), eo.sort_key, L.stream, lc);
         launch_trace(ta, L.stream, lc);

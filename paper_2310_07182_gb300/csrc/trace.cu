@@ -332,7 +332,7 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
 #define CR_TRACE_MAXNREG 56 // 36 warps resident per SM, no spills; 48 and 64 are within 1%, 40 costs 4%
 #endif
 
-template <bool kCount, bool kAny, int kSmemS, bool kOne, RangeKind kKind>
+template <bool kCount, bool kAny, int kSmemS, bool kOne, RangeKind kKind, bool kBeside>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __restrict__ scenes,
                                                            chained_ptr<kOne, uint16_t> slot_scene,
                                                            chained_ptr<kOne, float4> ray_o,
@@ -341,13 +341,14 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __res
                                                            chained_ptr<kOne, uint32_t> queue_count, uint32_t n_max,
                                                            int2* __restrict__ hit, unsigned long long* counters,
                                                            uint32_t* work) {
-    if (kOne) start_of_step();
+    if (kOne && !kBeside) start_of_step();
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     unsigned long long n_node = 0, n_tri = 0;
     QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit);
     if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemS, kOne, !kCount && !kAny && kKind != kPlain>(scenes, src, smem_stack, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
+    if (kBeside) start_of_step();
 }
 
 // A caller's rays and hit arrays, no scratch between: cr_trace_rays used to copy the rays into the
@@ -690,6 +691,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
     chained_ptr<kOne, uint32_t> group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
     unsigned long long* __restrict__ n_traced, uint32_t* work) {
     if (kOne) start_of_step();
+    next_may_start();
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
     ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
@@ -795,12 +797,12 @@ SceneDev scene_entry(const DevScene& s, bool bvh8) {
     return e;
 }
 
-template <bool kOne, auto kKernel, int kSmemS>
+template <bool kOne, bool kBeside, auto kKernel, int kSmemS>
 static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t st, LaunchCount& lc) {
     const size_t smem = (size_t)warp_smem(kSmemS) * (a.block / 32);
     if (smem > 48 * 1024) // 512-thread blocks with 32 entries need the opt-in beyond 48 KB
         cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_step(kOne && a.chained, kKernel, grid, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
+    launch_step(kBeside || (kOne && a.chained), kKernel, grid, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
                 a.queue_count, a.n_max, a.hit, a.counters, a.work);
     lc.n++;
 }
@@ -809,25 +811,38 @@ static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t s
 // out lane by lane where a.work allows it (kMore), else one per lane of as many blocks as it takes
 // (kPlain).  With fewer rays they are spread over all resident warps (kFew), unless other launches
 // share the device (a server's lanes): 24 requests took 6.65 ms against 6.54.
-template <bool kOne, bool kCount, bool kAny, int kSmemS>
+template <bool kOne, bool kCount, bool kAny, int kSmemS, bool kBeside>
 static void launch_bvh2_scenes(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    constexpr auto kM = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kMore>;
-    constexpr auto kF = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kFew>;
-    constexpr auto kP = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kPlain>;
+    constexpr auto kM = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kMore, kBeside>;
+    constexpr auto kF = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kFew, kBeside>;
+    constexpr auto kP = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kPlain, kBeside>;
     const uint32_t need = blocks_for(a.n_max, a.block);
     const uint32_t most = resident_blocks<kM>(a.block, (size_t)warp_smem(kSmemS) * (a.block / 32));
-    if (need <= most && a.alone) launch_bvh2_kernel<kOne, kF, kSmemS>(a, spread_blocks(a.n_max, a.block, most), st, lc);
-    else if (a.work && most && need > most) launch_bvh2_kernel<kOne, kM, kSmemS>(a, most, st, lc);
-    else launch_bvh2_kernel<kOne, kP, kSmemS>(a, need, st, lc);
+    if (need <= most && a.alone) launch_bvh2_kernel<kOne, kBeside, kF, kSmemS>(a, spread_blocks(a.n_max, a.block, most), st, lc);
+    else if (a.work && most && need > most) launch_bvh2_kernel<kOne, kBeside, kM, kSmemS>(a, most, st, lc);
+    else launch_bvh2_kernel<kOne, kBeside, kP, kSmemS>(a, need, st, lc);
 }
+
+// Queue positions up to which a launch over one scene runs beside the light samples' trace before it
+// (kBeside).  Interior, light samples, 4 bounces: 96x64 480 -> 360 us, 512x320 1020 -> 932, 1280x720 2965 ->
+// 2853; with 4 samples of that in a pass (3.7M positions) 9460 -> 9560, with 8 of them 36.1 -> 36.9 ms (the
+// variant's inner loop is a little slower).  Launches over several scenes gain at 6.5M positions still.
+constexpr uint32_t kBesideOne = 1u << 21;
 
 // kOneScene: whether launches over a single scene have a variant of their own.  Only these are set up
 // while the launch before ends: the plain pointers that this takes make launches over several scenes
 // 1% slower (16-job batch 5424 -> 5472 us) and those over one scene 1% faster (1024 x 1024 1185 -> 1175).
 template <bool kOneScene, bool kCount, bool kAny, int kSmemS>
 static void launch_bvh2(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    if (kOneScene && a.one_scene) launch_bvh2_scenes<kOneScene, kCount, kAny, kSmemS>(a, st, lc);
-    else launch_bvh2_scenes<false, kCount, kAny, kSmemS>(a, st, lc);
+    constexpr bool kMayBeside = !kCount && !kAny;
+    if (kOneScene && a.one_scene) {
+        if (kMayBeside && a.beside && a.n_max <= kBesideOne)
+            launch_bvh2_scenes<kOneScene, kCount, kAny, kSmemS, kMayBeside>(a, st, lc);
+        else launch_bvh2_scenes<kOneScene, kCount, kAny, kSmemS, false>(a, st, lc);
+    } else {
+        if (kMayBeside && a.beside) launch_bvh2_scenes<false, kCount, kAny, kSmemS, kMayBeside>(a, st, lc);
+        else launch_bvh2_scenes<false, kCount, kAny, kSmemS, false>(a, st, lc);
+    }
 }
 
 template <bool kCount, bool kAny>

@@ -219,17 +219,18 @@ __device__ __forceinline__ void trace_bvh8_warp(const SceneDev* __restrict__ sce
 #define CR_BVH8_MIN_BLOCKS 8 // resident 128-thread blocks per SM the register budget is sized for
 #endif
 
-template <bool kCount, bool kAny, RangeKind kKind>
+template <bool kCount, bool kAny, RangeKind kKind, bool kBeside>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8(const SceneDev* __restrict__ scenes,
                              const uint16_t* slot_scene, const float4* ray_o, const float4* ray_d,
                              const int32_t* queue, const uint32_t* queue_count,
                              uint32_t n_max, int2* __restrict__ hit, unsigned long long* counters, uint32_t* work) {
-    start_of_step();
+    if (!kBeside) start_of_step();
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     unsigned long long n_node = 0, n_tri = 0;
     QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit);
     if (src.more()) trace_bvh8_warp<kCount, kAny>(scenes, src, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
+    if (kBeside) start_of_step();
 }
 
 template <bool kCount, bool kAny, RangeKind kKind>
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_shadow8(
     const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
     unsigned long long* __restrict__ n_traced, uint32_t* work) {
     start_of_step();
+    next_may_start();
     const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
     ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
     if (!src.more()) return;
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_shadow8(
 
 // As for the BVH2: rays handed out lane by lane where the launch may hold more than lanes are
 // resident at once.
-template <bool kCount, bool kAny>
+template <bool kCount, bool kAny, bool kBeside>
 static void launch_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     const uint32_t need = blocks_for(a.n_max, a.block);
     if (a.user.rays) {
@@ -271,21 +273,22 @@ static void launch_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
         else
             k_trace_bvh8_user<kCount, kAny, kPlain><<<need, a.block, 0, st>>>(a.scenes, a.user, a.n_max, a.counters, nullptr);
     } else {
-        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8<kCount, kAny, kMore>>(a.block, 0) : 0u;
+        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8<kCount, kAny, kMore, kBeside>>(a.block, 0) : 0u;
         if (most && need > most)
-            launch_step(a.chained, k_trace_bvh8<kCount, kAny, kMore>, most, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
+            launch_step(kBeside || a.chained, k_trace_bvh8<kCount, kAny, kMore, kBeside>, most, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
                         a.ray_d, a.queue, a.queue_count, a.n_max, a.hit, a.counters, a.work);
         else
-            launch_step(a.chained, k_trace_bvh8<kCount, kAny, kPlain>, need, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
+            launch_step(kBeside || a.chained, k_trace_bvh8<kCount, kAny, kPlain, kBeside>, need, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
                         a.ray_d, a.queue, a.queue_count, a.n_max, a.hit, a.counters, nullptr);
     }
     lc.n++;
 }
 
 void launch_trace_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    if (a.any_hit) launch_bvh8<false, true>(a, st, lc);
-    else if (a.counters) launch_bvh8<true, false>(a, st, lc);
-    else launch_bvh8<false, false>(a, st, lc);
+    if (a.any_hit) launch_bvh8<false, true, false>(a, st, lc);
+    else if (a.counters) launch_bvh8<true, false, false>(a, st, lc);
+    else if (a.beside) launch_bvh8<false, false, true>(a, st, lc);
+    else launch_bvh8<false, false, false>(a, st, lc);
 }
 
 void launch_shadow_rays_bvh8(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o,

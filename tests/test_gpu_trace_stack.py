@@ -154,3 +154,31 @@ def test_chained_launches_and_a_graph_agree(cr, bvh, k, size, spp):
     for _ in range(20):
         images.append(S.render(cam, tile=(8, 8), k=k, bvh=getattr(cr, bvh), **kw)[0])
     assert all(torch.equal(images[0], i) for i in images[1:])
+
+
+@pytest.mark.parametrize("bvh", ["CR_BVH2", "CR_BVH8Q"])
+@pytest.mark.parametrize("size,spp", [((8, 8), 1), ((200, 120), 3), ((1500, 1000), 2)])
+def test_light_samples_beside_the_next_trace(cr, bvh, size, spp):
+    """The trace that runs beside the light samples' (below and above its size rule, one and two scenes, captured
+    and not) gives the images of the launches one after the other (a counting pass)."""
+    S = cr.Scene(scenes.interior(n_spheres=60, width=96, height=64), bvh_flags=cr.CR_BVH2 | cr.CR_BVH8Q)
+    T = cr.Scene(scenes.tiny(seed=6, n_soup=300, material_mix="mixed"), bvh_flags=cr.CR_BVH2 | cr.CR_BVH8Q)
+    c = scenes.interior(n_spheres=60, width=96, height=64).camera
+    cam = scenes.Camera(c.pos, c.look_at, c.up, c.vfov_deg, *size)
+    b = getattr(cr, bvh)
+    kw = dict(spp=spp, max_bounces=3, mode="direction_reuse", seed=9, nee=True)
+    want = S.render(cam, tile=(8, 8), k=8, bvh=b, flags=cr.CR_OPT_COUNT, stats=True, **kw)[0]
+    for _ in range(5):
+        assert torch.equal(want, S.render(cam, tile=(8, 8), k=8, bvh=b, **kw)[0])
+    out, other = torch.empty_like(want), torch.empty_like(want)
+    jobs = [cr.make_job(S.handle, cam, out, **kw), cr.make_job(T.handle, cam, other, **kw)]
+    for n in (1, 2):
+        for flags in (0, cr.CR_BATCH_GRAPH):
+            h = cr.cr_batch_create(jobs[:n], cr.make_batch_opts(tile=(8, 8), k=8, bvh=b, flags=flags))
+            try:
+                for _ in range(3):
+                    out.fill_(-1.0)
+                    cr.cr_batch_run(h)
+                    assert torch.equal(want, out)
+            finally:
+                cr.cr_batch_destroy(h)
