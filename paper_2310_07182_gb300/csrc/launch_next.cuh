@@ -14,8 +14,8 @@
 //  - chained is set only where the operation before on the stream is a kernel of the same call: the
 //    first launch of a call, and one behind a copy, a memset or an event of another stream, is an
 //    ordinary one.
-// Measured: 64 x 64 pixels, 6 launches, 98.4 -> 88.9 us; 512 x 512 in 64-slot groups, 18 launches,
-// 808 -> 769; 1024 x 1024, 1174 -> 1158; 24 server requests 6530 -> 6460.  Letting blocks start
+// Measured: 64 x 64 pixels, 6 launches, 98.4 -> 88.9 us; 500 x 333 in 64-slot groups, 20 launches,
+// 808 -> 769; 1920 x 1080, 1174 -> 1158; 24 server requests 6530 -> 6460.  Letting blocks start
 // while the one before is still running (an early trigger) gave nothing more: they then fill the
 // SMs in the order in which these drain, and the 64-slot groups took 781 to 800 us.  Nodes of a
 // captured graph follow each other closely already (16-job batch 5424 us against 5440), so a
