@@ -919,7 +919,7 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
         ta.queue_count = nullptr;
         ta.n_max = n_slots;
         ta.counters = nullptr;
-        ta.beside = false;
+        ta.shadow = nullptr;
         // primary rays of a warp end together: lanes that take new rays on their own mix pixel blocks
         // and cost 20% of this trace
         ta.work = eo.persistent ? b.counts + kWorkWord : nullptr;
@@ -935,10 +935,13 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
             ev.begin(stream, times ? &times->shade : &dummy, "cr shade");
             launch_shade(P, b, bnc == 1, !eo.ordered_queues, eo.debug, stream, lc);
             ev.end();
-            bool shadow = false;
-            if (P.nee && b.shadow_d) {
+            // the light samples' trace: by the launch of the closest-hit trace below where nothing comes
+            // between and the stages are not timed one by one
+            const ShadowArgs sh = shadow_args(P, b, bnc == 1, p.bvh8);
+            const bool together = !eo.ordered_queues && !p.sort && !times;
+            if (sh.n_groups_max && !together) {
                 ev.begin(stream, times ? &times->trace_shadow : &dummy, "cr trace shadow", true);
-                shadow = launch_shadow(P, b, bnc == 1, p.bvh8, stream, lc);
+                launch_shadow(sh, stream, lc);
                 ev.end();
             }
             if (eo.ordered_queues) {
@@ -956,7 +959,7 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
             }
             ta.counters = eo.count ? b.counters : nullptr;
             ta.work = b.counts + kWorkWord + bnc;
-            ta.beside = shadow && !eo.ordered_queues && !p.sort; // nothing was launched in between
+            ta.shadow = sh.n_groups_max && together ? &sh : nullptr;
             ta.two_phase = eo.phase_budget > 0 && ws.phase.state;
             ta.phase = ws.phase;
             ta.phase.budget = eo.phase_budget;

@@ -233,6 +233,24 @@ struct UserRays {
     bool aligned = false; // rays lie on a 16-byte boundary
 };
 
+// The light samples' rays of a shade (positions of its group queue): any-hit traversal, and the
+// contribution of each unblocked one added to the path radiance.  n_groups_max 0: none.
+struct ShadowArgs {
+    const SceneDev* scenes = nullptr;
+    const uint16_t* slot_scene = nullptr;
+    const float4* sh_o = nullptr;
+    const float4* sh_d = nullptr;
+    const float4* sh_c = nullptr;
+    const int32_t* group_queue = nullptr; // NULL: groups [0, n_groups_max)
+    const uint32_t* group_count = nullptr;
+    uint32_t n_groups_max = 0, K = 1;
+    float4* radiance = nullptr;
+    unsigned long long* n_traced = nullptr;
+    uint32_t* work = nullptr; // as in TraceArgs
+    bool bvh8 = false;
+    bool one_scene = false, alone = true, chained = false; // as in TraceArgs
+};
+
 // Arguments of one trace launch over a queue of slots, or over a caller's rays.
 struct TraceArgs {
     UserRays user; // rays != NULL: [0, n_max) of these instead of slots (scene 0 of the table)
@@ -251,7 +269,9 @@ struct TraceArgs {
     bool one_scene = false; // every ray is in scenes[0]
     bool alone = true;      // no other launches of the library run beside this one
     bool chained = false;   // may be set up while the launch before ends (launch_step)
-    bool beside = false;    // the launch before is launch_shadow's of the same bounce (next_may_start)
+    // light samples of the same shade, traced by the same launch where there is one for both, else
+    // by a launch before it; NULL: none
+    const ShadowArgs* shadow = nullptr;
     int block = 128;
     bool speculative = false; // parked-leaf speculative traversal (BVH2)
     bool packet = false;      // warp-packet traversal (BVH2)
@@ -319,20 +339,11 @@ struct PathBuffers {
 constexpr uint32_t kCountsWords = 256, kStatWord = 64, kCounterWord = 128, kShadowWord = 200;
 constexpr uint32_t kWorkWord = 136, kWorkWords = 64;
 constexpr uint32_t kQueueErrWord = 5, kQueueCountWords = kStatWord - 8;
-// Shadow rays of the last shade (positions of its group queue): any-hit traversal, and the
-// contribution of each unblocked one added to the path radiance.
-// launch_shadow*: false where nothing was launched (no light samples)
-bool launch_shadow(const PassArgs& p, PathBuffers& b, bool first, bool bvh8, cudaStream_t st, LaunchCount& lc);
+// Light samples of the last shade (n_groups_max 0 where it had none).
+ShadowArgs shadow_args(const PassArgs& p, PathBuffers& b, bool first, bool bvh8);
 void launch_trace_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc);
-void launch_shadow_rays_bvh8(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o,
-                             const float4* sh_d, const float4* sh_c, const int32_t* group_queue,
-                             const uint32_t* group_count, uint32_t n_groups_max, uint32_t K, float4* radiance,
-                             unsigned long long* n_traced, bool chained, uint32_t* work, cudaStream_t st, LaunchCount& lc);
-void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
-                        const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count,
-                        uint32_t n_groups_max, uint32_t K, float4* radiance, unsigned long long* n_traced, bool bvh8,
-                        bool one_scene, bool alone, bool chained, uint32_t* work, cudaStream_t st,
-                        LaunchCount& lc);
+void launch_shadow(const ShadowArgs& a, cudaStream_t st, LaunchCount& lc);
+void launch_shadow_bvh8(const ShadowArgs& a, cudaStream_t st, LaunchCount& lc);
 
 // A small job table (at most kSetupJobs entries) written from the launch's own arguments, and the
 // counts words cleared.
@@ -365,8 +376,7 @@ void launch_rays_from_user(const float* rays, const int32_t* skip, uint32_t n, f
 void launch_raygen_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_tiles, cudaStream_t st, LaunchCount& lc);
 void launch_shade_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max,
                           cudaStream_t st, LaunchCount& lc);
-bool launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max, bool bvh8,
-                           cudaStream_t st, LaunchCount& lc);
+ShadowArgs shadow_args_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max, bool bvh8);
 void launch_finish_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_slots, cudaStream_t st, LaunchCount& lc);
 void launch_finish_accumulate(const PassArgs& p, PathBuffers& b, const cr_debug* dbg, cudaStream_t st,
                               LaunchCount& lc);

@@ -6,8 +6,8 @@
 // before has ended, and each of its threads waits in start_of_step(), before its first access to
 // memory, until that grid is complete and its writes are visible.  Rules:
 //  - every kernel given to launch_step() begins with start_of_step(), in all its threads (a grid is
-//    then complete only after the one before it, so it also follows all earlier ones); one kernel
-//    ends with it instead (next_may_start);
+//    then complete only after the one before it, so it also follows all earlier ones).  Only behind
+//    that wait are an earlier grid's writes promised to be visible, so none reads anything before it;
 //  - what an earlier launch of the chain writes is read through plain pointers (chained_ptr):
 //    a const __restrict__ parameter may be read by loads that take memory as constant for the
 //    whole life of the grid, which begins before the wait;
@@ -27,16 +27,6 @@
 namespace cr {
 
 __device__ __forceinline__ void start_of_step() { cudaGridDependencySynchronize(); }
-
-// The light samples' trace and the closest-hit trace of a bounce need nothing from each other, and each
-// spends 80 us filling and draining the device.  So the first lets the next grid in as soon as
-// all its own blocks have started (which is after all earlier launches are complete), and the second,
-// launched with `beside`, takes the room as it drains and calls start_of_step() at its end instead of
-// its start: it is still complete only after the one before it.  It reads nothing that an unfinished
-// grid writes.  24 server requests 6390 -> 5740 us, a 16-job batch 5419 -> 5301 (in captured graphs too),
-// an interior of 96 x 64 pixels 480 -> 360, 992 -> 695 through the BVH8-Q; kBesideOne says where it
-// does not pay.
-__device__ __forceinline__ void next_may_start() { cudaTriggerProgrammaticLaunchCompletion(); }
 
 template <typename... P, typename... A>
 void launch_step(bool chained, void (*kernel)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t st,

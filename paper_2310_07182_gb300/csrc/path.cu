@@ -1772,13 +1772,29 @@ static ShadeArgs shade_args(const PassArgs& p, PathBuffers& b, bool first, bool 
     return a;
 }
 
-bool launch_shadow(const PassArgs& p, PathBuffers& b, bool first, bool bvh8, cudaStream_t st, LaunchCount& lc) {
-    if (!p.nee || !b.shadow_d || !b.n_groups) return false;
-    const ShadeArgs a = shade_args(p, b, first, false, nullptr);
-    launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
-                       a.n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
-                       bvh8, p.one_scene, true, p.chained, b.counts + kWorkWord + 32 + p.bounce, st, lc);
-    return true;
+static ShadowArgs shadow_args_of(const PassArgs& p, const PathBuffers& b, const ShadeArgs& a, bool bvh8, uint32_t* work) {
+    ShadowArgs s;
+    s.scenes = p.scenes;
+    s.slot_scene = b.slot_scene;
+    s.sh_o = b.shadow_o;
+    s.sh_d = b.shadow_d;
+    s.sh_c = b.shadow_c;
+    s.group_queue = a.group_queue;
+    s.group_count = a.group_count;
+    s.n_groups_max = a.n_groups_max;
+    s.K = p.k;
+    s.radiance = b.radiance;
+    s.n_traced = reinterpret_cast<unsigned long long*>(b.counts + kShadowWord);
+    s.work = work;
+    s.bvh8 = bvh8;
+    s.one_scene = p.one_scene;
+    s.chained = p.chained;
+    return s;
+}
+
+ShadowArgs shadow_args(const PassArgs& p, PathBuffers& b, bool first, bool bvh8) {
+    if (!p.nee || !b.shadow_d) return ShadowArgs();
+    return shadow_args_of(p, b, shade_args(p, b, first, false, nullptr), bvh8, b.counts + kWorkWord + 32 + p.bounce);
 }
 
 void launch_shade(const PassArgs& p, PathBuffers& b, bool first, bool compact, const cr_debug* dbg,
@@ -1838,14 +1854,12 @@ void launch_shade_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, ui
     lc.n++;
 }
 
-bool launch_shadow_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max, bool bvh8,
-                           cudaStream_t st, LaunchCount& lc) {
-    if (!p.nee || !b.shadow_d || !n_groups_max) return false;
-    const ShadeArgs a = shade_args_rolling(p, b, parity, n_groups_max);
-    launch_shadow_rays(p.scenes, b.slot_scene, b.shadow_o, b.shadow_d, b.shadow_c, a.group_queue, a.group_count,
-                       n_groups_max, p.k, b.radiance, reinterpret_cast<unsigned long long*>(b.counts + kShadowWord),
-                       bvh8, p.one_scene, false, p.chained, b.counts + 8 + 4 * (parity ^ 1u) + 3, st, lc);
-    return true;
+ShadowArgs shadow_args_rolling(const PassArgs& p, PathBuffers& b, uint32_t parity, uint32_t n_groups_max, bool bvh8) {
+    if (!p.nee || !b.shadow_d) return ShadowArgs();
+    ShadowArgs s = shadow_args_of(p, b, shade_args_rolling(p, b, parity, n_groups_max), bvh8,
+                                  b.counts + 8 + 4 * (parity ^ 1u) + 3);
+    s.alone = false;
+    return s;
 }
 
 void launch_finish_rolling(const PassArgs& p, PathBuffers& b, uint32_t n_slots, cudaStream_t st, LaunchCount& lc) {

@@ -497,8 +497,9 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
         launch_raygen_rolling(P, b, start_tiles, L.stream, lc);
         P.chained = true;
     }
-    // after the sums and the new samples' rays, which it does not touch, so that the trace runs beside it
-    const bool shadow = launch_shadow_rolling(P, b, par, n_groups, po.bvh8, L.stream, lc);
+    // after the sums and the new samples' rays, which it does not touch, so that one launch can trace both
+    const ShadowArgs sh = shadow_args_rolling(P, b, par, n_groups, po.bvh8);
+    if (sh.n_groups_max && (sort || !trace_max)) launch_shadow(sh, L.stream, lc);
     if (trace_max) {
         TraceArgs ta;
         ta.ray_o = b.ray_o;
@@ -514,7 +515,7 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
         ta.work = qn + 2;
         ta.alone = false;
         ta.chained = P.chained;
-        ta.beside = shadow && !sort;
+        ta.shadow = sh.n_groups_max && !sort ? &sh : nullptr;
         ta.n_max = trace_max;
         if (sort) ta.queue = launch_morton_sort(P, b, 2u * (par ^ 1u), eo.sort_key, L.stream, lc);
         launch_trace(ta, L.stream, lc);

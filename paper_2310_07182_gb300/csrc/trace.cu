@@ -332,7 +332,7 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
 #define CR_TRACE_MAXNREG 56 // 36 warps resident per SM, no spills; 48 and 64 are within 1%, 40 costs 4%
 #endif
 
-template <bool kCount, bool kAny, int kSmemS, bool kOne, RangeKind kKind, bool kBeside>
+template <bool kCount, bool kAny, int kSmemS, bool kOne, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __restrict__ scenes,
                                                            chained_ptr<kOne, uint16_t> slot_scene,
                                                            chained_ptr<kOne, float4> ray_o,
@@ -341,14 +341,13 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __res
                                                            chained_ptr<kOne, uint32_t> queue_count, uint32_t n_max,
                                                            int2* __restrict__ hit, unsigned long long* counters,
                                                            uint32_t* work) {
-    if (kOne && !kBeside) start_of_step();
+    if (kOne) start_of_step();
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     unsigned long long n_node = 0, n_tri = 0;
-    QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit);
+    QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit, blockIdx.x, gridDim.x);
     if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemS, kOne, !kCount && !kAny && kKind != kPlain>(scenes, src, smem_stack, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
-    if (kBeside) start_of_step();
 }
 
 // A caller's rays and hit arrays, no scratch between: cr_trace_rays used to copy the rays into the
@@ -543,7 +542,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
     const float4* tris = sc.tris;
     unsigned long long dummy = 0;
     if (!uniform_scene) { // rare: a warp straddling two jobs of different scenes
-        QueueSrc<kPlain> src(n, nullptr, slot_scene, ray_o, ray_d, queue, hit);
+        QueueSrc<kPlain> src(n, nullptr, slot_scene, ray_o, ray_d, queue, hit, blockIdx.x, gridDim.x);
         trace_bvh2_warp<false, false, kSmemStack, false, false>(scenes, src, smem_stack, dummy, dummy);
         return;
     }
@@ -691,14 +690,44 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
     chained_ptr<kOne, uint32_t> group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
     unsigned long long* __restrict__ n_traced, uint32_t* work) {
     if (kOne) start_of_step();
-    next_may_start();
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
-    ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K);
+    ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K, blockIdx.x, gridDim.x);
     if (!src.more()) return;
     unsigned long long dn = 0, dt = 0;
     trace_bvh2_warp<false, true, kSmemStack, kOne, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
     src.add_traced(n_traced);
+}
+
+// The next closest-hit rays of a bounce and its light samples in one launch: neither trace needs the
+// other's results, and each alone spends about 80 us filling the device and draining it to its longest
+// rays.  Blocks below `first` trace the closest hits, which take longer; the others come in as these end
+// (the other way round: 24 requests 5780 us against 5550, a batch of 16 jobs 5358 against 5314, single
+// renders alike).  Against a launch for each: an interior of 96 x 64 pixels 480 -> 350 us, 1280 x 720
+// 2965 -> 2805, with 16 samples 36.9 -> 36.5 ms, 24 requests 6390 -> 5550 us.
+template <int kSmemS, bool kOne, RangeKind kKind>
+__global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_both(
+    const SceneDev* __restrict__ scenes, chained_ptr<kOne, uint16_t> slot_scene, chained_ptr<kOne, float4> ray_o,
+    chained_ptr<kOne, float4> ray_d, chained_ptr<kOne, int32_t> queue, chained_ptr<kOne, uint32_t> queue_count,
+    uint32_t n_max, int2* __restrict__ hit, uint32_t* work, chained_ptr<kOne, float4> sh_o,
+    chained_ptr<kOne, float4> sh_d, chained_ptr<kOne, float4> sh_c, chained_ptr<kOne, int32_t> group_queue,
+    chained_ptr<kOne, uint32_t> group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
+    unsigned long long* __restrict__ n_traced, uint32_t* sh_work, uint32_t first) {
+    if (kOne) start_of_step();
+    extern __shared__ uint32_t smem_stack[];
+    unsigned long long dn = 0, dt = 0;
+    if (blockIdx.x < first) {
+        const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
+        QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit, blockIdx.x, first);
+        if (src.more()) trace_bvh2_warp<false, false, kSmemS, kOne, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
+    } else {
+        const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
+        ShadowSrc<kKind> src(n, sh_work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K, blockIdx.x - first,
+                             gridDim.x - first);
+        if (!src.more()) return;
+        trace_bvh2_warp<false, true, kSmemS, kOne, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
+        src.add_traced(n_traced);
+    }
 }
 
 __global__ void k_hits_to_user(const float4* __restrict__ tris, const int2* __restrict__ hit, uint32_t n,
@@ -721,16 +750,11 @@ __global__ void k_rays_from_user(const float* __restrict__ rays, const int32_t* 
 
 } // namespace
 
-void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
-                        const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count,
-                        uint32_t n_groups_max, uint32_t K, float4* radiance, unsigned long long* n_traced, bool bvh8,
-                        bool one_scene, bool alone, bool chained, uint32_t* work, cudaStream_t st,
-                        LaunchCount& lc) {
-    const uint32_t n_pos = n_groups_max * K;
+void launch_shadow(const ShadowArgs& a, cudaStream_t st, LaunchCount& lc) {
+    const uint32_t n_pos = a.n_groups_max * a.K;
     if (n_pos == 0) return;
-    if (bvh8) {
-        launch_shadow_rays_bvh8(scenes, slot_scene, sh_o, sh_d, sh_c, group_queue, group_count, n_groups_max, K,
-                                radiance, n_traced, chained, work, st, lc);
+    if (a.bvh8) {
+        launch_shadow_bvh8(a, st, lc);
         return;
     }
     const int block = kSecondaryBlock;
@@ -740,14 +764,14 @@ void launch_shadow_rays(const SceneDev* scenes, const uint16_t* slot_scene, cons
         constexpr bool kOne = decltype(one)::value;
         const uint32_t most = resident_blocks<k_trace_shadow<kOne, kMore>>(block, smem);
         auto run = [&](auto kernel, uint32_t grid) {
-            launch_step(kOne && chained, kernel, grid, block, smem, st, scenes, slot_scene, sh_o, sh_d, sh_c,
-                        group_queue, group_count, n_groups_max, K, radiance, n_traced, work);
+            launch_step(kOne && a.chained, kernel, grid, block, smem, st, a.scenes, a.slot_scene, a.sh_o, a.sh_d, a.sh_c,
+                        a.group_queue, a.group_count, a.n_groups_max, a.K, a.radiance, a.n_traced, a.work);
         };
-        if (need <= most && alone) run(k_trace_shadow<kOne, kFew>, spread_blocks(n_pos, block, most));
-        else if (work && most && need > most) run(k_trace_shadow<kOne, kMore>, most);
+        if (need <= most && a.alone) run(k_trace_shadow<kOne, kFew>, spread_blocks(n_pos, block, most));
+        else if (a.work && most && need > most) run(k_trace_shadow<kOne, kMore>, most);
         else run(k_trace_shadow<kOne, kPlain>, need);
     };
-    if (one_scene) go(std::true_type());
+    if (a.one_scene) go(std::true_type());
     else go(std::false_type());
     lc.n++;
 }
@@ -797,12 +821,12 @@ SceneDev scene_entry(const DevScene& s, bool bvh8) {
     return e;
 }
 
-template <bool kOne, bool kBeside, auto kKernel, int kSmemS>
+template <bool kOne, auto kKernel, int kSmemS>
 static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t st, LaunchCount& lc) {
     const size_t smem = (size_t)warp_smem(kSmemS) * (a.block / 32);
     if (smem > 48 * 1024) // 512-thread blocks with 32 entries need the opt-in beyond 48 KB
         cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_step(kBeside || (kOne && a.chained), kKernel, grid, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
+    launch_step(kOne && a.chained, kKernel, grid, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
                 a.queue_count, a.n_max, a.hit, a.counters, a.work);
     lc.n++;
 }
@@ -811,38 +835,56 @@ static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t s
 // out lane by lane where a.work allows it (kMore), else one per lane of as many blocks as it takes
 // (kPlain).  With fewer rays they are spread over all resident warps (kFew), unless other launches
 // share the device (a server's lanes): 24 requests took 6.65 ms against 6.54.
-template <bool kOne, bool kCount, bool kAny, int kSmemS, bool kBeside>
+template <bool kOne, bool kCount, bool kAny, int kSmemS>
 static void launch_bvh2_scenes(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    constexpr auto kM = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kMore, kBeside>;
-    constexpr auto kF = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kFew, kBeside>;
-    constexpr auto kP = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kPlain, kBeside>;
+    constexpr auto kM = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kMore>;
+    constexpr auto kF = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kFew>;
+    constexpr auto kP = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kPlain>;
     const uint32_t need = blocks_for(a.n_max, a.block);
     const uint32_t most = resident_blocks<kM>(a.block, (size_t)warp_smem(kSmemS) * (a.block / 32));
-    if (need <= most && a.alone) launch_bvh2_kernel<kOne, kBeside, kF, kSmemS>(a, spread_blocks(a.n_max, a.block, most), st, lc);
-    else if (a.work && most && need > most) launch_bvh2_kernel<kOne, kBeside, kM, kSmemS>(a, most, st, lc);
-    else launch_bvh2_kernel<kOne, kBeside, kP, kSmemS>(a, need, st, lc);
+    if (need <= most && a.alone) launch_bvh2_kernel<kOne, kF, kSmemS>(a, spread_blocks(a.n_max, a.block, most), st, lc);
+    else if (a.work && most && need > most) launch_bvh2_kernel<kOne, kM, kSmemS>(a, most, st, lc);
+    else launch_bvh2_kernel<kOne, kP, kSmemS>(a, need, st, lc);
 }
 
-// Queue positions up to which a launch over one scene runs beside the light samples' trace before it
-// (kBeside).  Interior, light samples, 4 bounces: 96x64 480 -> 360 us, 512x320 1020 -> 932, 1280x720 2965 ->
-// 2853; with 4 samples of that in a pass (3.7M positions) 9460 -> 9560, with 8 of them 36.1 -> 36.9 ms (the
-// variant's inner loop is a little slower).  Launches over several scenes gain at 6.5M positions still.
-constexpr uint32_t kBesideOne = 1u << 21;
+// One launch for a.shadow's rays too (k_trace_both): the kind of range that the longer list asks for.
+template <bool kOne, int kSmemS>
+static void launch_bvh2_both(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
+    const ShadowArgs& s = *a.shadow;
+    const size_t smem = (size_t)warp_smem(kSmemS) * (a.block / 32);
+    const uint32_t n_sh = s.n_groups_max * s.K;
+    const uint32_t need = blocks_for(a.n_max, a.block), need_sh = blocks_for(n_sh, a.block);
+    const uint32_t most = resident_blocks<k_trace_both<kSmemS, kOne, kMore>>(a.block, smem);
+    auto run = [&](auto kernel, uint32_t first, uint32_t rest) {
+        if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        launch_step(kOne && a.chained, kernel, first + rest, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d,
+                    a.queue, a.queue_count, a.n_max, a.hit, a.work, s.sh_o, s.sh_d, s.sh_c, s.group_queue, s.group_count,
+                    s.n_groups_max, s.K, s.radiance, s.n_traced, s.work, first);
+    };
+    if (need <= most && need_sh <= most && a.alone)
+        run(k_trace_both<kSmemS, kOne, kFew>, spread_blocks(a.n_max, a.block, most), spread_blocks(n_sh, a.block, most));
+    else if (a.work && s.work && most && (need > most || need_sh > most))
+        run(k_trace_both<kSmemS, kOne, kMore>, need < most ? need : most, need_sh < most ? need_sh : most);
+    else run(k_trace_both<kSmemS, kOne, kPlain>, need, need_sh);
+    lc.n++;
+}
 
 // kOneScene: whether launches over a single scene have a variant of their own.  Only these are set up
 // while the launch before ends: the plain pointers that this takes make launches over several scenes
 // 1% slower (16-job batch 5424 -> 5472 us) and those over one scene 1% faster (1024 x 1024 1185 -> 1175).
 template <bool kOneScene, bool kCount, bool kAny, int kSmemS>
 static void launch_bvh2(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    constexpr bool kMayBeside = !kCount && !kAny;
-    if (kOneScene && a.one_scene) {
-        if (kMayBeside && a.beside && a.n_max <= kBesideOne)
-            launch_bvh2_scenes<kOneScene, kCount, kAny, kSmemS, kMayBeside>(a, st, lc);
-        else launch_bvh2_scenes<kOneScene, kCount, kAny, kSmemS, false>(a, st, lc);
-    } else {
-        if (kMayBeside && a.beside) launch_bvh2_scenes<false, kCount, kAny, kSmemS, kMayBeside>(a, st, lc);
-        else launch_bvh2_scenes<false, kCount, kAny, kSmemS, false>(a, st, lc);
+    const bool one = kOneScene && a.one_scene;
+    if constexpr (!kCount && !kAny) {
+        if (a.shadow) {
+            if (one) launch_bvh2_both<kOneScene, kSmemS>(a, st, lc);
+            else launch_bvh2_both<false, kSmemS>(a, st, lc);
+            return;
+        }
     }
+    if (a.shadow) launch_shadow(*a.shadow, st, lc);
+    if (one) launch_bvh2_scenes<kOneScene, kCount, kAny, kSmemS>(a, st, lc);
+    else launch_bvh2_scenes<false, kCount, kAny, kSmemS>(a, st, lc);
 }
 
 template <bool kCount, bool kAny>
@@ -860,7 +902,10 @@ static void launch_bvh2_user(const TraceArgs& a, cudaStream_t st, LaunchCount& l
 }
 
 void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    if (a.n_max == 0) return;
+    if (a.n_max == 0) {
+        if (a.shadow) launch_shadow(*a.shadow, st, lc);
+        return;
+    }
     if (a.user.rays && !a.bvh8 && !(a.bvh4 && !a.any_hit)) { // a caller's rays through the BVH2
         if (a.any_hit) launch_bvh2_user<false, true>(a, st, lc);
         else if (a.counters) launch_bvh2_user<true, false>(a, st, lc);
@@ -873,6 +918,11 @@ void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
         launch_trace_bvh8(a, st, lc);
         return;
     }
+    // the BVH4 and the BVH2's variants trace closest hits only
+    const bool variant = (a.bvh4 && !a.any_hit) ||
+                         (!a.any_hit && !a.counters &&
+                          ((a.two_phase && a.phase.state && a.queue && a.queue_count) || a.packet || a.speculative));
+    if (a.shadow && variant) launch_shadow(*a.shadow, st, lc);
     if (a.bvh4 && !a.any_hit) { // BVH4 kernel (trace_bvh4.cu)
         launch_trace_bvh4(a, st, lc);
         return;

@@ -156,7 +156,7 @@ __global__ void __maxnreg__(CR_TRACE4_MAXNREG) k_trace_bvh4(const SceneDev* __re
                                                              int2* __restrict__ hit, unsigned long long* counters) {
     extern __shared__ uint32_t smem_stack[];
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
-    trace_bvh4_rays<kCount>(scenes, QueueSrc<kPlain>(n, nullptr, slot_scene, ray_o, ray_d, queue, hit), smem_stack, counters);
+    trace_bvh4_rays<kCount>(scenes, QueueSrc<kPlain>(n, nullptr, slot_scene, ray_o, ray_d, queue, hit, blockIdx.x, gridDim.x), smem_stack, counters);
 }
 
 template <bool kCount>

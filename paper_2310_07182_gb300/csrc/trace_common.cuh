@@ -330,8 +330,9 @@ struct WarpRange {
     uint32_t n, next, end;
     uint32_t* work;
     uint32_t first_free; // the first position that `work` hands out
-    __device__ __forceinline__ WarpRange(uint32_t n_, uint32_t* work_) : n(n_), work(work_) {
-        const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, warps = gridDim.x * blockDim.x >> 5;
+    // block, blocks: this block's place among those that share the list
+    __device__ __forceinline__ WarpRange(uint32_t n_, uint32_t* work_, uint32_t block, uint32_t blocks) : n(n_), work(work_) {
+        const uint32_t w = (block * blockDim.x + threadIdx.x) >> 5, warps = blocks * blockDim.x >> 5;
         // fewer positions than lanes: the same share for every warp
         const uint32_t each = kKind == RangeKind::kPlain ? kTraceChunk : min(max((n + warps - 1u) / warps, kTraceShare), kTraceChunk);
         next = min(w * each, n);
@@ -372,8 +373,8 @@ struct QueueSrc : WarpRange<kKind> {
     static constexpr bool kProbe = false;
     __device__ __forceinline__ void probe(bool, uint32_t) {}
     __device__ __forceinline__ QueueSrc(uint32_t n, uint32_t* work, const uint16_t* ss, const float4* o, const float4* d,
-                                        const int32_t* q, int2* h)
-        : WarpRange<kKind>(n, work), slot_scene(ss), ray_o(o), ray_d(d), queue(q), hit(h) {}
+                                        const int32_t* q, int2* h, uint32_t block, uint32_t blocks)
+        : WarpRange<kKind>(n, work, block, blocks), slot_scene(ss), ray_o(o), ray_d(d), queue(q), hit(h) {}
     __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) const {
         const int slot = queue ? queue[i] : (int)i;
         ro = ray_o[slot];
@@ -402,7 +403,7 @@ struct UserSrc : WarpRange<kKind>, UserRays {
     __device__ __forceinline__ void probe(bool live, uint32_t oct) {
         idle = __popc(__reduce_or_sync(0xffffffffu, live ? 1u << oct : 0u)) <= 1 ? 32 : kTraceIdle;
     }
-    __device__ __forceinline__ UserSrc(uint32_t n, uint32_t* work, const UserRays& u) : WarpRange<kKind>(n, work), UserRays(u) {}
+    __device__ __forceinline__ UserSrc(uint32_t n, uint32_t* work, const UserRays& u) : WarpRange<kKind>(n, work, blockIdx.x, gridDim.x), UserRays(u) {}
     __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) const {
         const float* r = rays + 8 * (size_t)i;
         if (aligned) {
@@ -445,8 +446,9 @@ struct ShadowSrc : WarpRange<kKind> {
     static constexpr bool kProbe = false;
     __device__ __forceinline__ void probe(bool, uint32_t) {}
     __device__ __forceinline__ ShadowSrc(uint32_t n, uint32_t* work, const uint16_t* ss, const float4* o, const float4* d,
-                                         const float4* c, const int32_t* gq, float4* rad, uint32_t k)
-        : WarpRange<kKind>(n, work), slot_scene(ss), sh_o(o), sh_d(d), sh_c(c), group_queue(gq), radiance(rad), K(k) {}
+                                         const float4* c, const int32_t* gq, float4* rad, uint32_t k, uint32_t block,
+                                         uint32_t blocks)
+        : WarpRange<kKind>(n, work, block, blocks), slot_scene(ss), sh_o(o), sh_d(d), sh_c(c), group_queue(gq), radiance(rad), K(k) {}
     __device__ __forceinline__ bool load(uint32_t i, int& key, float4& ro, float4& rd) {
         const uint32_t g = group_queue ? (uint32_t)group_queue[i / K] : i / K;
         const int slot = (int)(g * K + i % K);

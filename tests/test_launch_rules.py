@@ -1,0 +1,42 @@
+"""Kernels that may be set up while the one before on the stream ends (launch_next.cuh): an earlier grid's
+writes are promised to be visible only behind the wait, so it is the first statement of each of them."""
+import os
+import re
+
+import pytest
+
+from paper_2310_07182_gb300 import build
+
+SRC = {f: open(os.path.join(build.CSRC, f)).read() for f in os.listdir(build.CSRC) if f.endswith((".cu", ".cuh", ".cpp"))}
+
+
+def _kernels():
+    """(file, name, body) of every kernel."""
+    for f, s in SRC.items():
+        s = re.sub(r"#else\n__global__.*\n|#.*\n", "", s)  # a kernel's other heading; directives
+        for m in re.finditer(r"__global__\s+void\s+(?:__\w+__\((?:[^()]|\([^()]*\))*\)\s*)?(k_\w+)\s*\(", s):
+            i = s.index("{", m.end())
+            depth, j = 1, i + 1
+            while depth:
+                depth += {"{": 1, "}": -1}.get(s[j], 0)
+                j += 1
+            yield f, m.group(1), s[i + 1:j - 1]
+
+
+CHAINED = [k for k in _kernels() if "start_of_step" in k[2]]
+
+
+def test_kernels_are_found():
+    names = {k[1] for k in CHAINED}
+    assert {"k_raygen", "k_trace_bvh2", "k_trace_shadow", "k_trace_bvh8", "k_finish_accumulate"} <= names
+
+
+@pytest.mark.parametrize("f,name,body", CHAINED, ids=[k[1] for k in CHAINED])
+def test_nothing_comes_before_the_wait(f, name, body):
+    assert re.match(r"\s*(if \(kOne\) )?start_of_step\(\);", body)
+    assert body.count("start_of_step") == 1
+
+
+def test_no_kernel_lets_the_next_one_in_early():
+    for s in SRC.values():
+        assert "cudaTriggerProgrammaticLaunchCompletion" not in s and "griddepcontrol" not in s
