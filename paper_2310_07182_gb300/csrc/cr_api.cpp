@@ -890,7 +890,8 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
     ta.scenes = d_scenes;
     ta.slot_scene = b.slot_scene;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const bool chained = cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    // (stage events would lie between a launch and the kernel before it)
+    const bool chained = !times && cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
     ta.chained = chained;
     double dummy = 0.0;
     for (const Pass& ps : p.passes) {

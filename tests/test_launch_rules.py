@@ -40,3 +40,13 @@ def test_nothing_comes_before_the_wait(f, name, body):
 def test_no_kernel_lets_the_next_one_in_early():
     for s in SRC.values():
         assert "cudaTriggerProgrammaticLaunchCompletion" not in s and "griddepcontrol" not in s
+
+
+def test_stage_events_and_chained_launches_exclude_each_other():
+    """A launch behind a recorded event is not behind a kernel: no launch of a timed plan is chained."""
+    s = SRC["cr_api.cpp"]
+    plan = s[s.index("cr_status enqueue_plan("):]
+    plan = plan[:plan.index("\n}\n")]
+    decide = re.search(r"const bool chained = ([^;]*);", plan).group(1)
+    assert decide.startswith("!times && ")
+    assert all("chained" in v for v in re.findall(r"\.chained = ([^;]*);", plan))
