@@ -358,38 +358,245 @@ uint32_t plane_above(double g) {
 
 } // namespace
 
-DevBVH2 pack_bvh2(const HostBVH2& b, int n_threads) {
-    DevBVH2 out;
+namespace {
+
+struct Child2 {
+    float lo[3], hi[3];
+    int32_t link; // >= 0 inner node, < 0 leaf code
+};
+
+Child2 child2_of(const HostBVH2& b, uint32_t node, int which) {
+    const float* o = &b.nodes[16 * (size_t)node];
+    Child2 c;
+    const int x = which == 0 ? 0 : 4, z = which == 0 ? 8 : 10;
+    c.lo[0] = o[x]; c.hi[0] = o[x + 1]; c.lo[1] = o[x + 2]; c.hi[1] = o[x + 3]; c.lo[2] = o[z]; c.hi[2] = o[z + 1];
+    std::memcpy(&c.link, &o[12 + which], 4);
+    return c;
+}
+
+struct Grid {
+    float lo[3], scale[3];
+    uint32_t root, around; // root node; the grid around it (0 for the scene's own)
+    uint32_t nested;       // how many lie around it
+    int finer[3];          // scale is that of the grid around, times 2^finer
+};
+
+Grid grid_over(const float* blo, const float* bhi) {
+    Grid g = {};
     double big = 0.0, far = 0.0;
     for (int k = 0; k < 3; ++k) {
-        big = std::max(big, (double)b.hi[k] - (double)b.lo[k]);
-        far = std::max(far, std::max(std::fabs((double)b.lo[k]), std::fabs((double)b.hi[k])));
+        big = std::max(big, (double)bhi[k] - (double)blo[k]);
+        far = std::max(far, std::max(std::fabs((double)blo[k]), std::fabs((double)bhi[k])));
     }
     for (int k = 0; k < 3; ++k) {
         // a flat axis takes 2^-12 of the largest extent, a point a few units of its coordinates;
         // a margin of at least 2^-11 on both sides keeps the enlarged boxes inside the grid
-        const double ext = std::max({(double)b.hi[k] - (double)b.lo[k], big * 0x1.0p-12, far * 0x1.0p-22, 1e-30});
-        const double want = (double)b.lo[k] - ext * 0x1.0p-11;
-        out.lo[k] = (float)want;
-        if ((double)out.lo[k] > want) out.lo[k] = std::nextafterf(out.lo[k], -INFINITY);
-        out.scale[k] = (float)std::min(1.498 / ((double)b.lo[k] + ext - (double)out.lo[k]), 1e30);
+        const double ext = std::max({(double)bhi[k] - (double)blo[k], big * 0x1.0p-12, far * 0x1.0p-22, 1e-30});
+        const double want = (double)blo[k] - ext * 0x1.0p-11;
+        g.lo[k] = (float)want;
+        if ((double)g.lo[k] > want) g.lo[k] = std::nextafterf(g.lo[k], -INFINITY);
+        g.scale[k] = (float)std::min(1.498 / ((double)blo[k] + ext - (double)g.lo[k]), 1e30);
     }
-    out.words.resize((size_t)kDevNode2Words * b.n_nodes);
+    return g;
+}
+
+// The grid over a box within grid `around`; false where its steps cannot be fitted.
+bool grid_within(const float* blo, const float* bhi, const Grid& around, Grid& g) {
+    g = grid_over(blo, bhi);
+    for (int k = 0; k < 3; ++k) {
+        g.finer[k] = std::ilogb(g.scale[k] / around.scale[k]);
+        if (g.finer[k] < -100 || g.finer[k] > 100) return false;
+        g.scale[k] = std::ldexp(around.scale[k], g.finer[k]);
+    }
+    return true;
+}
+
+// How much larger a subtree's boxes are in a grid, in the terms of the surface area heuristic: a random
+// line that meets a box of half area A meets one inside it of half area a with probability a / A.  A
+// grid adds about two steps to a box along each axis, so with the sums over the subtree's child boxes
+// (a leaf's box once per triangle) what any grid adds follows from its steps alone.
+struct Extents {
+    double n = 0, x = 0, y = 0, z = 0, area = 0; // boxes, their extents and half areas
+    uint32_t inner = 0;                          // inner nodes of the subtree
+    void box(const float* lo, const float* hi, double w) {
+        const double dx = (double)hi[0] - lo[0], dy = (double)hi[1] - lo[1], dz = (double)hi[2] - lo[2];
+        n += w;
+        x += w * dx;
+        y += w * dy;
+        z += w * dz;
+        area += w * (dx * dy + dy * dz + dz * dx);
+    }
+    void add(const Extents& e) {
+        n += e.n;
+        x += e.x;
+        y += e.y;
+        z += e.z;
+        area += e.area;
+        inner += e.inner;
+    }
+    double added(const Grid& g) const {
+        const double px = 0x1.0p-15 / g.scale[0], py = 0x1.0p-15 / g.scale[1], pz = 0x1.0p-15 / g.scale[2];
+        return px * (y + z) + py * (x + z) + pz * (x + y) + n * (px * py + py * pz + pz * px);
+    }
+};
+
+// A subtree gets a grid of its own where the one around it costs a ray that enters the subtree more
+// than kGridShare of the visits that exact boxes take, and more than a few (kGridVisits; kGridVisitsSmall
+// in subtrees with less than 1/16 of the scene's nodes, a sphere's poles for instance: a scene with
+// several grids is traced by kernels that are 3 to 5% slower), and its own would take most of that away.
+constexpr double kGridVisits = 2.0, kGridVisitsSmall = 32.0, kGridShare = 0.05, kGridLeft = 1.0 / 16;
+
+bool too_coarse(const Child2& c, const Extents& e, const Grid& g, uint32_t n_nodes) {
+    Extents own;
+    own.box(c.lo, c.hi, 1.0);
+    const double add = e.added(g), visits = 16.0 * e.inner >= n_nodes ? kGridVisits : kGridVisitsSmall;
+    return add > kGridShare * e.area && add > visits * (own.area + own.added(g));
+}
+
+struct Grids {
+    const HostBVH2& b;
+    std::vector<Extents> sub;   // of the subtree at each inner node
+    std::vector<uint8_t> flag;  // too coarse in the scene's grid, or something below is
+    std::vector<uint32_t> of;   // grid of each node's record
+    std::vector<Grid> grids;
+
+    Grids(const HostBVH2& b_, int n_threads) : b(b_) {
+        grids.push_back(grid_over(b.lo, b.hi));
+        sub.resize(b.n_nodes);
+        flag.resize(b.n_nodes);
+        // the subtrees below the topmost nodes on several threads, then these
+        std::vector<uint32_t> top = {0}, parts = {0};
+        while (n_threads > 1 && parts.size() && parts.size() < 8 * (size_t)n_threads && b.n_nodes > 16384) {
+            std::vector<uint32_t> next;
+            for (uint32_t i : parts)
+                for (int w = 0; w < 2; ++w) {
+                    const int32_t l = child2_of(b, i, w).link;
+                    if (l >= 0) next.push_back((uint32_t)l);
+                }
+            top.insert(top.end(), next.begin(), next.end());
+            parts.swap(next);
+        }
+        std::atomic<size_t> turn{0};
+        auto work = [&]() {
+            for (size_t i; (i = turn++) < parts.size();) sum(parts[i]);
+        };
+        std::vector<std::thread> th;
+        for (size_t t = 1; t < std::min<size_t>((size_t)std::max(1, n_threads), parts.size()); ++t) {
+            try {
+                th.emplace_back(work);
+            } catch (const std::system_error&) { // no thread to be had
+                break;
+            }
+        }
+        work();
+        for (auto& t : th) t.join();
+        top.resize(top.size() - parts.size());
+        for (size_t i = top.size(); i-- > 0;) node(top[i]);
+        if (flag[0]) {
+            of.assign(b.n_nodes, 0);
+            place(0, 0);
+        }
+    }
+
+    void node(uint32_t i) { // after its children
+        Extents e;
+        e.inner = 1;
+        uint8_t f = 0;
+        for (int w = 0; w < 2; ++w) {
+            const Child2 c = child2_of(b, i, w);
+            e.box(c.lo, c.hi, c.link >= 0 ? 1.0 : (double)(((uint32_t)~c.link & 3u) + 1u));
+            if (c.link < 0) continue;
+            e.add(sub[c.link]);
+            f |= flag[c.link] | (uint8_t)too_coarse(c, sub[c.link], grids[0], b.n_nodes);
+        }
+        sub[i] = e;
+        flag[i] = f;
+    }
+    void sum(uint32_t i) {
+        for (int w = 0; w < 2; ++w) {
+            const int32_t l = child2_of(b, i, w).link;
+            if (l >= 0) sum((uint32_t)l);
+        }
+        node(i);
+    }
+    // The subtrees below node i, which is in grid g, that take grids of their own.  (A grid of its own has
+    // smaller steps, so what the scene's grid does not flag needs none.)
+    void place(uint32_t i, uint32_t g) {
+        for (int w = 0; w < 2; ++w) {
+            const Child2 c = child2_of(b, i, w);
+            if (c.link < 0) continue;
+            const uint32_t k = (uint32_t)c.link;
+            uint32_t in = g;
+            const uint32_t nested = grids[g].nested + 1;
+            if (nested <= kMaxNested && b.depth + nested < kBvh2StackCapacity && too_coarse(c, sub[k], grids[g], b.n_nodes)) {
+                Grid own;
+                if (grid_within(c.lo, c.hi, grids[g], own) &&
+                    sub[k].added(own) <= std::max(kGridLeft * sub[k].added(grids[g]), 0.02 * sub[k].area)) {
+                    own.root = k;
+                    own.around = g;
+                    own.nested = nested;
+                    in = (uint32_t)grids.size();
+                    grids.push_back(own);
+                    // a subtree's nodes follow each other, from the first of its root's children on
+                    of[k] = in;
+                    uint32_t first = b.n_nodes;
+                    for (int v = 0; v < 2; ++v) {
+                        const int32_t l = child2_of(b, k, v).link;
+                        if (l >= 0) first = std::min(first, (uint32_t)l);
+                    }
+                    if (sub[k].inner > 1) std::fill_n(of.begin() + first, sub[k].inner - 1, in);
+                }
+            }
+            if (flag[k]) place(k, in);
+        }
+    }
+};
+
+} // namespace
+
+DevBVH2 pack_bvh2(const HostBVH2& b, int n_threads) {
+    DevBVH2 out;
+    const Grids gr(b, n_threads);
+    for (int k = 0; k < 3; ++k) {
+        out.lo[k] = gr.grids[0].lo[k];
+        out.scale[k] = gr.grids[0].scale[k];
+    }
+    out.n_grids = (uint32_t)gr.grids.size();
+    const uint32_t first_grid = b.n_nodes + (b.n_nodes & 1u); // records of grid t: first_grid + 2 (t - 1)
+    out.words.resize((size_t)kDevNode2Words * ((size_t)first_grid + 2 * (size_t)(out.n_grids - 1)));
     auto run = [&](uint32_t first, uint32_t last) {
         for (uint32_t i = first; i < last; ++i) {
-            const float* o = &b.nodes[16 * (size_t)i];
+            const uint32_t at = gr.of.empty() ? 0u : gr.of[i];
+            const Grid& g = gr.grids[at];
             uint32_t* w = &out.words[(size_t)kDevNode2Words * i];
-            static const int at[3][2] = {{0, 4}, {2, 6}, {8, 10}}; // lower plane of (axis, child)
-            for (int c = 0; c < 2; ++c)
+            for (int s = 0; s < 2; ++s) {
+                const Child2 c = child2_of(b, i, s);
                 for (int a = 0; a < 3; ++a) {
-                    const double lo = 0.5 + ((double)o[at[a][c]] - (double)out.lo[a]) * (double)out.scale[a];
-                    const double hi = 0.5 + ((double)o[at[a][c] + 1] - (double)out.lo[a]) * (double)out.scale[a];
-                    w[3 * c + a] = plane_below(lo - kGridSlack) | plane_above(hi + kGridSlack) << 16;
+                    const double lo = 0.5 + ((double)c.lo[a] - (double)g.lo[a]) * (double)g.scale[a];
+                    const double hi = 0.5 + ((double)c.hi[a] - (double)g.lo[a]) * (double)g.scale[a];
+                    w[3 * s + a] = plane_below(lo - kGridSlack) | plane_above(hi + kGridSlack) << 16;
                 }
-            std::memcpy(&w[6], &o[12], 4);
-            std::memcpy(&w[7], &o[13], 4);
+                w[6 + s] = (uint32_t)c.link;
+                if (c.link >= 0 && !gr.of.empty() && gr.of[c.link] != at)
+                    w[6 + s] = ~(kGridLink | (first_grid + 2 * (gr.of[c.link] - 1)));
+            }
         }
     };
+    for (uint32_t t = 1; t < out.n_grids; ++t) {
+        const Grid& g = gr.grids[t];
+        const Grid& around = gr.grids[g.around];
+        uint32_t* w = &out.words[(size_t)kDevNode2Words * (first_grid + 2 * (t - 1))];
+        std::memcpy(w, g.lo, 12);
+        std::memcpy(w + 3, g.scale, 12);
+        std::memcpy(w + 8, around.lo, 12);
+        std::memcpy(w + 11, around.scale, 12);
+        for (int k = 0; k < 3; ++k) {
+            w[6] |= (uint32_t)(127 - g.finer[k]) << (8 * k);
+            w[14] |= (uint32_t)(127 + g.finer[k]) << (8 * k);
+        }
+        w[7] = g.root;
+        w[15] = g.around ? first_grid + 2 * (g.around - 1) : 0u;
+    }
     const uint32_t nt = (uint32_t)std::max(1, std::min(n_threads, (int)(b.n_nodes / 16384u)));
     std::vector<std::thread> th;
     for (uint32_t t = 0; t < nt; ++t) {
@@ -411,20 +618,6 @@ DevBVH2 pack_bvh2(const HostBVH2& b, int n_threads) {
 // Host verification of the BVH2 (used by cr_debug_bvh_check).
 namespace cr {
 namespace {
-
-struct Child2 {
-    float lo[3], hi[3];
-    int32_t link; // >= 0 inner node, < 0 leaf code
-};
-
-Child2 child2_of(const HostBVH2& b, uint32_t node, int which) {
-    const float* o = &b.nodes[16 * (size_t)node];
-    Child2 c;
-    const int x = which == 0 ? 0 : 4, z = which == 0 ? 8 : 10;
-    c.lo[0] = o[x]; c.hi[0] = o[x + 1]; c.lo[1] = o[x + 2]; c.hi[1] = o[x + 3]; c.lo[2] = o[z]; c.hi[2] = o[z + 1];
-    std::memcpy(&c.link, &o[12 + which], 4);
-    return c;
-}
 
 bool contains(const float* lo, const float* hi, const float* v) {
     for (int j = 0; j < 3; ++j)
@@ -463,21 +656,60 @@ void check_bvh2(const HostBVH2& b, const float* v, uint32_t n_tri, uint32_t& cov
             }
         }
     }
-    // the kernels' records: the same links, and boxes (as the kernels decode them) that contain
-    // each child box and kGridSlack around it
+    // the kernels' records, walked as the kernels do: links that lead to the same nodes, grids that lead
+    // back to the ones around them, and boxes (as the kernels decode them) that contain each child box
+    // and kGridSlack around it
     const DevBVH2 d = pack_bvh2(b, 2);
-    for (uint32_t i = 0; i < b.n_nodes; ++i)
+    const uint32_t n_rec = (uint32_t)(d.words.size() / kDevNode2Words);
+    struct At {
+        uint32_t node, in, nested; // the way in to its grid (0: the scene's)
+    };
+    std::vector<At> walk = {{0u, 0u, 0u}};
+    uint32_t visited = 0, entered = 1;
+    const auto grid_of = [&](uint32_t in, float* lo, float* scale) {
+        std::memcpy(lo, in ? (const void*)&d.words[(size_t)kDevNode2Words * in] : d.lo, 12);
+        std::memcpy(scale, in ? (const void*)&d.words[(size_t)kDevNode2Words * in + 3] : d.scale, 12);
+    };
+    while (!walk.empty()) {
+        const At at = walk.back();
+        walk.pop_back();
+        ++visited;
+        float glo[3], gscale[3];
+        grid_of(at.in, glo, gscale);
+        const uint32_t* rec = &d.words[(size_t)kDevNode2Words * at.node];
         for (int w = 0; w < 2; ++w) {
-            const Child2 c = child2_of(b, i, w);
-            const uint32_t* rec = &d.words[(size_t)kDevNode2Words * i];
-            if (rec[6 + w] != (uint32_t)c.link) ++violations;
+            const Child2 c = child2_of(b, at.node, w);
             for (int k = 0; k < 3; ++k) {
-                const double lo = 0.5 + ((double)c.lo[k] - (double)d.lo[k]) * (double)d.scale[k] - kGridSlack;
-                const double hi = 0.5 + ((double)c.hi[k] - (double)d.lo[k]) * (double)d.scale[k] + kGridSlack;
+                const double lo = 0.5 + ((double)c.lo[k] - (double)glo[k]) * (double)gscale[k] - kGridSlack;
+                const double hi = 0.5 + ((double)c.hi[k] - (double)glo[k]) * (double)gscale[k] + kGridSlack;
                 const uint32_t q = rec[3 * w + k];
                 if ((double)plane_value(q & 0xffffu) > lo || (double)plane_value(q >> 16) < hi) ++violations;
             }
+            At next = {(uint32_t)c.link, at.in, at.nested};
+            if (rec[6 + w] != (uint32_t)c.link) { // a grid of its own
+                const uint32_t r = ~rec[6 + w] & ~kGridLink;
+                if (c.link < 0 || !(~rec[6 + w] & kGridLink) || (r & 1u) || r < b.n_nodes || r + 1 >= n_rec) {
+                    ++violations;
+                    continue;
+                }
+                next.in = r;
+                ++next.nested;
+                ++entered;
+                if (next.nested > kMaxNested || b.depth + next.nested >= kBvh2StackCapacity) ++violations;
+                // in and out again: the root, the grid around, and scales that follow from each other
+                const uint32_t* g = &d.words[(size_t)kDevNode2Words * r];
+                float ilo[3], iscale[3];
+                grid_of(r, ilo, iscale);
+                if (g[7] != (uint32_t)c.link || g[15] != at.in || std::memcmp(g + 8, glo, 12) || std::memcmp(g + 11, gscale, 12)) ++violations;
+                for (int k = 0; k < 3; ++k) {
+                    const int in = (int)(g[6] >> (8 * k) & 0xffu) - 127, out = (int)(g[14] >> (8 * k) & 0xffu) - 127;
+                    if (in != -out || std::ldexp(iscale[k], in) != gscale[k]) ++violations;
+                }
+            }
+            if (c.link >= 0) walk.push_back(next);
         }
+    }
+    if (visited != b.n_nodes || entered != d.n_grids) ++violations;
     covered = 0;
     for (uint32_t t = 0; t < n_tri; ++t) covered += seen[t] >= 1 ? 1u : 0u;
     // the root-leaf case emits the same triangles twice on purpose; count distinct coverage

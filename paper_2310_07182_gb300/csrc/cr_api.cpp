@@ -358,6 +358,7 @@ extern "C" cr_status cr_scene_create(const float* tri_xyz, uint32_t n_tri, const
         s->dev.grid_lo[k] = d2.lo[k];
         s->dev.grid_scale[k] = d2.scale[k];
     }
+    s->dev.n_grids = d2.n_grids;
     s->dev.tris = static_cast<const float4*>(s->d_tris);
     s->dev.mats = static_cast<const float4*>(s->d_mats);
     for (int k = 0; k < 3; ++k) {
@@ -732,6 +733,7 @@ cr_status build_plan(const cr_job* jobs, uint32_t n_jobs, const PlanOpts& po, Re
     for (auto* sc : uniq) {
         plan.scenes.push_back(scene_entry(sc->dev, po.bvh8));
         plan.scenes.back().n_nodes4 = sc->dev.n_nodes4;
+        plan.grids |= sc->dev.n_grids > 1;
     }
     plan.npx_total = px;
     // passes: pass p renders sample p of every job with spp > p
@@ -887,6 +889,7 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
     ta.speculative = eo.speculative;
     ta.bvh8 = p.bvh8;
     ta.bvh4 = p.bvh4;
+    ta.grids = p.grids;
     ta.scenes = d_scenes;
     ta.slot_scene = b.slot_scene;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -909,6 +912,7 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
         P.npx = eo.debug_npx;
         P.nee = p.nee;
         P.one_scene = p.scenes.size() == 1;
+        P.grids = p.grids;
         P.accum_mode = fused_out ? 3u : 0u;
         const uint32_t n_slots = ps.n_tiles * p.m;
         b.n_groups = n_slots / p.k;
@@ -1234,6 +1238,7 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
     ta.any_hit = (o.flags & CR_OPT_ANY_HIT) != 0;
     ta.bvh8 = use8;
     ta.bvh4 = use4;
+    ta.grids = s->dev.n_grids > 1;
     ta.scenes = dev_scene_entry(s, use8);
     ta.slot_scene = nullptr;
     ta.one_scene = true;
@@ -1246,7 +1251,7 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
         if (count) ta.counters = reinterpret_cast<unsigned long long*>(s->d_work + 4);
     }
     // the traversal variants, and hit arrays that overlap the rays, go through ray and hit records
-    const bool records = ((ta.speculative || ta.packet) && !use8 && !use4 && !ta.any_hit && !count) ||
+    const bool records = ((ta.speculative || ta.packet) && !ta.grids && !use8 && !use4 && !ta.any_hit && !count) ||
                          !user_rays_apart(d_rays, d_skip, n, d_prim, d_t);
     DevMem ro, rd, hit;
     if (records) {

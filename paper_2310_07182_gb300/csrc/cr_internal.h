@@ -37,10 +37,24 @@ struct HostBVH2 {
 // scene into [0.5, 2).  A code q is the float with the bits 0x3f000000 | q << 8 (steps of 2^-16
 // below 1 and 2^-15 above).  Lower planes are rounded down and upper planes up, so that the
 // record's box contains the exact child box and kGridSlack beyond it on every side.
+//
+// Where that grid is too coarse for a subtree, its records are on a grid of its own (pack_bvh2 has the
+// rule), which may hold further ones; its steps are the steps around it divided by powers of two.  Such a
+// grid takes two records behind those of the nodes, r for the way in and r + 1 for the way out:
+//   words 0-2  lo, 3-5 scale of the grid entered
+//   word 6     per axis 8 bits: the exponent field of the power of two by which 1 / (d * scale) changes
+//   word 7     r: the subtree's root node;  r + 1: the way in to the grid around, 0 if that is the scene's
+// A link to such a subtree is ~(kGridLink | r); ~(kGridLink | r + 1), the link out of it, occurs on
+// traversal stacks only.  (r is even.)
 struct DevBVH2 {
-    std::vector<uint32_t> words; // 8 per inner node
-    float lo[3], scale[3];
+    std::vector<uint32_t> words; // 8 per inner node, then 16 per grid within the scene's
+    float lo[3], scale[3];       // the scene's grid
+    uint32_t n_grids = 1;        // the scene's among them
 };
+constexpr uint32_t kGridLink = 0x40000000u; // above every leaf code (triangles <= 2^28)
+// Traversal stack entries that a link back may take are within kBvh2StackCapacity: subtrees with a grid of
+// their own lie within each other at most this deep, and less deep in trees deeper than 63 - kMaxNested.
+constexpr uint32_t kMaxNested = 8;
 // Boxes are enlarged by this much on every side (grid units); see grid_ray in trace_common.cuh.
 constexpr double kGridSlack = 0x1.0p-18;
 constexpr uint32_t kDevNode2Words = 8;
@@ -98,6 +112,7 @@ void check_bvh8(const HostBVH8& b, const float* v, uint32_t n_tri, uint32_t& cov
 struct DevScene {
     const uint32_t* nodes2 = nullptr; // 8 words per node (DevBVH2)
     float grid_lo[3] = {0, 0, 0}, grid_scale[3] = {1, 1, 1}; // grid of its boxes
+    uint32_t n_grids = 1;                                    // DevBVH2::n_grids
     const uint4* nodes8 = nullptr;  // 5 per node
     const float4* nodes4 = nullptr; // 8 per node (BVH4, if built)
     const float4* tris = nullptr;   // 3 per triangle in leaf order: v0|orig, v1|mat, v2|0
@@ -184,6 +199,7 @@ struct PassArgs {
     uint32_t npx = 0;      // pixels of the debug capture (single-job renders)
     bool nee = false;      // some job of the plan uses next-event estimation
     bool one_scene = false; // the scene table has one entry
+    bool grids = false;     // some scene's BVH2 has several grids
     bool chained = false;   // launches may be set up while the one before ends (launch_step)
     // bit 0: a job's first sample writes its pixel sums without reading them (the buffer is
     // not cleared first); bit 1: its last sample writes the output instead of the sums
@@ -248,7 +264,7 @@ struct ShadowArgs {
     unsigned long long* n_traced = nullptr;
     uint32_t* work = nullptr; // as in TraceArgs
     bool bvh8 = false;
-    bool one_scene = false, alone = true, chained = false; // as in TraceArgs
+    bool one_scene = false, alone = true, chained = false, grids = false; // as in TraceArgs
 };
 
 // Arguments of one trace launch over a queue of slots, or over a caller's rays.
@@ -278,6 +294,7 @@ struct TraceArgs {
     bool any_hit = false;     // stop at the first hit before tmax (visibility)
     uint32_t stack = 16;      // BVH2 stack entries per thread in shared memory (8, 16, 32)
     bool two_phase = false;   // budgeted traversal, compaction of unfinished rays, resume (BVH2)
+    bool grids = false;       // some scene's BVH2 has several grids (the three variants above do not apply)
     PhaseBuffers phase;
     bool bvh8 = false;
     bool bvh4 = false; // closest hits through the BVH4 (any-hit queries stay on the BVH2)
@@ -434,6 +451,7 @@ struct RenderPlan {
     bool bvh8 = false, sort = false;
     bool bvh4 = false;
     bool nee = false; // some job uses next-event estimation
+    bool grids = false; // some scene's BVH2 has more than one grid
     uint32_t max_bounces = 0, max_slots = 0, npx_total = 0;
     // > 1: a pass renders up to `regions` samples of every job, each as a table entry of its own.  The
     // accumulation buffer then has `regions` regions of npx pixels (all jobs'), one per sample of

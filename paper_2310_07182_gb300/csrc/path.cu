@@ -1138,13 +1138,24 @@ __device__ __forceinline__ uint32_t hcut_path(const SceneDev& sc, float px, floa
     int node = 0;
     const float p[3] = {px, py, pz};
     float pg[3], inv[3];
+    auto grid = [&](const float lo[3], const float scale[3]) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        pg[k] = fmaf(p[k] - sc.grid_lo[k], sc.grid_scale[k], 0.5f);
-        inv[k] = 1.0f / sc.grid_scale[k];
-    }
+        for (int k = 0; k < 3; ++k) {
+            pg[k] = fmaf(p[k] - lo[k], scale[k], 0.5f);
+            inv[k] = 1.0f / scale[k];
+        }
+    };
+    grid(sc.grid_lo, sc.grid_scale);
     for (uint32_t l = 0; l < kHcutLevels; ++l) {
         code <<= 1;
+        if (node < 0 && ((uint32_t)~node & kGridLink)) { // a subtree with a grid of its own
+            const uint4* rec = reinterpret_cast<const uint4*>(sc.nodes2 + kDevNode2Words * (size_t)((uint32_t)~node & ~kGridLink));
+            const uint4 a = __ldg(rec), b = __ldg(rec + 1);
+            const float lo[3] = {__uint_as_float(a.x), __uint_as_float(a.y), __uint_as_float(a.z)};
+            const float scale[3] = {__uint_as_float(a.w), __uint_as_float(b.x), __uint_as_float(b.y)};
+            grid(lo, scale);
+            node = (int)b.w;
+        }
         if (node < 0) continue;
         const uint4* rec = reinterpret_cast<const uint4*>(sc.nodes2 + kDevNode2Words * (size_t)node);
         const uint4 a = __ldg(rec), b = __ldg(rec + 1);
@@ -1788,6 +1799,7 @@ static ShadowArgs shadow_args_of(const PassArgs& p, const PathBuffers& b, const 
     s.work = work;
     s.bvh8 = bvh8;
     s.one_scene = p.one_scene;
+    s.grids = p.grids;
     s.chained = p.chained;
     return s;
 }

@@ -136,6 +136,21 @@ __device__ __forceinline__ GridRay grid_ray(float4 o, float4 d, const SceneDev& 
     return g;
 }
 
+// A ray's way into another grid, by the record of that step (DevBVH2; a, b its words): the offsets are
+// made anew and the reciprocals scaled by powers of two, which is exact, so the errors are those above.
+__device__ __forceinline__ void cross_axis(float o, uint32_t lo, uint32_t scale, uint32_t two, float& i, float& n, float& f) {
+    const float og = fmaf(o - __uint_as_float(lo), __uint_as_float(scale), 0.5f);
+    i = __fmul_rn(i, __uint_as_float(two << 23));
+    const float oi = __fmul_rn(og, i), e = __fmul_rn(fabsf(oi), 0x1.0p-19f);
+    n = -oi - e;
+    f = -oi + e;
+}
+__device__ __forceinline__ void cross_grid(const RayPre& r, const uint4& a, const uint4& b, GridRay& g) {
+    cross_axis(r.ox, a.x, a.w, b.z & 0xffu, g.ix, g.nx, g.fx);
+    cross_axis(r.oy, a.y, b.x, b.z >> 8 & 0xffu, g.iy, g.ny, g.fy);
+    cross_axis(r.oz, a.z, b.y, b.z >> 16, g.iz, g.nz, g.fz);
+}
+
 struct NodeTest {
     float t0, t1; // entry distances of the boxes of child 0, 1 (0 from inside)
     float f0, f1; // exit distances
