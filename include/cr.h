@@ -433,7 +433,8 @@ cr_status cr_server_destroy(cr_server* server);
  *   prim      host or device, n int32: original index of the closest hit, -1 if none.
  *   t         host or device, n floats: hit distance in units of |d| (inf if none).
  * Hit rule: watertight test (Woop et al. 2013), t > 0, edges inclusive; equal t goes to the
- * smaller original index.  opts may be NULL (bvh, block, stream, flags are read).
+ * smaller original index.  Where the scene has triangles of more than 16 units, one that lies
+ * behind the origin along an axis is not hit even if rounding makes its t positive.  opts may be NULL (bvh, block, stream, flags are read).
  * With CR_OPT_ANY_HIT in opts->flags the traversal stops at the first triangle hit before
  * tmax (the shadow-ray kernel's traversal): prim is then some occluder (not necessarily the
  * closest) and t its distance, or -1 and inf if the ray reaches tmax unblocked. */

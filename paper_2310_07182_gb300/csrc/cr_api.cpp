@@ -223,11 +223,14 @@ extern "C" cr_status cr_scene_create(const float* tri_xyz, uint32_t n_tri, const
     }
     // triangles in leaf order: v0 | original index, v1 | material, v2 | 0
     std::vector<float> tris(12 * (size_t)n_tri);
+    float largest = 0.0f; // extent of a triangle along an axis
     for (uint32_t i = 0; i < n_tri; ++i) {
         const uint32_t t = b2.leaf_order[i];
         float* o = &tris[12 * (size_t)i];
         for (int v = 0; v < 3; ++v)
             for (int k = 0; k < 3; ++k) o[4 * v + k] = tri_xyz[9 * (size_t)t + 3 * v + k];
+        for (int k = 0; k < 3; ++k)
+            largest = std::max(largest, std::max({o[k], o[4 + k], o[8 + k]}) - std::min({o[k], o[4 + k], o[8 + k]}));
         int32_t orig = (int32_t)t, mat = (int32_t)tri_mat[t];
         std::memcpy(&o[3], &orig, 4);
         std::memcpy(&o[7], &mat, 4);
@@ -358,7 +361,7 @@ extern "C" cr_status cr_scene_create(const float* tri_xyz, uint32_t n_tri, const
         s->dev.grid_lo[k] = d2.lo[k];
         s->dev.grid_scale[k] = d2.scale[k];
     }
-    s->dev.n_grids = d2.n_grids;
+    s->dev.wide = d2.n_grids > 1 || largest > kWideTri;
     s->dev.tris = static_cast<const float4*>(s->d_tris);
     s->dev.mats = static_cast<const float4*>(s->d_mats);
     for (int k = 0; k < 3; ++k) {
@@ -733,7 +736,7 @@ cr_status build_plan(const cr_job* jobs, uint32_t n_jobs, const PlanOpts& po, Re
     for (auto* sc : uniq) {
         plan.scenes.push_back(scene_entry(sc->dev, po.bvh8));
         plan.scenes.back().n_nodes4 = sc->dev.n_nodes4;
-        plan.grids |= sc->dev.n_grids > 1;
+        plan.wide |= sc->dev.wide;
     }
     plan.npx_total = px;
     // passes: pass p renders sample p of every job with spp > p
@@ -889,7 +892,7 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
     ta.speculative = eo.speculative;
     ta.bvh8 = p.bvh8;
     ta.bvh4 = p.bvh4;
-    ta.grids = p.grids;
+    ta.wide = p.wide;
     ta.scenes = d_scenes;
     ta.slot_scene = b.slot_scene;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -912,7 +915,7 @@ cr_status enqueue_plan(const RenderPlan& p, const JobDev* d_jobs, const SceneDev
         P.npx = eo.debug_npx;
         P.nee = p.nee;
         P.one_scene = p.scenes.size() == 1;
-        P.grids = p.grids;
+        P.wide = p.wide;
         P.accum_mode = fused_out ? 3u : 0u;
         const uint32_t n_slots = ps.n_tiles * p.m;
         b.n_groups = n_slots / p.k;
@@ -1238,7 +1241,7 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
     ta.any_hit = (o.flags & CR_OPT_ANY_HIT) != 0;
     ta.bvh8 = use8;
     ta.bvh4 = use4;
-    ta.grids = s->dev.n_grids > 1;
+    ta.wide = s->dev.wide;
     ta.scenes = dev_scene_entry(s, use8);
     ta.slot_scene = nullptr;
     ta.one_scene = true;
@@ -1251,7 +1254,7 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
         if (count) ta.counters = reinterpret_cast<unsigned long long*>(s->d_work + 4);
     }
     // the traversal variants, and hit arrays that overlap the rays, go through ray and hit records
-    const bool records = ((ta.speculative || ta.packet) && !ta.grids && !use8 && !use4 && !ta.any_hit && !count) ||
+    const bool records = ((ta.speculative || ta.packet) && !ta.wide && !use8 && !use4 && !ta.any_hit && !count) ||
                          !user_rays_apart(d_rays, d_skip, n, d_prim, d_t);
     DevMem ro, rd, hit;
     if (records) {

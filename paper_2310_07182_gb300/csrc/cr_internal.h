@@ -107,12 +107,19 @@ constexpr uint32_t kBvh8StackCapacity = 48; // traversal stack entries of the BV
 void check_bvh2(const HostBVH2& b, const float* v, uint32_t n_tri, uint32_t& covered, uint32_t& violations);
 void check_bvh8(const HostBVH8& b, const float* v, uint32_t n_tri, uint32_t& covered, uint32_t& violations);
 
+// Triangle extent above which a path's ray may find, by rounding, a hit on a triangle that lies behind its
+// origin (behind() in trace_common.cuh): the test's distance is off by some 2^-22 of the extent, and a
+// ray starts 2^-18 or more off the surface that it leaves.
+constexpr float kWideTri = 16.0f;
+
 // ------------------------------------------------------------------------------------
 // Device-side scene description (host copy kept in the scene handle).
 struct DevScene {
     const uint32_t* nodes2 = nullptr; // 8 words per node (DevBVH2)
     float grid_lo[3] = {0, 0, 0}, grid_scale[3] = {1, 1, 1}; // grid of its boxes
-    uint32_t n_grids = 1;                                    // DevBVH2::n_grids
+    // the scene needs the kernels for wide scenes: its BVH2 has several grids, or some triangle is larger
+    // than kWideTri along an axis
+    bool wide = false;
     const uint4* nodes8 = nullptr;  // 5 per node
     const float4* nodes4 = nullptr; // 8 per node (BVH4, if built)
     const float4* tris = nullptr;   // 3 per triangle in leaf order: v0|orig, v1|mat, v2|0
@@ -199,7 +206,7 @@ struct PassArgs {
     uint32_t npx = 0;      // pixels of the debug capture (single-job renders)
     bool nee = false;      // some job of the plan uses next-event estimation
     bool one_scene = false; // the scene table has one entry
-    bool grids = false;     // some scene's BVH2 has several grids
+    bool wide = false;      // some scene is wide (DevScene::wide)
     bool chained = false;   // launches may be set up while the one before ends (launch_step)
     // bit 0: a job's first sample writes its pixel sums without reading them (the buffer is
     // not cleared first); bit 1: its last sample writes the output instead of the sums
@@ -264,7 +271,7 @@ struct ShadowArgs {
     unsigned long long* n_traced = nullptr;
     uint32_t* work = nullptr; // as in TraceArgs
     bool bvh8 = false;
-    bool one_scene = false, alone = true, chained = false, grids = false; // as in TraceArgs
+    bool one_scene = false, alone = true, chained = false, wide = false; // as in TraceArgs
 };
 
 // Arguments of one trace launch over a queue of slots, or over a caller's rays.
@@ -294,7 +301,7 @@ struct TraceArgs {
     bool any_hit = false;     // stop at the first hit before tmax (visibility)
     uint32_t stack = 16;      // BVH2 stack entries per thread in shared memory (8, 16, 32)
     bool two_phase = false;   // budgeted traversal, compaction of unfinished rays, resume (BVH2)
-    bool grids = false;       // some scene's BVH2 has several grids (the three variants above do not apply)
+    bool wide = false;        // some scene is wide (DevScene::wide; the three variants above do not apply)
     PhaseBuffers phase;
     bool bvh8 = false;
     bool bvh4 = false; // closest hits through the BVH4 (any-hit queries stay on the BVH2)
@@ -451,7 +458,7 @@ struct RenderPlan {
     bool bvh8 = false, sort = false;
     bool bvh4 = false;
     bool nee = false; // some job uses next-event estimation
-    bool grids = false; // some scene's BVH2 has more than one grid
+    bool wide = false; // some scene is wide (DevScene::wide)
     uint32_t max_bounces = 0, max_slots = 0, npx_total = 0;
     // > 1: a pass renders up to `regions` samples of every job, each as a table entry of its own.  The
     // accumulation buffer then has `regions` regions of npx pixels (all jobs'), one per sample of

@@ -1799,7 +1799,7 @@ static ShadowArgs shadow_args_of(const PassArgs& p, const PathBuffers& b, const 
     s.work = work;
     s.bvh8 = bvh8;
     s.one_scene = p.one_scene;
-    s.grids = p.grids;
+    s.wide = p.wide;
     s.chained = p.chained;
     return s;
 }

@@ -358,7 +358,7 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
     uint32_t* st_job = fin_job + 2 * kMaxRuns;
     uint32_t* st_pre = fin_job + 3 * kMaxRuns;
     uint32_t n_fin = 0, n_start = 0, fin_slots = 0, start_tiles = 0, n_groups = 0, trace_max = 0, max_run = 0;
-    bool nee = false, sort = false, grids = false, upload_scenes = false;
+    bool nee = false, sort = false, wide = false, upload_scenes = false;
     std::vector<SceneDev> scene_tab;
     std::vector<uint64_t> completing, host_copies;
     std::map<uint64_t, uint32_t> next_run;
@@ -402,7 +402,7 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
             tab[j.run] = d;
             max_run = std::max(max_run, j.run);
             nee = nee || d.nee;
-            grids = grids || dev_scene_of(j.job.scene)->n_grids > 1;
+            wide = wide || dev_scene_of(j.job.scene)->wide;
             sort = sort || j.job.mode == CR_MORTON_SORT;
             if (j.step >= 1) n_groups += j.slots / K; // its groups may be in the queue read now
             if (j.step == 0) {
@@ -466,7 +466,7 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
     P.m = m;
     P.k = K;
     P.nee = nee;
-    P.grids = grids;
+    P.wide = wide;
     P.rolling = true;
     P.chained = false; // behind the copies' event and the memset; then behind a kernel
     P.accum_mode = 3u;
@@ -516,7 +516,7 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
         ta.queue_count = qn;
         ta.work = qn + 2;
         ta.alone = false;
-        ta.grids = grids;
+        ta.wide = wide;
         ta.chained = P.chained;
         ta.shadow = sh.n_groups_max && !sort ? &sh : nullptr;
         ta.n_max = trace_max;

@@ -34,7 +34,7 @@ constexpr int kRefill = (int)0x80000001; // the stack's older entries wait in lo
 constexpr int kSteps = 2;                // node visits between two votes of the warp
 constexpr int kStealIdle = 16;           // idle lanes of a warp at which they take over parts of other lanes' rays
 // Shared-memory bytes of one warp: the lanes' stacks, three or four more words each.
-__host__ __device__ constexpr uint32_t warp_smem(int entries, bool grids) { return (uint32_t)(entries + (grids ? 4 : 3)) * 128u; }
+__host__ __device__ constexpr uint32_t warp_smem(int entries, bool wide) { return (uint32_t)(entries + (wide ? 4 : 3)) * 128u; }
 // Whether a link leads into or out of a grid (DevBVH2).
 __device__ __forceinline__ bool grid_link(int node) { return node < (int)~(kGridLink - 1u) && node > kRefill; }
 
@@ -56,7 +56,7 @@ __device__ __forceinline__ bool grid_link(int node) { return node < (int)~(kGrid
 //    which all of its lanes cull.  The closest hit does not depend on the order of visits, so it
 //    stays the same.  Short launches spread their rays over the whole device first (two to a
 //    warp or more): their time is that of their longest ray, one dependent load after another.
-//  - kGrids: some subtrees are on grids of their own (DevBVH2).  A lane that comes to a link into or out
+//  - kWide: some subtrees may be on grids of their own (DevBVH2).  A lane that comes to a link into or out
 //    of one crosses within the descent, the link out waits on its stack below the subtree's entries.
 //    A 1M-triangle sphere on a ground plane 500 times its size: 1M rays at it 0.89 ms with exact boxes (the
 //    64-byte nodes), 2.18 in one grid, 0.34 so; a 1280x720 frame of 3 bounces 0.98, 7.1, 0.74 ms.  (Crossing
@@ -73,7 +73,7 @@ __device__ __forceinline__ bool grid_link(int node) { return node < (int)~(kGrid
 // kSmemS: stack entries per lane kept in shared memory (8, 16 or 32), a launch-shape knob of
 // the autotuner.
 // kOne: every ray is in scenes[0], whose pointers then take no registers per lane.
-template <bool kCount, bool kAny, int kSmemS, bool kOne, bool kGrids, bool kSteal, class Src>
+template <bool kCount, bool kAny, int kSmemS, bool kOne, bool kWide, bool kSteal, class Src>
 __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ scenes, Src& src, uint32_t* smem,
                                                 unsigned long long& n_node, unsigned long long& n_tri) {
     constexpr uint32_t kLevel = 128u; // bytes between a lane's entries
@@ -89,12 +89,12 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
     // entry 0 holds kNoNode (or kRefill while older entries are in lstack), so a pop needs no
     // test for an empty stack
     const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem) + (threadIdx.x >> 5) * warp_smem(kSmemS, kGrids) + lane * 4u;
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem) + (threadIdx.x >> 5) * warp_smem(kSmemS, kWide) + lane * 4u;
     // kSteal: more words per lane
     const uint32_t lent = base + kSmemS * kLevel;      // lanes that trace part of this lane's ray
     const uint32_t bound = lent + kLevel;              // the smallest distance found for this lane's ray
     const uint32_t list = bound + kLevel - lane * 4u;  // scratch list of the warp
-    const uint32_t inside = bound + 2u * kLevel;       // kGrids: count << 29 | last, the grids that the lane has gone into
+    const uint32_t inside = bound + 2u * kLevel;       // kWide: count << 29 | last, the grids that the lane has gone into
     const uint32_t lim = base + (uint32_t)(kSmemS - kSteps + 1) * kLevel; // below it there is room for kSteps pushes
     uint32_t top = base + kLevel;                                         // next free entry
     int lstack[kStackTotal];
@@ -183,7 +183,7 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
                 if (kSteal) {
                     sts(lent, 0u);
                     sts(bound, __float_as_uint(rd.w));
-                    if (kGrids) sts(inside, 0u);
+                    if (kWide) sts(inside, 0u);
                 }
                 node = 0;
             }
@@ -234,7 +234,7 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
             // lanes without a ray take the oldest stack entry of a lane that has one
             const bool free = node == kNoNode && key < 0;
             bool gives = node != kNoNode && node != kRefill && lsp == 0 && top > bot + kLevel;
-            if (kGrids && gives) {
+            if (kWide && gives) {
                 // the oldest entry is in the grid that the lane started in: it gives only from there or from
                 // one step away, and drops a link out that has nothing below it
                 const uint32_t in = lds(inside), oldest = lds(bot + kLevel);
@@ -293,8 +293,8 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
                     }
                 }
                 if (takes) {
-                    const uint32_t in = kGrids ? lds(inside + (from - lane) * 4u) & 0x1fffffffu : 0u;
-                    if (kGrids && in) { // out of the giver's grid, into the entry's
+                    const uint32_t in = kWide ? lds(inside + (from - lane) * 4u) & 0x1fffffffu : 0u;
+                    if (kWide && in) { // out of the giver's grid, into the entry's
                         const uint4* rec = reinterpret_cast<const uint4*>(nodes + kDevNode2Words * (size_t)(in + 1u));
                         cross_grid(r, __ldg(rec), __ldg(rec + 1), g);
                     }
@@ -304,7 +304,7 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
                     best = Best{their_t, -1};
                     bot = base;
                     sts(bot, (uint32_t)kNoNode);
-                    if (kGrids) sts(inside, 0u);
+                    if (kWide) sts(inside, 0u);
                     top = base + kLevel;
                     lsp = 0;
                 }
@@ -327,8 +327,8 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
         const int half = __popc(alive) >> 1;
         bool run;
         do {
-            run = (node >= 0 || (kGrids && grid_link(node))) && top < lim;
-            if (kGrids && run && node < 0) {
+            run = (node >= 0 || (kWide && grid_link(node))) && top < lim;
+            if (kWide && run && node < 0) {
                 cross();
                 run = node >= 0;
             }
@@ -339,9 +339,9 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
                     run = node >= 0;
                 }
             }
-            run = (run || (kGrids && grid_link(node))) && top < lim;
+            run = (run || (kWide && grid_link(node))) && top < lim;
         } while (__popc(__ballot_sync(0xffffffffu, run)) > half);
-        const bool full = top >= lim && (node >= 0 || (kGrids && grid_link(node))); // room for a push is needed
+        const bool full = top >= lim && (node >= 0 || (kWide && grid_link(node))); // room for a push is needed
         if (kSteal && full && bot != base) { // the room of entries given away
             const uint32_t by = bot - base;
             for (uint32_t a = bot; a < top; a += kLevel) sts(a - by, lds(a));
@@ -354,7 +354,7 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
             lsp += kHalf;
             top -= kHalf * kLevel;
         }
-        if (node < 0 && node != kNoNode && !(kGrids && grid_link(node))) {
+        if (node < 0 && node != kNoNode && !(kWide && grid_link(node))) {
             if (node == kRefill) { // the stack is empty: its next entries come back
                 lsp -= kHalf;
                 for (int k = 0; k < kHalf; ++k) sts(base + (1 + k) * kLevel, (uint32_t)lstack[lsp + k]);
@@ -367,7 +367,7 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
                     lsp = 0;
                     continue;
                 })
-                test_leaf(tris, r, skip, code >> 2, (code & 3u) + 1u, best, n_tri);
+                test_leaf<kWide>(tris, r, g.ix, g.iy, g.iz, skip, code >> 2, (code & 3u) + 1u, best, n_tri);
                 tcull = __fmul_rn(best.t, kCullWiden);
                 if (kSteal && refill == 33 && best.leaf >= 0)
                     asm volatile("red.shared.min.s32 [%0], %1;" ::"r"(bound + (owner - lane) * 4u),
@@ -388,7 +388,7 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
 #define CR_TRACE_MAXNREG 56 // 36 warps resident per SM, no spills; 48 and 64 are within 1%, 40 costs 4%
 #endif
 
-template <bool kCount, bool kAny, int kSmemS, bool kOne, bool kGrids, RangeKind kKind>
+template <bool kCount, bool kAny, int kSmemS, bool kOne, bool kWide, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __restrict__ scenes,
                                                            chained_ptr<kOne, uint16_t> slot_scene,
                                                            chained_ptr<kOne, float4> ray_o,
@@ -402,21 +402,21 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2(const SceneDev* __res
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     unsigned long long n_node = 0, n_tri = 0;
     QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit, blockIdx.x, gridDim.x);
-    if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemS, kOne, kGrids, !kCount && !kAny && kKind != kPlain>(scenes, src, smem_stack, n_node, n_tri);
+    if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemS, kOne, kWide, !kCount && !kAny && kKind != kPlain>(scenes, src, smem_stack, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
 }
 
 // A caller's rays and hit arrays, no scratch between: cr_trace_rays used to copy the rays into the
 // render path's records, trace, and copy the hits out, in buffers allocated per call (1M surface
 // rays 952 us against 503, 300k camera rays 456 against 146, 1,000 rays 69 against 51).
-template <bool kCount, bool kAny, bool kGrids, RangeKind kKind>
+template <bool kCount, bool kAny, bool kWide, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_user(const SceneDev* __restrict__ scene, UserRays rays,
                                                                 uint32_t n, unsigned long long* counters,
                                                                 uint32_t* work) {
     extern __shared__ uint32_t smem_stack[];
     unsigned long long n_node = 0, n_tri = 0;
     UserSrc<kKind> src(n, work, rays);
-    if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemStack, true, kGrids, !kCount && !kAny && kKind != kPlain>(scene, src, smem_stack, n_node, n_tri);
+    if (src.more()) trace_bvh2_warp<kCount, kAny, kSmemStack, true, kWide, !kCount && !kAny && kKind != kPlain>(scene, src, smem_stack, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
 }
 
@@ -479,7 +479,7 @@ __device__ __forceinline__ int2 trace_bvh2_resumable(const SceneDev& sc, float4 
         if (suspended || node == 0x7fffffff) break;
         const uint32_t code = (uint32_t)(~node);
         unsigned long long dummy = 0;
-        test_leaf(tris, r, skip, code >> 2, (code & 3u) + 1u, best, dummy);
+        test_leaf<false>(tris, r, g.ix, g.iy, g.iz, skip, code >> 2, (code & 3u) + 1u, best, dummy);
         ++visits;
         if (sp == 0) break;
         STACK_POP(node);
@@ -633,7 +633,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
             }
         } else {
             const uint32_t code = (uint32_t)(~node);
-            if (valid) test_leaf(tris, r, skip, code >> 2, (code & 3u) + 1u, best, dummy);
+            if (valid) test_leaf<false>(tris, r, g.ix, g.iy, g.iz, skip, code >> 2, (code & 3u) + 1u, best, dummy);
         }
         if (sp == 0) break;
         STACK_POP(node);
@@ -724,7 +724,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_spec(
         // leaf phase: the parked leaf, then any leaf the descent stopped on
         while (leaf < 0) {
             const uint32_t code = (uint32_t)(~leaf);
-            test_leaf(tris, r, skip, code >> 2, (code & 3u) + 1u, best, dummy);
+            test_leaf<false>(tris, r, g.ix, g.iy, g.iz, skip, code >> 2, (code & 3u) + 1u, best, dummy);
             leaf = 0;
             if (node < 0) {
                 leaf = node;
@@ -739,7 +739,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_spec(
     }
 }
 
-template <bool kOne, bool kGrids, RangeKind kKind>
+template <bool kOne, bool kWide, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
     const SceneDev* __restrict__ scenes, chained_ptr<kOne, uint16_t> slot_scene, chained_ptr<kOne, float4> sh_o,
     chained_ptr<kOne, float4> sh_d, chained_ptr<kOne, float4> sh_c, chained_ptr<kOne, int32_t> group_queue,
@@ -751,7 +751,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
     ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K, blockIdx.x, gridDim.x);
     if (!src.more()) return;
     unsigned long long dn = 0, dt = 0;
-    trace_bvh2_warp<false, true, kSmemStack, kOne, kGrids, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
+    trace_bvh2_warp<false, true, kSmemStack, kOne, kWide, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
     src.add_traced(n_traced);
 }
 
@@ -761,7 +761,7 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_shadow(
 // (the other way round: 24 requests 5780 us against 5550, a batch of 16 jobs 5358 against 5314, single
 // renders alike).  Against a launch for each: an interior of 96 x 64 pixels 480 -> 350 us, 1280 x 720
 // 2965 -> 2805, with 16 samples 36.9 -> 36.5 ms, 24 requests 6390 -> 5550 us.
-template <int kSmemS, bool kOne, bool kGrids, RangeKind kKind>
+template <int kSmemS, bool kOne, bool kWide, RangeKind kKind>
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_both(
     const SceneDev* __restrict__ scenes, chained_ptr<kOne, uint16_t> slot_scene, chained_ptr<kOne, float4> ray_o,
     chained_ptr<kOne, float4> ray_d, chained_ptr<kOne, int32_t> queue, chained_ptr<kOne, uint32_t> queue_count,
@@ -775,13 +775,13 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_both(
     if (blockIdx.x < first) {
         const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
         QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit, blockIdx.x, first);
-        if (src.more()) trace_bvh2_warp<false, false, kSmemS, kOne, kGrids, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
+        if (src.more()) trace_bvh2_warp<false, false, kSmemS, kOne, kWide, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
     } else {
         const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
         ShadowSrc<kKind> src(n, sh_work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K, blockIdx.x - first,
                              gridDim.x - first);
         if (!src.more()) return;
-        trace_bvh2_warp<false, true, kSmemS, kOne, kGrids, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
+        trace_bvh2_warp<false, true, kSmemS, kOne, kWide, kKind != kPlain>(scenes, src, smem_stack, dn, dt);
         src.add_traced(n_traced);
     }
 }
@@ -815,19 +815,19 @@ void launch_shadow(const ShadowArgs& a, cudaStream_t st, LaunchCount& lc) {
     }
     const int block = kSecondaryBlock;
     const uint32_t need = blocks_for(n_pos, block); // the kinds of range as below
-    auto go = [&](auto one, auto grids) {
-        constexpr bool kOne = decltype(one)::value, kGrids = decltype(grids)::value;
-        const size_t smem = (size_t)warp_smem(kSmemStack, kGrids) * (block / 32);
-        const uint32_t most = resident_blocks<k_trace_shadow<kOne, kGrids, kMore>>(block, smem);
+    auto go = [&](auto one, auto wide) {
+        constexpr bool kOne = decltype(one)::value, kWide = decltype(wide)::value;
+        const size_t smem = (size_t)warp_smem(kSmemStack, kWide) * (block / 32);
+        const uint32_t most = resident_blocks<k_trace_shadow<kOne, kWide, kMore>>(block, smem);
         auto run = [&](auto kernel, uint32_t grid) {
             launch_step(kOne && a.chained, kernel, grid, block, smem, st, a.scenes, a.slot_scene, a.sh_o, a.sh_d, a.sh_c,
                         a.group_queue, a.group_count, a.n_groups_max, a.K, a.radiance, a.n_traced, a.work);
         };
-        if (need <= most && a.alone) run(k_trace_shadow<kOne, kGrids, kFew>, spread_blocks(n_pos, block, most));
-        else if (a.work && most && need > most) run(k_trace_shadow<kOne, kGrids, kMore>, most);
-        else run(k_trace_shadow<kOne, kGrids, kPlain>, need);
+        if (need <= most && a.alone) run(k_trace_shadow<kOne, kWide, kFew>, spread_blocks(n_pos, block, most));
+        else if (a.work && most && need > most) run(k_trace_shadow<kOne, kWide, kMore>, most);
+        else run(k_trace_shadow<kOne, kWide, kPlain>, need);
     };
-    if (a.grids) go(std::false_type(), std::true_type());
+    if (a.wide) go(std::false_type(), std::true_type());
     else if (a.one_scene) go(std::true_type(), std::false_type());
     else go(std::false_type(), std::false_type());
     lc.n++;
@@ -878,9 +878,9 @@ SceneDev scene_entry(const DevScene& s, bool bvh8) {
     return e;
 }
 
-template <bool kOne, bool kGrids, auto kKernel, int kSmemS>
+template <bool kOne, bool kWide, auto kKernel, int kSmemS>
 static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t st, LaunchCount& lc) {
-    const size_t smem = (size_t)warp_smem(kSmemS, kGrids) * (a.block / 32);
+    const size_t smem = (size_t)warp_smem(kSmemS, kWide) * (a.block / 32);
     if (smem > 48 * 1024) // 512-thread blocks with 32 entries need the opt-in beyond 48 KB
         cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     launch_step(kOne && a.chained, kKernel, grid, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
@@ -892,26 +892,26 @@ static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t s
 // out lane by lane where a.work allows it (kMore), else one per lane of as many blocks as it takes
 // (kPlain).  With fewer rays they are spread over all resident warps (kFew), unless other launches
 // share the device (a server's lanes): 24 requests took 6.65 ms against 6.54.
-template <bool kOne, bool kGrids, bool kCount, bool kAny, int kSmemS>
+template <bool kOne, bool kWide, bool kCount, bool kAny, int kSmemS>
 static void launch_bvh2_scenes(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    constexpr auto kM = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kGrids, kMore>;
-    constexpr auto kF = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kGrids, kFew>;
-    constexpr auto kP = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kGrids, kPlain>;
+    constexpr auto kM = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kWide, kMore>;
+    constexpr auto kF = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kWide, kFew>;
+    constexpr auto kP = k_trace_bvh2<kCount, kAny, kSmemS, kOne, kWide, kPlain>;
     const uint32_t need = blocks_for(a.n_max, a.block);
-    const uint32_t most = resident_blocks<kM>(a.block, (size_t)warp_smem(kSmemS, kGrids) * (a.block / 32));
-    if (need <= most && a.alone) launch_bvh2_kernel<kOne, kGrids, kF, kSmemS>(a, spread_blocks(a.n_max, a.block, most), st, lc);
-    else if (a.work && most && need > most) launch_bvh2_kernel<kOne, kGrids, kM, kSmemS>(a, most, st, lc);
-    else launch_bvh2_kernel<kOne, kGrids, kP, kSmemS>(a, need, st, lc);
+    const uint32_t most = resident_blocks<kM>(a.block, (size_t)warp_smem(kSmemS, kWide) * (a.block / 32));
+    if (need <= most && a.alone) launch_bvh2_kernel<kOne, kWide, kF, kSmemS>(a, spread_blocks(a.n_max, a.block, most), st, lc);
+    else if (a.work && most && need > most) launch_bvh2_kernel<kOne, kWide, kM, kSmemS>(a, most, st, lc);
+    else launch_bvh2_kernel<kOne, kWide, kP, kSmemS>(a, need, st, lc);
 }
 
 // One launch for a.shadow's rays too (k_trace_both): the kind of range that the longer list asks for.
-template <bool kOne, bool kGrids, int kSmemS>
+template <bool kOne, bool kWide, int kSmemS>
 static void launch_bvh2_both(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     const ShadowArgs& s = *a.shadow;
-    const size_t smem = (size_t)warp_smem(kSmemS, kGrids) * (a.block / 32);
+    const size_t smem = (size_t)warp_smem(kSmemS, kWide) * (a.block / 32);
     const uint32_t n_sh = s.n_groups_max * s.K;
     const uint32_t need = blocks_for(a.n_max, a.block), need_sh = blocks_for(n_sh, a.block);
-    const uint32_t most = resident_blocks<k_trace_both<kSmemS, kOne, kGrids, kMore>>(a.block, smem);
+    const uint32_t most = resident_blocks<k_trace_both<kSmemS, kOne, kWide, kMore>>(a.block, smem);
     auto run = [&](auto kernel, uint32_t first, uint32_t rest) {
         if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         launch_step(kOne && a.chained, kernel, first + rest, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d,
@@ -919,53 +919,53 @@ static void launch_bvh2_both(const TraceArgs& a, cudaStream_t st, LaunchCount& l
                     s.n_groups_max, s.K, s.radiance, s.n_traced, s.work, first);
     };
     if (need <= most && need_sh <= most && a.alone)
-        run(k_trace_both<kSmemS, kOne, kGrids, kFew>, spread_blocks(a.n_max, a.block, most), spread_blocks(n_sh, a.block, most));
+        run(k_trace_both<kSmemS, kOne, kWide, kFew>, spread_blocks(a.n_max, a.block, most), spread_blocks(n_sh, a.block, most));
     else if (a.work && s.work && most && (need > most || need_sh > most))
-        run(k_trace_both<kSmemS, kOne, kGrids, kMore>, need < most ? need : most, need_sh < most ? need_sh : most);
-    else run(k_trace_both<kSmemS, kOne, kGrids, kPlain>, need, need_sh);
+        run(k_trace_both<kSmemS, kOne, kWide, kMore>, need < most ? need : most, need_sh < most ? need_sh : most);
+    else run(k_trace_both<kSmemS, kOne, kWide, kPlain>, need, need_sh);
     lc.n++;
 }
 
 // kOneScene: whether launches over a single scene have a variant of their own.  Only these are set up
 // while the launch before ends: the plain pointers that this takes make launches over several scenes
 // 1% slower (16-job batch 5424 -> 5472 us) and those over one scene 1% faster (1024 x 1024 1185 -> 1175).
-// Launches with a scene of several grids have their own (they cost the others 2 to 3%).
+// Launches with a wide scene have kernels of their own (what these do more costs the others 2 to 3%).
 template <bool kOneScene, bool kCount, bool kAny, int kSmemS>
 static void launch_bvh2(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    const bool one = kOneScene && a.one_scene && !a.grids;
+    const bool one = kOneScene && a.one_scene && !a.wide;
     if constexpr (!kCount && !kAny) {
         if (a.shadow) {
-            if (a.grids) launch_bvh2_both<false, true, kSmemS>(a, st, lc);
+            if (a.wide) launch_bvh2_both<false, true, kSmemS>(a, st, lc);
             else if (one) launch_bvh2_both<kOneScene, false, kSmemS>(a, st, lc);
             else launch_bvh2_both<false, false, kSmemS>(a, st, lc);
             return;
         }
     }
     if (a.shadow) launch_shadow(*a.shadow, st, lc);
-    if (a.grids) launch_bvh2_scenes<false, true, kCount, kAny, kSmemS>(a, st, lc);
+    if (a.wide) launch_bvh2_scenes<false, true, kCount, kAny, kSmemS>(a, st, lc);
     else if (one) launch_bvh2_scenes<kOneScene, false, kCount, kAny, kSmemS>(a, st, lc);
     else launch_bvh2_scenes<false, false, kCount, kAny, kSmemS>(a, st, lc);
 }
 
-template <bool kCount, bool kAny, bool kGrids>
+template <bool kCount, bool kAny, bool kWide>
 static void launch_bvh2_user(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    const size_t smem = (size_t)warp_smem(kSmemStack, kGrids) * (a.block / 32);
+    const size_t smem = (size_t)warp_smem(kSmemStack, kWide) * (a.block / 32);
     const uint32_t need = blocks_for(a.n_max, a.block);
-    const uint32_t most = resident_blocks<k_trace_bvh2_user<kCount, kAny, kGrids, kMore>>(a.block, smem);
+    const uint32_t most = resident_blocks<k_trace_bvh2_user<kCount, kAny, kWide, kMore>>(a.block, smem);
     auto run = [&](auto kernel, uint32_t grid) {
         kernel<<<grid, a.block, smem, st>>>(a.scenes, a.user, a.n_max, a.counters, a.work);
     };
-    if (need <= most) run(k_trace_bvh2_user<kCount, kAny, kGrids, kFew>, spread_blocks(a.n_max, a.block, most));
-    else if (a.work && most) run(k_trace_bvh2_user<kCount, kAny, kGrids, kMore>, most);
-    else run(k_trace_bvh2_user<kCount, kAny, kGrids, kPlain>, need);
+    if (need <= most) run(k_trace_bvh2_user<kCount, kAny, kWide, kFew>, spread_blocks(a.n_max, a.block, most));
+    else if (a.work && most) run(k_trace_bvh2_user<kCount, kAny, kWide, kMore>, most);
+    else run(k_trace_bvh2_user<kCount, kAny, kWide, kPlain>, need);
     lc.n++;
 }
 
-template <bool kGrids>
+template <bool kWide>
 static void launch_bvh2_user(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
-    if (a.any_hit) launch_bvh2_user<false, true, kGrids>(a, st, lc);
-    else if (a.counters) launch_bvh2_user<true, false, kGrids>(a, st, lc);
-    else launch_bvh2_user<false, false, kGrids>(a, st, lc);
+    if (a.any_hit) launch_bvh2_user<false, true, kWide>(a, st, lc);
+    else if (a.counters) launch_bvh2_user<true, false, kWide>(a, st, lc);
+    else launch_bvh2_user<false, false, kWide>(a, st, lc);
 }
 
 void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
@@ -974,7 +974,7 @@ void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
         return;
     }
     if (a.user.rays && !a.bvh8 && !(a.bvh4 && !a.any_hit)) { // a caller's rays through the BVH2
-        if (a.grids) launch_bvh2_user<true>(a, st, lc);
+        if (a.wide) launch_bvh2_user<true>(a, st, lc);
         else launch_bvh2_user<false>(a, st, lc);
         return;
     }
@@ -986,7 +986,7 @@ void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     }
     // the BVH4 and the BVH2's variants trace closest hits only
     const bool variant = (a.bvh4 && !a.any_hit) ||
-                         (!a.any_hit && !a.counters && !a.grids &&
+                         (!a.any_hit && !a.counters && !a.wide &&
                           ((a.two_phase && a.phase.state && a.queue && a.queue_count) || a.packet || a.speculative));
     if (a.shadow && variant) launch_shadow(*a.shadow, st, lc);
     if (a.bvh4 && !a.any_hit) { // BVH4 kernel (trace_bvh4.cu)
@@ -997,7 +997,7 @@ void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
         launch_bvh2<false, false, true, kSmemStack>(a, st, lc);
         return;
     }
-    if (a.two_phase && !a.grids && !a.counters && a.phase.state && a.queue && a.queue_count) {
+    if (a.two_phase && !a.wide && !a.counters && a.phase.state && a.queue && a.queue_count) {
         const uint32_t grid = (a.n_max + block - 1) / block;
         const uint32_t nb = (a.n_max + 255) / 256;
         k_trace_bvh2_phase<<<grid, block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue, a.queue_count,
@@ -1012,14 +1012,14 @@ void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
         lc.n += 5;
         return;
     }
-    if (a.packet && !a.grids && !a.counters) {
+    if (a.packet && !a.wide && !a.counters) {
         const uint32_t grid = (a.n_max + block - 1) / block;
         k_trace_bvh2_packet<<<grid, block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
                                                        a.queue_count, a.n_max, a.hit);
         lc.n++;
         return;
     }
-    if (a.speculative && !a.grids && !a.counters) {
+    if (a.speculative && !a.wide && !a.counters) {
         const uint32_t grid = (a.n_max + block - 1) / block;
         k_trace_bvh2_spec<<<grid, block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue, a.queue_count,
                                                      a.n_max, a.hit);

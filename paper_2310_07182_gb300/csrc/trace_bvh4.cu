@@ -122,7 +122,7 @@ __device__ __forceinline__ int2 trace_bvh4_one(const float4* __restrict__ nodes,
         // leaf: a BVH2 leaf code
         const uint32_t code = (uint32_t)(~node);
         CR_DBG(if (!dbg_in_range(dsc, (code >> 2) + (code & 3u), kDbgTri, dsc->n_tris)) break;)
-        test_leaf(tris, r, skip, code >> 2, (code & 3u) + 1u, best, n_tri);
+        test_leaf<false>(tris, r, r.ix, r.iy, r.iz, skip, code >> 2, (code & 3u) + 1u, best, n_tri);
         tcull = __fmul_rn(best.t, kCullWiden);
         if (sp == 0) break;
         POP_CHILD(node);

@@ -54,7 +54,7 @@ __device__ __forceinline__ uint32_t visiting_order(uint32_t m, uint32_t s0, uint
 // 2.85 with lanes refilled, near and far words picked once per node instead of minima and maxima per
 // child, and no byte reordering of the node, 2.65 with the wait; shadow rays 2.67 -> 1.39 ->
 // 1.29 ms; primary 0.68 -> 0.51 ms.  Landscape secondary trace 1.75 -> 1.03 ms.
-template <bool kCount, bool kAny, class Src>
+template <bool kCount, bool kAny, bool kWide, class Src>
 __device__ __forceinline__ void trace_bvh8_warp(const SceneDev* __restrict__ scenes, Src& src,
                                                 unsigned long long& n_node, unsigned long long& n_tri) {
     constexpr bool kWait = Src::kMore;
@@ -206,7 +206,7 @@ __device__ __forceinline__ void trace_bvh8_warp(const SceneDev* __restrict__ sce
                 const uint32_t j = (uint32_t)__ffs(trimask) - 1u;
                 trimask &= trimask - 1u;
                 CR_DBG(if (!dbg_in_range(sc, tri_base + j, kDbgTri, sc->n_tris)) break;)
-                test_leaf(tris, r, skip, tri_base + j, 1u, best, n_tri);
+                test_leaf<kWide>(tris, r, r.ix, r.iy, r.iz, skip, tri_base + j, 1u, best, n_tri);
             } while (trimask);
             trimask = 0;
             tcull = __fmul_rn(best.t, kCullWiden);
@@ -219,7 +219,7 @@ __device__ __forceinline__ void trace_bvh8_warp(const SceneDev* __restrict__ sce
 #define CR_BVH8_MIN_BLOCKS 8 // resident 128-thread blocks per SM the register budget is sized for
 #endif
 
-template <bool kCount, bool kAny, RangeKind kKind>
+template <bool kCount, bool kAny, bool kWide, RangeKind kKind>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8(const SceneDev* __restrict__ scenes,
                              const uint16_t* slot_scene, const float4* ray_o, const float4* ray_d,
                              const int32_t* queue, const uint32_t* queue_count,
@@ -228,22 +228,22 @@ __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8(const Sc
     const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
     unsigned long long n_node = 0, n_tri = 0;
     QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit, blockIdx.x, gridDim.x);
-    if (src.more()) trace_bvh8_warp<kCount, kAny>(scenes, src, n_node, n_tri);
+    if (src.more()) trace_bvh8_warp<kCount, kAny, kWide>(scenes, src, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
 }
 
-template <bool kCount, bool kAny, RangeKind kKind>
+template <bool kCount, bool kAny, bool kWide, RangeKind kKind>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_bvh8_user(const SceneDev* __restrict__ scene,
                                                                              UserRays rays, uint32_t n,
                                                                              unsigned long long* counters, uint32_t* work) {
     unsigned long long n_node = 0, n_tri = 0;
     UserSrc<kKind> src(n, work, rays);
-    if (src.more()) trace_bvh8_warp<kCount, kAny>(scene, src, n_node, n_tri);
+    if (src.more()) trace_bvh8_warp<kCount, kAny, kWide>(scene, src, n_node, n_tri);
     if (kCount) add_counts(counters, n_node, n_tri);
 }
 
 // Shadow rays of next-event estimation over the BVH8-Q (see k_trace_shadow).
-template <RangeKind kKind>
+template <bool kWide, RangeKind kKind>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_shadow8(
     const SceneDev* __restrict__ scenes, const uint16_t* slot_scene, const float4* sh_o, const float4* sh_d,
     const float4* sh_c, const int32_t* group_queue, const uint32_t* group_count, uint32_t n_groups_max, uint32_t K, float4* __restrict__ radiance,
@@ -253,12 +253,12 @@ __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_shadow8(
     ShadowSrc<kKind> src(n, work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K, blockIdx.x, gridDim.x);
     if (!src.more()) return;
     unsigned long long dn = 0, dt = 0;
-    trace_bvh8_warp<false, true>(scenes, src, dn, dt);
+    trace_bvh8_warp<false, true, kWide>(scenes, src, dn, dt);
     src.add_traced(n_traced);
 }
 
 // Closest hits (blocks below `first`) and light samples in one launch (see k_trace_both).
-template <RangeKind kKind>
+template <bool kWide, RangeKind kKind>
 __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_both8(
     const SceneDev* __restrict__ scenes, const uint16_t* slot_scene, const float4* ray_o, const float4* ray_d,
     const int32_t* queue, const uint32_t* queue_count, uint32_t n_max, int2* __restrict__ hit, uint32_t* work,
@@ -270,13 +270,13 @@ __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_both8(
     if (blockIdx.x < first) {
         const uint32_t n = queue_count ? min(*queue_count, n_max) : n_max;
         QueueSrc<kKind> src(n, work, slot_scene, ray_o, ray_d, queue, hit, blockIdx.x, first);
-        if (src.more()) trace_bvh8_warp<false, false>(scenes, src, dn, dt);
+        if (src.more()) trace_bvh8_warp<false, false, kWide>(scenes, src, dn, dt);
     } else {
         const uint32_t n = (group_queue ? min(*group_count, n_groups_max) : n_groups_max) * K;
         ShadowSrc<kKind> src(n, sh_work, slot_scene, sh_o, sh_d, sh_c, group_queue, radiance, K, blockIdx.x - first,
                              gridDim.x - first);
         if (!src.more()) return;
-        trace_bvh8_warp<false, true>(scenes, src, dn, dt);
+        trace_bvh8_warp<false, true, kWide>(scenes, src, dn, dt);
         src.add_traced(n_traced);
     }
 }
@@ -285,64 +285,77 @@ __global__ void __launch_bounds__(128, CR_BVH8_MIN_BLOCKS) k_trace_both8(
 
 // As for the BVH2: rays handed out lane by lane where the launch may hold more than lanes are
 // resident at once.
-template <bool kCount, bool kAny>
+template <bool kCount, bool kAny, bool kWide>
 static void launch_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     const uint32_t need = blocks_for(a.n_max, a.block);
     if (a.user.rays) {
-        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8_user<kCount, kAny, kMore>>(a.block, 0) : 0u;
+        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8_user<kCount, kAny, kWide, kMore>>(a.block, 0) : 0u;
         if (most && need > most)
-            k_trace_bvh8_user<kCount, kAny, kMore><<<most, a.block, 0, st>>>(a.scenes, a.user, a.n_max, a.counters, a.work);
+            k_trace_bvh8_user<kCount, kAny, kWide, kMore><<<most, a.block, 0, st>>>(a.scenes, a.user, a.n_max, a.counters, a.work);
         else
-            k_trace_bvh8_user<kCount, kAny, kPlain><<<need, a.block, 0, st>>>(a.scenes, a.user, a.n_max, a.counters, nullptr);
+            k_trace_bvh8_user<kCount, kAny, kWide, kPlain><<<need, a.block, 0, st>>>(a.scenes, a.user, a.n_max, a.counters, nullptr);
     } else {
-        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8<kCount, kAny, kMore>>(a.block, 0) : 0u;
+        const uint32_t most = a.work ? resident_blocks<k_trace_bvh8<kCount, kAny, kWide, kMore>>(a.block, 0) : 0u;
         if (most && need > most)
-            launch_step(a.chained, k_trace_bvh8<kCount, kAny, kMore>, most, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
+            launch_step(a.chained, k_trace_bvh8<kCount, kAny, kWide, kMore>, most, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
                         a.ray_d, a.queue, a.queue_count, a.n_max, a.hit, a.counters, a.work);
         else
-            launch_step(a.chained, k_trace_bvh8<kCount, kAny, kPlain>, need, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
+            launch_step(a.chained, k_trace_bvh8<kCount, kAny, kWide, kPlain>, need, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o,
                         a.ray_d, a.queue, a.queue_count, a.n_max, a.hit, a.counters, nullptr);
     }
     lc.n++;
 }
 
+template <bool kWide>
 static void launch_bvh8_both(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     const ShadowArgs& s = *a.shadow;
     const uint32_t need = blocks_for(a.n_max, a.block), need_sh = blocks_for(s.n_groups_max * s.K, a.block);
-    const uint32_t most = a.work && s.work ? resident_blocks<k_trace_both8<kMore>>(a.block, 0) : 0u;
+    const uint32_t most = a.work && s.work ? resident_blocks<k_trace_both8<kWide, kMore>>(a.block, 0) : 0u;
     auto run = [&](auto kernel, uint32_t first, uint32_t rest, bool more) {
         launch_step(a.chained, kernel, first + rest, a.block, 0, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
                     a.queue_count, a.n_max, a.hit, more ? a.work : nullptr, s.sh_o, s.sh_d, s.sh_c, s.group_queue,
                     s.group_count, s.n_groups_max, s.K, s.radiance, s.n_traced, more ? s.work : nullptr, first);
     };
     if (most && (need > most || need_sh > most))
-        run(k_trace_both8<kMore>, need < most ? need : most, need_sh < most ? need_sh : most, true);
-    else run(k_trace_both8<kPlain>, need, need_sh, false);
+        run(k_trace_both8<kWide, kMore>, need < most ? need : most, need_sh < most ? need_sh : most, true);
+    else run(k_trace_both8<kWide, kPlain>, need, need_sh, false);
     lc.n++;
 }
 
-void launch_trace_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
+template <bool kWide>
+static void launch_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
     if (a.shadow && !a.any_hit && !a.counters && !a.user.rays) {
-        launch_bvh8_both(a, st, lc);
+        launch_bvh8_both<kWide>(a, st, lc);
         return;
     }
     if (a.shadow) launch_shadow(*a.shadow, st, lc);
-    if (a.any_hit) launch_bvh8<false, true>(a, st, lc);
-    else if (a.counters) launch_bvh8<true, false>(a, st, lc);
-    else launch_bvh8<false, false>(a, st, lc);
+    if (a.any_hit) launch_bvh8<false, true, kWide>(a, st, lc);
+    else if (a.counters) launch_bvh8<true, false, kWide>(a, st, lc);
+    else launch_bvh8<false, false, kWide>(a, st, lc);
 }
 
-void launch_shadow_bvh8(const ShadowArgs& a, cudaStream_t st, LaunchCount& lc) {
+void launch_trace_bvh8(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
+    if (a.wide) launch_bvh8<true>(a, st, lc);
+    else launch_bvh8<false>(a, st, lc);
+}
+
+template <bool kWide>
+static void launch_shadow8(const ShadowArgs& a, cudaStream_t st, LaunchCount& lc) {
     const int block = 128;
     const uint32_t need = blocks_for(a.n_groups_max * a.K, block);
-    const uint32_t most = a.work ? resident_blocks<k_trace_shadow8<kMore>>(block, 0) : 0u;
+    const uint32_t most = a.work ? resident_blocks<k_trace_shadow8<kWide, kMore>>(block, 0) : 0u;
     auto run = [&](auto kernel, uint32_t grid, uint32_t* work) {
         launch_step(a.chained, kernel, grid, block, 0, st, a.scenes, a.slot_scene, a.sh_o, a.sh_d, a.sh_c, a.group_queue,
                     a.group_count, a.n_groups_max, a.K, a.radiance, a.n_traced, work);
     };
-    if (most && need > most) run(k_trace_shadow8<kMore>, most, a.work);
-    else run(k_trace_shadow8<kPlain>, need, nullptr);
+    if (most && need > most) run(k_trace_shadow8<kWide, kMore>, most, a.work);
+    else run(k_trace_shadow8<kWide, kPlain>, need, nullptr);
     lc.n++;
+}
+
+void launch_shadow_bvh8(const ShadowArgs& a, cudaStream_t st, LaunchCount& lc) {
+    if (a.wide) launch_shadow8<true>(a, st, lc);
+    else launch_shadow8<false>(a, st, lc);
 }
 
 } // namespace cr

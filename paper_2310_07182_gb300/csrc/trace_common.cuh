@@ -227,7 +227,10 @@ __device__ __forceinline__ bool box_hit_fma(const RayPre& r, float lox, float hi
 // fallback: edge functions of exactly zero count as inside, so shared edges are covered.
 // kx and ky are not exchanged for rays that run down the kz axis: that negates U, V, W, det
 // and T exactly, which leaves the sign test and t = T / det as they are.
-__device__ __forceinline__ bool tri_test(const RayPre& r, float4 a4, float4 b4, float4 c4, float& t_out) {
+// near (kNear): the hit is nearer than 1/16 of the farthest vertex (along kz), where rounding may have moved it
+// past the origin (the error is some 2^-22 of that distance unless the ray all but lies in the plane).
+template <bool kNear>
+__device__ __forceinline__ bool tri_test(const RayPre& r, float4 a4, float4 b4, float4 c4, float& t_out, bool& near) {
     const float Ax3 = a4.x - r.ox, Ay3 = a4.y - r.oy, Az3 = a4.z - r.oz;
     const float Bx3 = b4.x - r.ox, By3 = b4.y - r.oy, Bz3 = b4.z - r.oz;
     const float Cx3 = c4.x - r.ox, Cy3 = c4.y - r.oy, Cz3 = c4.z - r.oz;
@@ -247,6 +250,7 @@ __device__ __forceinline__ bool tri_test(const RayPre& r, float4 a4, float4 b4, 
     const float T = __fadd_rn(__fadd_rn(__fmul_rn(U, Az), __fmul_rn(V, Bz)), __fmul_rn(W, Cz));
     const float t = __fdiv_rn(T, det);
     if (!(t > 0.0f)) return false;
+    if (kNear) near = t < 0.0625f * max3f(fabsf(Az), fabsf(Bz), fabsf(Cz));
     t_out = t;
     return true;
 }
@@ -256,7 +260,31 @@ struct Best {
     int leaf; // triangle in leaf order, -1 none
 };
 
-__device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, const RayPre& r, int skip, uint32_t first,
+// Whether a triangle lies behind the origin along an axis, by more than 2^-22 of the origin's coordinate
+// (i: any value with the direction component's sign).  Such a triangle is not hit, but the test above can
+// say so when it is large and the origin lies just off its plane: a ray that leaves a ground of a
+// kilometre met the coplanar triangle beside its own at t = 3e-5.  Exact boxes keep most of these from
+// the test; enlarged ones do not.  The vertices are read again (this is rare, see tri_test; kept in
+// registers since the test, they cost the traces 4 to 9%, read again 2%), and only the kernels for wide
+// scenes look (kWideTri).
+__device__ __forceinline__ float4 reload(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ bool behind_axis(float o, float i, float a, float b, float c) {
+    const float e = __fmul_rn(fabsf(o), 0x1.0p-22f);
+    return __float_as_int(i) < 0 ? min3f(a, b, c) > __fadd_rn(o, e) : max3f(a, b, c) < __fsub_rn(o, e);
+}
+__device__ __forceinline__ bool behind(const RayPre& r, float ix, float iy, float iz, const float4* tri) {
+    const float4 a = reload(tri), b = reload(tri + 1), c = reload(tri + 2);
+    return behind_axis(r.ox, ix, a.x, b.x, c.x) || behind_axis(r.oy, iy, a.y, b.y, c.y) || behind_axis(r.oz, iz, a.z, b.z, c.z);
+}
+
+// kWide: look for triangles behind the origin; ix, iy, iz: values with the signs of the direction's components.
+template <bool kWide>
+__device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, const RayPre& r, float ix, float iy, float iz,
+                                          int skip, uint32_t first,
                                           uint32_t count, Best& best, unsigned long long& n_tri) {
     for (uint32_t i = 0; i < count; ++i) {
         const uint32_t tri = first + i;
@@ -267,9 +295,13 @@ __device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, const
         const float4 c = __ldg(&tris[3 * tri + 2]);
         ++n_tri;
         float t;
+        bool near = false;
         // a tie goes to the smaller original index (any hit at exactly tmax is taken)
-        if (tri_test(r, a, b, c, t) &&
+        if (tri_test<kWide>(r, a, b, c, t, near) &&
             (t < best.t || (t == best.t && (best.leaf < 0 || orig < __float_as_int(__ldg(&tris[3 * best.leaf]).w))))) {
+            if constexpr (kWide) {
+                if (near && behind(r, ix, iy, iz, &tris[3 * tri])) continue;
+            }
             best.t = t;
             best.leaf = (int)tri;
         }

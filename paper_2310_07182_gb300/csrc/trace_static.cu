@@ -106,7 +106,7 @@ extern "C" cr_status cr_trace_rays_static(cr_scene* scene, const float* rays, co
     ta.block = 128;
     ta.scenes = dev_scene_entry(scene, false);
     ta.one_scene = true;
-    ta.grids = dev_scene_of(scene)->n_grids > 1;
+    ta.wide = dev_scene_of(scene)->wide;
     if (user_rays_apart(rays, skip_prim, n, prim, t)) {
         ta.user.rays = rays;
         ta.user.skip = skip_prim;
