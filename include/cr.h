@@ -337,8 +337,8 @@ cr_status cr_batch_create(const cr_job* jobs, uint32_t n_jobs, const cr_batch_op
 cr_status cr_batch_run(cr_batch* batch, cr_stats* stats);
 cr_status cr_batch_destroy(cr_batch* batch);
 /* Path-state bytes a batch of these jobs would allocate (admission by device footprint).  Samples of
- * its jobs share passes up to 2^23 slots; cr_batch_create falls back to a sample per pass when that
- * much cannot be had. */
+ * its jobs share passes up to 2^23 slots; cr_batch_create lets fewer of them share one, at last one, when
+ * that much cannot be had. */
 cr_status cr_batch_device_bytes(const cr_job* jobs, uint32_t n_jobs, const cr_batch_opts* opts, uint64_t* bytes);
 
 /* Autotuner: times candidate (W,H) in {4x4, 8x8, 16x16}, K <= W*H/4 (larger K loses image

@@ -828,6 +828,25 @@ cr_status build_plan(const cr_job* jobs, uint32_t n_jobs, const PlanOpts& po, Re
     return CR_OK;
 }
 
+// The plan of these jobs and the path state for it: samples share passes as far as memory can be had
+// (half as many after each allocation that fails, at last a sample per pass).
+static cr_status fit_plan(const cr_job* jobs, uint32_t n_jobs, PlanOpts po, bool two_phase, Workspace& ws, RenderPlan& plan) {
+    while (true) {
+        cr_status st = build_plan(jobs, n_jobs, po, plan);
+        if (st != CR_OK) return st;
+        st = ws.ensure(plan.max_slots, plan.npx_total);
+        if (st == CR_OK && plan.nee) st = ws.ensure_nee(plan.max_slots);
+        if (st == CR_OK && two_phase) st = ws.ensure_phase(plan.max_slots);
+        if (st == CR_OK) {
+            g_err.clear(); // of the attempts before
+            return CR_OK;
+        }
+        if (st != CR_ERR_OOM || plan.regions == 1) return st;
+        ws.release();
+        po.samples = plan.regions / 2;
+    }
+}
+
 // Room for the tables, grown on demand (they are reused across calls).
 cr_status Plan::reserve(size_t bj, size_t bs) {
     if (bj <= cap_jobs && bs <= cap_scenes) return CR_OK;
@@ -1058,17 +1077,8 @@ extern "C" cr_status cr_render_ex(cr_scene* s, const cr_camera* cam, uint32_t sp
         if (po.tile_end == 0) return fail(CR_ERR_INVALID_ARG, "cr_render: tile_end is 0 with tile_begin %u", o.tile_begin);
     }
     RenderPlan plan;
-    while (true) {
-        st = build_plan(&job, 1, po, plan);
-        if (st != CR_OK) return st;
-        st = s->ws.ensure(plan.max_slots, plan.npx_total);
-        if (st == CR_OK && plan.nee) st = s->ws.ensure_nee(plan.max_slots);
-        if (st == CR_OK) break;
-        if (st != CR_ERR_OOM || plan.regions == 1) return st;
-        s->ws.release(); // one sample per pass needs less memory
-        po.samples = 1;
-    }
-    g_err.clear();
+    st = fit_plan(&job, 1, po, (o.flags & CR_OPT_TWO_PHASE) != 0, s->ws, plan);
+    if (st != CR_OK) return st;
     // the job table (the scene's own entry is its scene table): from the arguments of a first launch
     // where it is small
     Plan& dev = s->plan_dev;
@@ -1090,11 +1100,7 @@ extern "C" cr_status cr_render_ex(cr_scene* s, const cr_camera* cam, uint32_t sp
     eo.count = (o.flags & CR_OPT_COUNT) != 0;
     if (o.sort_key > CR_SORT_HIERARCHY_CUT) return fail(CR_ERR_INVALID_ARG, "cr_render: sort_key %u", o.sort_key);
     eo.sort_key = o.sort_key;
-    if (o.flags & CR_OPT_TWO_PHASE) {
-        eo.phase_budget = CR_PHASE_BUDGET;
-        st = s->ws.ensure_phase(plan.max_slots);
-        if (st != CR_OK) return st;
-    }
+    if (o.flags & CR_OPT_TWO_PHASE) eo.phase_budget = CR_PHASE_BUDGET;
     eo.debug = o.debug;
     eo.debug_npx = npx;
     eo.stats_traces_only = (o.flags & CR_OPT_STATS_TRACES) && !(o.flags & CR_OPT_STATS);
@@ -1535,17 +1541,8 @@ extern "C" cr_status cr_batch_create(const cr_job* jobs, uint32_t n_jobs, const 
     if (!b) return fail(CR_ERR_OOM, "cr_batch_create: host allocation");
     b->jobs.assign(jobs, jobs + n_jobs);
     b->opts = *opts;
-    while (true) {
-        st = build_plan(b->jobs.data(), n_jobs, po, b->plan);
-        if (st != CR_OK) return st;
-        st = b->ws.ensure(b->plan.max_slots, b->plan.npx_total);
-        if (st == CR_OK && b->plan.nee) st = b->ws.ensure_nee(b->plan.max_slots);
-        if (st == CR_OK) break;
-        if (st != CR_ERR_OOM || b->plan.regions == 1) return st;
-        b->ws.release(); // one sample per pass needs less memory
-        po.samples = 1;
-    }
-    g_err.clear();
+    st = fit_plan(b->jobs.data(), n_jobs, po, false, b->ws, b->plan);
+    if (st != CR_OK) return st;
     if (opts->stream) {
         b->stream = static_cast<cudaStream_t>(opts->stream);
     } else {
