@@ -257,6 +257,10 @@ cr_status cr_render_opts_default(cr_render_opts* opts);
  * bounces, mode, W, H, K, interleave, seed, frame_base, reuse_depth): random numbers are
  * keyed by (pixel, frame, bounce), never by ray order, so CR_MORTON_SORT gives the same
  * image as CR_INDEPENDENT bit for bit.
+ * Memory: the scene keeps the path state of its largest render until it is destroyed, 125 to 173 bytes per
+ * slot (the pixels of whole tiles).  Samples of a render share passes of up to 2^23 slots, which takes a
+ * multiple of one sample's state: at most an eighth of the free device memory, and 1/16 of the device's
+ * memory over all scenes and batches; with less room fewer samples share a pass, with the same image.
  * Errors: CR_ERR_INVALID_ARG, CR_ERR_OOM, CR_ERR_CUDA. */
 cr_status cr_render(cr_scene* scene, const cr_camera* camera, uint32_t spp, uint32_t max_bounces,
                     cr_reuse_mode mode, uint32_t group_w, uint32_t group_h, float* out_rgb);
@@ -336,9 +340,9 @@ cr_status cr_batch_create(const cr_job* jobs, uint32_t n_jobs, const cr_batch_op
  * stats (may be NULL): ms_total (CUDA events around the run), secondary rays, launches. */
 cr_status cr_batch_run(cr_batch* batch, cr_stats* stats);
 cr_status cr_batch_destroy(cr_batch* batch);
-/* Path-state bytes a batch of these jobs would allocate (admission by device footprint).  Samples of
- * its jobs share passes up to 2^23 slots; cr_batch_create lets fewer of them share one, at last one, when
- * that much cannot be had. */
+/* Path-state bytes a batch of these jobs needs (admission by device footprint): what one sample of each
+ * job per pass takes.  Where memory is plentiful more samples share a pass and cr_batch_create takes more
+ * (see cr_render_ex); it never fails for want of more than this. */
 cr_status cr_batch_device_bytes(const cr_job* jobs, uint32_t n_jobs, const cr_batch_opts* opts, uint64_t* bytes);
 
 /* Autotuner: times candidate (W,H) in {4x4, 8x8, 16x16}, K <= W*H/4 (larger K loses image

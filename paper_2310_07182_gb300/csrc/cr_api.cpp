@@ -4,6 +4,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
@@ -513,7 +514,39 @@ struct StageEvents {
 
 namespace cr {
 
+// Bytes per device that all workspaces hold for samples sharing passes, beyond what a sample per pass
+// needs: at most a kSharedPart-th of the device's memory, so that scenes and batches do not fill it by
+// having rendered once (a workspace is kept until its scene or batch is destroyed).  One workspace takes
+// at most a kSharedFree-th of what is free, so that its caller's next allocation is not the one to fail.
+// (1280x720 with light samples takes 0.16 GB for a sample per pass and 1.45 GB for nine.)
+constexpr uint64_t kSharedPart = 16, kSharedFree = 8;
+static std::atomic<uint64_t> g_shared[64];
+
+static void unshare_memory(Workspace& ws) {
+    if (ws.shared) g_shared[ws.shared_device] -= ws.shared;
+    ws.shared = 0;
+}
+// Counts `bytes` for ws instead of what it holds so; false, and nothing changed, where that is too much.
+// free: what is free to it, its own buffers among it.
+static bool share_memory(Workspace& ws, int dev, uint64_t bytes, uint64_t free, uint64_t total) {
+    if (dev < 0 || dev >= 64 || bytes > free / kSharedFree) return false;
+    const uint64_t own = ws.shared_device == dev ? ws.shared : 0;
+    uint64_t held = g_shared[dev].load();
+    do {
+        if (held - own + bytes > total / kSharedPart) return false;
+    } while (!g_shared[dev].compare_exchange_weak(held, held - own + bytes));
+    if (ws.shared_device != dev) unshare_memory(ws);
+    ws.shared = bytes;
+    ws.shared_device = dev;
+    return true;
+}
+
 void Workspace::release() {
+    free_buffers();
+    unshare_memory(*this);
+}
+
+void Workspace::free_buffers() {
     if (base) cudaFree(base);
     base = nullptr;
     bytes = 0;
@@ -579,7 +612,7 @@ cr_status Workspace::ensure_phase(uint32_t n_slots) {
 cr_status Workspace::ensure(uint32_t n_slots, uint32_t npx) {
     if (base && pb.n_slots >= n_slots && pb.n_px_cap >= npx) return CR_OK;
     cudaDeviceSynchronize();
-    release();
+    free_buffers();
     const size_t ns = n_slots, np = npx;
     const size_t n_cblocks = compact_blocks(n_slots) + 1;
     const size_t n_hist = sort_hist_len(n_slots);
@@ -762,6 +795,7 @@ cr_status build_plan(const cr_job* jobs, uint32_t n_jobs, const PlanOpts& po, Re
         uint64_t r = po.samples ? po.samples : std::max<uint64_t>(1, kPassSlots / slots);
         r = std::min<uint64_t>({r, max_spp, 65535u / n_jobs, (1ull << 27) / slots, ((1ull << 28) / px) - 1});
         plan.regions = (uint32_t)std::max<uint64_t>(1, r);
+        plan.one_slots = (uint32_t)slots;
     }
     if (plan.regions > 1) {
         plan.npx = px;
@@ -828,12 +862,37 @@ cr_status build_plan(const cr_job* jobs, uint32_t n_jobs, const PlanOpts& po, Re
     return CR_OK;
 }
 
+// Device bytes of path state (the two-phase buffers as Workspace::ensure_phase takes them).
+static uint64_t state_bytes(uint32_t slots, uint32_t npx, bool nee, bool two_phase) {
+    return workspace_bytes(slots, npx) + (nee ? 48ull * slots : 0) +
+           (two_phase ? (sizeof(TraceState) + 5ull) * slots + 8ull * ((slots + 255ull) / 256 + 1) + 1024 : 0);
+}
+
 // The plan of these jobs and the path state for it: samples share passes as far as memory can be had
-// (half as many after each allocation that fails, at last a sample per pass).
+// (half as many after each attempt that fails, at last a sample per pass).
 static cr_status fit_plan(const cr_job* jobs, uint32_t n_jobs, PlanOpts po, bool two_phase, Workspace& ws, RenderPlan& plan) {
+    int dev = -1;
+    size_t free = 0, total = 0; // asked for once, where the workspace has to grow
     while (true) {
         cr_status st = build_plan(jobs, n_jobs, po, plan);
         if (st != CR_OK) return st;
+        const bool fits = ws.base && ws.pb.n_slots >= plan.max_slots && ws.pb.n_px_cap >= plan.npx_total &&
+                          (!plan.nee || (ws.nee_base && ws.nee_slots >= plan.max_slots)) &&
+                          (!two_phase || (ws.phase_base && ws.phase_slots >= plan.max_slots));
+        if (!fits && plan.regions > 1) {
+            if (!total) {
+                if (cudaGetDevice(&dev) != cudaSuccess || cudaMemGetInfo(&free, &total) != cudaSuccess) cudaGetLastError();
+                if (!total) dev = -1;
+                free += ws.bytes + (ws.nee_base ? 48 * (size_t)ws.nee_slots : 0) +
+                        (ws.phase_base ? (sizeof(TraceState) + 5) * (size_t)ws.phase_slots : 0);
+            }
+            const uint64_t more = state_bytes(plan.max_slots, plan.npx_total, plan.nee, two_phase) -
+                                  state_bytes(plan.one_slots, plan.npx, plan.nee, two_phase);
+            if (!share_memory(ws, dev, more, free, total)) {
+                po.samples = plan.regions / 2;
+                continue;
+            }
+        }
         st = ws.ensure(plan.max_slots, plan.npx_total);
         if (st == CR_OK && plan.nee) st = ws.ensure_nee(plan.max_slots);
         if (st == CR_OK && two_phase) st = ws.ensure_phase(plan.max_slots);
@@ -1520,10 +1579,11 @@ extern "C" cr_status cr_batch_device_bytes(const cr_job* jobs, uint32_t n_jobs, 
     cr_status st = batch_opts_check(opts, po, eo);
     if (st != CR_OK) return st;
     RenderPlan plan;
+    po.samples = 1;
     st = build_plan(jobs, n_jobs, po, plan);
     if (st != CR_OK) return st;
-    *bytes = workspace_bytes(plan.max_slots, plan.npx_total) + sizeof(JobDev) * plan.jobs.size() +
-             sizeof(SceneDev) * plan.scenes.size() + (plan.nee ? 48 * (uint64_t)plan.max_slots : 0);
+    *bytes = state_bytes(plan.max_slots, plan.npx_total, plan.nee, false) + sizeof(JobDev) * plan.jobs.size() +
+             sizeof(SceneDev) * plan.scenes.size();
     return CR_OK;
 }
 

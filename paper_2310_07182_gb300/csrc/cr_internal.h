@@ -434,6 +434,11 @@ struct Workspace {
     PhaseBuffers phase;
     cr_status ensure(uint32_t n_slots, uint32_t npx);
     cr_status ensure_phase(uint32_t n_slots);
+    // what it holds beyond the need of a sample per pass, and the device that this counts against
+    // (share_memory in cr_api.cpp)
+    uint64_t shared = 0;
+    int shared_device = -1;
+    void free_buffers();
     void release();
     ~Workspace() { release(); }
 };
@@ -446,8 +451,8 @@ struct PlanOpts {
     bool bvh8 = false;
     bool bvh4 = false; // closest-hit traces through the BVH4 (single renders; shadow rays stay on the BVH2)
     uint32_t tile_begin = 0, tile_end = 0; // single-job plans: render only these tiles (0, 0 = all)
-    // samples of each job that share a pass (RenderPlan::regions; whole images only): 0 = as many as
-    // keep a pass within kPassSlots slots
+    // samples of each job that share a pass at most (RenderPlan::regions; whole images only): 0 = as many
+    // as keep a pass within kPassSlots slots
     uint32_t samples = 0;
 };
 struct Pass {
@@ -465,6 +470,7 @@ struct RenderPlan {
     // the pass; after each pass they are added in sample order to the running sums in the region
     // after them, and a job's last pass writes its output.  jobs[sum_offset ...] has one entry per job.
     uint32_t regions = 1, npx = 0, sum_offset = 0, n_jobs = 0;
+    uint32_t one_slots = 0; // slots of a pass of one sample per job
     std::vector<JobDev> jobs;     // all passes' tables, pass by pass
     std::vector<SceneDev> scenes; // scene table
     std::vector<Pass> passes;

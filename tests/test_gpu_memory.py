@@ -1,4 +1,5 @@
-"""Renders of several samples when device memory is short: fewer samples share a pass, the images stay."""
+"""Device memory of renders of several samples: bounded over all scenes and batches, and when little is free fewer
+samples share a pass; the images stay."""
 import pytest
 import torch
 
@@ -37,7 +38,7 @@ def _scene(cr):
 
 
 # 16 samples of 640 x 360 in a pass: 524 MB of path state, 177 more with light samples, 490 more for the two
-# phases.  At 900 MB the first fit and the last do not, at 300 MB none does; a sample per pass takes 41.
+# phases.  At 900 MB the first fit and the last do not, at 300 MB none does; a sample per pass takes 33.
 @pytest.mark.parametrize("free", [900 * MB, 300 * MB])
 @pytest.mark.parametrize("flags,nee", [(0, False), (0, True), (128, False), (128, True)])
 def test_renders_when_memory_is_short(cr, leave, free, flags, nee):
@@ -74,4 +75,65 @@ def test_batches_when_memory_is_short(cr, leave, free):
             assert all(torch.equal(w, o) for w, o in zip(want, outs))
         finally:
             cr.cr_batch_destroy(b)
+    S.close()
+
+
+def _held(f):
+    """Device bytes that f() leaves allocated."""
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    f()
+    torch.cuda.synchronize()
+    return before - torch.cuda.mem_get_info()[0]
+
+
+def test_scenes_that_have_rendered_hold_a_bounded_share(cr):
+    """64 samples of 640 x 360 take 1.2 GB in passes of 36: not of every scene that has rendered once."""
+    kw = dict(spp=64, max_bounces=1, tile=(8, 8), k=8, seed=9)
+    out = torch.empty((360, 640, 3), device="cuda")
+    S = _scene(cr)
+    first = _held(lambda: S.render(_cam(640, 360), out=out, **kw))
+    assert first > 600 * MB
+    want = out.clone()
+    many = [_scene(cr) for _ in range(40)]
+    held = _held(lambda: [s.render(_cam(640, 360), out=out, **kw) for s in many])
+    total = torch.cuda.mem_get_info()[1]
+    assert first + held < total // 16 + 41 * 64 * MB  # a sample per pass takes 33 MB
+    assert torch.equal(out, want)
+    for s in many + [S]:
+        s.close()
+    S = _scene(cr)  # what they held has been given back
+    assert _held(lambda: S.render(_cam(640, 360), out=out, **kw)) > 600 * MB
+    S.close()
+
+
+def test_renders_leave_most_of_the_free_memory(cr, leave):
+    kw = dict(spp=64, max_bounces=1, tile=(8, 8), k=8, seed=9)
+    out = torch.empty((360, 640, 3), device="cuda")
+    S = _scene(cr)
+    S.render(_cam(640, 360), out=out, **kw)
+    want = out.clone()
+    S.close()
+    S = _scene(cr)
+    leave(3000 * MB)
+    launches = []
+    for _ in range(3):
+        held = _held(lambda: launches.append(S.render(_cam(640, 360), out=out, stats=True, **kw)[1]["kernel_launches"]))
+        assert held < 3000 * MB // 8 + 64 * MB and torch.equal(out, want)
+    assert held == 0 and launches[0] == launches[1] == launches[2]  # the workspace that was found is kept
+    S.close()
+
+
+def test_device_bytes_are_what_a_batch_needs(cr, leave):
+    S = _scene(cr)
+    out = torch.empty((360, 640, 3), device="cuda")
+    opts = cr.make_batch_opts(tile=(8, 8), k=8)
+    def job(n):
+        return [cr.make_job(S.handle, _cam(640, 360), out, spp=n, max_bounces=1)]
+    one, many = (cr.cr_batch_device_bytes(job(n), opts) for n in (1, 64))
+    assert one <= many < one + 64 * 1024  # the tables of 64 passes
+    leave(many + 64 * MB)
+    b = cr.cr_batch_create(job(64), opts)
+    cr.cr_batch_run(b)
+    cr.cr_batch_destroy(b)
     S.close()
