@@ -881,8 +881,7 @@ SceneDev scene_entry(const DevScene& s, bool bvh8) {
 template <bool kOne, bool kWide, auto kKernel, int kSmemS>
 static void launch_bvh2_kernel(const TraceArgs& a, uint32_t grid, cudaStream_t st, LaunchCount& lc) {
     const size_t smem = (size_t)warp_smem(kSmemS, kWide) * (a.block / 32);
-    if (smem > 48 * 1024) // 512-thread blocks with 32 entries need the opt-in beyond 48 KB
-        cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem<kKernel>(smem); // blocks of 352 threads or more with 32 entries
     launch_step(kOne && a.chained, kKernel, grid, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
                 a.queue_count, a.n_max, a.hit, a.counters, a.work);
     lc.n++;
@@ -904,6 +903,9 @@ static void launch_bvh2_scenes(const TraceArgs& a, cudaStream_t st, LaunchCount&
     else launch_bvh2_kernel<kOne, kWide, kP, kSmemS>(a, need, st, lc);
 }
 
+template <auto kKernel>
+using kernel_of = std::integral_constant<decltype(kKernel), kKernel>;
+
 // One launch for a.shadow's rays too (k_trace_both): the kind of range that the longer list asks for.
 template <bool kOne, bool kWide, int kSmemS>
 static void launch_bvh2_both(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
@@ -913,16 +915,17 @@ static void launch_bvh2_both(const TraceArgs& a, cudaStream_t st, LaunchCount& l
     const uint32_t need = blocks_for(a.n_max, a.block), need_sh = blocks_for(n_sh, a.block);
     const uint32_t most = resident_blocks<k_trace_both<kSmemS, kOne, kWide, kMore>>(a.block, smem);
     auto run = [&](auto kernel, uint32_t first, uint32_t rest) {
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_step(kOne && a.chained, kernel, first + rest, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d,
+        constexpr auto kKernel = decltype(kernel)::value;
+        allow_smem<kKernel>(smem);
+        launch_step(kOne && a.chained, kKernel, first + rest, a.block, smem, st, a.scenes, a.slot_scene, a.ray_o, a.ray_d,
                     a.queue, a.queue_count, a.n_max, a.hit, a.work, s.sh_o, s.sh_d, s.sh_c, s.group_queue, s.group_count,
                     s.n_groups_max, s.K, s.radiance, s.n_traced, s.work, first);
     };
     if (need <= most && need_sh <= most && a.alone)
-        run(k_trace_both<kSmemS, kOne, kWide, kFew>, spread_blocks(a.n_max, a.block, most), spread_blocks(n_sh, a.block, most));
+        run(kernel_of<k_trace_both<kSmemS, kOne, kWide, kFew>>(), spread_blocks(a.n_max, a.block, most), spread_blocks(n_sh, a.block, most));
     else if (a.work && s.work && most && (need > most || need_sh > most))
-        run(k_trace_both<kSmemS, kOne, kWide, kMore>, need < most ? need : most, need_sh < most ? need_sh : most);
-    else run(k_trace_both<kSmemS, kOne, kWide, kPlain>, need, need_sh);
+        run(kernel_of<k_trace_both<kSmemS, kOne, kWide, kMore>>(), need < most ? need : most, need_sh < most ? need_sh : most);
+    else run(kernel_of<k_trace_both<kSmemS, kOne, kWide, kPlain>>(), need, need_sh);
     lc.n++;
 }
 

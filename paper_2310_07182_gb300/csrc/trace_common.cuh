@@ -532,6 +532,13 @@ __device__ __forceinline__ void add_counts(unsigned long long* counters, unsigne
     }
 }
 
+// Launches of a kernel with more than 48 KB of shared memory per block need the opt-in first, and so does
+// the question how many of them are resident.
+template <auto kKernel>
+static void allow_smem(size_t smem) {
+    if (smem > 48 * 1024) cudaFuncSetAttribute(kKernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 // Blocks of a trace kernel that are resident on the current device at once (0: unknown).
 template <auto kKernel>
 static uint32_t resident_blocks(int block, size_t smem) {
@@ -543,6 +550,7 @@ static uint32_t resident_blocks(int block, size_t smem) {
     uint32_t v = r.load(std::memory_order_relaxed);
     if (!v) {
         int sms = 0, nb = 0;
+        allow_smem<kKernel>(smem);
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kKernel, block, smem) != cudaSuccess || sms <= 0 || nb <= 0)
             return 0;

@@ -50,3 +50,12 @@ def test_stage_events_and_chained_launches_exclude_each_other():
     decide = re.search(r"const bool chained = ([^;]*);", plan).group(1)
     assert decide.startswith("!times && ")
     assert all("chained" in v for v in re.findall(r"\.chained = ([^;]*);", plan))
+
+
+def test_shared_memory_beyond_48_kb_is_allowed_before_occupancy_is_asked():
+    """Otherwise the answer is 0 blocks, and such launches (32 stack entries, 352 threads or more) get the plain
+    variant."""
+    s = SRC["trace_common.cuh"]
+    body = s[s.index("static uint32_t resident_blocks("):]
+    body = body[:body.index("\n}\n")]
+    assert 0 < body.find("allow_smem<kKernel>(smem)") < body.index("cudaOccupancyMaxActiveBlocksPerMultiprocessor")
