@@ -559,9 +559,9 @@ __global__ void __launch_bounds__(256) k_susp_scatter(const uint8_t* __restrict_
 // superset of the boxes its own ray enters, with the same triangle test and tie rule, so
 // the hits are the single-ray kernel's bit for bit.  Control flow is warp-uniform, which
 // pays off when the rays of a warp are coherent (primary rays, reused directions) and
-// costs extra box and triangle tests when they are not.
+// costs extra box and triangle tests when they are not.  Every ray is in scenes[0].
 __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
-    const SceneDev* __restrict__ scenes, const uint16_t* __restrict__ slot_scene, const float4* __restrict__ ray_o,
+    const SceneDev* __restrict__ scenes, const float4* __restrict__ ray_o,
     const float4* __restrict__ ray_d, const int32_t* __restrict__ queue, const uint32_t* __restrict__ queue_count,
     uint32_t n_max, int2* __restrict__ hit) {
     extern __shared__ uint32_t smem_stack[];
@@ -575,12 +575,10 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
     RayPre r;
     int skip = -1;
     Best best{-1.0f, -1}; // t < 0: a lane without a ray never enters a box
-    uint32_t sid = 0;
     if (i < n) {
         slot = queue ? queue[i] : (int)i;
         const float4 ro = ray_o[slot];
         const float4 rd = ray_d[slot];
-        sid = slot_scene ? slot_scene[slot] : 0;
         if (rd.w >= 0.0f) {
             r = prep_ray(ro, rd);
             skip = __float_as_int(ro.w);
@@ -590,18 +588,10 @@ __global__ void __maxnreg__(CR_TRACE_MAXNREG) k_trace_bvh2_packet(
             hit[slot] = make_int2(-1, __float_as_int(INFINITY));
         }
     }
-    // a warp shares one scene (slots of one tile are one job); mixed warps take the slow path
-    const uint32_t sid0 = __shfl_sync(0xffffffffu, sid, 0);
-    const bool uniform_scene = __all_sync(0xffffffffu, !valid || sid == sid0);
-    const SceneDev& sc = scenes[uniform_scene ? sid0 : sid];
+    const SceneDev& sc = scenes[0];
     const uint32_t* nodes = sc.nodes2;
     const float4* tris = sc.tris;
     unsigned long long dummy = 0;
-    if (!uniform_scene) { // rare: a warp straddling two jobs of different scenes
-        QueueSrc<kPlain> src(n, nullptr, slot_scene, ray_o, ray_d, queue, hit, blockIdx.x, gridDim.x);
-        trace_bvh2_warp<false, false, kSmemStack, false, false, false>(scenes, src, smem_stack, dummy, dummy);
-        return;
-    }
     constexpr int kSmemS = kSmemStack;
 #if CR_TRACE_LOCAL_STACK
     int lstack_all[kStackTotal];
@@ -988,10 +978,10 @@ void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
         return;
     }
     // the BVH4 and the BVH2's variants trace closest hits only
-    const bool variant = (a.bvh4 && !a.any_hit) ||
-                         (!a.any_hit && !a.counters && !a.wide &&
-                          ((a.two_phase && a.phase.state && a.queue && a.queue_count) || a.packet || a.speculative));
-    if (a.shadow && variant) launch_shadow(*a.shadow, st, lc);
+    const bool variants = !a.wide && !a.counters && !a.any_hit;
+    const bool two_phase = variants && a.two_phase && a.phase.state && a.queue && a.queue_count;
+    const bool packet = variants && a.packet && a.one_scene, speculative = variants && a.speculative;
+    if (a.shadow && ((a.bvh4 && !a.any_hit) || two_phase || packet || speculative)) launch_shadow(*a.shadow, st, lc);
     if (a.bvh4 && !a.any_hit) { // BVH4 kernel (trace_bvh4.cu)
         launch_trace_bvh4(a, st, lc);
         return;
@@ -1000,7 +990,7 @@ void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
         launch_bvh2<false, false, true, kSmemStack>(a, st, lc);
         return;
     }
-    if (a.two_phase && !a.wide && !a.counters && a.phase.state && a.queue && a.queue_count) {
+    if (two_phase) {
         const uint32_t grid = (a.n_max + block - 1) / block;
         const uint32_t nb = (a.n_max + 255) / 256;
         k_trace_bvh2_phase<<<grid, block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue, a.queue_count,
@@ -1015,14 +1005,14 @@ void launch_trace(const TraceArgs& a, cudaStream_t st, LaunchCount& lc) {
         lc.n += 5;
         return;
     }
-    if (a.packet && !a.wide && !a.counters) {
+    if (packet) {
         const uint32_t grid = (a.n_max + block - 1) / block;
-        k_trace_bvh2_packet<<<grid, block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue,
+        k_trace_bvh2_packet<<<grid, block, smem, st>>>(a.scenes, a.ray_o, a.ray_d, a.queue,
                                                        a.queue_count, a.n_max, a.hit);
         lc.n++;
         return;
     }
-    if (a.speculative && !a.wide && !a.counters) {
+    if (speculative) {
         const uint32_t grid = (a.n_max + block - 1) / block;
         k_trace_bvh2_spec<<<grid, block, smem, st>>>(a.scenes, a.slot_scene, a.ray_o, a.ray_d, a.queue, a.queue_count,
                                                      a.n_max, a.hit);
