@@ -618,7 +618,8 @@ def run_ours(args):
 def trace_bytes_per_ray(nodes_per_ray: float, tris_per_ray: float, node_bytes: int = 64) -> float:
     """Algorithmic bytes one secondary ray moves through the trace kernel: its ray record
     (32 B), the queue entry (4 B) and the hit (8 B), every node visited (node_bytes: 32 for a
-    BVH2 record, 80 for BVH8-Q, 112 for BVH4) and every triangle tested (48 B)."""
+    BVH2 record, 80 for BVH8-Q, 112 for BVH4; the default is the exact 64-byte BVH2 node) and
+    every triangle tested (48 B)."""
     return 32 + 4 + 8 + node_bytes * nodes_per_ray + 48 * tris_per_ray
 
 

@@ -493,8 +493,8 @@ cr_status cr_debug_bvh_check(const float* tri_xyz, uint32_t n_tri, uint32_t flag
 /* ---------------------------------------------------------------------------------- */
 /* Tracing without allocation.  The paper has no counterpart: this is a library service.
  *
- * cr_trace_rays allocates device staging buffers on every call.  Some callers cannot allow
- * that: a host framework that owns all device memory through its own pool allocator and
+ * cr_trace_rays allocates device staging buffers for host arrays, and for hit arrays that
+ * overlap the rays.  Some callers need a call that never allocates: a host framework that owns all device memory through its own pool allocator and
  * forbids raw cudaMalloc, a latency-critical loop that cannot afford the device-wide
  * synchronisation of cudaMalloc/cudaFree, or a process that has reserved nearly all device
  * memory, so an allocation could fail mid-frame.  cr_trace_rays_static computes exactly

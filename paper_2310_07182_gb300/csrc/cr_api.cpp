@@ -723,7 +723,7 @@ JobDev job_dev(const cr_job& j, const PlanOpts& po, uint32_t scene_idx, uint32_t
 }
 
 // Slots up to which samples of a plan's jobs share a pass (1.6 GB of path state with light samples).  A
-// trace launch costs about 90 us beyond its rays at full rate (the device fills, then drains to the
+// trace launch costs about 80 us beyond its rays at full rate (the device fills, then drains to the
 // longest rays).  1280x720, 16 samples, 4 bounces, light samples: 48.2 ms with a pass per sample,
 // 42.1 / 38.9 / 37.3 with 2^21 / 2^22 / 2^23 slots; 853x479 with 4 samples through the BVH8-Q: 7.42 ms,
 // 5.58 with 2^21 or more; 500x333 with 4 samples and 8 bounces: 1.92 ms, 0.82 from 2^20 on;
@@ -1310,8 +1310,8 @@ extern "C" cr_status cr_trace_rays(cr_scene* s, const float* rays, const int32_t
     ta.scenes = dev_scene_entry(s, use8);
     ta.slot_scene = nullptr;
     ta.one_scene = true;
-    // four work words of the scene: the rays taken (more rays than resident lanes only), then the
-    // counts of a counting pass
+    // eight work words of the scene: from word 0 the rays taken (more rays than resident lanes only), from
+    // word 4 the counts of a counting pass
     const bool count = (o.flags & CR_OPT_COUNT) != 0;
     if (count || n > kTraceWorkMin) {
         CR_CUDA(cudaMemsetAsync(s->d_work, 0, 32, stream));

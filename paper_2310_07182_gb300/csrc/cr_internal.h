@@ -287,7 +287,7 @@ struct TraceArgs {
     const uint16_t* slot_scene = nullptr; // per-slot scene index (NULL: scene 0)
     unsigned long long* counters = nullptr; // [0] node visits, [1] triangle tests (counting pass)
     // device counter, zero before the launch: warps of a resident grid take further rays as
-    // theirs end (BVH2); NULL: one ray per lane
+    // theirs end (BVH2 and BVH8-Q); NULL: one ray per lane
     uint32_t* work = nullptr;
     bool one_scene = false; // every ray is in scenes[0]
     bool alone = true;      // no other launches of the library run beside this one

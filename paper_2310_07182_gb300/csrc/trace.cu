@@ -385,7 +385,9 @@ __device__ __forceinline__ void trace_bvh2_warp(const SceneDev* __restrict__ sce
 }
 
 #ifndef CR_TRACE_MAXNREG
-#define CR_TRACE_MAXNREG 56 // 36 warps resident per SM, no spills; 48 and 64 are within 1%, 40 costs 4%
+// 36 warps resident per SM; 48 and 64 are within 1%, 40 costs 4%.  Variants for one scene spill up to 32 bytes
+// per lane (44 where k_trace_both takes new rays), those for several 8 to 172.
+#define CR_TRACE_MAXNREG 56
 #endif
 
 template <bool kCount, bool kAny, int kSmemS, bool kOne, bool kWide, RangeKind kKind>

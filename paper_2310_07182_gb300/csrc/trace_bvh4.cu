@@ -2,8 +2,8 @@
 // collapsed from the BVH2 in bvh4_build.cpp), one ray per thread.
 //
 // A node visit loads the node's seven 16-byte words (the near and far plane words of each
-// axis picked by the ray's direction signs), tests the four child boxes with the BVH2
-// kernel's conservative slab test (unused slots have NaN planes and never pass), and
+// axis picked by the ray's direction signs), tests the four child boxes with a
+// conservative slab test (unused slots have NaN planes and never pass), and
 // orders the hit children by entry distance: the distance bits with the child slot in the
 // two low bits, sorted by a five-exchange network (the slot bits only reorder children whose
 // distances agree to 21 bits, which changes the visit order, never the closest hit).  The
@@ -24,9 +24,13 @@ namespace {
 #define CR_TRACE4_MAXNREG 64
 #endif
 
-// The slab test of box_hit_fma with the near and far planes chosen by the ray: three min /
-// max operations per box instead of nine.  Unused slots (NaN planes) still miss: the exit
-// distance is NaN and the comparison fails.
+constexpr float kFarWiden = 1.0f + 0x1.0p-21f;
+
+// One FMA per plane, near and far planes chosen by the ray.  Each plane distance fma(x, 1/d, offset)
+// differs from (x - o) * (1/d) by at most the rounding of o/d and of the offset (<= 2^-23 |o/d|) plus a
+// relative 2^-24; the offsets are moved apart by 2^-22 |o/d| (prep_ray) and the exit is widened by
+// 1 + 2^-21 > 1 + 2 gamma_3 (Ize 2013), so no box that the exact form would enter is rejected.  Unused
+// slots (NaN planes) miss: the exit distance is NaN and the comparison fails.
 __device__ __forceinline__ bool box_hit_nf(const RayPre& r, float nx, float fx, float ny, float fy, float nz, float fz,
                                            float onx, float ofx, float ony, float ofy, float onz, float ofz, float tcull,
                                            float& tn) {

@@ -4,9 +4,12 @@
 //
 // Closest-hit rule, identical for every kernel: accept t > 0 if t < t_best, or t == t_best
 // and the original triangle index is smaller.  Boxes are culled only if their entry distance
-// exceeds t_best (1 + 2^-16) and the slab exit is widened by (1 + 2^-21) > 1 + 2 gamma_3
-// (Ize 2013), so no box that holds a candidate triangle is ever skipped and every layout
-// returns the same hit bit for bit.
+// exceeds t_best (1 + 2^-16), and no slab test rejects a box that a ray enters:
+//   BVH2    records enlarged by kGridSlack, entry and exit offsets moved apart (grid_axis)
+//   BVH8-Q  entry and exit offsets of each node moved apart (trace_bvh8.cu)
+//   BVH4    offsets moved apart by 2^-22 |o / d|, the exit widened by 1 + 2^-21 (box_hit_nf)
+// so every layout returns the same hit bit for bit, up to triangles that a ray misses and the
+// triangle test accepts by rounding (behind() keeps out the ones that matter).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -20,7 +23,6 @@ namespace {
 
 constexpr int kSmemStack = 16;  // entries per thread in shared memory
 constexpr int kStackTotal = (int)kBvh2StackCapacity; // > BVH2 depth (checked at scene creation)
-constexpr float kFarWiden = 1.0f + 0x1.0p-21f;
 constexpr float kCullWiden = 1.0f + 0x1.0p-16f;
 
 struct RayPre {
@@ -31,7 +33,7 @@ struct RayPre {
     float dx, dy, dz;
     // slab offsets for t = fma(plane, 1/d, offset): -o/d biased outward by 2^-22 |o/d|, which
     // bounds the rounding of o/d and of the offset, so the FMA interval contains the one the
-    // exact (plane - o) / d form gives (see box_entry_fma)
+    // exact (plane - o) / d form gives (see box_hit_nf in trace_bvh4.cu)
     float lox, loy, loz, hix, hiy, hiz;
 };
 
@@ -185,42 +187,6 @@ __device__ __forceinline__ NodeTest node_test(const GridRay& g, const uint32_t* 
     r.c0 = (int)w6;
     r.c1 = (int)w7;
     return r;
-}
-
-// Slab test of one box; returns the entry distance, or +inf if the box is missed or culled.
-__device__ __forceinline__ float box_entry(const RayPre& r, float lox, float hix, float loy, float hiy, float loz,
-                                           float hiz, float tcull) {
-    const float tx0 = __fmul_rn(__fsub_rn(lox, r.ox), r.ix), tx1 = __fmul_rn(__fsub_rn(hix, r.ox), r.ix);
-    const float ty0 = __fmul_rn(__fsub_rn(loy, r.oy), r.iy), ty1 = __fmul_rn(__fsub_rn(hiy, r.oy), r.iy);
-    const float tz0 = __fmul_rn(__fsub_rn(loz, r.oz), r.iz), tz1 = __fmul_rn(__fsub_rn(hiz, r.oz), r.iz);
-    const float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.0f));
-    const float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fmaxf(tz0, tz1));
-    return (tn <= __fmul_rn(tf, kFarWiden) && tn <= tcull) ? tn : INFINITY;
-}
-
-// The same test with one FMA per plane.  Each plane distance fma(x, 1/d, offset) differs
-// from (x - o) * (1/d) by at most the rounding of o/d and of the offset (<= 2^-23 |o/d|) plus a
-// relative 2^-24; the offsets are pre-biased by 2^-22 |o/d| toward a larger interval and the
-// exit is widened by (1 + 2^-21), so no box that the exact form would enter is rejected.
-__device__ __forceinline__ float box_entry_fma(const RayPre& r, float lox, float hix, float loy, float hiy, float loz,
-                                               float hiz, float tcull) {
-    const float tx0 = fmaf(lox, r.ix, r.lox), tx1 = fmaf(hix, r.ix, r.hix);
-    const float ty0 = fmaf(loy, r.iy, r.loy), ty1 = fmaf(hiy, r.iy, r.hiy);
-    const float tz0 = fmaf(loz, r.iz, r.loz), tz1 = fmaf(hiz, r.iz, r.hiz);
-    const float tn = max3f(fminf(tx0, tx1), fminf(ty0, ty1), fmaxf(fminf(tz0, tz1), 0.0f));
-    const float tf = min3f(fmaxf(tx0, tx1), fmaxf(ty0, ty1), fmaxf(tz0, tz1));
-    return (tn <= __fmul_rn(tf, kFarWiden) && tn <= tcull) ? tn : INFINITY;
-}
-
-// box_entry_fma as a hit flag plus the entry distance (no +inf sentinel to test again).
-__device__ __forceinline__ bool box_hit_fma(const RayPre& r, float lox, float hix, float loy, float hiy, float loz,
-                                            float hiz, float tcull, float& tn) {
-    const float tx0 = fmaf(lox, r.ix, r.lox), tx1 = fmaf(hix, r.ix, r.hix);
-    const float ty0 = fmaf(loy, r.iy, r.loy), ty1 = fmaf(hiy, r.iy, r.hiy);
-    const float tz0 = fmaf(loz, r.iz, r.loz), tz1 = fmaf(hiz, r.iz, r.hiz);
-    tn = max3f(fminf(tx0, tx1), fminf(ty0, ty1), fmaxf(fminf(tz0, tz1), 0.0f));
-    const float tf = min3f(fmaxf(tx0, tx1), fmaxf(ty0, ty1), fmaxf(tz0, tz1));
-    return tn <= __fmul_rn(tf, kFarWiden) && tn <= tcull;
 }
 
 // Watertight ray/triangle test (Woop, Benthin, Wald 2013) without the double-precision
