@@ -41,6 +41,15 @@ def dist_info():
     return int(os.environ.get("RANK", 0)), int(os.environ.get("WORLD_SIZE", 1)), int(os.environ.get("LOCAL_RANK", 0))
 
 
+def emit(line: dict, legs: dict) -> None:
+    """The benchmark's JSON line on stdout; the legs' figures (precision, sweep, quality, batches,
+    serving: 15 KB and more) as one JSON line on stderr, so that the line stays short enough for
+    whoever keeps only the end of the output."""
+    if legs:
+        print(json.dumps({"legs": legs}), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
+
+
 def frame_of(rank: int, step: int, world: int) -> int:
     """Frame index rendered by ``rank`` at ``step``: ranks render disjoint frames."""
     return step * world + rank
@@ -599,7 +608,6 @@ def run_ours(args):
                                  "peak": peak, "unit": "GB/s", "frac": None if gbs is None else round(gbs / peak, 4),
                                  "share_of_step": round(rm["ms_sort"] / rm["ms_per_step"], 4),
                                  "timing": "stage events of 3 untimed steps (events between all stages)"}
-    line.update(extras)
     if not args.no_cpu_baseline and world == 1:  # the oracle's rate is a single-GPU context figure
         v, thr, sample, dt = cpu_oracle_rate(sc, args.cpu_seconds)
         line["cpu_baseline"] = {"value": round(v, 4), "unit": "Mrays/s", "cores": thr, "kind": "oracle",
@@ -611,8 +619,8 @@ def run_ours(args):
             for name, scn, b in (("tiny", scenes.tiny(), 1), ("interior", scenes.interior(), 4)):
                 v2, thr2, sample2, dt2 = cpu_oracle_rate(scn, 4.0, bounces=b)
                 extra[name] = {"mrays": round(v2, 4), "cores": thr2, "sample": sample2, "seconds": round(dt2, 2)}
-            line["cpu_baseline"]["other_workloads"] = extra
-    print(json.dumps(line), flush=True)
+            extras["cpu_other_workloads"] = extra
+    emit(line, extras)
 
 
 def trace_bytes_per_ray(nodes_per_ray: float, tris_per_ray: float, node_bytes: int = 64) -> float:
