@@ -388,6 +388,9 @@ extern "C" cr_status cr_scene_create(const float* tri_xyz, uint32_t n_tri, const
         s->d_work = reinterpret_cast<uint32_t*>(static_cast<char*>(de.p) + 2 * sizeof(SceneDev) + 16);
         de.p = nullptr;
     }
+    // copies from pageable memory may still be on their way when they return, and streams that do not wait
+    // for the legacy one read the scene next
+    CR_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     std::memset(&s->info, 0, sizeof(s->info));
     s->info.n_tri = n_tri;
     s->info.n_mat = n_mat;

@@ -455,8 +455,10 @@ bool cr_server::iterate(Lane& L, LaunchCount& lc) {
     }
     cudaEventRecord(L.ev_copied[set], L.copy_stream);
     cudaStreamWaitEvent(L.stream, L.ev_copied[set], 0);
-    if (upload_scenes) // append-only: entries in-flight iterations read do not change
+    if (upload_scenes) { // append-only: entries in-flight iterations read do not change
         cudaMemcpy(d_scenes, scene_tab.data(), sizeof(SceneDev) * scene_tab.size(), cudaMemcpyHostToDevice);
+        cudaStreamSynchronize(cudaStreamLegacy); // the copy from pageable memory may still be on its way
+    }
     PassArgs P;
     P.jobs = L.d_table[set];
     P.n_jobs = max_run + 1;
@@ -742,7 +744,7 @@ extern "C" cr_status cr_server_submit(cr_server* s, const cr_job* job, uint64_t*
     j.ray_steps = (uint64_t)j.npx * job->spp * (job->max_bounces + 1ull);
     std::lock_guard<std::mutex> lk(s->mu);
     if (s->fatal != CR_OK) {
-        set_last_error("cr_server_submit: the server stopped after a device error");
+        set_last_error(("cr_server_submit: the server stopped after a device error: " + s->fatal_msg).c_str());
         return s->fatal;
     }
     if (j.tiles > s->lanes[0].tiles_cap || j.npx > s->arena_px || (j.host_out && j.npx > s->staging_px)) {

@@ -59,3 +59,14 @@ def test_shared_memory_beyond_48_kb_is_allowed_before_occupancy_is_asked():
     body = s[s.index("static uint32_t resident_blocks("):]
     body = body[:body.index("\n}\n")]
     assert 0 < body.find("allow_smem<kKernel>(smem)") < body.index("cudaOccupancyMaxActiveBlocksPerMultiprocessor")
+
+
+def test_uploads_from_pageable_memory_are_waited_for():
+    """cudaMemcpy from pageable memory may return before the data has arrived, and the render streams do not
+    wait for the legacy stream that it runs on: a wait follows the scene's uploads and the server's table."""
+    s = SRC["cr_api.cpp"]
+    create = s[s.index("cr_status cr_scene_create("):s.index("static void free_workspace(")]
+    assert create.rindex("cudaStreamSynchronize(cudaStreamLegacy)") > create.rindex("cudaMemcpyHostToDevice")
+    t = SRC["server.cpp"]
+    for i in [m.end() for m in re.finditer(r"cudaMemcpy\(", t)]:
+        assert "cudaStreamSynchronize(cudaStreamLegacy)" in t[i:i + 250]
