@@ -674,6 +674,7 @@ extern "C" cr_status cr_server_create(const cr_server_opts* o, cr_server** out) 
     if (e == cudaSuccess) e = cudaMalloc(&r->arena, 16ull * r->arena_px);
     if (e == cudaSuccess) e = cudaMalloc(&r->staging, 12ull * r->staging_px);
     if (e == cudaSuccess) e = cudaMalloc(&r->d_scenes, sizeof(SceneDev) * kMaxScenes);
+    if (e == cudaSuccess) e = cudaMemset(r->d_scenes, 0, sizeof(SceneDev) * kMaxScenes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_last_error("cr_server_create: device allocation failed");
@@ -685,6 +686,18 @@ extern "C" cr_status cr_server_create(const cr_server_opts* o, cr_server** out) 
         Workspace& ws = r->lanes[l].ws;
         st = ws.ensure(r->lanes[l].tiles_cap * m, 1);
         if (st == CR_OK) st = ws.ensure_nee(r->lanes[l].tiles_cap * m);
+        // all of it, and the job tables, not only the counters: a queue position that was never written then
+        // names slot 0 of job 0, not whatever the memory held
+        if (st == CR_OK) {
+            cudaError_t z = cudaMemset(ws.base, 0, ws.bytes);
+            for (uint32_t q = 0; q < kDepth && z == cudaSuccess; ++q)
+                z = cudaMemset(r->lanes[l].d_table[q], 0, sizeof(JobDev) * kMaxRuns);
+            if (z != cudaSuccess) {
+                cudaGetLastError();
+                set_last_error("cr_server_create: clearing the path state failed");
+                st = CR_ERR_CUDA;
+            }
+        }
         if (st == CR_OK && cudaMemset(ws.pb.counts, 0, 4 * kCountsWords) != cudaSuccess) {
             cudaGetLastError();
             set_last_error("cr_server_create: clearing the counters failed");

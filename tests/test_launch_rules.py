@@ -70,3 +70,13 @@ def test_uploads_from_pageable_memory_are_waited_for():
     t = SRC["server.cpp"]
     for i in [m.end() for m in re.finditer(r"cudaMemcpy\(", t)]:
         assert "cudaStreamSynchronize(cudaStreamLegacy)" in t[i:i + 250]
+
+
+def test_the_server_clears_its_path_state():
+    """A queue position that was reserved but not written must not hold uninitialised memory: it is used as
+    an index.  The lanes' state, job tables and the scene table are cleared before the first iteration."""
+    s = SRC["server.cpp"]
+    body = s[s.index("cr_status cr_server_create("):s.index("r->loop()")]
+    wait = body.index("cudaStreamSynchronize(cudaStreamLegacy)")
+    for clear in ("cudaMemset(ws.base, 0, ws.bytes)", "cudaMemset(r->lanes[l].d_table[q], 0,", "cudaMemset(r->d_scenes, 0,"):
+        assert 0 < body.index(clear) < wait
